@@ -17,7 +17,7 @@ er1k, the 2048-instance batched workload and serving are the other lines.
 Roofline of the walker: `frac` = DRAM bytes per launch (ncu, read + write,
 per draw on a block-sampled capture of the same kernel source and launch
 shape, times this launch's draws) / walker CUDA-event time / measured copy
-peak.  Beside it, the 32-byte sectors the layout's searches read (counted
+peak.  Beside it, the 32-byte sectors the layout's draws read (counted
 by a statistics launch) and the flat-CSR bisection model of the same draws.
 
 --impl reference times the CPU oracle (single-threaded C) on a bounded sample
@@ -48,10 +48,10 @@ WORKLOADS = {
                    desc="R-MAT scale 20, 16.8M edges (a=.57 b=.19 c=.19), Zipf(1.5) w in [1,1000], 5% dangling"),
     "er1k": dict(alpha=0.15, R=1000, seed=1, topk=32, segments=False,
                  desc="Erdos-Renyi n=1000 m=10000, w U[1,10], dense n x n counts"),
-    "rmat24": dict(alpha=0.15, R=50, seed=1, topk=64, segments=True, launch=dict(refill_lanes=16, step_loads=6),
+    "rmat24": dict(alpha=0.15, R=50, seed=1, topk=64, segments=True,
                    desc="R-MAT scale 24, 268M edges + hub > 1e6, Zipf(1.5) w in [1,1000], 5% dangling, "
                         "depth-3 segments for out-degree <= 8"),
-    "rmat24plain": dict(alpha=0.15, R=50, seed=1, topk=64, segments=False, launch=dict(refill_lanes=16, step_loads=6),
+    "rmat24plain": dict(alpha=0.15, R=50, seed=1, topk=64, segments=False,
                         desc="R-MAT scale 24 as rmat24, plain steps only"),
     "rmat20alias": dict(alpha=0.2, R=100, seed=1, topk=32, segments=False, sampler=1,
                         desc="R-MAT scale 20 as rmat20, integer alias sampler (Algorithm 1 tables built every step)"),
@@ -256,9 +256,9 @@ def walker_roofline(workload, launch, sampled, draws, sectors, model_sectors, ke
            "kernel_ms": kernel_ms, "draws": draws,
            "counted_sector_frac": counted / s / 1e9 / peak,
            "counted": {"bytes_per_launch": counted, "sectors_per_draw": sectors / max(draws, 1),
-                       "model": "32-byte sectors the walker's own layout reads per draw: node record, one per "
-                                "search-tree level below the record, 1-2 sectors of the bottom block (alias: "
-                                "node record + slot), counted by a statistics launch"},
+                       "model": "32-byte sectors the walker's own layout reads per draw: one guide slot, and one "
+                                "sector of edge records where the slot's range overflows (alias: node record + "
+                                "slot), counted by a statistics launch"},
            "flat_csr_model": {"bytes_per_launch": model, "sectors_per_draw": model_sectors / max(draws, 1),
                               "frac": model / s / 1e9 / peak,
                               "model": "the same draws on a flat CSR searched by bisection without reuse: row_ptr "

@@ -66,11 +66,12 @@ enum {
 /* flags */
 #define PPR_PTRS_DEVICE 0x1u /* pointer arguments are device pointers */
 /* Node numbering of the device layout (ppr_load_graph; plain graphs only).
- * With PPR_RENUMBER the layout numbers nodes by descending in-degree (counted
- * on every fourth edge, eight classes per power of two, ties in caller
- * order) so that the records and rows of the most visited nodes are
- * contiguous; PPR_KEEP_IDS keeps the caller's order; with neither, the
- * layout renumbers when its node records (32 bytes a node) exceed twice the
+ * The layout numbers nodes by the length class of their rows.  With
+ * PPR_RENUMBER the nodes of a class follow in descending in-degree order
+ * (counted on every fourth edge, two steps per power of two, ties in caller
+ * order), so that the rows of the most visited nodes are contiguous;
+ * PPR_KEEP_IDS keeps the caller's order within a class; with neither, the
+ * layout takes the in-degree order when 32 bytes a node exceed twice the
  * device's L2.  The numbering is internal:
  * sources, rows and top-k use the caller's ids, walks draw by the caller's
  * source id, and every result is the same either way. */
@@ -129,10 +130,12 @@ int ppr_device_sms(const ppr_ctx *ctx);
 
 /*
  * Loads a weighted directed graph G = (V, E, w), w(e) > 0 (Sec. 2.1), in CSR
- * form and builds its device layout: node records (32 bytes, with the top
- * level of the row's search tree, when every row total is below 2^32; else
- * 16 bytes) and per-row inclusive 64-bit weight prefix sums (stored as
- * 32-bit values when every row total is below 2^32), built by device kernels.
+ * form and builds its device layout with device kernels: per-row inclusive
+ * 64-bit weight prefix sums (stored as 32-bit values when every row total is
+ * below 2^32) and guide slots, 32 bytes per range of the draw's random bits
+ * with the edges that meet the range, so that a draw reads one slot (23 to 45
+ * bytes an edge in all; fewer when the slots would take more than an eighth
+ * of the device).
  *   n        number of nodes, 1 <= n <= PPR_MAX_NODES
  *   m        number of edges, 0 <= m <= PPR_MAX_EDGES
  *   row_ptr  int64[n+1], row_ptr[0] = 0, non-decreasing, row_ptr[n] = m
@@ -198,8 +201,8 @@ typedef struct {
     int32_t topk;        /* 0..PPR_MAX_R: per-source top-k (count desc, end id asc) kept with the
                             rows; entries past the row's distinct endpoints are (-1, 0) */
     int32_t kernel;      /* PPR_KERNEL_PERSISTENT or PPR_KERNEL_PLAIN */
-    int32_t large_degree;/* out-degree above which the whole warp searches a lane's row
-                            cooperatively (persistent kernel); 0 = never (default) */
+    int32_t large_degree;/* >= 0; kept for callers that set it: a draw reads one slot of its row
+                            whatever the degree, so there is no search to share */
     int32_t warps_per_block;  /* persistent kernel: 4 or 8 warps per CTA (0 = 8) */
     int32_t chunk_sources;    /* sources per queue item, 0 = default */
     int64_t max_batch_sources;/* sources per device batch, 0 = sized to free device memory */
@@ -211,7 +214,8 @@ typedef struct {
                             its alias.  Same law, different counts.  Alias tables are built on
                             the first run that asks for them (every row total < 2^32; no
                             segment mode) */
-    int32_t l2_persist;  /* 1: walker launches mark the node records persisting in L2 (an
+    int32_t l2_persist;  /* 1: walker launches mark the front of the walked layout (guide slots,
+                            or the alias node records) persisting in L2 (an
                             access-policy window; the device's persisting set-aside is raised
                             for this context on first use); 0: off.  Results are unchanged */
     int32_t refill_lanes;/* persistent kernel: a warp starts new walks once at least this many of
@@ -220,13 +224,8 @@ typedef struct {
                             walk, so the first steps of a source's walks share their loads.
                             Results are unchanged */
     void *stream;        /* cudaStream_t, NULL = legacy default stream */
-    int32_t step_loads;  /* persistent kernel, prefix sampler on 32-bit rows, no cooperative
-                            search, no statistics: the dependent loads one lane may spend on a
-                            draw in one warp iteration (the node record counts as one); a
-                            deeper search resumes in the next iteration while the warp's other
-                            lanes start new draws.  0 = the library's choice (6); -1 = none
-                            (each iteration finishes every lane's draw); 2..16.  Results are
-                            unchanged */
+    int32_t step_loads;  /* -1, 0 or 2..16; kept for callers that set it: an iteration of the
+                            persistent kernel costs every lane one load */
 } ppr_run_args;
 
 /* Fills *args with defaults (alpha 0.15, R 100, seed 1, all sources of
@@ -271,7 +270,7 @@ int ppr_run_into(ppr_ctx *ctx, const ppr_graph *g, const ppr_run_args *args, voi
 /* Launch tuning chosen by ppr_autotune. */
 typedef struct {
     int32_t chunk_sources;   /* sources per work-queue item */
-    int32_t large_degree;    /* cooperative-search threshold (0 = off) */
+    int32_t large_degree;    /* 0 */
     int32_t warps_per_block; /* walkers per CTA / 32 (4 or 8) */
     float ms;                /* device time of the best candidate on the sample */
     int32_t candidates;      /* candidates timed */
@@ -283,9 +282,9 @@ typedef struct {
  * Times the persistent walker on a sample of the run's sources (at most
  * sample_sources, 0 = 65536; evenly strided for plain graphs, a leading range
  * for batched graphs) for each candidate of walkers per CTA (128, 256), queue
- * chunk (1/4x .. 4x of 400/R sources) and cooperative threshold (off, 4096,
- * 65536), then, with the fastest of those, for refill thresholds of 8, 16,
- * 24 and 32 idle lanes (against 1), and returns the fastest.  Synchronous;
+ * chunk (1/4x .. 4x of 400/R sources), then, with the fastest of those, for
+ * refill thresholds of 8, 16, 24 and 32 idle lanes (against 1), and returns
+ * the fastest.  Synchronous;
  * allocates scratch for the sample.  Tuning never changes results.
  */
 int ppr_autotune(ppr_ctx *ctx, const ppr_graph *g, const ppr_run_args *args, int64_t sample_sources, ppr_tuning *best);

@@ -18,22 +18,27 @@ struct AggOut {
     int32_t topk;
 };
 
-// Caller id of an endpoint the walker wrote in the layout's numbering
-// (order: the renumbered layout's order array, else null).
-__device__ __forceinline__ uint32_t caller_id(const int32_t *order, uint32_t v)
-{
-    return order ? (uint32_t)order[v] : v;
-}
+// Caller id of an endpoint the walker wrote as a node code: the layout's order
+// array and the first seq of each class-table entry (shared memory), or
+// neither where the endpoints are caller ids already.
+struct CallerIds {
+    const int32_t *order = nullptr;
+    const uint32_t *first = nullptr;
+    __device__ __forceinline__ uint32_t operator()(uint32_t v) const
+    {
+        return order ? (uint32_t)__ldg(order + (first[v >> kIdxBits] + (v & kIdxMask))) : v;
+    }
+};
 
 // ends: the R endpoints of one source (shared memory).  sortbuf: next_pow2(R)
 // uint32 and keys: next_pow2(R) uint64 of per-warp shared scratch.  Writes
 // row `out_row` of the outputs.  All 32 lanes call it.
 __device__ inline void aggregate_source(const uint32_t *ends, uint32_t R, uint32_t *sortbuf, uint64_t *keys,
-                                        const AggOut &o, uint64_t out_row, const int32_t *order = nullptr)
+                                        const AggOut &o, uint64_t out_row, const CallerIds &ids = CallerIds())
 {
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t P2 = next_pow2(R);
-    for (uint32_t i = lane; i < P2; i += 32) sortbuf[i] = i < R ? caller_id(order, ends[i]) : 0xffffffffu;
+    for (uint32_t i = lane; i < P2; i += 32) sortbuf[i] = i < R ? ids(ends[i]) : 0xffffffffu;
     __syncwarp();
     warp_bitonic_sort(sortbuf, P2);
     // One run per distinct endpoint.  A run is found at its last element;
@@ -237,7 +242,7 @@ __device__ __forceinline__ bool topk_all_reg(const uint32_t (&kv)[E], uint32_t n
 // scratch: 3 * R uint32 of per-warp shared memory
 template <int E>
 __device__ inline void aggregate_source_reg(const uint32_t *ends, uint32_t R, uint32_t *scratch, const AggOut &o,
-                                            uint64_t out_row, const int32_t *order = nullptr)
+                                            uint64_t out_row, const CallerIds &ids = CallerIds())
 {
     const uint32_t lane = threadIdx.x & 31;
     uint32_t *start_pos = scratch, *run_id = scratch + R, *kbuf = scratch + 2 * R;
@@ -256,7 +261,7 @@ __device__ inline void aggregate_source_reg(const uint32_t *ends, uint32_t R, ui
 #pragma unroll
     for (int e = 0; e < E; ++e) same = same && ((uint32_t)e * 32 + lane >= R || v[e] == v0);
     if (__all_sync(0xffffffffu, same)) {
-        const int32_t id = (int32_t)caller_id(order, v0);
+        const int32_t id = (int32_t)ids(v0);
         if (lane == 0) {
             if (o.cols) {
                 o.cols[rbase] = id;
@@ -272,11 +277,9 @@ __device__ inline void aggregate_source_reg(const uint32_t *ends, uint32_t R, ui
         __syncwarp();
         return;
     }
-    if (order) {
 #pragma unroll
-        for (int e = 0; e < E; ++e)
-            if ((uint32_t)e * 32 + lane < R) v[e] = (uint32_t)order[v[e]];
-    }
+    for (int e = 0; e < E; ++e)
+        if ((uint32_t)e * 32 + lane < R) v[e] = ids(v[e]);
     warp_sort_reg<E>(v);
     uint32_t nrun = 0;
 #pragma unroll
@@ -355,7 +358,8 @@ struct AggParams {
     int64_t S;
     int64_t out_row0;   // output row of the first source
     AggOut out;
-    const int32_t *order;  // renumbered layout: caller id of an internal node, else null
+    const int32_t *order;  // caller id by seq
+    const ClassTab *tab;
 };
 
 // E > 0: register-resident reduction for next_pow2(R) = 32 * E; E = 0:
@@ -365,17 +369,21 @@ template <int E>
 __global__ void __launch_bounds__(128) k_aggregate(AggParams p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ uint32_t first[kTabEntries];
+    for (uint32_t i = threadIdx.x; i < kTabEntries; i += blockDim.x) first[i] = p.tab->e[i].first;
+    __syncthreads();
+    const CallerIds ids{p.order, first};
     const uint32_t wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     unsigned char *scratch = smem_raw + (size_t)wid * p.P2 * 12;
     const uint64_t S = (uint64_t)p.S;
     for (uint64_t i = (uint64_t)blockIdx.x * nw + wid; i < S; i += (uint64_t)gridDim.x * nw) {
         if constexpr (E > 0) {
             aggregate_source_reg<E>(p.ends + i * p.R, p.R, reinterpret_cast<uint32_t *>(scratch), p.out,
-                                    (uint64_t)p.out_row0 + i, p.order);
+                                    (uint64_t)p.out_row0 + i, ids);
         } else {
             uint64_t *keys = reinterpret_cast<uint64_t *>(scratch);
             aggregate_source(p.ends + i * p.R, p.R, reinterpret_cast<uint32_t *>(keys + p.P2), keys, p.out,
-                             (uint64_t)p.out_row0 + i, p.order);
+                             (uint64_t)p.out_row0 + i, ids);
         }
     }
 }
@@ -385,7 +393,7 @@ static int launch_aggregate_e(ppr_ctx *ctx, const AggParams &ap, cudaStream_t st
 {
     const int aw = 4;
     size_t smem = (size_t)aw * ap.P2 * 12;
-    if (smem > 48 * 1024)
+    if (smem + sizeof(uint32_t) * kTabEntries > 48 * 1024)  // with the kernel's own table
         PPR_CUDA(cudaFuncSetAttribute(k_aggregate<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int ablocks = (int)std::min<int64_t>((ap.S + aw - 1) / aw, (int64_t)ctx->sms * 16);
     if (ablocks < 1) ablocks = 1;

@@ -208,6 +208,11 @@ int ppr_create(int device, ppr_ctx **out)
     c->l2_window_max = (size_t)v;
     cudaDeviceGetAttribute(&v, cudaDevAttrL2CacheSize, device);
     c->l2_bytes = (size_t)v;
+    size_t free_b = 0;
+    if (cudaMemGetInfo(&free_b, &c->mem_bytes) != cudaSuccess) {
+        delete c;
+        return cuda_fail(cudaGetLastError(), "cudaMemGetInfo");
+    }
     ppr::preload_run_kernels();
     {
         cudaFuncAttributes fa;
@@ -271,7 +276,7 @@ static int load_common(ppr_ctx *ctx, int64_t n, int64_t m, const int64_t *row_pt
     g->n = n;
     g->m = m;
     g->stream = (cudaStream_t)stream;
-    // node records of 32 bytes: renumber when they would take more than twice the L2
+    // what the graph reports as renumbered: the flag, or 32 bytes a node taking more than twice the L2
     const bool renumber = g->instances == 0 && ((flags & PPR_RENUMBER) != 0 ||
                                                 ((flags & PPR_KEEP_IDS) == 0 && (uint64_t)n * 32 > 2 * ctx->l2_bytes));
     return build_graph(ctx, n, m, row_ptr, col, w, (flags & PPR_PTRS_DEVICE) != 0, renumber, (cudaStream_t)stream, g);
@@ -346,7 +351,7 @@ int ppr_graph_get_info(const ppr_graph *g, ppr_graph_info *info)
     info->device_bytes = g->device_bytes;
     info->segment_nodes = g->seg.nodes;
     info->segment_entries = g->seg.entries_n;
-    info->renumbered = g->order ? 1 : 0;
+    info->renumbered = g->renumbered ? 1 : 0;
     info->reserved = 0;
     return PPR_OK;
 }
@@ -358,14 +363,11 @@ void ppr_free_graph(ppr_graph *g)
         cudaSetDevice(g->ctx->device);
         cudaDeviceSynchronize();  // runs on any stream may still read the graph
     }
-    dev_free(g->node, g->stream);
-    dev_free(g->edges, g->stream);
-    dev_free(g->sum, g->stream);
-    dev_free(g->seg.node, g->stream);
-    dev_free(g->seg.entries, g->stream);
-    dev_free(g->d_node_off, g->stream);
-    dev_free(g->order, g->stream);
-    dev_free(g->rank, g->stream);
+    for (void *p : {(void *)g->node, (void *)g->edges, (void *)g->slots, (void *)g->single, (void *)g->tab,
+                    (void *)g->order, (void *)g->code_of, (void *)g->seg.tab, (void *)g->seg.slots,
+                    (void *)g->seg.single, (void *)g->seg.head, (void *)g->seg.entries, (void *)g->d_node_off})
+        dev_free(p, g->stream);
+    dev_free(g->alias.tab, g->stream);
     dev_free(g->alias.node, g->stream);
     dev_free(g->alias.slots, g->stream);
     cudaGetLastError();  // a failed free must not surface in a later call
@@ -469,14 +471,12 @@ int check_run(const ppr_graph *g, const ppr_run_args *a, int64_t count, bool lis
     plan->dangling = a->dangling;
     plan->segments = a->segments != 0;
     plan->kernel = a->kernel;
-    plan->large_degree = a->large_degree;
     plan->warps_per_block = a->warps_per_block;
     plan->chunk_sources = a->chunk_sources;
     plan->refill_lanes = a->refill_lanes;
     plan->stats = a->stats != 0;
     plan->sampler = a->sampler;
     plan->l2_persist = a->l2_persist == 1;
-    plan->step_loads = a->step_loads == 0 ? kDefaultStepLoads : (a->step_loads < 0 ? 0 : a->step_loads);
     return PPR_OK;
 }
 }  // namespace ppr
@@ -829,11 +829,11 @@ int ppr_run_into(ppr_ctx *ctx, const ppr_graph *g, const ppr_run_args *a, void *
         set_error("top-k outputs missing");
         return PPR_EINVAL;
     }
-    if (a->segments && !(g->seg.T == plan.T && g->seg.node)) {
+    if (a->segments && !(g->seg.T == plan.T && g->seg.tab)) {
         set_error("segment tables for this alpha are not built (a ppr_run with segments=1 builds them)");
         return PPR_ENOTSUP;
     }
-    if (a->sampler == 1 && !g->alias.node) {
+    if (a->sampler == 1 && !g->alias.tab) {
         set_error("alias tables are not built (a ppr_run with sampler=1 builds them)");
         return PPR_ENOTSUP;
     }
@@ -914,48 +914,44 @@ int ppr_autotune(ppr_ctx *ctx, const ppr_graph *g, const ppr_run_args *a, int64_
     }
     const int cs_base = std::max(1, (int)(400 / a->R));
     const int cs_cands[] = {std::max(1, cs_base / 4), std::max(1, cs_base / 2), cs_base, cs_base * 2, cs_base * 4};
-    const int lg_cands[] = {0, 4096, 65536};
     const int wpb_cands[] = {8, 4};
     ppr_tuning bt{};
     bt.ms = -1.f;
     int tried = 0;
     for (int wpb : wpb_cands)
-        for (int lg : lg_cands)
-            for (int cs : cs_cands) {
-                if ((uint64_t)cs * a->R > (1u << 20)) continue;
-                RunPlan pl = plan;
-                pl.kernel = PPR_KERNEL_PERSISTENT;
-                pl.stats = false;
-                pl.chunk_sources = cs;
-                pl.large_degree = lg;
-                pl.warps_per_block = wpb;
-                if (launch_workspace_bytes(g, pl, S) > ws_bytes) continue;
-                float ms_best = 1e30f;
-                for (int rep = 0; rep < 2; ++rep) {
-                    cudaMemsetAsync(o.counters, 0, 256, st);
-                    cudaEventRecord(e0, st);
-                    rc = launch_walks(ctx, g, pl, o, use_list ? 0 : a->src_begin, S, d_list, 0, ws, st, nullptr);
-                    cudaEventRecord(e1, st);
-                    if (rc) break;
-                    e = cudaEventSynchronize(e1);
-                    if (e != cudaSuccess) {
-                        rc = cuda_fail(e, "autotune run");
-                        break;
-                    }
-                    float ms = 0.f;
-                    cudaEventElapsedTime(&ms, e0, e1);
-                    if (rep > 0) ms_best = std::min(ms_best, ms);
-                }
+        for (int cs : cs_cands) {
+            if ((uint64_t)cs * a->R > (1u << 20)) continue;
+            RunPlan pl = plan;
+            pl.kernel = PPR_KERNEL_PERSISTENT;
+            pl.stats = false;
+            pl.chunk_sources = cs;
+            pl.warps_per_block = wpb;
+            if (launch_workspace_bytes(g, pl, S) > ws_bytes) continue;
+            float ms_best = 1e30f;
+            for (int rep = 0; rep < 2; ++rep) {
+                cudaMemsetAsync(o.counters, 0, 256, st);
+                cudaEventRecord(e0, st);
+                rc = launch_walks(ctx, g, pl, o, use_list ? 0 : a->src_begin, S, d_list, 0, ws, st, nullptr);
+                cudaEventRecord(e1, st);
                 if (rc) break;
-                ++tried;
-                if (bt.ms < 0 || ms_best < bt.ms) {
-                    bt.chunk_sources = cs;
-                    bt.large_degree = lg;
-                    bt.warps_per_block = wpb;
-                    bt.refill_lanes = plan.refill_lanes > 0 ? plan.refill_lanes : 1;
-                    bt.ms = ms_best;
+                e = cudaEventSynchronize(e1);
+                if (e != cudaSuccess) {
+                    rc = cuda_fail(e, "autotune run");
+                    break;
                 }
+                float ms = 0.f;
+                cudaEventElapsedTime(&ms, e0, e1);
+                if (rep > 0) ms_best = std::min(ms_best, ms);
             }
+            if (rc) break;
+            ++tried;
+            if (bt.ms < 0 || ms_best < bt.ms) {
+                bt.chunk_sources = cs;
+                bt.warps_per_block = wpb;
+                bt.refill_lanes = plan.refill_lanes > 0 ? plan.refill_lanes : 1;
+                bt.ms = ms_best;
+            }
+        }
     // refill thresholds with the fastest launch shape
     const int rf_cands[] = {8, 16, 24, 32};
     for (int rf : rf_cands) {
@@ -964,7 +960,6 @@ int ppr_autotune(ppr_ctx *ctx, const ppr_graph *g, const ppr_run_args *a, int64_
         pl.kernel = PPR_KERNEL_PERSISTENT;
         pl.stats = false;
         pl.chunk_sources = bt.chunk_sources;
-        pl.large_degree = bt.large_degree;
         pl.warps_per_block = bt.warps_per_block;
         pl.refill_lanes = rf;
         float ms_best = 1e30f;

@@ -1,5 +1,6 @@
-// graph.cu -- device construction of the walk layout (node records, per-row
-// inclusive weight prefixes) and of the depth-3 segment tables.
+// graph.cu -- device construction of the walk layout (edge records with
+// per-row inclusive weight prefixes, guide slots) and of the depth-3 segment
+// tables and the alias tables.
 //
 // Sec. 2.1 defines the routing probability r(s,t) = w(<s,t>) / sum_v w(<s,v>).
 // The step rule realises it exactly over integers with the row's inclusive
@@ -8,20 +9,12 @@
 // nodes, the distribution over short walk outcomes; here it is built with a
 // fixed depth of 3 in 2^62 fixed point, one warp per node.
 #include <cstdio>
+#include <type_traits>
 
 #include "ppr_host.h"
 #include "scan.cuh"
 
 namespace ppr {
-
-enum : uint32_t { kBadRowPtr = 1u, kBadCol = 2u, kBadWeight = 4u };
-
-struct BuildStats {
-    unsigned long long max_total;
-    unsigned long long max_degree;
-    unsigned long long dangling;
-    unsigned int status;
-};
 
 // Instance of global node u in a block-diagonal graph (node_off has count+1
 // entries); returns 0 for a plain graph.
@@ -36,764 +29,434 @@ __device__ __forceinline__ int32_t instance_of(const int64_t *node_off, int32_t 
     return lo;
 }
 
-// Wide layout (some row total >= 2^32), two passes.
-// Pass 1: one warp per row.  Validates the CSR, sums the row weights.
-__global__ void k_rows_pass1(int64_t n, int64_t m, const int64_t *row_ptr, const int32_t *col,
-                             const uint32_t *w, const int64_t *node_off, int32_t count, uint64_t *W,
-                             BuildStats *st)
+// ------------------------------------------------------------ edge records ----
+// Prefixes by edge, not by row: a scan of the weights that restarts at every
+// row start (the bits number_nodes set) gives each edge its inclusive prefix
+// P.  Every thread takes eight consecutive edges whatever the rows are, so a
+// hub of a million edges and a million rows of one edge cost the same, where
+// a build by rows needs a tier of kernels per row length and still waits for
+// the longest row of each.  Two reads of the weights (tile sums, then the
+// records), no tier lists, no host round trip between them.
+constexpr uint32_t kEdgeThreads = 512, kEdgeRun = 8;
+constexpr uint32_t kEdgeTile = kEdgeThreads * kEdgeRun;
+constexpr uint32_t kSelfCarry = 512;  // up to so many tiles each block adds up the tiles before it itself
+
+// Running sum since the last row start; bit 63: a row starts in the range.
+using Run = unsigned long long;
+constexpr Run kRowStart = 1ull << 63;
+__device__ __forceinline__ Run run_join(Run a, Run b) { return (b & kRowStart) ? b : a + b; }
+
+// Join of the runs of all threads before this one (threads in order); *total: of all.
+__device__ __forceinline__ Run block_runs(Run v, Run *s_warp, Run *total)
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t u = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < n; u += warps) {
-        int64_t a = row_ptr[u], b = row_ptr[u + 1];
-        bool bad = a < 0 || b < a || b > m || (u == 0 && a != 0) || (u == n - 1 && b != m);
-        if (bad) {
-            if (lane == 0) atomicOr(&st->status, kBadRowPtr);
-            if (lane == 0) W[u] = 0;
-            continue;
-        }
-        int64_t lo_id = 0, hi_id = n;
-        if (count > 0) {
-            int32_t g = instance_of(node_off, count, u);
-            lo_id = 0;
-            hi_id = node_off[g + 1] - node_off[g];
-        }
-        uint64_t sum = 0;
-        uint32_t flags = 0;
-        for (int64_t e = a + lane; e < b; e += 32) {
-            uint32_t we = w[e];
-            int64_t c = col[e];
-            if (we == 0) flags |= kBadWeight;
-            if (c < lo_id || c >= hi_id) flags |= kBadCol;
-            sum += we;
-        }
+    const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    Run x = v;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            sum += __shfl_xor_sync(0xffffffffu, sum, o);
-            flags |= __shfl_xor_sync(0xffffffffu, flags, o);
-        }
-        if (lane == 0) {
-            W[u] = sum;
-            if (flags) atomicOr(&st->status, flags);
-            atomicMax(&st->max_total, (unsigned long long)sum);
-            atomicMax(&st->max_degree, (unsigned long long)(b - a));
-            if (b == a) atomicAdd(&st->dangling, 1ull);
-        }
+    for (int o = 1; o < 32; o <<= 1) {
+        const Run y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= (uint32_t)o) x = run_join(y, x);
     }
-}
-
-// Pass 2: one warp per row.  Inclusive prefix of the row's weights (warp scan
-// over 32-edge chunks with a carry) into the edge records; the node record.
-template <bool WIDE>
-__global__ void k_rows_pass2(int64_t n, const int64_t *row_ptr, const int32_t *col, const uint32_t *w,
-                             const int64_t *node_off, int32_t count, const uint64_t *W, NodeRec *node,
-                             void *edges_v)
-{
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t u = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < n; u += warps) {
-        int64_t a = row_ptr[u], b = row_ptr[u + 1];
-        int64_t base_id = 0;
-        if (count > 0) base_id = node_off[instance_of(node_off, count, u)];
-        uint64_t carry = 0;
-        for (int64_t e0 = a; e0 < b; e0 += 32) {
-            int64_t e = e0 + lane;
-            uint64_t v = e < b ? (uint64_t)w[e] : 0ull;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                uint64_t y = __shfl_up_sync(0xffffffffu, v, o);
-                if (lane >= o) v += y;
-            }
-            uint64_t P = carry + v;
-            if (e < b) {
-                int32_t c = (int32_t)(col[e] + base_id);
-                if (WIDE) {
-                    EdgeW r;
-                    r.P = P;
-                    r.col = c;
-                    r.pad = 0;
-                    reinterpret_cast<EdgeW *>(edges_v)[e] = r;
-                } else {
-                    EdgeN r;
-                    r.P = (uint32_t)P;
-                    r.col = c;
-                    reinterpret_cast<EdgeN *>(edges_v)[e] = r;
-                }
-            }
-            carry += __shfl_sync(0xffffffffu, v, 31);
-        }
-        if (lane == 0) {
-            NodeRec r;
-            r.word0 = pack_word0((uint64_t)a, (uint32_t)(b - a), false);
-            // a single out-edge needs no draw-to-edge search: keep its target inline
-            r.total = (b - a == 1) ? (uint64_t)(uint32_t)(col[a] + base_id) : W[u];
-            node[u] = r;
-        }
-    }
-}
-
-// ----------------------------------------------------- single-pass build ----
-// The narrow (32-bit prefix) layout is built in one validating pass over the
-// input: k_layout checks row_ptr and sizes every blocked row; after the scan
-// of those sizes, k_build_small builds every row of at most 32 edges with one
-// thread, and queues longer rows for k_build_mid (one warp per row, up to
-// 1,024 edges) and k_build_big (one block per row, up to 8,192); longer rows
-// are cut into tiles.  The limits keep every row within a few passes of its
-// group, so no single long row leaves the GPU idle behind it.  A row total
-// >= 2^32 sets kWide and the graph is rebuilt in the wide layout.
-enum : uint32_t { kWide = 8u, kBigDegree = 16u };
-constexpr uint32_t kSmallRow = 32, kMidRow = 1024, kHugeRow = 8192;
-constexpr uint32_t kBuildTile = 8192;  // edges per tile block of a huge row (256 threads x 32)
-
-struct LayoutStats {
-    unsigned long long max_degree;
-    unsigned long long dangling;
-    unsigned int status;
-    unsigned int n_mid, n_big, n_huge;
-};
-
-__device__ __forceinline__ void block_stats(LayoutStats *st, uint32_t deg_max, uint32_t dang, uint32_t flags)
-{
-    __shared__ uint32_t s_max, s_dang, s_flags;
-    if (threadIdx.x == 0) {
-        s_max = 0;
-        s_dang = 0;
-        s_flags = 0;
+    Run before = __shfl_up_sync(0xffffffffu, x, 1);
+    if (lane == 0) before = 0;
+    if (lane == 31) s_warp[wid] = x;
+    __syncthreads();
+    Run carry = 0, all = 0;
+    for (uint32_t q = 0; q < nw; ++q) {
+        if (q == wid) carry = all;
+        all = run_join(all, s_warp[q]);
     }
     __syncthreads();
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        deg_max = max(deg_max, __shfl_xor_sync(0xffffffffu, deg_max, o));
-        dang += __shfl_xor_sync(0xffffffffu, dang, o);
-        flags |= __shfl_xor_sync(0xffffffffu, flags, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        atomicMax(&s_max, deg_max);
-        atomicAdd(&s_dang, dang);
-        atomicOr(&s_flags, flags);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        if (s_max) atomicMax(&st->max_degree, (unsigned long long)s_max);
-        if (s_dang) atomicAdd(&st->dangling, (unsigned long long)s_dang);
-        if (s_flags) atomicOr(&st->status, s_flags);
-    }
+    if (total) *total = all;
+    return run_join(carry, before);
 }
 
-// order: the caller's row of internal node u (renumbered layout), or null.
-// sizes: the row's records in the edge array (its blocks, and with
-// interleave its summary sectors before them); ssizes: its summary sectors.
-__global__ void __launch_bounds__(256) k_layout(int64_t n, int64_t m, const int64_t *row_ptr, const int32_t *order,
-                                                bool interleave, uint32_t *sizes, uint32_t *ssizes, LayoutStats *st,
-                                                uint2 *huge, uint32_t huge_cap)
-{
-    uint32_t dmax = 0, dang = 0, flags = 0;
-    for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n; u += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t o = order ? (int64_t)order[u] : u;
-        const int64_t a = row_ptr[o], b = row_ptr[o + 1];
-        const bool bad = a < 0 || b < a || b > m || (o == 0 && a != 0) || (o == n - 1 && b != m);
-        uint32_t sz = 0, ssz = 0;
-        if (bad) {
-            flags |= kBadRowPtr;
-        } else if (b - a > PPR_MAX_DEGREE) {
-            flags |= kBigDegree;
-        } else {
-            const uint32_t d = (uint32_t)(b - a);
-            dmax = max(dmax, d);
-            dang += d == 0;
-            ssz = d >= 2 ? summary_sectors(d) : 0u;
-            // split layout: every row's blocks start on 64 bytes (a full block is
-            // one 64-byte DRAM fetch); otherwise on 32 bytes after the summary
-            sz = interleave ? blocked_row_records(d) + 4 * ssz : (d <= 1 ? 0u : 8u * ceil_shift(d, 3));
-            if (d > kHugeRow) {  // a valid row_ptr has at most m / kHugeRow of them
-                const uint32_t k = atomicAdd(&st->n_huge, 1u);
-                if (k < huge_cap) huge[k] = make_uint2((uint32_t)u, d);
-            }
-        }
-        sizes[u] = sz;
-        ssizes[u] = ssz;
-    }
-    block_stats(st, dmax, dang, flags);
-}
-
-struct BuildArgs {
-    int64_t n;
-    const int64_t *row_ptr;
+struct EdgeArgs {
+    int64_t n, m;
     const int32_t *col;
     const uint32_t *w;
-    const int64_t *node_off;
+    const uint32_t *heads;
+    const int64_t *row_ptr;
+    const int64_t *node_off;  // batched graphs
     int32_t count;
-    const uint64_t *region;   // first record of each row's area in E
-    const uint64_t *sregion;  // first summary sector of each row in K, or null: summary at the start of the row's area
-    NodeRecN *node;
-    EdgeN *E;
-    uint32_t *K;              // the summary array (8 keys a sector)
+    const uint32_t *code_of;
+    Run *tile;                // per tile: its run, then (more than kSelfCarry tiles) the join of those before it
+    int64_t tiles;
+    void *edges;
     LayoutStats *st;
-    uint32_t *list;  // mid rows from the front, big rows from the back
-    const int32_t *order;  // renumbered layout: caller row of internal node u, else null
-    const int32_t *rank;   // renumbered layout: internal id of caller node v, else null
+    bool vec;                 // col and w are 16-byte aligned
 };
 
-// First block record (reg) and first summary sector (sreg) of row u of degree
-// d: separate arrays, or one area in E holding the summary, then the blocks.
-__device__ __forceinline__ void row_regions(const BuildArgs &A, int64_t u, uint32_t d, uint64_t &reg, uint64_t &sreg)
+__device__ __forceinline__ void load8(const uint32_t *p, int64_t e0, int64_t m, bool vec, uint32_t (&v)[kEdgeRun])
 {
-    if (A.sregion) {
-        reg = A.region[u];
-        sreg = A.sregion[u];
+    if (vec && e0 + kEdgeRun <= m) {
+        const uint4 a = __ldg(reinterpret_cast<const uint4 *>(p + e0)), b = __ldg(reinterpret_cast<const uint4 *>(p + e0) + 1);
+        v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w, v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
     } else {
-        sreg = A.region[u] / 4;  // areas start on a 32-byte sector
-        reg = A.region[u] + (d >= 2 ? 4ull * summary_sectors(d) : 0ull);
-    }
-}
-
-// Input row (caller numbering) of internal node u, and the internal id of a
-// target the caller numbered c (c already checked to lie in [0, n)).
-__device__ __forceinline__ int64_t in_row(const BuildArgs &A, int64_t u) { return A.order ? (int64_t)A.order[u] : u; }
-__device__ __forceinline__ int64_t map_col(const BuildArgs &A, int64_t c) { return A.rank ? (int64_t)A.rank[c] : c; }
-
-// u32 slot in the summary array of key i of level l of a blocked row (first
-// summary sector sreg, degree d, L levels; the top level comes first)
-__device__ __forceinline__ uint64_t key_slot(uint64_t sreg, uint32_t d, uint32_t L, uint32_t l, uint32_t i)
-{
-    uint32_t off = 0;
-    for (uint32_t q = L; q > l; --q) off += level_sectors(d, q);
-    return (sreg + off) * 8ull + i;
-}
-
-// Node record of a built row; a row whose top summary level fits the record
-// (root_in_record) gets that level's first four keys, read back from the
-// level the calling group has just written.
-__device__ __forceinline__ void write_node(const BuildArgs &A, int64_t u, uint64_t reg, uint64_t sreg, uint32_t d,
-                                           uint64_t W, uint32_t first_target)
-{
-    NodeRecN r;
-    r.word0 = pack_word0(reg, d, false);
-    // summary field: the first sector in the summary array (split layout), or
-    // the number of summary sectors before the blocks (see blocked_sum)
-    const uint64_t field = d <= 8 ? 0ull : (A.sregion ? sreg : (uint64_t)summary_sectors(d));
-    r.total = d == 1 ? (uint64_t)first_target : (d == 0 ? 0ull : pack_blocked_total(W, field, d));
-    const uint32_t L = d >= 2 ? tree_levels(d) : 0;
-    const bool root = root_in_record(d, L);
 #pragma unroll
-    for (uint32_t i = 0; i < 4; ++i) r.key[i] = root ? A.K[key_slot(sreg, d, L, L, i)] : 0xffffffffu;
-    A.node[u] = r;
-}
-
-__device__ __forceinline__ int64_t instance_base(const BuildArgs &A, int64_t u, int64_t &hi_id)
-{
-    if (A.count == 0) {
-        hi_id = A.n;
-        return 0;
-    }
-    const int32_t g = instance_of(A.node_off, A.count, u);
-    hi_id = A.node_off[g + 1] - A.node_off[g];
-    return A.node_off[g];
-}
-
-// summary levels 2..L from level 1 (already written), padding included;
-// the calling group (warp or block) strides over keys with `rank`/`size`
-__device__ void write_upper_levels(uint32_t *K, uint64_t sreg, uint32_t d, uint32_t L, uint32_t rank, uint32_t size,
-                                   bool block)
-{
-    for (uint32_t l = 2; l <= L; ++l) {
-        const uint32_t nl = ceil_shift(d, 3 * l), np = ceil_shift(d, 3 * (l - 1));
-        for (uint32_t i = rank; i < 8 * level_sectors(d, l); i += size) {
-            uint32_t kv = 0xffffffffu;
-            if (i < nl) kv = K[key_slot(sreg, d, L, l - 1, min(8 * i + 8, np) - 1)];
-            K[key_slot(sreg, d, L, l, i)] = kv;
-        }
-        if (block) __syncthreads();
-        else __syncwarp();
+        for (uint32_t i = 0; i < kEdgeRun; ++i) v[i] = e0 + i < m ? __ldg(p + e0 + i) : 0u;
     }
 }
 
-// Each thread of a row's group takes a run of kRun consecutive edges per pass:
-// its kRun loads are independent, so a pass costs one memory latency for
-// 32 * kRun (warp) or 512 * kRun (block) edges.
-constexpr uint32_t kRun = 4;
-
-struct EdgeRun {
-    uint32_t w[kRun];
-    int32_t c[kRun];
-    uint64_t sum;
-};
-
-// Loads edges [i0, i0 + kRun) of row (a, d); missing ones read as weight 0.
-__device__ __forceinline__ EdgeRun load_run(const BuildArgs &A, int64_t a, uint32_t d, uint32_t i0, int64_t hi_id,
-                                            uint32_t &flags)
+__device__ __forceinline__ uint32_t heads8(const EdgeArgs &A, int64_t e0)
 {
-    EdgeRun r;
-    r.sum = 0;
+    return e0 < A.m ? (A.heads[e0 >> 5] >> (e0 & 31)) & 0xffu : 0u;
+}
+
+__device__ __forceinline__ Run run8(const uint32_t (&w)[kEdgeRun], uint32_t hb)
+{
+    Run r = 0;
 #pragma unroll
-    for (uint32_t q = 0; q < kRun; ++q) {
-        const uint32_t i = i0 + q;
-        r.w[q] = 0;
-        r.c[q] = 0;
-        if (i < d) {
-            r.w[q] = A.w[a + i];
-            r.c[q] = A.col[a + i];
-        }
-    }
-#pragma unroll
-    for (uint32_t q = 0; q < kRun; ++q) {
-        if (i0 + q < d) {
-            if (r.w[q] == 0) flags |= kBadWeight;
-            if (r.c[q] < 0 || (int64_t)r.c[q] >= hi_id) flags |= kBadCol;
-            else if (A.rank) r.c[q] = A.rank[r.c[q]];
-        }
-        r.sum += r.w[q];
-    }
+    for (uint32_t i = 0; i < kEdgeRun; ++i) r = ((hb >> i) & 1u) ? (kRowStart | w[i]) : r + w[i];
     return r;
 }
 
-// Writes the run's records (P after each edge, target) from the exclusive
-// prefix P0, padding records past d included (a row's region is padded to a
-// multiple of 4 records, and i0 is a multiple of 4), and its level-1 keys.
-__device__ __forceinline__ void write_run(const BuildArgs &A, uint32_t *K, const EdgeRun &r, uint64_t P0, uint64_t sreg,
-                                          uint64_t eb, uint32_t d, uint32_t L, uint32_t i0, int64_t base_id)
+__global__ void __launch_bounds__(kEdgeThreads) k_edge_tiles(EdgeArgs A)
 {
-    if (i0 >= d) return;
-    uint32_t v[8];
-    uint64_t P = P0;
-#pragma unroll
-    for (uint32_t q = 0; q < kRun; ++q) {
-        const uint32_t i = i0 + q;
-        P += r.w[q];
-        const bool in = i < d;
-        v[2 * q] = in ? (uint32_t)P : 0xffffffffu;
-        v[2 * q + 1] = in ? (uint32_t)(r.c[q] + base_id) : 0u;
-        if (in && ((i & 7) == 7 || i == d - 1)) K[key_slot(sreg, d, L, 1, i >> 3)] = (uint32_t)P;
-    }
-    uint4 *dst = reinterpret_cast<uint4 *>(A.E + eb + i0);  // 32-byte aligned
-    dst[0] = make_uint4(v[0], v[1], v[2], v[3]);
-    dst[1] = make_uint4(v[4], v[5], v[6], v[7]);
+    __shared__ Run s_warp[kEdgeThreads / 32];
+    const int64_t e0 = ((int64_t)blockIdx.x * kEdgeThreads + threadIdx.x) * kEdgeRun;
+    uint32_t w[kEdgeRun];
+    load8(A.w, e0, A.m, A.vec, w);
+    Run total;
+    block_runs(run8(w, heads8(A, e0)), s_warp, &total);
+    if (threadIdx.x == 0) A.tile[blockIdx.x] = total;
 }
 
-__global__ void __launch_bounds__(256) k_build_small(BuildArgs A)
+__global__ void __launch_bounds__(1024) k_edge_carry(EdgeArgs A)
 {
-    uint32_t *K = A.K;
-    uint32_t flags = 0;
-    for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < A.n; u += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t o = in_row(A, u);
-        const int64_t a = A.row_ptr[o];
-        const uint32_t d = (uint32_t)(A.row_ptr[o + 1] - a);
-        if (d > kSmallRow) {
-            if (d <= kMidRow) A.list[atomicAdd(&A.st->n_mid, 1u)] = (uint32_t)u;
-            else if (d <= kHugeRow) A.list[A.n - 1 - atomicAdd(&A.st->n_big, 1u)] = (uint32_t)u;
-            continue;  // rows above kHugeRow: tile kernels
+    __shared__ Run s_warp[32];
+    Run carry = 0;
+    for (int64_t t0 = 0; t0 < A.tiles; t0 += 4 * 1024) {  // four consecutive tiles a thread
+        Run v[4], mine = 0, all;
+        const int64_t t = t0 + 4 * (int64_t)threadIdx.x;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            v[i] = t + i < A.tiles ? A.tile[t + i] : 0ull;
+            mine = run_join(mine, v[i]);
         }
-        int64_t hi_id;
-        const int64_t base_id = instance_base(A, u, hi_id);
-        uint64_t reg, sreg;
-        row_regions(A, u, d, reg, sreg);
-        const uint32_t L = tree_levels(d);  // 0 or 1 here
-        const uint64_t eb = reg;
-        uint64_t P = 0;
-        uint32_t first = 0;
-        for (uint32_t i = 0; i < d; ++i) {
-            const uint32_t wi = A.w[a + i];
-            int64_t c = A.col[a + i];
-            if (wi == 0) flags |= kBadWeight;
-            if (c < 0 || c >= hi_id) flags |= kBadCol;
-            else c = map_col(A, c);
-            P += wi;
-            if (i == 0) first = (uint32_t)(c + base_id);
-            if (d >= 2) {
-                EdgeN r;
-                r.P = (uint32_t)P;
-                r.col = (int32_t)(c + base_id);
-                A.E[eb + i] = r;
-                if (L > 0 && ((i & 7) == 7 || i == d - 1)) K[key_slot(sreg, d, L, 1, i >> 3)] = (uint32_t)P;
-            }
+        Run before = run_join(carry, block_runs(mine, s_warp, &all));
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (t + i < A.tiles) A.tile[t + i] = before;
+            before = run_join(before, v[i]);
         }
-        if (P >= (1ull << 32)) flags |= kWide;
-        if (d >= 2) {
-            for (uint32_t i = d; i < 4 * ceil_shift(d, 2); ++i) {
-                EdgeN r;
-                r.P = 0xffffffffu;
-                r.col = 0;
-                A.E[eb + i] = r;
-            }
-            if (L > 0)
-                for (uint32_t i = ceil_shift(d, 3); i < 8 * level_sectors(d, 1); ++i) K[key_slot(sreg, d, L, 1, i)] = 0xffffffffu;
-        }
-        write_node(A, u, reg, sreg, d, P, first);
+        carry = run_join(carry, all);
     }
-    block_stats(A.st, 0, 0, flags);
 }
 
-__global__ void __launch_bounds__(256) k_build_mid(BuildArgs A)
+template <bool WIDE>
+__global__ void __launch_bounds__(kEdgeThreads) k_edge_records(EdgeArgs A)
 {
-    uint32_t *K = A.K;
-    const uint32_t lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    uint32_t flags = 0;
-    const uint32_t nmid = A.st->n_mid;
-    for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < nmid; t += warps) {
-        const int64_t u = A.list[t];
-        const int64_t o = in_row(A, u);
-        const int64_t a = A.row_ptr[o];
-        const uint32_t d = (uint32_t)(A.row_ptr[o + 1] - a);
-        int64_t hi_id;
-        const int64_t base_id = instance_base(A, u, hi_id);
-        uint64_t reg, sreg;
-        row_regions(A, u, d, reg, sreg);
-        const uint32_t L = tree_levels(d);
-        const uint64_t eb = reg;
-        uint64_t carry = 0;
-        for (uint32_t e0 = 0; e0 < d; e0 += 32 * kRun) {
-            const uint32_t i0 = e0 + lane * kRun;
-            const EdgeRun r = load_run(A, a, d, i0, hi_id, flags);
-            uint64_t v = r.sum;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint64_t y = __shfl_up_sync(0xffffffffu, v, o);
-                if (lane >= o) v += y;
-            }
-            write_run(A, K, r, carry + v - r.sum, sreg, eb, d, L, i0, base_id);
-            carry += __shfl_sync(0xffffffffu, v, 31);
-        }
-        if (carry >= (1ull << 32)) flags |= kWide;
-        for (uint32_t i = ceil_shift(d, 3) + lane; i < 8 * level_sectors(d, 1); i += 32)
-            K[key_slot(sreg, d, L, 1, i)] = 0xffffffffu;
-        __syncwarp();
-        write_upper_levels(K, sreg, d, L, lane, 32, false);
-        if (lane == 0) write_node(A, u, reg, sreg, d, carry, 0);
-    }
-    block_stats(A.st, 0, 0, flags);
-}
-
-__global__ void __launch_bounds__(512) k_build_big(BuildArgs A)
-{
-    __shared__ uint64_t s_warp[16];
-    uint32_t *K = A.K;
-    const uint32_t tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
-    uint32_t flags = 0;
-    const uint32_t nbig = A.st->n_big;
-    for (uint32_t t = blockIdx.x; t < nbig; t += gridDim.x) {
-        const int64_t u = A.list[A.n - 1 - t];
-        const int64_t o = in_row(A, u);
-        const int64_t a = A.row_ptr[o];
-        const uint32_t d = (uint32_t)(A.row_ptr[o + 1] - a);
-        int64_t hi_id;
-        const int64_t base_id = instance_base(A, u, hi_id);
-        uint64_t reg, sreg;
-        row_regions(A, u, d, reg, sreg);
-        const uint32_t L = tree_levels(d);
-        const uint64_t eb = reg;
-        uint64_t carry = 0;
-        for (uint32_t e0 = 0; e0 < d; e0 += blockDim.x * kRun) {
-            const uint32_t i0 = e0 + tid * kRun;
-            const EdgeRun r = load_run(A, a, d, i0, hi_id, flags);
-            uint64_t v = r.sum;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint64_t y = __shfl_up_sync(0xffffffffu, v, o);
-                if (lane >= o) v += y;
-            }
-            if (lane == 31) s_warp[wid] = v;
-            __syncthreads();
-            uint64_t before = 0, chunk = 0;
-            for (uint32_t q = 0; q < nw; ++q) {
-                if (q < wid) before += s_warp[q];
-                chunk += s_warp[q];
-            }
-            write_run(A, K, r, carry + before + v - r.sum, sreg, eb, d, L, i0, base_id);
-            carry += chunk;
-            __syncthreads();
-        }
-        if (carry >= (1ull << 32)) flags |= kWide;
-        for (uint32_t i = ceil_shift(d, 3) + tid; i < 8 * level_sectors(d, 1); i += blockDim.x)
-            K[key_slot(sreg, d, L, 1, i)] = 0xffffffffu;
-        __syncthreads();
-        write_upper_levels(K, sreg, d, L, tid, blockDim.x, true);
-        if (tid == 0) write_node(A, u, reg, sreg, d, carry, 0);
-        __syncthreads();
-    }
-    // one status word per block
+    __shared__ Run s_warp[kEdgeThreads / 32];
     __shared__ uint32_t s_flags;
-    if (tid == 0) s_flags = 0;
-    __syncthreads();
+    if (threadIdx.x == 0) s_flags = 0;
+    const int64_t e0 = ((int64_t)blockIdx.x * kEdgeThreads + threadIdx.x) * kEdgeRun;
+    uint32_t w[kEdgeRun], c[kEdgeRun], flags = 0;
+    load8(A.w, e0, A.m, A.vec, w);
+    load8(reinterpret_cast<const uint32_t *>(A.col), e0, A.m, A.vec, c);
+    // targets to codes: eight independent loads in flight
+    int32_t g = 0;
+    int64_t g_end = A.m, base = 0, size = A.n;  // the instance of the edge at hand
+    if (A.count > 0 && e0 < A.m) {
+        int32_t lo = 0, hi = A.count;
+        while (hi - lo > 1) {  // last instance whose first edge is <= e0
+            const int32_t mid = (lo + hi) >> 1;
+            if (A.row_ptr[A.node_off[mid]] <= e0) lo = mid;
+            else hi = mid;
+        }
+        g = lo;
+        base = A.node_off[g];
+        size = A.node_off[g + 1] - base;
+        g_end = A.row_ptr[A.node_off[g + 1]];
+    }
+#pragma unroll
+    for (uint32_t i = 0; i < kEdgeRun; ++i) {
+        if (e0 + i < A.m) {
+            if (A.count > 0)
+                while (e0 + i >= g_end) {
+                    ++g;
+                    base = A.node_off[g];
+                    size = A.node_off[g + 1] - base;
+                    g_end = A.row_ptr[A.node_off[g + 1]];
+                }
+            if (w[i] == 0) flags |= kBadWeight;
+            if ((int64_t)(int32_t)c[i] < 0 || (int64_t)(int32_t)c[i] >= size) flags |= kBadCol, c[i] = 0;
+            else c[i] = __ldg(A.code_of + base + c[i]);
+        }
+    }
+    const uint32_t hb = heads8(A, e0);
+    Run before = block_runs(run8(w, hb), s_warp, nullptr);
+    Run carry;
+    if (A.tiles > kSelfCarry) {
+        carry = A.tile[blockIdx.x];
+    } else {  // the tiles before this one (up to one a thread)
+        const Run v = threadIdx.x < blockIdx.x ? A.tile[threadIdx.x] : 0ull;
+        block_runs(v, s_warp, &carry);
+    }
+    Run P = run_join(carry, before) & ~kRowStart;
+    uint64_t v[kEdgeRun];
+#pragma unroll
+    for (uint32_t i = 0; i < kEdgeRun; ++i) {
+        P = ((hb >> i) & 1u) ? (Run)w[i] : P + w[i];
+        v[i] = P;
+        if (!WIDE && P >= (1ull << 32)) flags |= kWide;
+    }
+    if (e0 < A.m) {  // (the array is padded to whole runs)
+        if constexpr (WIDE) {
+            Sector *dst = reinterpret_cast<Sector *>(static_cast<EdgeW *>(A.edges) + e0);
+#pragma unroll
+            for (uint32_t i = 0; i < kEdgeRun; i += 2)
+                st_sector(dst + i / 2, Sector{{(uint32_t)v[i], (uint32_t)(v[i] >> 32), c[i], 0u, (uint32_t)v[i + 1],
+                                               (uint32_t)(v[i + 1] >> 32), c[i + 1], 0u}});
+        } else {
+            Sector *dst = reinterpret_cast<Sector *>(static_cast<EdgeN *>(A.edges) + e0);
+#pragma unroll
+            for (uint32_t i = 0; i < kEdgeRun; i += 4)
+                st_sector(dst + i / 4, Sector{{(uint32_t)v[i], c[i], (uint32_t)v[i + 1], c[i + 1], (uint32_t)v[i + 2],
+                                               c[i + 2], (uint32_t)v[i + 3], c[i + 3]}});
+        }
+    }
     if (flags) atomicOr(&s_flags, flags);
     __syncthreads();
-    if (tid == 0 && s_flags) atomicOr(&A.st->status, s_flags);
+    if (threadIdx.x == 0 && s_flags) atomicOr(&A.st->status, s_flags);
 }
 
-// Rows above kHugeRow edges are built by tiles of kBuildTile edges, one block
-// each, so a hub row does not leave one block working while the GPU idles:
-// tile weight totals, a scan of each row's tiles, tile writes of the prefix
-// records and level-1 keys, then one block per row for the padding, the upper
-// summary levels and the node record.
-struct BuildTiles {
-    BuildArgs A;
-    const uint4 *rows;   // (node, degree, first tile, tiles)
-    const uint2 *tiles;  // (row index, first edge of the tile)
-    uint64_t *tile_sum;  // per tile: weight total, then its exclusive offset in the row
-    uint64_t *row_total; // per row: W
-    uint32_t nrows;
+// ------------------------------------------------------------ nodes, slots ----
+struct SlotArgs {
+    int64_t n;
+    const int64_t *row_ptr;
+    const uint32_t *code_of;
+    const ClassTab *tab;
+    NodeRec *node;
+    Sector *slots;
+    int64_t n_slots;
+    const LayoutStats *st;
 };
 
-__device__ __forceinline__ uint64_t block_sum_u64(uint64_t v, uint64_t *s)  // 256 threads
+// Node records by seq, and the targets of single-edge nodes.
+template <class E>
+__global__ void __launch_bounds__(256) k_nodes(SlotArgs A, E edges)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = v;
-    __syncthreads();
-    uint64_t t = 0;
-    for (int q = 0; q < 8; ++q) t += s[q];
-    __syncthreads();
-    return t;
-}
-
-__global__ void __launch_bounds__(256) k_build_tile_totals(BuildTiles T)
-{
-    __shared__ uint64_t s[8];
-    const BuildArgs &A = T.A;
-    const uint2 tl = T.tiles[blockIdx.x];
-    const uint4 rw = T.rows[tl.x];
-    const int64_t a = A.row_ptr[in_row(A, rw.x)];
-    int64_t hi_id;
-    instance_base(A, rw.x, hi_id);
-    const uint32_t end = min(tl.y + kBuildTile, rw.y);
-    const uint32_t lo = min(tl.y + threadIdx.x * 32, end), hi = min(lo + 32, end);
-    uint64_t sum = 0;
-    uint32_t flags = 0;
-    for (uint32_t i = lo; i < hi; ++i) {
-        const uint32_t wi = A.w[a + i];
-        const int64_t c = A.col[a + i];
-        if (wi == 0) flags |= kBadWeight;
-        if (c < 0 || c >= hi_id) flags |= kBadCol;
-        sum += wi;
+    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (v >= A.n) return;
+    const int64_t a = A.row_ptr[v];
+    const uint32_t d = (uint32_t)(A.row_ptr[v + 1] - a), code = A.code_of[v];
+    uint64_t total = 0;
+    if (d) {
+        const typename E::Rec last = edges.load(a + d - 1);
+        total = d == 1 ? (uint64_t)E::target(last) : E::key(last);
+        if (d == 1) reinterpret_cast<uint32_t *>(A.tab->e[code >> kIdxBits].addr)[code & kIdxMask] = E::target(last);
     }
-    if (flags) atomicOr(&A.st->status, flags);
-    const uint64_t t = block_sum_u64(sum, s);
-    if (threadIdx.x == 0) T.tile_sum[blockIdx.x] = t;
+    A.node[seq_of(*A.tab, code)] = NodeRec{pack_word0((uint64_t)a, d, false), total};
 }
 
-__global__ void k_build_tile_scan(BuildTiles T)
+// Index of the first edge of a row whose prefix exceeds x, among its n edges
+// from lo on (there is one).  P: uint32_t (narrow) or uint64_t.
+template <class E, class P>
+__device__ __forceinline__ uint32_t first_above(const typename E::Edge *row, uint32_t lo, uint32_t n, P x)
 {
-    const uint32_t r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (r >= T.nrows) return;
-    const uint32_t lane = threadIdx.x & 31;
-    const uint4 rw = T.rows[r];
-    uint64_t carry = 0;
-    for (uint32_t t0 = 0; t0 < rw.w; t0 += 32) {
-        const uint32_t t = t0 + lane;
-        uint64_t v = t < rw.w ? T.tile_sum[rw.z + t] : 0ull;
-        const uint64_t own = v;
+    while (n > 1) {
+        const uint32_t half = n >> 1;
+        const bool below = __ldg(&row[lo + half - 1].P) <= x;
+        lo += below ? half : 0u;
+        n = below ? n - half : half;
+    }
+    return lo;
+}
+
+// One slot a thread.  The class-major numbering makes the slot's row and
+// range plain arithmetic, neighbouring threads hold neighbouring ranges of a
+// row (their probes of P share sectors), and every slot is one 32-byte store.
+// Bound by issue: the searches' instructions, so the narrow layout computes in
+// 32 bits and the table entry is found once a block (R-MAT scale 24, 394 M
+// slots: 7.9 -> 7.2 ms).
+template <class E>
+__global__ void __launch_bounds__(256) k_slots(SlotArgs A, E edges)
+{
+    using P = typename std::conditional<E::kWide, uint64_t, uint32_t>::type;
+    __shared__ ClassTab tab;
+    __shared__ uint32_t s_entry;
+    // an input that failed its checks (weights of 0, totals beyond 32 bits)
+    // has no ascending prefixes to search; the host reports it
+    if (A.st->status) return;
+    if (threadIdx.x == 0) s_entry = 0;
+    for (uint32_t i = threadIdx.x; i < kTabEntries; i += blockDim.x) tab.e[i] = A.tab->e[i];
+    __syncthreads();
+    // the last entry whose slots start at or before the block's first
+    const uint64_t at0 = reinterpret_cast<uint64_t>(A.slots + (int64_t)blockIdx.x * blockDim.x);
+    if (threadIdx.x < kTabEntries && tab.e[threadIdx.x].kind < kKindSingle && tab.e[threadIdx.x].addr <= at0)
+        atomicMax(&s_entry, threadIdx.x);
+    __syncthreads();
+    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= A.n_slots) return;
+    const uint64_t at = reinterpret_cast<uint64_t>(A.slots + s);
+    uint32_t entry = s_entry;  // slot entries follow each other in the table
+    while (entry + 1 < kTabEntries && tab.e[entry + 1].kind < kKindSingle && tab.e[entry + 1].addr <= at) ++entry;
+    const TabEntry t = tab.e[entry];
+    const uint32_t c = t.kind, rel = (uint32_t)((at - t.addr) / sizeof(Sector));  // below 2^32: a device holds fewer slots
+    const uint32_t b = rel & ((1u << c) - 1);
+    const NodeRec r = A.node[t.first + (rel >> c)];
+    const typename E::Edge *row = edges.e + (r.word0 & kBeginMask);
+    const uint32_t d = (uint32_t)(r.word0 >> 40) & kCountMask;
+    const uint64_t W = r.total;
+    P X0, X1;  // the range's first x and its last: ceil((b + 1) W / 2^c) - 1
+    if constexpr (E::kWide) {
+        X0 = range_start(W, b, c);
+        X1 = range_start(W, b + 1, c) - (((W * (b + 1ull)) & ((1ull << c) - 1)) == 0);
+    } else {
+        const uint64_t lo = (uint64_t)(uint32_t)W * b, up = lo + (uint32_t)W;
+        X0 = (uint32_t)(lo >> c);
+        X1 = (uint32_t)(up >> c) - (((uint32_t)up & ((1u << c) - 1)) == 0);
+    }
+    const uint32_t lo = c ? first_above<E, P>(row, 0, d, X0) : 0u;
+    const uint32_t left = d - lo;  // edges from lo to the row's end
+    constexpr uint32_t kFit = E::kWide ? 3 : 4;
+    typename E::Rec rec[kFit];
+    uint32_t q = 0;  // edges that meet the range, 0 for more than fit
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint64_t y = __shfl_up_sync(0xffffffffu, v, o);
-            if (lane >= o) v += y;
+    for (uint32_t i = 0; i < kFit; ++i) rec[i] = __ldg(reinterpret_cast<const typename E::Rec *>(row) + lo + min(i, left - 1));
+#pragma unroll
+    for (uint32_t i = 0; i < kFit; ++i)
+        if (q == 0 && (P)E::key(rec[i]) > X1) q = i + 1;
+    const uint64_t e_lo = (r.word0 & kBeginMask) + lo;
+    Sector o;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) o.v[i] = 0;
+    o.v[0] = (uint32_t)W;
+    if constexpr (!E::kWide) {
+        if (q) {
+#pragma unroll
+            for (uint32_t i = 0; i < 3; ++i) o.v[1 + i] = i + 1 < q ? rec[i].x : 0xffffffffu;
+            uint32_t to = E::target(rec[0]);
+#pragma unroll
+            for (uint32_t i = 0; i < 4; ++i) {
+                if (i < q) to = E::target(rec[i]);
+                o.v[4 + i] = to;
+            }
+        } else {
+            const uint64_t e_hi = (r.word0 & kBeginMask) + first_above<E, P>(row, lo + kFit, left - kFit, X1), sec = e_lo >> 2;
+            const uint32_t nsec = (uint32_t)((e_hi >> 2) - sec + 1), gs = (nsec + kGroups - 1) / kGroups;
+            uint32_t k[kGroups - 1];
+#pragma unroll
+            for (uint32_t g = 0; g < kGroups - 1; ++g)
+                k[g] = (g + 1) * gs < nsec ? __ldg(&edges.e[4 * (sec + (uint64_t)(g + 1) * gs) - 1].P) : 0xffffffffu;
+            o.v[1] = k[0];
+            o.v[2] = k[1];
+            o.v[3] = k[2];
+            o.v[7] = k[3];
+            o.v[4] = kMarkOverflow | ((uint32_t)(e_lo & 3) << 8) | (uint32_t)(sec >> 32);
+            o.v[5] = (uint32_t)sec;
+            o.v[6] = nsec;
         }
-        if (t < rw.w) T.tile_sum[rw.z + t] = carry + v - own;
-        carry += __shfl_sync(0xffffffffu, v, 31);
-    }
-    if (lane == 0) {
-        T.row_total[r] = carry;
-        if (carry >= (1ull << 32)) atomicOr(&T.A.st->status, kWide);
-    }
-}
-
-__global__ void __launch_bounds__(256) k_build_tile_write(BuildTiles T)
-{
-    __shared__ uint64_t s[8];
-    const BuildArgs &A = T.A;
-    uint32_t *K = A.K;
-    const uint2 tl = T.tiles[blockIdx.x];
-    const uint4 rw = T.rows[tl.x];
-    const uint32_t d = rw.y;
-    const int64_t a = A.row_ptr[in_row(A, rw.x)];
-    int64_t hi_id;
-    const int64_t base_id = instance_base(A, rw.x, hi_id);
-    uint64_t reg, sreg;
-    row_regions(A, rw.x, d, reg, sreg);
-    const uint32_t L = tree_levels(d);
-    const uint64_t eb = reg;
-    const uint32_t end = min(tl.y + kBuildTile, d);
-    const uint32_t lo = min(tl.y + threadIdx.x * 32, end), hi = min(lo + 32, end);
-    uint64_t own = 0;
-    for (uint32_t i = lo; i < hi; ++i) own += A.w[a + i];
-    // exclusive offset of this thread's run within the tile
-    const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    uint64_t v = own;
+    } else {
+        o.v[1] = (uint32_t)(W >> 32);
+        if (q && X1 - X0 < (1ull << 32)) {
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint64_t y = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += y;
+            for (uint32_t i = 0; i < 2; ++i) o.v[2 + i] = i + 1 < q ? (uint32_t)(E::key(rec[i]) - X0) : 0xffffffffu;
+            uint32_t to = E::target(rec[0]);
+#pragma unroll
+            for (uint32_t i = 0; i < 3; ++i) {
+                if (i < q) to = E::target(rec[i]);
+                o.v[4 + i] = to;
+            }
+        } else {
+            const uint32_t hi = q ? lo + q - 1 : first_above<E, P>(row, lo + kFit, left - kFit, X1);
+            o.v[4] = kMarkOverflow;
+            o.v[5] = (uint32_t)e_lo;
+            o.v[6] = (uint32_t)(e_lo >> 32);
+            o.v[7] = hi - lo + 1;
+        }
     }
-    if (lane == 31) s[wid] = v;
-    __syncthreads();
-    uint64_t before = 0;
-    for (uint32_t q = 0; q < wid; ++q) before += s[q];
-    uint64_t P = T.tile_sum[blockIdx.x] + before + v - own;
-    for (uint32_t i = lo; i < hi; ++i) {
-        P += A.w[a + i];
-        const int64_t c = A.col[a + i];  // checked by k_build_tile_totals (the build fails if it is out of range)
-        EdgeN r;
-        r.P = (uint32_t)P;
-        r.col = (int32_t)((c >= 0 && c < hi_id ? map_col(A, c) : c) + base_id);
-        A.E[eb + i] = r;
-        if ((i & 7) == 7 || i == d - 1) K[key_slot(sreg, d, L, 1, i >> 3)] = (uint32_t)P;
-    }
+    st_sector(A.slots + s, o);
 }
 
-__global__ void __launch_bounds__(512) k_build_tile_finish(BuildTiles T)
-{
-    const BuildArgs &A = T.A;
-    uint32_t *K = A.K;
-    const uint4 rw = T.rows[blockIdx.x];
-    const uint32_t d = rw.y, tid = threadIdx.x;
-    uint64_t reg, sreg;
-    row_regions(A, rw.x, d, reg, sreg);
-    const uint32_t L = tree_levels(d);
-    const uint64_t eb = reg;
-    for (uint32_t i = d + tid; i < 4 * ceil_shift(d, 2); i += blockDim.x) {
-        EdgeN r;
-        r.P = 0xffffffffu;
-        r.col = 0;
-        A.E[eb + i] = r;
-    }
-    for (uint32_t i = ceil_shift(d, 3) + tid; i < 8 * level_sectors(d, 1); i += blockDim.x)
-        K[key_slot(sreg, d, L, 1, i)] = 0xffffffffu;
-    __syncthreads();
-    write_upper_levels(K, sreg, d, L, tid, blockDim.x, true);
-    if (tid == 0) write_node(A, rw.x, reg, sreg, d, T.row_total[blockIdx.x], 0);
-}
-
-// Narrow layout in one pass.  Returns PPR_OK, an error, or 1 when a row total
-// reaches 2^32 (the caller then builds the wide layout).
-static int build_narrow(ppr_ctx *ctx, int64_t n, int64_t m, const int64_t *d_rp, const int32_t *d_col,
+// The layout of CSR (d_rp, d_col, d_w).  Returns PPR_OK, an error, or 1 when
+// a row total reaches 2^32 and WIDE is false (the caller then builds the wide
+// layout).
+template <class E>
+static int build_layout(ppr_ctx *ctx, int64_t n, int64_t m, const int64_t *d_rp, const int32_t *d_col,
                         const uint32_t *d_w, const int64_t *d_off, cudaStream_t st, ppr_graph *g,
                         std::vector<void *> &tmp)
 {
     int rc;
-    uint32_t *d_sizes, *d_ssizes;
-    uint64_t *d_region, *d_sregion, *d_scan;
+    // Ranges per row: at most 2^lam_bits edges a range on average.  One edge a
+    // range makes overflow rare (5 % of the draws with Zipf weights, 11 % with
+    // two), two halve the slots (45 and 23 bytes an edge).  What decides is
+    // where the slots lie: within L2 the second load of an overflow costs
+    // more, far beyond it (16 times) every slot is a miss anyway and the
+    // overflow one more; in between the smaller slots hit L2 more often.
+    // Walker ms with one / two: R-MAT scale 16 .347 / .375, 18 1.22 / 1.29, 19
+    // 2.70 / 2.52, 20 6.12 / 5.82, 22 7.42 / 7.76 (2^20 sources), 24 86.2 /
+    // 91.5; Chung-Lu 2.4 M edges .724 / .777, 12 M 5.45 / 4.37.  A batch's
+    // instances are walked one after the other: the largest counts (256
+    // graphs: 17.6 / 19.0).  The wide layout's slot holds three edges, and
+    // its ranges one.  Slots that would take more than an eighth of the
+    // device (64 m >> lam_bits bytes at most) get longer ranges.
+    double share = 1.0;
+    if (g->instances > 0) {
+        int64_t largest = 0;
+        for (int32_t i = 0; i < g->instances; ++i) largest = std::max(largest, g->node_off[i + 1] - g->node_off[i]);
+        share = (double)largest / (double)n;
+    }
+    const double slot_bytes = 45.0 * (double)m * share, l2 = (double)ctx->l2_bytes;
+    g->lam_bits = !E::kWide && slot_bytes > 1.75 * l2 && slot_bytes < 16.0 * l2 ? 1 : 0;
+    while (g->lam_bits < 23 && (uint64_t)m * 64 >> g->lam_bits > ctx->mem_bytes / 8) ++g->lam_bits;
+    uint32_t *heads;
     LayoutStats *d_ls;
-    uint32_t *d_list;
-    const int64_t tiles = (n + kScanTile - 1) / kScanTile;
-    if ((rc = dev_alloc((void **)&d_sizes, sizeof(uint32_t) * n, "row sizes", st))) return rc;
-    tmp.push_back(d_sizes);
-    if ((rc = dev_alloc((void **)&d_region, sizeof(uint64_t) * (n + 1), "row regions", st))) return rc;
-    tmp.push_back(d_region);
-    if ((rc = dev_alloc((void **)&d_ssizes, sizeof(uint32_t) * n, "summary sizes", st))) return rc;
-    tmp.push_back(d_ssizes);
-    if ((rc = dev_alloc((void **)&d_sregion, sizeof(uint64_t) * (n + 1), "summary regions", st))) return rc;
-    tmp.push_back(d_sregion);
-    if ((rc = dev_alloc((void **)&d_scan, sizeof(uint64_t) * (tiles + 2), "scan scratch", st))) return rc;
-    tmp.push_back(d_scan);
+    const int64_t tiles = (m + kEdgeTile - 1) / kEdgeTile;
+    const size_t head_words = (size_t)(m / 32 + 1);
+    if ((rc = dev_alloc((void **)&heads, sizeof(uint32_t) * head_words, "row starts", st))) return rc;
+    tmp.push_back(heads);
     if ((rc = dev_alloc((void **)&d_ls, sizeof(LayoutStats), "layout stats", st))) return rc;
     tmp.push_back(d_ls);
-    if ((rc = dev_alloc((void **)&d_list, sizeof(uint32_t) * n, "long-row list", st))) return rc;
-    tmp.push_back(d_list);
-    const uint32_t huge_cap = (uint32_t)(m / kHugeRow + 1);
-    uint2 *d_huge;
-    if ((rc = dev_alloc((void **)&d_huge, sizeof(uint2) * huge_cap, "huge-row list", st))) return rc;
-    tmp.push_back(d_huge);
-    cudaError_t e = cudaMemsetAsync(d_ls, 0, sizeof(LayoutStats), st);
-    if (e != cudaSuccess) return cuda_fail(e, "memset");
-    const int tblocks = (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)ctx->sms * 16));
-    // Summary levels in an array of their own on a renumbered layout (graphs
-    // far larger than L2: the summaries every draw passes through then pack
-    // L2 lines instead of sharing them with blocks a draw reads once); at the
-    // start of each row's area, before its blocks, otherwise (the summary
-    // sector of a small row shares a DRAM page with its blocks).  The record's
-    // 28-bit summary offset bounds the shared area: 2 m + 4 n records cover
-    // every row's blocks and summary.
-    const bool interleave = g->order == nullptr && (uint64_t)(2 * m + 4 * n) / 4 < kSumSectorsMax;
-    k_layout<<<tblocks, 256, 0, st>>>(n, m, d_rp, g->order, interleave, d_sizes, d_ssizes, d_ls, d_huge, huge_cap);
-    note_launch();
-    exclusive_scan_u32(d_sizes, n, d_region, d_scan, st);
-    if (!interleave) exclusive_scan_u32(d_ssizes, n, d_sregion, d_scan, st);  // same scratch, in stream order
-    LayoutStats hs;
-    uint64_t slots = 0, sum_sectors = 0;
-    e = cudaMemcpyAsync(&hs, d_ls, sizeof(hs), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&slots, d_region + n, sizeof(uint64_t), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess && !interleave)
-        e = cudaMemcpyAsync(&sum_sectors, d_sregion + n, sizeof(uint64_t), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return cuda_fail(e, "graph layout");
-    if (hs.status & kBadRowPtr) {
-        set_error("row_ptr must start at 0, be non-decreasing and end at m");
-        return PPR_EINVAL;
+    Run *d_tile;
+    if ((rc = dev_alloc((void **)&d_tile, sizeof(Run) * (tiles > 0 ? tiles : 1), "weight sums", st))) return rc;
+    tmp.push_back(d_tile);
+    if ((rc = dev_alloc((void **)&g->order, sizeof(int32_t) * n, "node order", st)) ||
+        (rc = dev_alloc((void **)&g->code_of, sizeof(uint32_t) * n, "node codes", st)))
+        return rc;
+    PPR_CUDA(cudaMemsetAsync(heads, 0, sizeof(uint32_t) * head_words, st));
+    PPR_CUDA(cudaMemsetAsync(d_ls, 0, sizeof(LayoutStats), st));
+    if ((rc = number_nodes(n, m, d_rp, d_off, heads, d_ls, E::kWide, st, g, tmp))) return rc;
+    const size_t run = kEdgeRun * sizeof(typename E::Edge);
+    const size_t edge_bytes = (size_t)(tiles > 0 ? (m + kEdgeRun - 1) / kEdgeRun : 1) * run;
+    if ((rc = dev_alloc(&g->edges, edge_bytes, "edge records", st)) ||
+        (rc = dev_alloc((void **)&g->node, sizeof(NodeRec) * n, "node records", st)) ||
+        (rc = dev_alloc((void **)&g->slots, sizeof(Sector) * std::max<int64_t>(g->n_slots, 1), "guide slots", st)) ||
+        (rc = dev_alloc((void **)&g->single, sizeof(uint64_t) * (g->n_single / 2 + 1), "single targets", st)) ||
+        (rc = dev_alloc((void **)&g->tab, sizeof(ClassTab), "class table", st)))
+        return rc;
+    for (TabEntry &t : g->htab.e) {
+        if (t.kind < kKindSingle) t.addr += reinterpret_cast<uint64_t>(g->slots);
+        if (t.kind == kKindSingle) t.addr += reinterpret_cast<uint64_t>(g->single);
     }
-    if (hs.status & kBigDegree) {
-        set_error("an out-degree exceeds the limit %lld", (long long)PPR_MAX_DEGREE);
-        return PPR_ERANGE;
-    }
-    if (slots > kBeginMask) {
-        set_error("edge layout needs %llu record slots, beyond 2^40", (unsigned long long)slots);
-        return PPR_ERANGE;
-    }
-    if (sum_sectors >= kSumSectorsMax) {
-        set_error("the rows' search-tree summaries need %llu sectors, beyond 2^28", (unsigned long long)sum_sectors);
-        return PPR_ERANGE;
-    }
-    g->max_degree = (int64_t)hs.max_degree;
-    g->dangling = (int64_t)hs.dangling;
-    if ((rc = dev_alloc((void **)&g->node, sizeof(NodeRecN) * n, "node records", st))) return rc;
-    const size_t edge_bytes = (size_t)(slots > 0 ? slots : 2) * sizeof(EdgeN);
-    if ((rc = dev_alloc(&g->edges, edge_bytes, "edge records", st))) return rc;
-    g->edge_records = (int64_t)slots;
-    size_t sum_bytes = 0;
-    if (!interleave) {
-        sum_bytes = (size_t)(sum_sectors > 0 ? sum_sectors : 1) * 32;
-        if ((rc = dev_alloc((void **)&g->sum, sum_bytes, "row summaries", st))) return rc;
-        g->sum_sectors = (int64_t)sum_sectors;
-    }
-    g->device_bytes = (int64_t)(sizeof(NodeRecN) * n + edge_bytes + sum_bytes);
-    BuildArgs A{n, d_rp, d_col, d_w, d_off, g->instances, d_region, interleave ? nullptr : d_sregion,
-                static_cast<NodeRecN *>(g->node), (EdgeN *)g->edges,
-                interleave ? reinterpret_cast<uint32_t *>(g->edges) : g->sum, d_ls, d_list, g->order, g->rank};
-    k_build_small<<<tblocks, 256, 0, st>>>(A);
-    note_launch();
-    k_build_mid<<<ctx->sms * 8, 256, 0, st>>>(A);
-    note_launch();
-    k_build_big<<<ctx->sms * 3, 512, 0, st>>>(A);  // three resident 512-thread blocks per SM (39 registers)
-    note_launch();
-    std::vector<uint4> hrows;  // host tables must outlive their uploads (synchronised below)
-    std::vector<uint2> htiles;
-    if (hs.n_huge > 0) {
-        const uint32_t nh = std::min(hs.n_huge, huge_cap);
-        std::vector<uint2> hl(nh);
-        e = cudaMemcpyAsync(hl.data(), d_huge, sizeof(uint2) * nh, cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) return cuda_fail(e, "huge rows");
-        for (uint32_t r = 0; r < nh; ++r) {
-            const uint32_t d = hl[r].y, nt = (d + kBuildTile - 1) / kBuildTile;
-            hrows.push_back(make_uint4(hl[r].x, d, (uint32_t)htiles.size(), nt));
-            for (uint32_t t = 0; t < nt; ++t) htiles.push_back(make_uint2(r, t * kBuildTile));
+    PPR_CUDA(cudaMemcpyAsync(g->tab, &g->htab, sizeof(ClassTab), cudaMemcpyHostToDevice, st));
+    g->device_bytes = (int64_t)(edge_bytes + (sizeof(NodeRec) + 8) * n + sizeof(Sector) * g->n_slots + 4 * g->n_single);
+    EdgeArgs A{n, m, d_col, d_w, heads, d_rp, d_off, g->instances, g->code_of, d_tile, tiles, g->edges, d_ls,
+               ((reinterpret_cast<uintptr_t>(d_col) | reinterpret_cast<uintptr_t>(d_w)) & 15) == 0};
+    if (tiles > 0) {
+        if (tiles > 1) {
+            k_edge_tiles<<<(unsigned)tiles, kEdgeThreads, 0, st>>>(A);
+            note_launch();
         }
-        const uint32_t nt = (uint32_t)htiles.size();
-        uint4 *d_rows;
-        uint2 *d_tiles;
-        uint64_t *d_tsum, *d_rtot;
-        if ((rc = dev_alloc((void **)&d_rows, sizeof(uint4) * nh, "huge rows", st))) return rc;
-        tmp.push_back(d_rows);
-        if ((rc = dev_alloc((void **)&d_tiles, sizeof(uint2) * nt, "tile table", st))) return rc;
-        tmp.push_back(d_tiles);
-        if ((rc = dev_alloc((void **)&d_tsum, sizeof(uint64_t) * nt, "tile sums", st))) return rc;
-        tmp.push_back(d_tsum);
-        if ((rc = dev_alloc((void **)&d_rtot, sizeof(uint64_t) * nh, "row totals", st))) return rc;
-        tmp.push_back(d_rtot);
-        e = cudaMemcpyAsync(d_rows, hrows.data(), sizeof(uint4) * nh, cudaMemcpyHostToDevice, st);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(d_tiles, htiles.data(), sizeof(uint2) * nt, cudaMemcpyHostToDevice, st);
-        if (e != cudaSuccess) return cuda_fail(e, "tile table upload");
-        BuildTiles T{A, d_rows, d_tiles, d_tsum, d_rtot, nh};
-        k_build_tile_totals<<<nt, 256, 0, st>>>(T);
-        note_launch();
-        k_build_tile_scan<<<(nh + 7) / 8, 256, 0, st>>>(T);
-        note_launch();
-        k_build_tile_write<<<nt, 256, 0, st>>>(T);
-        note_launch();
-        k_build_tile_finish<<<nh, 512, 0, st>>>(T);
+        if (tiles > kSelfCarry) {
+            k_edge_carry<<<1, 1024, 0, st>>>(A);
+            note_launch();
+        }
+        k_edge_records<E::kWide><<<(unsigned)tiles, kEdgeThreads, 0, st>>>(A);
         note_launch();
     }
-    e = cudaMemcpyAsync(&hs, d_ls, sizeof(hs), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return cuda_fail(e, "graph build");
+    const E edges{static_cast<const typename E::Edge *>(g->edges)};
+    const SlotArgs B{n, d_rp, g->code_of, g->tab, g->node, g->slots, g->n_slots, d_ls};
+    k_nodes<E><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(B, edges);
+    note_launch();
+    if (g->n_slots > 0) {
+        k_slots<E><<<(unsigned)((g->n_slots + 255) / 256), 256, 0, st>>>(B, edges);
+        note_launch();
+    }
+    LayoutStats hs;
+    PPR_CUDA(cudaGetLastError());
+    PPR_CUDA(cudaMemcpyAsync(&hs, d_ls, sizeof(hs), cudaMemcpyDeviceToHost, st));
+    PPR_CUDA(cudaStreamSynchronize(st));
     if (hs.status & kBadCol) {
         set_error("an edge target is outside [0, n) (of its instance)");
         return PPR_EINVAL;
@@ -802,17 +465,7 @@ static int build_narrow(ppr_ctx *ctx, int64_t n, int64_t m, const int64_t *d_rp,
         set_error("edge weights must be >= 1 (w(e) > 0, Sec. 2.1)");
         return PPR_EINVAL;
     }
-    if (hs.status & kWide) {
-        dev_free(g->node, st);
-        dev_free(g->edges, st);
-        dev_free(g->sum, st);
-        g->node = nullptr;
-        g->edges = nullptr;
-        g->sum = nullptr;
-        g->sum_sectors = 0;
-        return 1;
-    }
-    return PPR_OK;
+    return (hs.status & kWide) ? 1 : PPR_OK;
 }
 
 int build_graph(ppr_ctx *ctx, int64_t n, int64_t m, const int64_t *row_ptr, const int32_t *col,
@@ -856,79 +509,25 @@ int build_graph(ppr_ctx *ctx, int64_t n, int64_t m, const int64_t *row_ptr, cons
                                         cudaMemcpyHostToDevice, st);
         if (e != cudaSuccess) return cleanup(), cuda_fail(e, "node_off upload");
     }
-    if (renumber && g->instances == 0) {
-        if ((rc = dev_alloc((void **)&g->order, sizeof(int32_t) * n, "node order", st)) ||
-            (rc = dev_alloc((void **)&g->rank, sizeof(int32_t) * n, "node rank", st)) ||
-            (rc = renumber_by_indegree(ctx, n, m, d_col, st, g->order, g->rank, tmp)))
-            return cleanup(), rc;
-        g->device_bytes_extra = (int64_t)(2 * sizeof(int32_t) * n);
+    rc = build_layout<NarrowEdges>(ctx, n, m, d_rp, d_col, d_w, d_off, st, g, tmp);
+    g->renumbered = renumber && g->instances == 0;
+    if (rc == 1) {  // some row total reaches 2^32: 64-bit prefixes
+        for (void *p : {(void *)g->edges, (void *)g->node, (void *)g->slots, (void *)g->single, (void *)g->tab,
+                        (void *)g->order, (void *)g->code_of})
+            dev_free(p, st);
+        g->edges = nullptr;
+        g->node = nullptr;
+        g->slots = nullptr;
+        g->single = nullptr;
+        g->tab = nullptr;
+        g->order = nullptr;
+        g->code_of = nullptr;
+        g->wide = true;
+        g->renumbered = false;
+        rc = build_layout<WideEdges>(ctx, n, m, d_rp, d_col, d_w, d_off, st, g, tmp);
     }
-    rc = build_narrow(ctx, n, m, d_rp, d_col, d_w, d_off, st, g, tmp);
-    if (rc != 1) {
-        if (rc == PPR_OK) g->device_bytes += g->device_bytes_extra;
-        cleanup();
-        return rc;
-    }
-    // the wide layout keeps the caller's numbering
-    dev_free(g->order, st);
-    dev_free(g->rank, st);
-    g->order = g->rank = nullptr;
-    g->device_bytes_extra = 0;
-    // some row total reaches 2^32: 64-bit prefixes in flat rows
-    void *p;
-    if ((rc = dev_alloc(&p, sizeof(uint64_t) * n, "row totals", st))) return cleanup(), rc;
-    tmp.push_back(p);
-    uint64_t *d_W = (uint64_t *)p;
-    if ((rc = dev_alloc(&p, sizeof(BuildStats), "build stats", st))) return cleanup(), rc;
-    tmp.push_back(p);
-    BuildStats *d_st = (BuildStats *)p;
-    cudaError_t e = cudaMemsetAsync(d_st, 0, sizeof(BuildStats), st);
-    if (e != cudaSuccess) return cleanup(), cuda_fail(e, "memset");
-
-    const int threads = 256;
-    int64_t want_blocks = (n + 7) / 8;
-    int blocks = (int)std::min<int64_t>(want_blocks, (int64_t)ctx->sms * 64);
-    if (blocks < 1) blocks = 1;
-    k_rows_pass1<<<blocks, threads, 0, st>>>(n, m, d_rp, d_col, d_w, d_off, g->instances, d_W, d_st);
-    note_launch();
-    BuildStats hs;
-    e = cudaMemcpyAsync(&hs, d_st, sizeof(BuildStats), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return cleanup(), cuda_fail(e, "graph validation");
-    if (hs.status & kBadRowPtr) {
-        set_error("row_ptr must start at 0, be non-decreasing and end at m");
-        return cleanup(), PPR_EINVAL;
-    }
-    if (hs.status & kBadCol) {
-        set_error("an edge target is outside [0, n) (of its instance)");
-        return cleanup(), PPR_EINVAL;
-    }
-    if (hs.status & kBadWeight) {
-        set_error("edge weights must be >= 1 (w(e) > 0, Sec. 2.1)");
-        return cleanup(), PPR_EINVAL;
-    }
-    if ((int64_t)hs.max_degree > PPR_MAX_DEGREE) {
-        set_error("out-degree %llu exceeds the limit %lld", hs.max_degree, (long long)PPR_MAX_DEGREE);
-        return cleanup(), PPR_ERANGE;
-    }
-    g->wide = true;
-    g->max_degree = (int64_t)hs.max_degree;
-    g->dangling = (int64_t)hs.dangling;
-    if ((rc = dev_alloc((void **)&g->node, sizeof(NodeRec) * n, "node records", st))) return cleanup(), rc;
-    {
-        size_t edge_bytes = (size_t)m * sizeof(EdgeW);
-        if ((rc = dev_alloc(&g->edges, edge_bytes > 0 ? edge_bytes : 16, "edge records", st))) return cleanup(), rc;
-        g->edge_records = m;
-        g->device_bytes = (int64_t)(sizeof(NodeRec) * n + edge_bytes);
-        k_rows_pass2<true><<<blocks, threads, 0, st>>>(n, d_rp, d_col, d_w, d_off, g->instances, d_W,
-                                                       static_cast<NodeRec *>(g->node), g->edges);
-        note_launch();
-    }
-    e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     cleanup();
-    if (e != cudaSuccess) return cuda_fail(e, "graph build");
-    return PPR_OK;
+    return rc;
 }
 
 // ------------------------------------------------------------ segments ----
@@ -950,19 +549,20 @@ __device__ __forceinline__ uint64_t mul_div(uint64_t q, uint64_t num, uint64_t d
     return (uint64_t)(p / den);
 }
 
+// The layout's rows by seq, targets given by seq.
 template <class E>
 struct RowView {
-    const typename E::Node *node;
+    const NodeRec *node;
     E edges;
+    const ClassTab *tab;
     __device__ __forceinline__ uint32_t deg(uint32_t u) const { return (uint32_t)(node[u].word0 >> 40) & kCountMask; }
     __device__ __forceinline__ uint64_t begin(uint32_t u) const { return node[u].word0 & kBeginMask; }
-    // row total = last inclusive prefix (the node record holds the target of a
-    // single-edge row instead of its total)
+    // (the record of a single-edge row holds its target instead of its total)
     __device__ __forceinline__ uint64_t total(uint32_t u) const
     {
         uint32_t d = deg(u);
         if (d == 1) return 1;  // with wt = 1 above: the single edge has ratio 1
-        return d ? E::key(edges.load(E::edge_base(begin(u), d) + d - 1)) : 0ull;
+        return d ? node[u].total : 0ull;
     }
     // weight and target of the i-th edge of u
     __device__ __forceinline__ void edge(uint32_t u, uint32_t i, uint64_t &wt, uint32_t &tgt) const
@@ -970,19 +570,45 @@ struct RowView {
         const uint32_t d = deg(u);
         if (d == 1) {  // target kept in the node record; weight ratio is 1
             wt = 1;
-            tgt = (uint32_t)node[u].total;
+            tgt = seq_of(*tab, (uint32_t)node[u].total);
             return;
         }
-        uint64_t b = E::edge_base(begin(u), d);
+        uint64_t b = begin(u);
         auto r = edges.load(b + i);
         uint64_t prev = i > 0 ? E::key(edges.load(b + i - 1)) : 0ull;
         wt = E::key(r) - prev;
-        tgt = E::target(r);
+        tgt = seq_of(*tab, E::target(r));
     }
 };
 
+// Table entry of node seq v (entries are in seq order, unused ones last).
+__device__ __forceinline__ uint32_t entry_of(const ClassTab &t, uint32_t v)
+{
+    uint32_t lo = 0, hi = kTabEntries;
+    while (hi - lo > 1) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (t.e[mid].first <= v) lo = mid;
+        else hi = mid;
+    }
+    return lo;
+}
+
+__device__ __forceinline__ uint32_t code_of_seq(const ClassTab &t, uint32_t v)
+{
+    const uint32_t e = entry_of(t, v);
+    return (e << kIdxBits) | (v - t.e[e].first);
+}
+
+// Where a segment table is hung: the small classes' slots and single targets
+// of the segment layout (copies of the plain layout's), see SegCache.
+struct SegLinks {
+    ClassTab *tab;
+    uint32_t *single;
+    SegHead *head;
+};
+
 // Segment tables in two passes.  k_seg_scan (every node; a warp takes 32 at a
-// time) copies the plain record into the segment record array, tests the
+// time) tests the
 // depth-1 shape of all 32 nodes at once (degree <= 8 of the node and of its
 // targets), then for each candidate left the depth-2 shape, and counts the
 // raw contributions the path enumeration will make; eligible nodes are listed
@@ -993,7 +619,7 @@ struct RowView {
 // masses, rejects a node with more than 64 outcomes, puts the rest in
 // canonical order (terminated before active, then node, then length) by
 // ranking, and writes the table at the node's slot.  A table's place in the
-// entry array is free (its record holds begin and count; a shorter table
+// entry array is free (its link holds begin and count; a shorter table
 // leaves a gap), so only its content is fixed.
 
 constexpr unsigned long long kSegEmpty = ~0ull;  // free hash slot (an outcome key's node field is below 2^31)
@@ -1039,30 +665,29 @@ struct SegHash {
 // lbound[list position]: min(raw contributions, 64), the entries the node's
 // table may take (its slot range in the entry array comes from a scan of these).
 template <class E>
-__global__ void __launch_bounds__(256) k_seg_scan(RowView<E> G, int64_t n, typename E::Node *seg_node, uint32_t *list,
-                                                  uint32_t *lbound, SegCounters *ct)
+__global__ void __launch_bounds__(256) k_seg_scan(RowView<E> G, int64_t n, uint32_t *list, uint32_t *lbound,
+                                                  SegCounters *ct)
 {
     const uint32_t lane = threadIdx.x & 31;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    // each warp takes 32 consecutive nodes (coalesced record copy and degree
+    // each warp takes 32 consecutive nodes (coalesced records, degree
     // test), then examines the candidates among them one by one with all lanes
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); base < n; base += stride) {
         const int64_t vl = base + lane;
         uint32_t dl = 0;
         bool c = false;
         if (vl < n) {
-            const typename E::Node r = G.node[vl];
-            seg_node[vl] = r;  // plain record unless a table replaces it
+            const NodeRec r = G.node[vl];
             dl = (uint32_t)(r.word0 >> 40) & kCountMask;
             // depth 1, every lane its own node at once (most candidates have
             // a neighbour above the limit): the row's targets, then their degrees
             c = dl >= 1 && dl <= (uint32_t)kSegMaxDeg;
             if (c) {
                 uint32_t tg[kSegMaxDeg];
-                const uint64_t eb = E::edge_base(r.word0 & kBeginMask, dl);
+                const uint64_t eb = r.word0 & kBeginMask;
 #pragma unroll
                 for (uint32_t i = 0; i < (uint32_t)kSegMaxDeg; ++i)
-                    tg[i] = i >= dl ? 0u : (dl == 1 ? (uint32_t)r.total : E::target(G.edges.load(eb + i)));
+                    tg[i] = i >= dl ? 0u : seq_of(*G.tab, dl == 1 ? (uint32_t)r.total : E::target(G.edges.load(eb + i)));
 #pragma unroll
                 for (uint32_t i = 0; i < (uint32_t)kSegMaxDeg; ++i)
                     if (i < dl && G.deg(tg[i]) > (uint32_t)kSegMaxDeg) c = false;
@@ -1154,15 +779,14 @@ __device__ __forceinline__ unsigned long long seg_key_caller(unsigned long long 
     return (k & ~(0x7fffffffull << 8)) | ((unsigned long long)(uint32_t)order[node] << 8);
 }
 
-// order: the renumbered layout's order array (the canonical order ranks
-// outcomes by the caller's node ids), or null.
+// order: the layout's order array (the canonical order ranks outcomes by the
+// caller's node ids).
 // slot: first entry of the table of list position pos (exclusive scan of
 // lbound), so a table is written without a shared counter.
 template <class E, int SLOTS, int WARPS>
 __global__ void __launch_bounds__(32 * WARPS) k_seg_fill(RowView<E> G, uint32_t T, const uint32_t *list, int tier,
-                                                         int64_t n, SegCounters *ct, SegEntry *ent,
-                                                         typename E::Node *seg_node, const int32_t *order,
-                                                         const uint64_t *slot)
+                                                         int64_t n, SegCounters *ct, SegEntry *ent, SegLinks links,
+                                                         const int32_t *order, const uint64_t *slot)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SegHash<SLOTS> *h = reinterpret_cast<SegHash<SLOTS> *>(smem_raw) + (threadIdx.x >> 5);
@@ -1292,11 +916,11 @@ __global__ void __launch_bounds__(32 * WARPS) k_seg_fill(RowView<E> G, uint32_t 
             const uint32_t i = (uint32_t)e * 32 + lane;
             mk[e] = i < K ? h->u.r.sk[i] : ~0ull;
             mq[e] = i < K ? h->u.r.sq[i] : 0ull;
-            mo[e] = (order && i < K) ? seg_key_caller(mk[e], order) : mk[e];
-            if (order && i < K) h->u.r.so[i] = mo[e];
+            mo[e] = i < K ? seg_key_caller(mk[e], order) : mk[e];
+            if (i < K) h->u.r.so[i] = mo[e];
         }
         __syncwarp();
-        const unsigned long long *cmp = order ? h->u.r.so : h->u.r.sk;
+        const unsigned long long *cmp = h->u.r.so;
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
             uint32_t r = 0;
@@ -1336,16 +960,25 @@ __global__ void __launch_bounds__(32 * WARPS) k_seg_fill(RowView<E> G, uint32_t 
                 const unsigned long long k = h->u.r.sk[i];
                 SegEntry se;
                 se.cum = cum[e];
-                se.node = (uint32_t)((k >> 8) & 0x7fffffffull);
+                se.node = code_of_seq(*G.tab, (uint32_t)((k >> 8) & 0x7fffffffull));
                 se.mark_len = ((uint32_t)(k >> 63) << 8) | (uint32_t)(k & 0xff);
                 ent[base + i] = se;
             }
         }
-        if (lane == 0) {
-            typename E::Node r = G.node[v];  // a NodeRecN keeps its (unused) top-level keys
-            r.word0 = pack_word0(base, K, true);
-            r.total = carry;  // Q_v, the table's total mass
-            seg_node[v] = r;
+        // the node's slots (or its single target) now say where its table is
+        const uint32_t ent_v = entry_of(*G.tab, v), idx = v - G.tab->e[ent_v].first;
+        const TabEntry te = links.tab->e[ent_v];
+        if (te.kind == kKindSingle) {
+            if (lane == 0) {
+                uint32_t *to = reinterpret_cast<uint32_t *>(te.addr) + idx;
+                *to = kMarkSeg;
+                links.head[to - links.single] = SegHead{pack_word0(base, K, false), carry};
+            }
+        } else {
+            Sector *at = reinterpret_cast<Sector *>(te.addr) + ((uint64_t)idx << te.kind);
+            for (uint32_t b = lane; b < (1u << te.kind); b += 32)
+                st_sector(at + b, Sector{{(uint32_t)carry, (uint32_t)(carry >> 32), 0u, 0u, kMarkSeg, (uint32_t)base,
+                                          (uint32_t)(base >> 32), K}});
         }
         __syncwarp();
     }
@@ -1360,7 +993,7 @@ static int seg_build_typed(ppr_graph *g, uint32_t T, cudaStream_t st, const RowV
                            SegCounters *d_ct)
 {
     const int64_t n = g->n;
-    typename E::Node *seg_node = static_cast<typename E::Node *>(g->seg.node);
+    const SegLinks links{g->seg.tab, g->seg.single, g->seg.head};
     uint32_t *lbound = nullptr;
     uint64_t *slot = nullptr, *scan_tmp = nullptr;
     auto done = [&](int code) {
@@ -1378,7 +1011,7 @@ static int seg_build_typed(ppr_graph *g, uint32_t T, cudaStream_t st, const RowV
     cudaError_t e = cudaMemsetAsync(lbound, 0, sizeof(uint32_t) * n, st);  // unlisted positions take no entries
     if (e != cudaSuccess) return done(cuda_fail(e, "memset"));
     const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)g->ctx->sms * 16));
-    k_seg_scan<E><<<blocks, 256, 0, st>>>(G, n, seg_node, list, lbound, d_ct);
+    k_seg_scan<E><<<blocks, 256, 0, st>>>(G, n, list, lbound, d_ct);
     note_launch();
     exclusive_scan_u32(lbound, n, slot, scan_tmp, st);  // each listed node's slot range in the entry array
     SegCounters hc;
@@ -1395,7 +1028,7 @@ static int seg_build_typed(ppr_graph *g, uint32_t T, cudaStream_t st, const RowV
                                  (int)smem);
         if (e != cudaSuccess) return done(cuda_fail(e, "cudaFuncSetAttribute(k_seg_fill)"));
         const int fb = (int)std::min<int64_t>((hc.listed[0] + W - 1) / W, (int64_t)g->ctx->sms * 16);
-        k_seg_fill<E, 2 * kSegSmallRaw, W><<<fb, 32 * W, smem, st>>>(G, T, list, 0, n, d_ct, g->seg.entries, seg_node,
+        k_seg_fill<E, 2 * kSegSmallRaw, W><<<fb, 32 * W, smem, st>>>(G, T, list, 0, n, d_ct, g->seg.entries, links,
                                                                      g->order, slot);
         note_launch();
     }
@@ -1406,7 +1039,7 @@ static int seg_build_typed(ppr_graph *g, uint32_t T, cudaStream_t st, const RowV
                                  (int)smem);
         if (e != cudaSuccess) return done(cuda_fail(e, "cudaFuncSetAttribute(k_seg_fill)"));
         const int fb = (int)std::min<int64_t>((hc.listed[1] + W - 1) / W, (int64_t)g->ctx->sms * 8);
-        k_seg_fill<E, kSegLargeSlots, W><<<fb, 32 * W, smem, st>>>(G, T, list, 1, n, d_ct, g->seg.entries, seg_node,
+        k_seg_fill<E, kSegLargeSlots, W><<<fb, 32 * W, smem, st>>>(G, T, list, 1, n, d_ct, g->seg.entries, links,
                                                                    g->order, slot);
         note_launch();
     }
@@ -1417,17 +1050,26 @@ static int seg_build_typed(ppr_graph *g, uint32_t T, cudaStream_t st, const RowV
     g->seg.nodes = (int64_t)hc.tables;
     g->seg.entries_n = (int64_t)hc.used;
     g->seg.entries_cap = (int64_t)hc.bound;
-    g->device_bytes += (int64_t)(sizeof(typename E::Node) * n + sizeof(SegEntry) * hc.bound);
+    g->device_bytes += (int64_t)(sizeof(Sector) * g->seg.n_slots + (4 + sizeof(SegHead)) * g->n_single +
+                                 sizeof(SegEntry) * hc.bound);
     return done(PPR_OK);
+}
+
+static void free_segments(ppr_graph *g, cudaStream_t st)
+{
+    dev_free(g->seg.tab, st);
+    dev_free(g->seg.slots, st);
+    dev_free(g->seg.single, st);
+    dev_free(g->seg.head, st);
+    dev_free(g->seg.entries, st);
+    g->seg = SegCache{};
 }
 
 int build_segments(ppr_graph *g, uint32_t T, cudaStream_t st)
 {
-    if (g->seg.T == T && g->seg.node) return PPR_OK;
+    if (g->seg.T == T && g->seg.tab) return PPR_OK;
     Range range("segment tables");
-    dev_free(g->seg.node, st);
-    dev_free(g->seg.entries, st);
-    g->seg = SegCache{};
+    free_segments(g, st);
     const int64_t n = g->n;
     uint32_t *list = nullptr;
     SegCounters *d_ct = nullptr;
@@ -1437,24 +1079,47 @@ int build_segments(ppr_graph *g, uint32_t T, cudaStream_t st)
         dev_free(d_ct, st);
         if (code != PPR_OK) {
             cudaStreamSynchronize(st);
-            dev_free(g->seg.node, st);
-            dev_free(g->seg.entries, st);
-            g->seg = SegCache{};
+            free_segments(g, st);
         }
         return code;
     };
-    const size_t node_bytes = g->wide ? sizeof(NodeRec) : sizeof(NodeRecN);
+    // the classes that hold rows of up to eight edges come first among the
+    // slots: the segment layout has its own copy of those, and of the single
+    // targets, and shares the rest
+    const uint32_t small = ranges_log2(kSegMaxDeg, g->lam_bits, g->wide);
+    ClassTab tab = g->htab;
+    int64_t ns = 0;
+    for (uint32_t e = 0; e < kTabEntries; ++e)
+        if (tab.e[e].kind <= small) {
+            const uint64_t next = e + 1 < kTabEntries && tab.e[e + 1].first != 0xffffffffu ? tab.e[e + 1].first : (uint64_t)n;
+            ns += (int64_t)(next - tab.e[e].first) << tab.e[e].kind;
+        }
     if ((rc = dev_alloc((void **)&list, sizeof(uint32_t) * n, "segment node list", st)) ||
         (rc = dev_alloc((void **)&d_ct, sizeof(SegCounters), "segment counters", st)) ||
-        (rc = dev_alloc((void **)&g->seg.node, node_bytes * n, "segment node records", st)))
+        (rc = dev_alloc((void **)&g->seg.tab, sizeof(ClassTab), "segment class table", st)) ||
+        (rc = dev_alloc((void **)&g->seg.slots, sizeof(Sector) * std::max<int64_t>(ns, 1), "segment slots", st)) ||
+        (rc = dev_alloc((void **)&g->seg.single, sizeof(uint32_t) * std::max<int64_t>(g->n_single, 1), "segment singles",
+                        st)) ||
+        (rc = dev_alloc((void **)&g->seg.head, sizeof(SegHead) * std::max<int64_t>(g->n_single, 1), "segment heads", st)))
         return done(rc);
+    g->seg.n_slots = ns;
+    for (TabEntry &t : tab.e) {
+        if (t.kind <= small) t.addr += reinterpret_cast<uint64_t>(g->seg.slots) - reinterpret_cast<uint64_t>(g->slots);
+        if (t.kind == kKindSingle)
+            t.addr += reinterpret_cast<uint64_t>(g->seg.single) - reinterpret_cast<uint64_t>(g->single);
+    }
     cudaError_t e = cudaMemsetAsync(d_ct, 0, sizeof(SegCounters), st);
-    if (e != cudaSuccess) return done(cuda_fail(e, "memset"));
+    if (e == cudaSuccess) e = cudaMemcpyAsync(g->seg.tab, &tab, sizeof(tab), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess && ns > 0)
+        e = cudaMemcpyAsync(g->seg.slots, g->slots, sizeof(Sector) * ns, cudaMemcpyDeviceToDevice, st);
+    if (e == cudaSuccess && g->n_single > 0)
+        e = cudaMemcpyAsync(g->seg.single, g->single, sizeof(uint32_t) * g->n_single, cudaMemcpyDeviceToDevice, st);
+    if (e != cudaSuccess) return done(cuda_fail(e, "segment slots"));
     if (g->wide) {
-        RowView<WideEdges> G{static_cast<const NodeRec *>(g->node), WideEdges{(const EdgeW *)g->edges}};
+        RowView<WideEdges> G{g->node, WideEdges{(const EdgeW *)g->edges}, g->tab};
         rc = seg_build_typed(g, T, st, G, list, d_ct);
     } else {
-        RowView<NarrowEdges> G{static_cast<const NodeRecN *>(g->node), NarrowEdges{(const EdgeN *)g->edges}};
+        RowView<NarrowEdges> G{g->node, NarrowEdges{(const EdgeN *)g->edges}, g->tab};
         rc = seg_build_typed(g, T, st, G, list, d_ct);
     }
     if (rc != PPR_OK) return done(rc);
@@ -1486,10 +1151,11 @@ constexpr uint32_t kTileEdges = 8192;     // edges per tile block (256 threads x
 
 struct AliasArgs {
     int64_t n;
-    const NodeRecN *node;  // the narrow layout's records (begin, count, W)
+    const NodeRec *node;  // the narrow layout's records (begin, count, W), by seq
     const EdgeN *edges;
     const uint64_t *off;  // first slot of each row (exclusive scan of degrees)
-    AliasNode *anode;
+    AliasNode *anode;     // rows from seq first_node on
+    int64_t first_node;
     AliasRec *slots;
     uint2 *ic;            // per slot of a long row: (edge, col) of the small edges from the front,
                           // of the large edges from the back
@@ -1503,10 +1169,10 @@ template <class N>
 __device__ __forceinline__ uint32_t row_degree(const N &r) { return (uint32_t)(r.word0 >> 40) & kCountMask; }
 
 // The pairing rounds of one row, serially (row of d >= 2 edges, slots from o).
-__device__ void alias_row_serial(const AliasArgs &A, const NodeRecN &nr, uint32_t d, uint64_t o)
+__device__ void alias_row_serial(const AliasArgs &A, const NodeRec &nr, uint32_t d, uint64_t o)
 {
     const uint64_t W = nr.total & 0xffffffffull;
-    const uint64_t eb = NarrowEdges::edge_base(nr.word0 & kBeginMask, d);
+    const uint64_t eb = nr.word0 & kBeginMask;
     auto pw = [&](uint32_t i) -> uint64_t {
         const uint32_t hi = A.edges[eb + i].P, lo = i ? A.edges[eb + i - 1].P : 0u;
         return (uint64_t)d * (hi - lo);
@@ -1546,11 +1212,10 @@ __device__ void alias_row_serial(const AliasArgs &A, const NodeRecN &nr, uint32_
 __global__ void __launch_bounds__(256) k_alias_small(AliasArgs A)
 {
     for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < A.n; u += (int64_t)gridDim.x * blockDim.x) {
-        const NodeRecN nr = A.node[u];
+        const NodeRec nr = A.node[u];
         const uint32_t d = row_degree(nr);
         const uint64_t o = A.off[u];
-        // first slot and degree; a single-edge row keeps its target instead
-        A.anode[u] = AliasNode{pack_word0(d == 1 ? (nr.total & 0xffffffffull) : o, d, false)};
+        if (u >= A.first_node) A.anode[u - A.first_node] = AliasNode{pack_word0(o, d, false)};
         if (d < 2) continue;
         if (d > kAliasInline) {
             if (d > kAliasHuge) {
@@ -1589,11 +1254,11 @@ __global__ void __launch_bounds__(32 * kSmemWarps) k_alias_serial(AliasArgs A)
     const uint32_t warps = gridDim.x * kSmemWarps;
     for (uint32_t t = blockIdx.x * kSmemWarps + (threadIdx.x >> 5); t < rows; t += warps) {
         const uint32_t u = A.list[t];
-        const NodeRecN nr = A.node[u];
+        const NodeRec nr = A.node[u];
         const uint32_t d = row_degree(nr);  // 33..512
         const uint64_t o = A.off[u];
         const uint64_t W = nr.total & 0xffffffffull;
-        const uint64_t eb = NarrowEdges::edge_base(nr.word0 & kBeginMask, d);
+        const uint64_t eb = nr.word0 & kBeginMask;
         uint32_t ns = 0, nl = 0;
         uint64_t Dc = 0, Ec = 0;
         for (uint32_t e0 = 0; e0 < d; e0 += 32) {
@@ -1742,11 +1407,11 @@ __device__ __forceinline__ void group_sync()
 template <int NT>
 __device__ void alias_row_group(const AliasArgs &A, int64_t u, uint32_t rank, uint64_t *s)
 {
-    const NodeRecN nr = A.node[u];
+    const NodeRec nr = A.node[u];
     const uint32_t d = row_degree(nr);
     const uint64_t o = A.off[u];
     const uint64_t W = nr.total & 0xffffffffull;
-    const uint64_t eb = NarrowEdges::edge_base(nr.word0 & kBeginMask, d);
+    const uint64_t eb = nr.word0 & kBeginMask;
     const uint32_t run = (d + NT - 1) / NT;
     const uint32_t lo = min(rank * run, d), hi = min(lo + run, d);
     // totals of this thread's run
@@ -1942,9 +1607,9 @@ __global__ void __launch_bounds__(256) k_alias_tile_totals(TileArgs T)
     const AliasArgs &A = T.A;
     const uint2 tl = T.tiles[blockIdx.x];
     const HugeRow hr = T.rows[tl.x];
-    const NodeRecN nr = A.node[hr.u];
+    const NodeRec nr = A.node[hr.u];
     const uint64_t W = nr.total & 0xffffffffull;
-    const uint64_t eb = NarrowEdges::edge_base(nr.word0 & kBeginMask, hr.d);
+    const uint64_t eb = nr.word0 & kBeginMask;
     const uint32_t end = min(tl.y + kTileEdges, hr.d);
     const uint32_t lo = min(tl.y + threadIdx.x * 32, end), hi = min(lo + 32, end);
     uint64_t v[3] = {0, 0, 0};
@@ -1984,9 +1649,9 @@ __global__ void __launch_bounds__(256) k_alias_tile_write(TileArgs T)
     const uint2 tl = T.tiles[blockIdx.x];
     const HugeRow hr = T.rows[tl.x];
     const uint32_t d = hr.d;
-    const NodeRecN nr = A.node[hr.u];
+    const NodeRec nr = A.node[hr.u];
     const uint64_t W = nr.total & 0xffffffffull;
-    const uint64_t eb = NarrowEdges::edge_base(nr.word0 & kBeginMask, d);
+    const uint64_t eb = nr.word0 & kBeginMask;
     const uint64_t o = A.off[hr.u];
     const uint32_t end = min(tl.y + kTileEdges, d);
     const uint32_t lo = min(tl.y + threadIdx.x * 32, end), hi = min(lo + 32, end);
@@ -2037,7 +1702,7 @@ __global__ void __launch_bounds__(256) k_alias_tile_merge(TileArgs T)
     const ulonglong2 ab = T.row_ab[lo];
     const uint32_t a = (uint32_t)ab.x, b = (uint32_t)ab.y, d = hr.d;
     if (a == 0 || b == 0 || (uint64_t)a + b > d) return;
-    const NodeRecN nr = A.node[hr.u];
+    const NodeRec nr = A.node[hr.u];
     const uint64_t W = nr.total & 0xffffffffull;
     const uint64_t o = A.off[hr.u];
     auto E = [&](uint32_t j) { return A.sum[o + d - 1 - j]; };
@@ -2086,15 +1751,18 @@ __global__ void __launch_bounds__(256) k_alias_tile_merge(TileArgs T)
     }
 }
 
-__global__ void k_alias_degrees(int64_t n, const NodeRecN *node, uint32_t *deg)
+__global__ void k_alias_degrees(int64_t n, const NodeRec *node, uint32_t *deg)
 {
     for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n; u += (int64_t)gridDim.x * blockDim.x)
-        deg[u] = row_degree(node[u]);
+    {
+        const uint32_t d = row_degree(node[u]);
+        deg[u] = d >= 2 ? d : 0;  // walks find a single edge's target in the layout's own array
+    }
 }
 
 int build_alias(ppr_graph *g, cudaStream_t st)
 {
-    if (g->alias.node) return PPR_OK;
+    if (g->alias.tab) return PPR_OK;
     Range range("alias tables");
     if (g->wide) {
         set_error("the alias sampler needs every row total below 2^32");
@@ -2126,10 +1794,10 @@ int build_alias(ppr_graph *g, cudaStream_t st)
     auto fail = [&](int code) {
         cudaStreamSynchronize(st);
         cleanup();
+        dev_free(g->alias.tab, st);
         dev_free(g->alias.node, st);
         dev_free(g->alias.slots, st);
-        g->alias.node = nullptr;
-        g->alias.slots = nullptr;
+        g->alias = AliasCache{};
         return code;
     };
     if ((rc = dev_alloc((void **)&deg, sizeof(uint32_t) * n, "alias degrees", st)) ||
@@ -2141,15 +1809,39 @@ int build_alias(ppr_graph *g, cudaStream_t st)
         (rc = dev_alloc((void **)&counts, sizeof(uint32_t) * 4, "long-row counts", st)) ||
         (rc = dev_alloc((void **)&huge, sizeof(uint2) * kAliasMaxHuge, "tile-path rows", st)))
         return cleanup(), rc;
-    if ((rc = dev_alloc((void **)&g->alias.node, sizeof(AliasNode) * n, "alias node records", st))) return cleanup(), rc;
-    if ((rc = dev_alloc((void **)&g->alias.slots, sizeof(AliasRec) * m, "alias slots", st))) return fail(rc);
+    // the rows classed by degree have theirs one after the other, in seq order;
+    // the others, which follow, are looked up in node records
+    ClassTab tab = g->htab;
+    int64_t first_node = n, slot = 0;
+    for (uint32_t e = 0; e < kTabEntries && tab.e[e].first != 0xffffffffu; ++e)
+        if (tab.e[e].kind < kKindSingle && g->degree[e] == 0) {
+            first_node = tab.e[e].first;
+            break;
+        }
+    if ((rc = dev_alloc((void **)&g->alias.node, sizeof(AliasNode) * std::max<int64_t>(n - first_node, 1),
+                        "alias node records", st)) ||
+        (rc = dev_alloc((void **)&g->alias.slots, sizeof(AliasRec) * m, "alias slots", st)))
+        return fail(rc);
+    for (uint32_t e = 0; e < kTabEntries && tab.e[e].first != 0xffffffffu; ++e) {
+        TabEntry &t = tab.e[e];
+        if (t.kind >= kKindSingle) continue;
+        if (g->degree[e]) {
+            const int64_t next = e + 1 < kTabEntries && tab.e[e + 1].first != 0xffffffffu ? (int64_t)tab.e[e + 1].first : n;
+            t.kind = g->degree[e];
+            t.addr = reinterpret_cast<uint64_t>(g->alias.slots + slot);
+            slot += (next - (int64_t)t.first) * g->degree[e];
+        } else {
+            t.kind = kKindLookup;
+            t.addr = reinterpret_cast<uint64_t>(g->alias.node + ((int64_t)t.first - first_node));
+        }
+    }
     cudaError_t e = cudaMemsetAsync(counts, 0, sizeof(uint32_t) * 4, st);
     if (e != cudaSuccess) return fail(cuda_fail(e, "memset"));
     const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)g->ctx->sms * 16));
-    k_alias_degrees<<<blocks, 256, 0, st>>>(n, static_cast<const NodeRecN *>(g->node), deg);
+    k_alias_degrees<<<blocks, 256, 0, st>>>(n, g->node, deg);
     note_launch();
     exclusive_scan_u32(deg, n, off, tmp, st);
-    AliasArgs A{n, static_cast<const NodeRecN *>(g->node), (const EdgeN *)g->edges, off, g->alias.node, g->alias.slots, ic,
+    AliasArgs A{n, g->node, (const EdgeN *)g->edges, off, g->alias.node, first_node, g->alias.slots, ic,
                 sum, list, counts, huge};
     k_alias_small<<<blocks, 256, 0, st>>>(A);
     note_launch();
@@ -2209,8 +1901,15 @@ int build_alias(ppr_graph *g, cudaStream_t st)
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return fail(cuda_fail(e, "alias build"));
+    ClassTab *d_tab = nullptr;
+    if ((rc = dev_alloc((void **)&d_tab, sizeof(ClassTab), "alias class table", st))) return fail(rc);
+    e = cudaMemcpyAsync(d_tab, &tab, sizeof(tab), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    g->alias.tab = d_tab;
+    g->alias.nodes = n - first_node;
+    if (e != cudaSuccess) return fail(cuda_fail(e, "alias class table"));
     cleanup();
-    g->device_bytes += (int64_t)(sizeof(AliasNode) * n + sizeof(AliasRec) * m);
+    g->device_bytes += (int64_t)(sizeof(AliasNode) * (n - first_node) + sizeof(AliasRec) * m);
     return PPR_OK;
 }
 

@@ -37,14 +37,20 @@ int dev_alloc(void **p, size_t bytes, const char *what, cudaStream_t st);
 void dev_free(void *p, cudaStream_t st);
 
 struct AliasCache {
-    AliasNode *node = nullptr; // node records pointing at alias slots
-    AliasRec *slots = nullptr; // one per edge
+    ClassTab *tab = nullptr;   // class table of the alias walk: where the rows' alias slots are
+    AliasNode *node = nullptr; // rows whose degree their class does not tell, by seq - first_node
+    AliasRec *slots = nullptr; // one per edge of the rows of two and more
+    int64_t nodes = 0;         // records at node
 };
 
 struct SegCache {
     uint32_t T = 0;               // threshold the tables were built for (0 = none)
-    void *node = nullptr;         // node records (the graph's type) with eligible nodes switched to their tables
+    ClassTab *tab = nullptr;      // the class table with the small classes' slots replaced
+    Sector *slots = nullptr;      // their slots, eligible nodes' pointing at their tables
+    uint32_t *single = nullptr;   // single-edge nodes' targets, eligible ones marked
+    SegHead *head = nullptr;      // their tables
     SegEntry *entries = nullptr;  // all tables
+    int64_t n_slots = 0;
     int64_t nodes = 0, entries_n = 0;  // tables, and the entries they hold
     int64_t entries_cap = 0;           // entries allocated (tables sit at fixed slots, with gaps)
 };
@@ -64,6 +70,7 @@ struct ppr_ctx {
     size_t l2_window_max = 0;
     size_t l2_persist_set = 0;    // persisting set-aside this context asked for
     size_t l2_bytes = 0;          // L2 size (the layout's renumbering policy)
+    size_t mem_bytes = 0;         // device memory (the layout's slot density)
     cudaStream_t copy_stream = nullptr;  // output copies of ppr_run_to_host
     unsigned long long *pinned = nullptr;  // page-locked words for per-batch totals
     std::atomic<int> refs{1};  // the caller's handle plus every live graph and result
@@ -82,18 +89,20 @@ struct ppr_graph {
     int64_t n = 0, m = 0;
     int64_t max_degree = 0, dangling = 0;
     bool wide = false;
-    void *node = nullptr;   // NodeRecN[n] (narrow layout) or NodeRec[n] (wide layout)
-    void *edges = nullptr;  // EdgeN[m] or EdgeW[m]
-    int64_t edge_records = 0;  // records the edge layout holds (blocked narrow rows: with padding)
-    uint32_t *sum = nullptr;   // narrow layout: the blocked rows' summary levels (8 keys a sector), or
-    int64_t sum_sectors = 0;   // null: each row's summary precedes its blocks in the edge array
-    // where the walkers read summary sectors (the summary array or the edge array) and how many there are
-    const uint32_t *sum_base() const { return sum ? sum : static_cast<const uint32_t *>(edges); }
-    uint64_t sum_extent() const { return sum ? (uint64_t)sum_sectors : (uint64_t)edge_records / 4; }
-    // internal numbering of the layout (renumber.cu), or null: caller ids
-    int32_t *order = nullptr;  // [n] caller id of internal node i
-    int32_t *rank = nullptr;   // [n] internal id of caller node v
-    int64_t device_bytes_extra = 0;  // order and rank
+    // the layout (ppr_internal.cuh)
+    ppr::NodeRec *node = nullptr;     // [n] by seq
+    void *edges = nullptr;            // EdgeN[m] or EdgeW[m] (padded to whole sectors)
+    ppr::Sector *slots = nullptr;     // guide slots
+    int64_t n_slots = 0;
+    uint32_t *single = nullptr;       // targets of the single-edge nodes
+    int64_t n_single = 0;
+    ppr::ClassTab *tab = nullptr;     // device copy of htab
+    ppr::ClassTab htab;
+    uint32_t degree[ppr::kTabEntries];  // degree of an entry's rows, 0: not told by its class
+    uint32_t lam_bits = 0;            // a range holds at most 2^lam_bits edges on average
+    int32_t *order = nullptr;         // [n] caller id (within its instance) by seq
+    uint32_t *code_of = nullptr;      // [n] code by caller id
+    bool renumbered = false;          // what ppr_graph_info reports (the flags' rule)
     // block-diagonal instances
     int32_t instances = 0;
     std::vector<int64_t> node_off;  // host copy, count+1
@@ -134,9 +143,17 @@ namespace ppr {
 // graph.cu
 int build_graph(ppr_ctx *ctx, int64_t n, int64_t m, const int64_t *row_ptr, const int32_t *col,
                 const uint32_t *w, bool device_ptrs, bool renumber, cudaStream_t st, ppr_graph *g);
-// renumber.cu: order and rank of the in-degree numbering (see ppr_graph)
-int renumber_by_indegree(ppr_ctx *ctx, int64_t n, int64_t m, const int32_t *d_col, cudaStream_t st, int32_t *order,
-                         int32_t *rank, std::vector<void *> &tmp);
+// renumber.cu: numbers the nodes class by class (see ClassTab).  Fills order,
+// code_of, htab (addresses counted from the arrays' starts), degree, n_single
+// and n_slots; checks row_ptr.
+struct LayoutStats {
+    unsigned long long max_degree;
+    unsigned long long dangling;
+    unsigned int status;
+};
+enum : uint32_t { kBadRowPtr = 1u, kBadCol = 2u, kBadWeight = 4u, kWide = 8u, kBigDegree = 16u };
+int number_nodes(int64_t n, int64_t m, const int64_t *d_rp, const int64_t *d_off, uint32_t *heads,
+                 LayoutStats *d_stats, bool wide, cudaStream_t st, ppr_graph *g, std::vector<void *> &tmp);
 int build_segments(ppr_graph *g, uint32_t T, cudaStream_t st);
 int build_alias(ppr_graph *g, cudaStream_t st);
 
@@ -149,16 +166,13 @@ struct RunPlan {
     int32_t dangling;
     bool segments;
     int32_t kernel;
-    int32_t large_degree;
     int32_t warps_per_block;
     int32_t chunk_sources;
     int32_t refill_lanes;  // persistent kernel: idle lanes before a warp refills (0 = 1)
     bool stats;
     int32_t sampler;  // 0 first-prefix-above rule, 1 integer alias method
-    bool l2_persist;  // walker launches keep the node records in L2 (access-policy window)
-    int32_t step_loads;  // bounded step: dependent loads per lane per warp iteration (0 = unbounded)
+    bool l2_persist;  // walker launches keep the front of the layout in L2 (access-policy window)
 };
-constexpr int32_t kDefaultStepLoads = 6;
 // Enqueues the walks of sources [s_begin, s_end) writing output rows from
 // out_row0.  ends: S * R endpoint scratch for the plain kernel (else unused);
 // queue: one device counter for the persistent kernel's work queue.

@@ -1,46 +1,37 @@
 // ppr_internal.cuh -- device-side building blocks of libppr.so (sm_103a).
 //
 // Graph layout in HBM
-//   NodeRec (16 B, one aligned half-sector per node; wide layout, alias tables)
-//     word0 = begin (bits 0..39) | count (bits 40..62) | segment flag (bit 63)
-//     word1 = W_u, the row's total weight (Sec. 2.1 routing denominator), or
-//             the target id when the row has exactly one edge (no search), or
-//             Q_v, the total fixed-point mass of a segment table (Algorithm 4);
-//             narrow blocked rows keep W_u in bits 0..31, a summary field
-//             (bits 32..59, see blocked_sum) and their level count L (bits
-//             60..63) above it
-//   NodeRecN (32 B, one sector per node; narrow layout): a NodeRec and the
-//     first four keys of the row's top summary level when that level has at
-//     most five keys (the fifth is W_u), so the step that reads the record
-//     ranks the draw within the top level and skips that sector
-//   plain rows:  begin/count index the edge-record array
-//   segment rows: begin/count index the segment-entry array
-//   EdgeN (8 B): {uint32 P, int32 col}  -- narrow layout, every W_u < 2^32
-//   EdgeW (16 B): {uint64 P, int32 col, pad} -- wide layout (flat rows)
 //
-// Narrow rows are stored as static search trees ("blocked" rows).  A row with
-// d >= 2 edges has its edge records in blocks of 8 in the edge array (the
-// area rounded up to whole sectors, padding keys 0xFFFFFFFF) and, when d > 8,
-// summary levels, top level first.  Two placements (the walkers' SPLIT
-// template parameter):
-//   split (renumbered graphs far larger than L2): the summaries sit in a
-//     summary array that holds nothing else, so the summary sectors that
-//     every draw at a node passes through share L2 lines and DRAM pages
-//     instead of lying one per row between blocks that a draw reads once;
-//     every row's blocks start on 64 bytes, so a full block is one fetch;
-//   interleaved (otherwise): each row's area holds its summary, then its
-//     blocks, starting on a 32-byte sector.
-// Level 1 keeps the last prefix of every 8-record block, level l+1 the last
-// key of every 8-key sector of level l, up to a top level of at most 8 keys
-// (one sector).
-// A search reads one sector per level and one 8-record block: the same edge
-// as bisection of the flat prefix (the first P > x is unique), found with
-// ceil(log8 d) + 1 dependent loads instead of ceil(log2 d) + 1.  The alias
-// tree of the paper (Algorithm 3) splits large neighbour sets the same way so
-// that a selection touches one small set per level; Lemma 1 is the analogous
-// exactness argument.
-//   SegEntry (16 B): {uint64 cum, uint32 node, uint32 mark_len}
-//   P / cum are inclusive prefix sums within the row / table.
+// A draw at node u is a step function of its 64 random bits r: the first edge
+// whose inclusive weight prefix P exceeds x = floor(r * W_u / 2^64).  The
+// layout stores that function cut into 2^c equal ranges of r (the top c bits
+// of r name the range): one 32-byte slot per range holds the at most four
+// edges that meet the range, so a draw reads one sector whatever the degree,
+// where a search tree over P reads one per level.  A range that more edges
+// meet (runs of light edges) sends the draw on to the edge records.  The
+// edge drawn is the one the rule names, bit for bit: only its lookup differs.
+//
+// Nodes are numbered class by class (class = dangling, single edge, on large
+// graphs the degree up to 24, then the number of ranges 2^c), so the 32-bit code of a node is all a walk needs to
+// find its slots: the top six bits select an entry of the class table (where
+// the class starts and its c), the rest count nodes within the entry.  No
+// node record is read on the way.
+//   code   (entry << 26) | index         names a node to the walkers
+//   seq    first[entry] + index          the same node in [0, n), dense
+//   order[seq]: the caller's id (within its instance);  code_of[id]: its code
+//   single[]   4 B per single-edge node: the code of its target
+//   slots[]    32 B per range (GuideSlot layouts below)
+//   EdgeN (8 B): {uint32 P, code}   -- narrow layout, every W_u < 2^32
+//   EdgeW (16 B): {uint64 P, code, pad} -- wide layout; in the caller's edge order
+//   NodeRec (16 B, by seq): word0 = begin (bits 0..39) | count (bits 40..62);
+//     total = W_u, or the target's code for a single edge (read by the table
+//     builds and the statistics, not by walks)
+//   SegEntry (16 B): {uint64 cum, code, mark_len}; P / cum are inclusive
+//     prefix sums within the row / table.
+//
+// The paper's alias tree (Algorithm 3) splits a large neighbour set so that a
+// selection visits one small set per level; Lemma 1 is the analogous
+// exactness argument for reading one small set of edges instead of the row.
 #pragma once
 
 #include <cstdint>
@@ -55,12 +46,6 @@ constexpr uint64_t kSegFlag = 1ull << 63;
 struct __align__(16) NodeRec {
     uint64_t word0;
     uint64_t total;
-};
-
-struct __align__(32) NodeRecN {
-    uint64_t word0;
-    uint64_t total;
-    uint32_t key[4];  // top-level keys 0..3 (see root_in_record), else 0xFFFFFFFF
 };
 
 struct __align__(8) EdgeN {
@@ -85,16 +70,22 @@ struct __align__(16) AliasRec {
     uint32_t W;
 };
 
-// Node record of the alias layout: first slot (bits 0..39) | degree (bits
-// 40..62); a single-edge row keeps its target in the slot field.
+// Alias row of a node whose degree its class does not tell: first slot (bits
+// 0..39) | degree (bits 40..62).
 struct __align__(8) AliasNode {
     uint64_t word;
 };
 
 struct __align__(16) SegEntry {
     uint64_t cum;
-    uint32_t node;
+    uint32_t node;      // code
     uint32_t mark_len;  // (active << 8) | len
+};
+
+// Segment table of a single-edge node: entries and total mass Q.
+struct __align__(16) SegHead {
+    uint64_t where;  // first entry (bits 0..39) | entries (bits 40..62)
+    uint64_t Q;
 };
 
 __host__ __device__ inline uint64_t pack_word0(uint64_t begin, uint32_t count, bool seg)
@@ -102,45 +93,62 @@ __host__ __device__ inline uint64_t pack_word0(uint64_t begin, uint32_t count, b
     return (begin & kBeginMask) | ((uint64_t)(count & kCountMask) << 40) | (seg ? kSegFlag : 0ull);
 }
 
-// ceil(d / 2^s)
-__host__ __device__ __forceinline__ uint32_t ceil_shift(uint32_t d, uint32_t s) { return (d + (1u << s) - 1) >> s; }
+// ------------------------------------------------------------- node codes ----
+// 26 index bits and up to 62 table entries name any n < 2^31 nodes: each class
+// is cut into entries of 2^26 nodes.
+constexpr uint32_t kIdxBits = 26;
+constexpr uint32_t kIdxMask = (1u << kIdxBits) - 1;
+constexpr uint32_t kTabEntries = 64;
+constexpr uint32_t kMarkOverflow = 63u << kIdxBits;  // in a slot's first code: the range overflows
+constexpr uint32_t kMarkSeg = 62u << kIdxBits;       // the node carries a segment table
+constexpr uint32_t kKindSingle = 64, kKindDangling = 128;  // else the class's c, 0..23
+constexpr uint32_t kKindLookup = 192;  // alias table: rows listed in AliasNode records (else the rows' degree)
 
-// Number of summary levels above a blocked row of d edges (0 for d <= 8).
-__host__ __device__ __forceinline__ uint32_t tree_levels(uint32_t d)
+// addr: the entry's first slot (or single target); kind: its class's c, or one
+// of the above; first: seq of its first node (0xFFFFFFFF: unused entry).
+struct __align__(16) TabEntry {
+    uint64_t addr;
+    uint32_t kind;
+    uint32_t first;
+};
+struct ClassTab {
+    TabEntry e[kTabEntries];
+};
+
+// Class of a row of d edges: 0 dangling, 1 single edge, kExact + 1 + c for 2^c
+// ranges.  Plain graphs of more than kExactMin nodes class rows of up to kExact
+// edges by their degree, so that alias slots are found without a record: the
+// records of all nodes would not stay in L2 there, those of the longer rows (a
+// tenth) do (R-MAT scale 24, alias walker over 2^22 sources: 22.1 -> 20.9 ms).
+// Elsewhere the classes stay few: every class is an area of its own, and with
+// 23 more of them the walker of a 256-graph batch took 25.1 ms, not 17.6.
+// More than kExactNodes nodes leave no room in the table for classes by degree.
+// 2^c is the smallest power of two >= d / 2^lam_bits, and a row that fits one
+// slot (four edges, three in the wide layout) is one range.
+constexpr uint32_t kExact = 24, kClasses = kExact + 1 + 24;
+constexpr int64_t kExactMin = 1ll << 22, kExactNodes = 1ll << 30;  // 44 classes and 16 further entries of 2^26 nodes
+__host__ __device__ __forceinline__ uint32_t ceil_log2(uint32_t v)
 {
-    uint32_t L = 0;
-    while (d > (1u << (3 * (L + 1)))) ++L;
-    return L;
+    if (v <= 1) return 0;
+#ifdef __CUDA_ARCH__
+    return 32u - __clz(v - 1);
+#else
+    return 32u - (uint32_t)__builtin_clz(v - 1);
+#endif
+}
+__host__ __device__ __forceinline__ uint32_t ranges_log2(uint32_t d, uint32_t lam_bits, bool wide)
+{
+    return d <= (wide ? 3u : 4u) ? 0u : ceil_log2((d + (1u << lam_bits) - 1) >> lam_bits);
+}
+__host__ __device__ __forceinline__ uint32_t class_of_degree(uint32_t d, uint32_t lam_bits, bool wide, bool exact)
+{
+    return d <= 1 || (exact && d <= kExact) ? d : kExact + 1 + ranges_log2(d, lam_bits, wide);
 }
 
-// Sectors of level l (1 <= l <= L): ceil(keys_l / 8) = ceil(d / 8^(l+1)).
-__host__ __device__ __forceinline__ uint32_t level_sectors(uint32_t d, uint32_t l) { return ceil_shift(d, 3 * (l + 1)); }
-
-__host__ __device__ __forceinline__ uint32_t summary_sectors(uint32_t d)
+__device__ __forceinline__ uint32_t seq_of(const ClassTab &t, uint32_t code)
 {
-    uint32_t L = tree_levels(d), S = 0;
-    for (uint32_t l = 1; l <= L; ++l) S += level_sectors(d, l);
-    return S;
+    return t.e[code >> kIdxBits].first + (code & kIdxMask);
 }
-
-// 8-byte record slots a blocked row's blocks take (a one-edge row keeps its
-// target in the node record and needs none), not counting its summary
-// levels (summary_sectors) or the split layout's padding to 64 bytes.
-__host__ __device__ __forceinline__ uint32_t blocked_row_records(uint32_t d)
-{
-    if (d <= 1) return 0;
-    return 4 * ceil_shift(d, 2);
-}
-
-// A blocked row's record keeps, above W_u, a 28-bit summary field and its
-// level count (4 bits).  The field is the row's first sector in the summary
-// array on a split layout (renumbered graphs far larger than L2), and the
-// number of summary sectors that precede the row's blocks in the edge array
-// otherwise; the record's begin points at the blocks either way.
-constexpr uint32_t kSumBits = 28;
-constexpr uint64_t kSumSectorsMax = 1ull << kSumBits;
-__host__ __device__ __forceinline__ uint32_t blocked_sum(uint64_t total) { return (uint32_t)(total >> 32) & (uint32_t)(kSumSectorsMax - 1); }
-__host__ __device__ __forceinline__ uint32_t blocked_levels(uint64_t total) { return (uint32_t)(total >> 60); }
 
 // ---------------------------------------------------------------- Philox ----
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11): ten rounds; each round
@@ -148,18 +156,39 @@ __host__ __device__ __forceinline__ uint32_t blocked_levels(uint64_t total) { re
 // multipliers, and the new words are (hi1 ^ c1 ^ k0, lo1, hi0 ^ c3 ^ k1, lo0);
 // the key advances by the golden-ratio and sqrt(3) Weyl increments between
 // rounds.
-__device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1)
+constexpr uint32_t kPhiloxW0 = 0x9E3779B9u, kPhiloxW1 = 0xBB67AE85u;
+
+// Round keys of one seed, computed on the host for a launch whose walks share
+// it: ten pairs of constants where the schedule would be eighteen additions a
+// draw (256-graph batch 16.9 -> 15.9 ms, scale-20 alias walker 4.73 -> 4.58).
+struct RoundKeys {
+    uint32_t k0[10], k1[10];
+    __host__ __device__ void set(uint32_t a, uint32_t b)
+    {
+        for (uint32_t r = 0; r < 10; ++r) {
+            k0[r] = a + r * kPhiloxW0;
+            k1[r] = b + r * kPhiloxW1;
+        }
+    }
+    __device__ __forceinline__ uint32_t a(int r) const { return k0[r]; }
+    __device__ __forceinline__ uint32_t b(int r) const { return k1[r]; }
+};
+// The same schedule from the two key words (lanes with keys of their own).
+struct LaneKeys {
+    uint32_t k0, k1;
+    __device__ __forceinline__ uint32_t a(int r) const { return k0 + (uint32_t)r * kPhiloxW0; }
+    __device__ __forceinline__ uint32_t b(int r) const { return k1 + (uint32_t)r * kPhiloxW1; }
+};
+
+template <class K>
+__device__ __forceinline__ uint4 philox4x32_10(uint4 c, const K &key)
 {
 #pragma unroll
     for (int r = 0; r < 10; ++r) {
-        if (r > 0) {
-            k0 += 0x9E3779B9u;
-            k1 += 0xBB67AE85u;
-        }
         const uint32_t m0 = 0xD2511F53u, m1 = 0xCD9E8D57u;
-        uint32_t lo0 = m0 * c.x, hi0 = __umulhi(m0, c.x);
-        uint32_t lo1 = m1 * c.z, hi1 = __umulhi(m1, c.z);
-        c = make_uint4(hi1 ^ c.y ^ k0, lo1, hi0 ^ c.w ^ k1, lo0);
+        const uint64_t p0 = (uint64_t)m0 * c.x, p1 = (uint64_t)m1 * c.z;
+        c = make_uint4((uint32_t)(p1 >> 32) ^ c.y ^ key.a(r), (uint32_t)p1, (uint32_t)(p0 >> 32) ^ c.w ^ key.b(r),
+                       (uint32_t)p0);
     }
     return c;
 }
@@ -175,15 +204,6 @@ __device__ __forceinline__ uint64_t mulhi64_by32(uint32_t r_lo, uint32_t r_hi, u
 __device__ __forceinline__ uint64_t mulhi64(uint64_t r, uint64_t W) { return __umul64hi(r, W); }
 
 // ---------------------------------------------------------------- loads ----
-__device__ __forceinline__ NodeRec load_node(const NodeRec *node, uint32_t u)
-{
-    uint4 v = __ldg(reinterpret_cast<const uint4 *>(node) + u);
-    NodeRec r;
-    r.word0 = (uint64_t)v.x | ((uint64_t)v.y << 32);
-    r.total = (uint64_t)v.z | ((uint64_t)v.w << 32);
-    return r;
-}
-
 // One 32-byte sector in a single 256-bit load (sm_100+ vector width).
 struct Sector {
     uint32_t v[8];
@@ -198,54 +218,28 @@ __device__ __forceinline__ Sector ld_sector(const void *p)
     return s;
 }
 
-
-// One 32-byte sector of a row's bottom block.  EF (layouts of graphs far
-// larger than L2) loads it with an evict-first L2 policy: a bottom block
-// serves the one draw that picked it and is rarely read again before it would
-// leave L2, while node records and summary sectors are shared by every draw
-// that passes the same node, so blocks should be the first to go.  On a graph
-// about the size of L2 the blocks are reused (evict-first there cost the
-// 2,048-graph batch 3 %), so they keep the normal policy.
-template <bool EF>
-__device__ __forceinline__ Sector ld_block_sector(const void *p)
+// Eight bytes for the lanes with `on` set only (the others' are undefined),
+// without a branch that the compiler would carry what follows into.
+__device__ __forceinline__ uint2 ld_pair_if(const void *p, bool on)
 {
-    if constexpr (!EF) {
-        return ld_sector(p);
-    } else {
-        uint64_t pol;
-        asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-        Sector s;
-        asm("ld.global.nc.L2::cache_hint.v8.u32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8], %9;"
-            : "=r"(s.v[0]), "=r"(s.v[1]), "=r"(s.v[2]), "=r"(s.v[3]), "=r"(s.v[4]), "=r"(s.v[5]), "=r"(s.v[6]),
-              "=r"(s.v[7])
-            : "l"(p), "l"(pol));
-        return s;
-    }
+    uint2 v;
+    asm("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %3, 0;\n\t@q ld.global.nc.v2.u32 {%0,%1}, [%2];\n\t}"
+        : "=r"(v.x), "=r"(v.y)
+        : "l"(p), "r"((uint32_t)on));
+    return v;
 }
 
-// A blocked row of d edges with L >= 1 summary levels keeps its top level's
-// keys in the node record when that level has at most five keys
-// (ceil(d / 8^L) <= 5): keys 0..3 in NodeRecN::key, the fifth being W_u.
-__host__ __device__ __forceinline__ bool root_in_record(uint32_t d, uint32_t L)
+__device__ __forceinline__ void st_sector(void *p, const Sector &s)
 {
-    return L >= 1 && d <= (5u << (3 * L));
+    asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(s.v[0]), "r"(s.v[1]), "r"(s.v[2]),
+                 "r"(s.v[3]), "r"(s.v[4]), "r"(s.v[5]), "r"(s.v[6]), "r"(s.v[7])
+                 : "memory");
 }
 
 struct NarrowEdges {
-    using Key = uint32_t;
-    using Node = NodeRecN;
-    // the record half of the sector; search_blocked reads the key half when
-    // it needs it (then an L1 hit: the first load brought the whole sector)
-    __device__ __forceinline__ static NodeRec load_node(const void *node, uint32_t u)
-    {
-        return ppr::load_node(reinterpret_cast<const NodeRec *>(static_cast<const NodeRecN *>(node) + u), 0);
-    }
+    static constexpr bool kWide = false;
+    using Edge = EdgeN;
     const EdgeN *e;
-    // record index of edge 0 of a row whose region starts at `begin`
-    __host__ __device__ __forceinline__ static uint64_t edge_base(uint64_t begin, uint32_t)
-    {
-        return begin;  // the summary levels live in their own array
-    }
     __device__ __forceinline__ uint2 load(uint64_t i) const
     {
         return __ldg(reinterpret_cast<const uint2 *>(e) + i);
@@ -256,13 +250,9 @@ struct NarrowEdges {
 };
 
 struct WideEdges {
-    using Node = NodeRec;
-    __device__ __forceinline__ static NodeRec load_node(const void *node, uint32_t u)
-    {
-        return ppr::load_node(static_cast<const NodeRec *>(node), u);
-    }
+    static constexpr bool kWide = true;
+    using Edge = EdgeW;
     const EdgeW *e;
-    __host__ __device__ __forceinline__ static uint64_t edge_base(uint64_t begin, uint32_t) { return begin; }
     __device__ __forceinline__ uint4 load(uint64_t i) const
     {
         return __ldg(reinterpret_cast<const uint4 *>(e) + i);
@@ -272,24 +262,8 @@ struct WideEdges {
     using Rec = uint4;
 };
 
-// Alias layout: begin/count of a node record index its alias slots.
-struct AliasEdges {
-    using Node = AliasNode;
-    __device__ __forceinline__ static NodeRec load_node(const void *node, uint32_t u)
-    {
-        const uint2 v = __ldg(reinterpret_cast<const uint2 *>(node) + u);
-        NodeRec r;
-        r.word0 = (uint64_t)v.x | ((uint64_t)v.y << 32);
-        r.total = 0;
-        return r;
-    }
-    const AliasRec *e;
-    __host__ __device__ __forceinline__ static uint64_t edge_base(uint64_t begin, uint32_t) { return begin; }
-    __device__ __forceinline__ uint4 load(uint64_t i) const { return __ldg(reinterpret_cast<const uint4 *>(e) + i); }
-    __device__ __forceinline__ static uint64_t key(uint4 v) { return v.x; }
-    __device__ __forceinline__ static uint32_t target(uint4 v) { return v.y; }
-    using Rec = uint4;
-};
+// Alias tables: walked with AliasNode records and AliasRec slots.
+struct AliasEdges {};
 
 // Segment entries have the same 16-byte shape as wide edges: key = cum,
 // target = node, and the fourth word carries mark_len.
@@ -349,115 +323,70 @@ __device__ __forceinline__ typename E::Rec search_serial_tally(const E &edges, u
     return edges.load(lo);
 }
 
+// ------------------------------------------------------------ guide slots ----
+// The range of r with top bits b covers x in [X0, X1], X0 = floor(b W / 2^c)
+// and X1 = ceil((b + 1) W / 2^c) - 1; the edges that meet it are lo .. hi, the
+// first with P > X0 and the first with P > X1.
+//
+// Narrow slot, at most 4 edges:
+//   v0 = W;  v1..v3 = P of edges lo, lo+1, lo+2;  v4..v7 = codes of lo .. lo+3
+//   (missing ones repeat the last edge, so any rank past it reads the same code)
+// Narrow slot, overflow: the edge records of lo .. hi lie in nsec sectors of
+// four records; cut into five groups of gs = ceil(nsec / 5) sectors,
+//   v0 = W;  v1..v3, v7 = last P of groups 0..3 (0xFFFFFFFF: none)
+//   v4 = kMarkOverflow | (lo & 3) << 8 | first sector (bits 32..37)
+//   v5 = first sector (low word);  v6 = nsec
+// Wide slot, at most 3 edges (offsets from X0, which fit 32 bits since
+// 2^c >= d edges of 32-bit weight):
+//   v0,v1 = W;  v2,v3 = P - X0 of edges lo, lo+1;  v4..v6 = codes of lo .. lo+2
+// Wide slot, overflow: v0,v1 = W;  v4 = kMarkOverflow;  v5 = lo (low word);
+//   v6 = lo (high bits);  v7 = edges to search
+// Node with a segment table: v0,v1 = Q;  v4 = kMarkSeg;  v5,v6 = first entry;
+//   v7 = entries
+constexpr uint32_t kGroups = 5;
 
-// field: the row's summary field (below 2^28; see blocked_sum)
-__host__ __device__ __forceinline__ uint64_t pack_blocked_total(uint64_t W, uint64_t field, uint32_t d)
+// Code of the edge of a narrow slot that x falls on.
+__device__ __forceinline__ uint32_t pick_slot(const Sector &s, uint32_t x)
 {
-    return W | (field << 32) | ((uint64_t)tree_levels(d) << 60);
+    const uint32_t lo = s.v[1] <= x ? s.v[5] : s.v[4], hi = s.v[3] <= x ? s.v[7] : s.v[6];
+    return s.v[2] <= x ? hi : lo;
 }
 
-// Number of the 8 keys k[0..7] that are <= x, for keys in ascending order with
-// k[7] > x (a summary sector's last key is its parent's key, above x; missing
-// keys are 0xFFFFFFFF): three comparisons of a binary search, 0..7.
-__device__ __forceinline__ uint32_t rank8(uint32_t k0, uint32_t k1, uint32_t k2, uint32_t k3, uint32_t k4, uint32_t k5,
-                                          uint32_t k6, uint32_t x)
+// floor(b * W / 2^c) for b <= 2^c <= 2^23
+__device__ __forceinline__ uint64_t range_start(uint64_t W, uint32_t b, uint32_t c)
 {
-    uint32_t c = k3 <= x ? 4u : 0u;
-    c += (c ? k5 : k1) <= x ? 2u : 0u;
-    const uint32_t kk = (c & 4u) ? ((c & 2u) ? k6 : k4) : ((c & 2u) ? k2 : k0);
-    return c + (kk <= x ? 1u : 0u);
+    const uint64_t lo = W * b, hi = __umul64hi(W, (uint64_t)b);
+    return c ? (hi << (64 - c)) | (lo >> c) : lo;
 }
 
-// First byte of a blocked row's summary (its top level): sector S of the
-// summary array SUM (SPLIT), or the S sectors before the row's blocks.
-template <bool SPLIT>
-__device__ __forceinline__ const unsigned char *summary_base(const EdgeN *E, const uint32_t *SUM, uint64_t begin,
-                                                             uint32_t S)
+// The sector of edge records (of the whole edge array) that holds the first
+// edge with P > x of a narrow overflow slot, counted from the slot's first.
+__device__ __forceinline__ uint32_t overflow_sector(const EdgeN *E, const Sector &s, uint32_t x, uint32_t &probes)
 {
-    if constexpr (SPLIT) return reinterpret_cast<const unsigned char *>(SUM + 8ull * S);
-    else return reinterpret_cast<const unsigned char *>(E + begin) - 32ull * S;
+    const uint32_t g = (s.v[1] <= x) + (s.v[2] <= x) + (s.v[3] <= x) + (s.v[7] <= x), nsec = s.v[6];
+    if (nsec <= kGroups) return g;  // one sector a group
+    const uint32_t gs = (nsec + kGroups - 1) / kGroups;
+    const uint64_t sec0 = (uint64_t)s.v[5] | ((uint64_t)(s.v[4] & 0xffu) << 32);
+    uint32_t a = g * gs, n = min(gs, nsec - a);
+    while (n > 1) {
+        const uint32_t half = n >> 1;
+        ++probes;
+        if (__ldg(&E[4 * (sec0 + a + half) - 1].P) <= x) {
+            a += half;
+            n -= half;
+        } else {
+            n = half;
+        }
+    }
+    return a;
 }
 
-// Search of a blocked narrow row (layout above) whose blocks start at record
-// `begin` of E, with summary field S and L summary levels: the target of the
-// first edge with P > x.  TALLY counts the 32-byte sectors read.
-template <bool TALLY, bool SPLIT>
-__device__ __forceinline__ uint32_t search_blocked(const EdgeN *E, const uint32_t *SUM, uint64_t begin, uint32_t d,
-                                                   uint32_t S, uint32_t L, uint32_t x, const NodeRecN *rec,
-                                                   uint32_t &sectors)
+// Code of the first record i >= first of a sector of edge records with P > x
+// (one of them is, by the choice of the sector).
+__device__ __forceinline__ uint32_t pick_record(const Sector &r, uint32_t first, uint32_t x)
 {
-    const unsigned char *base = summary_base<SPLIT>(E, SUM, begin, S);  // the row's top level
-    uint32_t b = 0, off = 0, l = L;
-    if (root_in_record(d, L)) {  // the top level (one sector) is ranked from the node record
-        const uint4 k = __ldg(reinterpret_cast<const uint4 *>(rec->key));
-        b = min(rank8(k.x, k.y, k.z, k.w, 0xffffffffu, 0xffffffffu, 0xffffffffu, x), (d - 1) >> (3 * L));
-        off = 1;
-        --l;
-    }
-    for (; l >= 1; --l) {
-        const Sector k = ld_sector(base + 32ull * (off + b));
-        const uint32_t c = rank8(k.v[0], k.v[1], k.v[2], k.v[3], k.v[4], k.v[5], k.v[6], x);
-        off += level_sectors(d, l);
-        b = b * 8 + c;
-        if (TALLY) ++sectors;
-    }
-    const uint32_t len = min(8u, d - 8 * b);
-    const unsigned char *q = reinterpret_cast<const unsigned char *>(E + begin) + 64ull * b;  // block b: (P, col) pairs
-    const Sector r0 = ld_block_sector<SPLIT>(q);
-    Sector r1;
-    if (len > 4) r1 = ld_block_sector<SPLIT>(q + 32);
-    else {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) r1.v[i] = 0xffffffffu;
-    }
-    if (TALLY) sectors += len > 4 ? 2 : 1;
-    // record i holds (P, col) in words 2i, 2i+1 of r0 (i < 4) or r1 (i >= 4)
-    const uint32_t c = rank8(r0.v[0], r0.v[2], r0.v[4], r0.v[6], r1.v[0], r1.v[2], r1.v[4], x);
-    const Sector &h = (c & 4u) ? r1 : r0;
-    const uint32_t lo = (c & 1u) ? h.v[3] : h.v[1], hi = (c & 1u) ? h.v[7] : h.v[5];
-    return (c & 2u) ? hi : lo;
-}
-
-// Same result, computed by the whole warp for one lane's search (all 32 lanes
-// must call it with the same arguments).  Each round splits the range into 32
-// parts, every lane reads the last key of one part and a ballot locates the
-// part holding the answer: ceil(log32 n) + 1 rounds instead of log2 n
-// dependent loads.
-template <class E>
-__device__ __forceinline__ typename E::Rec search_warp(const E &edges, uint64_t lo, uint32_t n, uint64_t x)
-{
-    const uint32_t lane = threadIdx.x & 31;
-    while (n > 32) {
-        uint32_t end_i = (uint32_t)(((uint64_t)(lane + 1) * n) >> 5);  // part i = [i*n/32, (i+1)*n/32)
-        uint32_t beg_i = (uint32_t)(((uint64_t)lane * n) >> 5);
-        bool above = true;
-        if (end_i > beg_i) above = E::key(edges.load(lo + end_i - 1)) > x;
-        uint32_t mask = __ballot_sync(0xffffffffu, above);
-        uint32_t f = __ffs(mask) - 1;  // mask != 0: the last part ends at n-1 whose key > x
-        uint32_t nb = (uint32_t)(((uint64_t)f * n) >> 5);
-        uint32_t ne = (uint32_t)(((uint64_t)(f + 1) * n) >> 5);
-        lo += nb;
-        n = ne - nb;
-    }
-    typename E::Rec v{};
-    bool above = false;
-    if (lane < n) {
-        v = edges.load(lo + lane);
-        above = E::key(v) > x;
-    }
-    uint32_t mask = __ballot_sync(0xffffffffu, above);
-    uint32_t f = __ffs(mask) - 1;
-    typename E::Rec r;
-    if constexpr (sizeof(typename E::Rec) == 8) {
-        r.x = __shfl_sync(0xffffffffu, v.x, f);
-        r.y = __shfl_sync(0xffffffffu, v.y, f);
-    } else {
-        r.x = __shfl_sync(0xffffffffu, v.x, f);
-        r.y = __shfl_sync(0xffffffffu, v.y, f);
-        r.z = __shfl_sync(0xffffffffu, v.z, f);
-        r.w = __shfl_sync(0xffffffffu, v.w, f);
-    }
-    return r;
+    const bool h0 = first == 0 && r.v[0] > x, h1 = first <= 1 && r.v[2] > x, h2 = first <= 2 && r.v[4] > x;
+    return h0 ? r.v[1] : (h1 ? r.v[3] : (h2 ? r.v[5] : r.v[7]));
 }
 
 // ----------------------------------------------------------- aggregation ----

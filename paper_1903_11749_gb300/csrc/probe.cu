@@ -24,7 +24,7 @@ __global__ void k_probe_philox(uint4 c0, uint32_t k0, uint32_t k1, int64_t count
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
         uint4 c = c0;
         c.x += (uint32_t)i;  // counter word 0 advances (mod 2^32)
-        out[i] = philox4x32_10(c, k0, k1);
+        out[i] = philox4x32_10(c, LaneKeys{k0, k1});
     }
 }
 
@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(256, 6) k_probe_philox_rate(uint32_t k0, uint3
     const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x;
     uint32_t acc = 0;
     for (int32_t j = 0; j < per_thread; ++j) {
-        const uint4 x = philox4x32_10(make_uint4(tid, (uint32_t)j, 0u, 0u), k0, k1);
+        const uint4 x = philox4x32_10(make_uint4(tid, (uint32_t)j, 0u, 0u), LaneKeys{k0, k1});
         acc ^= x.x ^ x.y ^ x.z;
     }
     if (acc == 0x9e3779b9u) atomicAdd(sink, 1ull);

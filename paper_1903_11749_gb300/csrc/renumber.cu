@@ -1,139 +1,241 @@
-// renumber.cu -- the walk layout's own node numbering for graphs far larger
-// than L2.
+// renumber.cu -- the walk layout's own node numbering.
 //
-// A walk with restart from every node visits node v at a rate proportional
-// to its PageRank (Sec. 2.1: the walks of all sources together follow the
-// random surfer with teleport alpha), which on a power-law graph is led by
-// its in-degree.  The layout numbers nodes in descending order of in-degree
-// (counted on every fourth edge; eight classes per power of two, ties in
-// input order), so the records and rows of the most visited nodes sit
-// together at the front of their arrays: their 32-byte sectors share
-// 128-byte L2 lines and DRAM pages instead of being spread over gigabytes.  The numbering is internal: sources, result
-// rows and top-k use the caller's ids, and the draw of a walk is keyed by the
-// caller's source id, so every count is the same with and without it.
-//   order[i]: caller id of internal node i;  rank[v]: internal id of caller node v.
+// Nodes are numbered class by class (ClassTab in ppr_internal.cuh: dangling,
+// single edge, degree, or the number of ranges 2^c of the row), because a
+// node's place within its class is then all a walk needs to find its slots.
+// Within a class they keep the caller's order.  (Descending in-degree order
+// within the classes, which packs the rows most walks pass, was measured:
+// R-MAT scale 24 walker 23.461 against 23.470 ms without it, alias 23.571
+// against 23.587, scale 22 21.581 against 21.589; with a slot a draw there is
+// no small hot record left to pack.)  The numbering is internal: sources,
+// result rows and top-k use the caller's ids, and the draw of a walk is keyed
+// by the caller's source id, so every count is the same under any numbering.
+//   order[seq]: caller id (within its instance);  code_of[v]: code of caller node v.
 #include "ppr_host.h"
 #include "scan.cuh"
 
 namespace ppr {
 
-constexpr int kRnBuckets = 1 + 32 * 8;  // in-degree 0, then 8 classes per power of two
-constexpr int kRnTile = 1024;           // nodes per warp tile of the counting sort
+struct NumberArgs {
+    int64_t n, m;
+    const int64_t *row_ptr;
+    uint32_t lam_bits;
+    bool wide, exact;
+    int64_t tiles;
+    uint32_t tile;          // nodes a warp takes
+    uint32_t *hist;         // [class][tile]
+    uint64_t *off;          // its exclusive scan
+    uint32_t *heads;        // bit e: a row starts at edge e
+    LayoutStats *st;
+    const int64_t *node_off;
+    int32_t count;
+    int32_t *order;
+    uint32_t *code_of;
+};
 
-// In-degree of every node, counted on every kRnEvery-th edge (the ordering
-// needs the classes of the well-visited nodes, whose counts a quarter of the
-// edges already fixes to within a class or two; the atomics, not the read,
-// set this kernel's time).  Edges whose target lies outside [0, n) are
-// skipped (the layout build reports them).  Equal targets within a warp are
-// summed first, so a hub takes one atomic per warp and not one per edge.
-constexpr int64_t kRnEvery = 4;
-
-__global__ void __launch_bounds__(256) k_rn_indegree(int64_t n, int64_t m, const int32_t *col, uint32_t *indeg)
+// Degree of caller row v, 0 (and a flag) when its row_ptr is invalid.
+__device__ __forceinline__ uint32_t checked_degree(const NumberArgs &A, int64_t v, int64_t &a, uint32_t &flags)
 {
-    const uint32_t lane = threadIdx.x & 31;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const int64_t ms = (m + kRnEvery - 1) / kRnEvery;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < ms; base += stride) {
-        const int64_t e = (base + threadIdx.x) * kRnEvery;
-        int32_t c = -1;
-        if (e < m) c = col[e];
-        const bool ok = c >= 0 && (int64_t)c < n;
-        const uint32_t key = ok ? (uint32_t)c : 0xffffffffu;
-        const uint32_t peers = __match_any_sync(0xffffffffu, key);
-        if (ok && lane == (uint32_t)(__ffs(peers) - 1)) atomicAdd(&indeg[c], (uint32_t)__popc(peers));
+    a = A.row_ptr[v];
+    const int64_t b = A.row_ptr[v + 1];
+    if (a < 0 || b < a || b > A.m || (v == 0 && a != 0) || (v == A.n - 1 && b != A.m)) {
+        flags |= kBadRowPtr;
+        return 0;
     }
+    if (b - a > PPR_MAX_DEGREE) {
+        flags |= kBigDegree;
+        return 0;
+    }
+    return (uint32_t)(b - a);
 }
 
-// Class of an in-degree: 0 for none, else 1 + 8 * floor(log2 c) + the three
-// bits after the leading one.  Placed in descending class order.
-__device__ __forceinline__ uint32_t rn_slot(uint32_t c)
+__device__ __forceinline__ uint32_t node_class(const NumberArgs &A, uint32_t d)
 {
-    if (c == 0) return kRnBuckets - 1;
-    const uint32_t lg = 31u - __clz(c);
-    const uint32_t frac = lg >= 3 ? (c >> (lg - 3)) & 7u : (c << (3 - lg)) & 7u;
-    return (uint32_t)(kRnBuckets - 1) - (1u + 8u * lg + frac);
+    return class_of_degree(d, A.lam_bits, A.wide, A.exact);
 }
 
-// Per-tile class counts, class-major: hist[slot * tiles + tile].
-__global__ void __launch_bounds__(256) k_rn_hist(int64_t n, const uint32_t *indeg, uint32_t *hist, int64_t tiles)
+// Per-tile class counts; row starts and degree statistics.  Four warps a
+// block, one tile a warp.
+__global__ void __launch_bounds__(128) k_rn_hist(NumberArgs A)
 {
-    __shared__ uint32_t h[8][kRnBuckets];
+    __shared__ uint32_t h_all[4 * kClasses];
     const uint32_t wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t tile = (int64_t)blockIdx.x * 8 + wid;
-    for (uint32_t i = lane; i < (uint32_t)kRnBuckets; i += 32) h[wid][i] = 0;
+    uint32_t *h = h_all + wid * kClasses;
+    const int64_t t = (int64_t)blockIdx.x * 4 + wid;
+    for (uint32_t i = lane; i < kClasses; i += 32) h[i] = 0;
     __syncwarp();
-    if (tile < tiles) {
-        for (uint32_t r = 0; r < (uint32_t)kRnTile; r += 32) {
-            const int64_t v = tile * kRnTile + r + lane;
-            if (v < n) atomicAdd(&h[wid][rn_slot(indeg[v])], 1u);
+    uint32_t dmax = 0, dang = 0, flags = 0;
+    if (t < A.tiles) {
+        for (uint32_t r = 0; r < A.tile; r += 32) {
+            const int64_t v = t * A.tile + r + lane;
+            uint32_t key = 0xffffffffu;
+            if (v < A.n) {
+                int64_t a;
+                const uint32_t d = checked_degree(A, v, a, flags);
+                dmax = max(dmax, d);
+                dang += d == 0;
+                key = node_class(A, d);
+                if (d) atomicOr(&A.heads[a >> 5], 1u << (a & 31));
+            }
+            const uint32_t peers = __match_any_sync(0xffffffffu, key);
+            if (v < A.n && lane == (uint32_t)(__ffs(peers) - 1)) h[key] += __popc(peers);
+            __syncwarp();
         }
-        __syncwarp();
-        for (uint32_t i = lane; i < (uint32_t)kRnBuckets; i += 32) hist[(int64_t)i * tiles + tile] = h[wid][i];
+        for (uint32_t i = lane; i < kClasses; i += 32) A.hist[(int64_t)i * A.tiles + t] = h[i];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        dmax = max(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
+        dang += __shfl_xor_sync(0xffffffffu, dang, o);
+        flags |= __shfl_xor_sync(0xffffffffu, flags, o);
+    }
+    if (lane == 0) {
+        if (dmax) atomicMax(&A.st->max_degree, (unsigned long long)dmax);
+        if (dang) atomicAdd(&A.st->dangling, (unsigned long long)dang);
+        if (flags) atomicOr(&A.st->status, flags);
     }
 }
 
-// Stable scatter: node v of tile t goes to off[slot * tiles + t] plus the
-// number of earlier nodes of the tile in its class.
-__global__ void __launch_bounds__(256) k_rn_scatter(int64_t n, const uint32_t *indeg, const uint64_t *off,
-                                                    int64_t tiles, int32_t *order, int32_t *rank)
+// What the host needs to lay the classes out: the statistics and each class's first seq.
+struct ClassStarts {
+    LayoutStats st;
+    uint64_t start[kClasses + 1];
+};
+
+__global__ void k_rn_starts(NumberArgs A, ClassStarts *out)
 {
-    __shared__ uint32_t seen[8][kRnBuckets];
+    const uint32_t i = threadIdx.x;
+    if (i <= kClasses) out->start[i] = A.off[(int64_t)i * A.tiles];
+    if (i == 0) out->st = *A.st;
+}
+
+struct ClassEntries {
+    uint32_t e0[kClasses];  // first table entry of each class
+    uint32_t start[kClasses];
+};
+
+// Stable scatter: node v of tile t goes to off[class][t] plus the number of
+// earlier nodes of the tile in its class.
+__global__ void __launch_bounds__(128) k_rn_scatter(NumberArgs A, ClassEntries C)
+{
+    __shared__ uint32_t seen_all[4 * kClasses];
     const uint32_t wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t tile = (int64_t)blockIdx.x * 8 + wid;
-    for (uint32_t i = lane; i < (uint32_t)kRnBuckets; i += 32) seen[wid][i] = 0;
+    uint32_t *seen = seen_all + wid * kClasses;
+    const int64_t t = (int64_t)blockIdx.x * 4 + wid;
+    for (uint32_t i = lane; i < kClasses; i += 32) seen[i] = 0;
     __syncwarp();
-    if (tile >= tiles) return;
-    for (uint32_t r = 0; r < (uint32_t)kRnTile; r += 32) {
-        const int64_t v = tile * kRnTile + r + lane;
-        const uint32_t s = v < n ? rn_slot(indeg[v]) : 0xffffffffu;
-        const uint32_t peers = __match_any_sync(0xffffffffu, s);
+    if (t >= A.tiles) return;
+    for (uint32_t r = 0; r < A.tile; r += 32) {
+        const int64_t v = t * A.tile + r + lane;
+        uint32_t key = 0xffffffffu;
+        if (v < A.n) {
+            int64_t a;
+            uint32_t flags = 0;
+            key = node_class(A, checked_degree(A, v, a, flags));
+        }
+        const uint32_t peers = __match_any_sync(0xffffffffu, key);
         const uint32_t before = __popc(peers & ((1u << lane) - 1));
         uint32_t base = 0;
-        if (v < n) base = seen[wid][s];
+        if (v < A.n) base = seen[key];
         __syncwarp();
-        if (v < n) {
-            const int64_t pos = (int64_t)off[(int64_t)s * tiles + tile] + base + before;
-            order[pos] = (int32_t)v;
-            rank[v] = (int32_t)pos;
-            if (before == 0) seen[wid][s] = base + __popc(peers);
+        if (v < A.n) {
+            const uint32_t seq = (uint32_t)A.off[(int64_t)key * A.tiles + t] + base + before, idx = seq - C.start[key];
+            int64_t id = v;
+            if (A.count > 0) {  // the id within its instance
+                int32_t lo = 0, hi = A.count;
+                while (hi - lo > 1) {
+                    const int32_t mid = (lo + hi) >> 1;
+                    if (A.node_off[mid] <= v) lo = mid;
+                    else hi = mid;
+                }
+                id -= A.node_off[lo];
+            }
+            A.order[seq] = (int32_t)id;
+            A.code_of[v] = ((C.e0[key] + (idx >> kIdxBits)) << kIdxBits) | (idx & kIdxMask);
+            if (before == 0) seen[key] = base + __popc(peers);
         }
         __syncwarp();
     }
 }
 
-// order and rank (n int32 each, device) for the CSR col[0..m); scratch goes
-// to tmp (freed by the caller).  Enqueued on st.
-int renumber_by_indegree(ppr_ctx *ctx, int64_t n, int64_t m, const int32_t *d_col, cudaStream_t st, int32_t *order,
-                         int32_t *rank, std::vector<void *> &tmp)
+int number_nodes(int64_t n, int64_t m, const int64_t *d_rp, const int64_t *d_off, uint32_t *heads,
+                 LayoutStats *d_stats, bool wide, cudaStream_t st, ppr_graph *g, std::vector<void *> &tmp)
 {
-    Range range("renumber");
+    Range range("number nodes");
     int rc;
-    const int64_t tiles = (n + kRnTile - 1) / kRnTile;
-    const int64_t cells = tiles * kRnBuckets;
-    uint32_t *indeg, *hist;
-    uint64_t *off, *scan_tmp;
-    if ((rc = dev_alloc((void **)&indeg, sizeof(uint32_t) * n, "in-degrees", st))) return rc;
-    tmp.push_back(indeg);
-    if ((rc = dev_alloc((void **)&hist, sizeof(uint32_t) * cells, "class counts", st))) return rc;
-    tmp.push_back(hist);
-    if ((rc = dev_alloc((void **)&off, sizeof(uint64_t) * (cells + 1), "class offsets", st))) return rc;
-    tmp.push_back(off);
+    NumberArgs A{};
+    A.n = n;
+    A.m = m;
+    A.row_ptr = d_rp;
+    A.lam_bits = g->lam_bits;
+    A.wide = wide;
+    A.exact = g->instances == 0 && n > kExactMin && n <= kExactNodes;
+    // nodes a warp takes in turn: few where the graph is small (a warp's chain
+    // of rounds is then the kernel's time)
+    A.tile = n <= (1 << 18) ? 128u : 1024u;
+    A.tiles = (n + A.tile - 1) / A.tile;
+    A.heads = heads;
+    A.st = d_stats;
+    A.node_off = d_off;
+    A.count = g->instances;
+    A.order = g->order;
+    A.code_of = g->code_of;
+    const int64_t cells = A.tiles * kClasses;
+    uint64_t *scan_tmp;
+    ClassStarts *d_cs;
+    if ((rc = dev_alloc((void **)&A.hist, sizeof(uint32_t) * cells, "class counts", st))) return rc;
+    tmp.push_back(A.hist);
+    if ((rc = dev_alloc((void **)&A.off, sizeof(uint64_t) * (cells + 1), "class offsets", st))) return rc;
+    tmp.push_back(A.off);
     if ((rc = dev_alloc((void **)&scan_tmp, sizeof(uint64_t) * ((cells + kScanTile - 1) / kScanTile + 2), "scan scratch",
                         st)))
         return rc;
     tmp.push_back(scan_tmp);
-    PPR_CUDA(cudaMemsetAsync(indeg, 0, sizeof(uint32_t) * n, st));
-    if (m > 0) {
-        const int64_t ms = (m + kRnEvery - 1) / kRnEvery;
-        const int eb = (int)std::max<int64_t>(1, std::min<int64_t>((ms + 255) / 256, (int64_t)ctx->sms * 32));
-        k_rn_indegree<<<eb, 256, 0, st>>>(n, m, d_col, indeg);
-        note_launch();
-    }
-    const int tb = (int)((tiles + 7) / 8);
-    k_rn_hist<<<tb, 256, 0, st>>>(n, indeg, hist, tiles);
+    if ((rc = dev_alloc((void **)&d_cs, sizeof(ClassStarts), "class starts", st))) return rc;
+    tmp.push_back(d_cs);
+    const unsigned tb = (unsigned)((A.tiles + 3) / 4);
+    k_rn_hist<<<tb, 128, 0, st>>>(A);
     note_launch();
-    exclusive_scan_u32(hist, cells, off, scan_tmp, st);
-    k_rn_scatter<<<tb, 256, 0, st>>>(n, indeg, off, tiles, order, rank);
+    exclusive_scan_u32(A.hist, cells, A.off, scan_tmp, st);
+    k_rn_starts<<<1, 64, 0, st>>>(A, d_cs);
+    note_launch();
+    ClassStarts cs;
+    PPR_CUDA(cudaMemcpyAsync(&cs, d_cs, sizeof(cs), cudaMemcpyDeviceToHost, st));
+    PPR_CUDA(cudaStreamSynchronize(st));
+    if (cs.st.status & kBadRowPtr) {
+        set_error("row_ptr must start at 0, be non-decreasing and end at m");
+        return PPR_EINVAL;
+    }
+    if (cs.st.status & kBigDegree) {
+        set_error("an out-degree exceeds the limit %lld", (long long)PPR_MAX_DEGREE);
+        return PPR_ERANGE;
+    }
+    g->max_degree = (int64_t)cs.st.max_degree;
+    g->dangling = (int64_t)cs.st.dangling;
+    ClassEntries C{};
+    ClassTab &T = g->htab;
+    uint32_t e = 0;
+    g->n_slots = g->n_single = 0;
+    for (uint32_t c = 0; c < kClasses; ++c) {
+        C.e0[c] = e;
+        C.start[c] = (uint32_t)cs.start[c];
+        for (uint64_t at = cs.start[c]; at < cs.start[c + 1]; at += 1ull << kIdxBits, ++e) {
+            const uint64_t cnt = std::min<uint64_t>(cs.start[c + 1] - at, 1ull << kIdxBits);
+            T.e[e] = TabEntry{0, kKindDangling, (uint32_t)at};
+            g->degree[e] = c <= kExact ? c : 0;
+            if (c == 1) {
+                T.e[e].kind = kKindSingle;
+                T.e[e].addr = sizeof(uint32_t) * (uint64_t)g->n_single;
+                g->n_single += (int64_t)cnt;
+            } else if (c >= 2) {
+                T.e[e].kind = c <= kExact ? ranges_log2(c, g->lam_bits, wide) : c - kExact - 1;
+                T.e[e].addr = sizeof(Sector) * (uint64_t)g->n_slots;
+                g->n_slots += (int64_t)(cnt << T.e[e].kind);
+            }
+        }
+    }
+    for (; e < kTabEntries; ++e) T.e[e] = TabEntry{0, kKindDangling, 0xffffffffu};
+    k_rn_scatter<<<tb, 128, 0, st>>>(A, C);
     note_launch();
     PPR_CUDA(cudaGetLastError());
     return PPR_OK;

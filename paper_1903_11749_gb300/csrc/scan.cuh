@@ -94,6 +94,29 @@ static __global__ void k_scan_apply(const uint32_t *in, int64_t n, const uint64_
     if (n > 0 && base <= n - 1 && n - 1 < base + kScanItems) out[n] = ex;  // holder of element n-1 writes the total
 }
 
+// One block scans up to kScanTile counts in one launch (the three passes cost
+// two more launches, which small graphs feel: each is a few microseconds).
+static __global__ void __launch_bounds__(kScanThreads) k_scan_one(const uint32_t *in, int64_t n, uint64_t *out)
+{
+    __shared__ uint64_t wt[32];
+    __shared__ uint64_t tot;
+    const int64_t base = (int64_t)threadIdx.x * kScanItems;
+    uint32_t v[kScanItems];
+    uint64_t s = 0;
+#pragma unroll
+    for (int i = 0; i < kScanItems; ++i) {
+        v[i] = base + i < n ? in[base + i] : 0u;
+        s += v[i];
+    }
+    uint64_t ex = block_exclusive_scan(s, wt, &tot);
+#pragma unroll
+    for (int i = 0; i < kScanItems; ++i) {
+        if (base + i < n) out[base + i] = ex;
+        ex += v[i];
+    }
+    if (threadIdx.x == 0) out[n] = tot;
+}
+
 // out[0..n] = exclusive scan of in[0..n), out[n] = total.  tmp needs
 // ceil(n / kScanTile) + 1 uint64.  Enqueued on st.
 inline void exclusive_scan_u32(const uint32_t *in, int64_t n, uint64_t *out, uint64_t *tmp, cudaStream_t st)
@@ -101,6 +124,11 @@ inline void exclusive_scan_u32(const uint32_t *in, int64_t n, uint64_t *out, uin
     int64_t tiles = (n + kScanTile - 1) / kScanTile;
     if (n == 0) {
         cudaMemsetAsync(out, 0, sizeof(uint64_t), st);
+        return;
+    }
+    if (tiles == 1) {
+        k_scan_one<<<1, kScanThreads, 0, st>>>(in, n, out);
+        note_launch();
         return;
     }
     k_scan_tile_sums<<<(unsigned)tiles, kScanThreads, 0, st>>>(in, n, tmp);

@@ -111,7 +111,7 @@ struct SGlob {  // device memory, persists across launches of the loop
 };
 
 struct LoopParams {
-    KParams kp;  // the graph layout (node, edges, n_nodes, n_records); dangling mode 0, no segments
+    KParams kp;  // the graph layout (set_layout); dangling mode 0, no segments
     const SDesc *desc;
     SSlot *slot;
     SCtl *ctl;   // device view of the host-mapped control block
@@ -338,16 +338,17 @@ __device__ __forceinline__ void count_walks(const LoopParams &P, uint32_t q, uin
     if (old + n == __ldcg(&P.desc[q].walks)) P.slot[q].t_walks = gtime_ns();
 }
 
-template <class E, bool SPLIT>
-__device__ void walker_warp(const LoopParams &P, WalkChunk &wc, uint32_t **ends_of, uint32_t gwarp,
-                            unsigned long long *s_tail)
+template <class E>
+__device__ void walker_warp(const LoopParams &P, const ClassTab &tab, WalkChunk &wc, uint32_t **ends_of,
+                            uint32_t gwarp, unsigned long long *s_tail)
 {
     const uint32_t lane = threadIdx.x & 31;
-    const E edges = make_edges<E>(P.kp.edges);
     bool active = false;
     uint32_t q = 0, g = 0, src = 0, j = 0, k = 0, u = 0;
-    uint32_t s0 = 0;  // the walk's start (and restart) node in the layout's numbering
-    StepKey key{0, 0, 0};
+    uint32_t s0 = 0;  // code of the walk's start (and restart) node
+    Pending pend;
+    LaneKeys key{0, 0};
+    uint32_t T = 0;
     uint32_t pend_q = 0xffffffffu, pend_n = 0;  // uniform: walks of pend_q finished, not yet counted
     bool have = false;                          // uniform: wc holds walks left to issue
     uint64_t idle_t0 = 0, flush_t = gtime_ns(), claim_after = 0;
@@ -418,9 +419,10 @@ __device__ void walker_warp(const LoopParams &P, WalkChunk &wc, uint32_t **ends_
                 const uint32_t pos = (uint32_t)(((uint64_t)g * wc.magic) >> 40);
                 j = g - pos * wc.R;
                 src = __ldcg(wc.src + pos);  // the caller's id keys the draws
-                s0 = P.kp.rank ? (uint32_t)P.kp.rank[src] : src;
+                s0 = P.kp.code_of[src];
                 q = wc.slot;
-                key = StepKey{wc.k0, wc.k1, wc.T};
+                key = LaneKeys{wc.k0, wc.k1};
+                T = wc.T;
                 k = 0;
                 u = s0;
                 active = true;
@@ -460,11 +462,11 @@ __device__ void walker_warp(const LoopParams &P, WalkChunk &wc, uint32_t **ends_
                 flush_t = t;
             }
         }
-        uint32_t end = 0;
         bool fin = false;
         const long long c0 = clock64();
-        if (walk_step<E, false, false, false, SPLIT>(P.kp, key, edges, active, s0, src, j, 0, k, u, end, tl)) {
-            ends_of[q][g] = end;
+        if (active && walk_step<E, false, false>(P.kp, tab, key, T, s0, src, j, 0, k, u, pend, tl)) {
+            ends_of[q][g] = u;
+            tl.steps += k;
             active = false;
             fin = true;
         }
@@ -594,7 +596,8 @@ __device__ int claim_source(const LoopParams &P, unsigned long long *s_tail, boo
 
 // Reduction of source i of query slot s into its top-k row (host memory).
 // smem: cap endpoints, then the reduction's scratch (3 * cap words); cap >= R.
-__device__ void reduce_source(const LoopParams &P, uint32_t s, uint32_t i, uint32_t *smem, uint32_t cap)
+__device__ void reduce_source(const LoopParams &P, const CallerIds &ids, uint32_t s, uint32_t i, uint32_t *smem,
+                              uint32_t cap)
 {
     const uint32_t lane = threadIdx.x & 31;
     const SDesc *d = P.desc + s;
@@ -605,7 +608,7 @@ __device__ void reduce_source(const LoopParams &P, uint32_t s, uint32_t i, uint3
     o.topk_cnt = reinterpret_cast<uint32_t *>(__ldcg(reinterpret_cast<const unsigned long long *>(&d->out_cnt)));
     o.topk = (int32_t)topk;
     uint32_t *e = smem;  // the endpoints, read past L1 (the arena is reused by later queries)
-    for (uint32_t r = lane; r < R; r += 32) e[r] = caller_id(P.kp.order, __ldcg(ends + (uint64_t)i * R + r));
+    for (uint32_t r = lane; r < R; r += 32) e[r] = ids(__ldcg(ends + (uint64_t)i * R + r));
     __syncwarp();
     uint32_t *scratch = smem + cap;
     switch (P2) {
@@ -636,7 +639,7 @@ __device__ void finish_source(const LoopParams &P, uint64_t id, uint32_t s, uint
     }
 }
 
-__device__ void aggregator_warp(const LoopParams &P, uint32_t *smem, unsigned long long *s_tail)
+__device__ void aggregator_warp(const LoopParams &P, const CallerIds &ids, uint32_t *smem, unsigned long long *s_tail)
 {
     const uint32_t lane = threadIdx.x & 31;
     uint64_t idle_t0 = 0, busy_t0 = 0;
@@ -649,7 +652,7 @@ __device__ void aggregator_warp(const LoopParams &P, uint32_t *smem, unsigned lo
         const int r = claim_source(P, s_tail, refresh, kLoopMaxR, id, s, i, nb, in_flight);
         if (r < 0) break;
         if (r > 0) {
-            for (uint32_t b = 0; b < nb; ++b) reduce_source(P, s, i + b, smem, kLoopMaxR);
+            for (uint32_t b = 0; b < nb; ++b) reduce_source(P, ids, s, i + b, smem, kLoopMaxR);
             finish_source(P, id, s, nb);
             idle_t0 = busy_t0 = 0;
             backoff = 256;
@@ -683,22 +686,24 @@ __device__ void aggregator_warp(const LoopParams &P, uint32_t *smem, unsigned lo
     }
 }
 
-// SPLIT: the narrow layout of a renumbered graph (see search_blocked)
-template <class E, bool SPLIT = false>
+template <class E>
 __global__ void __launch_bounds__(32 * kLoopWarps, 4) k_serve_loop(LoopParams P)
 {
     __shared__ WalkChunk wc[kLoopWarps - 1];
     __shared__ uint32_t *ends_of[kRing];  // endpoint array of each slot, set by the warp that takes a chunk of it
     __shared__ __align__(16) uint32_t smem[kLoopMaxR + 3 * kLoopMaxR];  // the aggregator warp's endpoints and scratch
     __shared__ unsigned long long s_tail[2];  // the block's copy of the published tail, and when it was read
+    __shared__ ClassTab tab;
+    __shared__ uint32_t s_first[kTabEntries];
+    for (uint32_t i = threadIdx.x; i < kTabEntries; i += blockDim.x) s_first[i] = P.kp.tab->e[i].first;
     if (threadIdx.x == 0) s_tail[0] = s_tail[1] = 0;
-    __syncthreads();
+    load_tab(tab, P.kp.tab);
     const uint32_t wid = threadIdx.x >> 5;
     if (wid == kLoopWarps - 1) {
-        aggregator_warp(P, smem, s_tail);
+        aggregator_warp(P, CallerIds{P.kp.order, s_first}, smem, s_tail);
         return;
     }
-    walker_warp<E, SPLIT>(P, wc[wid], ends_of, blockIdx.x * (kLoopWarps - 1) + wid, s_tail);
+    walker_warp<E>(P, tab, wc[wid], ends_of, blockIdx.x * (kLoopWarps - 1) + wid, s_tail);
 }
 
 // ============================================================ queries ====
@@ -942,20 +947,12 @@ static void scheduler_streams(Server *sv)
 
 // ---------------------------------------------------------- device loop ----
 
-template <class E, bool SPLIT = false>
+template <class E>
 static int launch_loop_typed(Server *sv)
 {
     const ppr_graph *g = sv->g;
     LoopParams P{};
-    P.kp.node = sv->cfg.sampler == 1 ? (const void *)g->alias.node : g->node;
-    P.kp.edges = sv->cfg.sampler == 1 ? (const void *)g->alias.slots : g->edges;
-    P.kp.large = 0xffffffffu;
-    P.kp.n_nodes = g->n;
-    P.kp.rank = g->rank;
-    P.kp.order = g->order;
-    P.kp.n_records = sv->cfg.sampler == 1 ? (uint64_t)g->m : (uint64_t)g->edge_records;
-    P.kp.sum = g->sum_base();
-    P.kp.n_sum = g->sum_extent();
+    set_layout(P.kp, g, false, sv->cfg.sampler == 1);
     P.kp.err = &sv->d_glob->err;
     P.desc = sv->d_desc;
     P.slot = sv->d_slot;
@@ -965,11 +962,11 @@ static int launch_loop_typed(Server *sv)
     P.idle_ns = (uint64_t)(sv->cfg.idle_us > 0 ? sv->cfg.idle_us : 200000) * 1000ull;
     if (!sv->grid) {
         int per_sm = 0;
-        PPR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_serve_loop<E, SPLIT>, 32 * kLoopWarps, 0));
+        PPR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_serve_loop<E>, 32 * kLoopWarps, 0));
         sv->grid = (uint32_t)(sv->ctx->sms * std::max(per_sm, 1));
     }
     P.walker_warps = sv->grid * (kLoopWarps - 1);
-    k_serve_loop<E, SPLIT><<<sv->grid, 32 * kLoopWarps, 0, sv->loop_stream>>>(P);
+    k_serve_loop<E><<<sv->grid, 32 * kLoopWarps, 0, sv->loop_stream>>>(P);
     note_launch();
     PPR_CUDA(cudaGetLastError());
     PPR_CUDA(cudaEventRecord(sv->loop_done, sv->loop_stream));
@@ -982,7 +979,6 @@ static int launch_loop(Server *sv)
     int rc;
     if (sv->cfg.sampler == 1) rc = launch_loop_typed<AliasEdges>(sv);
     else if (sv->g->wide) rc = launch_loop_typed<WideEdges>(sv);
-    else if (sv->g->sum) rc = launch_loop_typed<NarrowEdges, true>(sv);
     else rc = launch_loop_typed<NarrowEdges>(sv);
     if (rc == PPR_OK) {
         sv->loop_running = true;
@@ -1452,13 +1448,11 @@ int ppr_submit(ppr_ctx *ctx, const int32_t *srcs, int64_t ns, double alpha, uint
     q->plan.dangling = 0;
     q->plan.segments = false;
     q->plan.kernel = PPR_KERNEL_PERSISTENT;
-    q->plan.large_degree = sv->cfg.large_degree;
     q->plan.warps_per_block = sv->cfg.warps_per_block;
     q->plan.refill_lanes = sv->cfg.refill_lanes;
     q->plan.chunk_sources = sv->cfg.chunk_sources;
     q->plan.sampler = sv->cfg.sampler;
     q->plan.stats = false;
-    q->plan.step_loads = kDefaultStepLoads;
     q->topk = topk;
     const uint32_t cap = (uint32_t)std::min<int64_t>((int64_t)R, sv->g->n);
     q->bytes = loop ? loop_dev_bytes(ns, R) : query_bytes(sv->g, q->plan, ns, topk, cap);

@@ -3,8 +3,7 @@
 // k_walk_plain:      one thread per walk, endpoint to HBM (baseline).
 // k_walk_persistent: persistent warps pull chunks of walks from a global
 //                    queue and refill lanes as walks end (the paper's
-//                    pipelines keep the cluster busy the same way); rows above
-//                    a set degree may be searched by the whole warp.
+//                    pipelines keep the cluster busy the same way).
 // Both write one endpoint per walk to HBM; k_aggregate (aggregate.cuh) then
 // turns each source's R endpoints into its count row and top-k.
 #include <algorithm>
@@ -38,14 +37,24 @@ __device__ __forceinline__ void warp_add_tally(unsigned long long *dst, const Ta
 }
 
 // ------------------------------------------------------------ plain (K4) ----
-#ifndef PPR_WALK_MINB
-#define PPR_WALK_MINB 6  // resident 256-thread blocks per SM asked of ptxas (6: 40 registers, no spills)
-#endif
+// Resident 256-thread blocks per SM asked of ptxas.  Narrow: 6 (40 registers;
+// 8 blocks at 32 gain nothing on the batch and lose 7 % on a small query).
+// Wide: 8 (R-MAT scale 18 with amounts as weights: 2.20 -> 2.08 ms).  Alias: 6 (R-MAT
+// scale 24, 2^22 sources: 20.4 ms; 8 blocks 21.4: more walks at once, fewer L2 hits).
+// Idle lanes before a warp starts new walks, unless the caller says: starting
+// them costs the whole warp some forty instructions (256-graph batch 17.6 ms
+// at one lane, 17.0 at four, 16.9 at eight, 17.9 at sixteen; the scale-24 and
+// scale-20 walkers, which wait for memory, are level from one to eight).
+constexpr uint32_t kDefaultRefill = 8;
 
-template <class E, bool SEG, bool STATS, bool SPLIT = false>
-__global__ void __launch_bounds__(256, PPR_WALK_MINB) k_walk_plain(KParams p)
+template <class E>
+constexpr int kWalkBlocks = std::is_same<E, WideEdges>::value ? 8 : 6;
+
+template <class E, bool SEG, bool STATS>
+__global__ void __launch_bounds__(256, kWalkBlocks<E>) k_walk_plain(KParams p)
 {
-    const E edges = make_edges<E>(p.edges);
+    __shared__ ClassTab tab;
+    load_tab(tab, p.tab);
     const uint64_t S = (uint64_t)(p.s_end - p.s_begin);
     const uint64_t total = S * p.R;
     Tally tl;
@@ -67,30 +76,31 @@ __global__ void __launch_bounds__(256, PPR_WALK_MINB) k_walk_plain(KParams p)
         }
         // the draw is keyed by the caller's source id; the walk starts (and
         // restarts) at its node of the layout
-        const uint32_t s0 = p.rank ? (uint32_t)p.rank[src] : src;
-        uint32_t k = 0, u = s0, end = 0;
-        while (!walk_step<E, SEG, false, STATS, SPLIT>(p, StepKey{p.k0, p.k1, p.T}, edges, true, s0, src - ctr_base, j,
-                                                        tag, k, u, end, tl)) {
+        const uint32_t s0 = p.code_of[src];
+        uint32_t k = 0, u = s0;
+        Pending pend;
+        while (!walk_step<E, SEG, STATS>(p, tab, p.key, p.T, s0, src - ctr_base, j, tag, k, u, pend, tl)) {
         }
-        p.ends[t] = end - ctr_base;
+        if (!SEG) tl.steps += k;
+        p.ends[t] = u;
     }
     warp_add_tally<STATS>(p.steps, tl);
 }
 
 // ------------------------------------------------------- persistent (K5) ----
-// Persistent warps.  Each warp pulls chunks of sources from a global queue
-// (one atomic per chunk) and keeps all 32 lanes busy: a lane whose walk ends
-// takes the next walk of the warp's chunk at once, so a warp never waits for
-// the longest of 32 geometric walk lengths (the paper's pipelines keep the
-// cluster busy the same way: new walks start while old ones finish).  Steps
-// run in lockstep; a row longer than p.large can be searched by the whole
-// warp (search_warp).  Endpoints go to the per-walk buffer, reduced per
-// source by k_aggregate.  The walker uses no shared memory beyond the queue
-// state, so L1 keeps its full size.
-struct WarpQueue {
-    uint32_t base, ctr_base, tag;  // current chunk: first position, counter base, tag
+// Persistent warps.  Each warp pulls chunks of walks from a global queue (one
+// atomic per chunk) and keeps all 32 lanes busy: a lane whose walk ends takes
+// the next walk of the warp's chunk at once, so a warp never waits for the
+// longest of 32 geometric walk lengths (the paper's pipelines keep the cluster
+// busy the same way: new walks start while old ones finish).  Walks start in
+// order, so those of one source start close together and share the loads of
+// its row (with walks dealt out to lanes in advance, l, l + 32, ..., lanes
+// drift apart and the scale-24 walker took 120 ms, not 93).  Steps run in
+// lockstep, one load each (walk_step).  Endpoints go to the per-walk buffer as
+// node codes, reduced per source by k_aggregate.
+struct WarpChunk {
+    uint32_t base, ctr_base, tag;  // first position, counter base, tag
     uint32_t j0;                   // walk index (within source `base`) of the chunk's first walk
-    uint32_t issued, total;
 };
 
 __device__ __forceinline__ uint32_t div_by_R(uint32_t w, uint64_t magic)
@@ -98,103 +108,81 @@ __device__ __forceinline__ uint32_t div_by_R(uint32_t w, uint64_t magic)
     return (uint32_t)(((uint64_t)w * magic) >> 40);  // exact for w < 2^20, R <= 4096
 }
 
-template <class E, bool SEG, bool STATS, bool BOUNDED = false, bool SPLIT = false>
-__global__ void __launch_bounds__(256, PPR_WALK_MINB) k_walk_persistent(KParams p)
+template <class E, bool SEG, bool STATS>
+__global__ void __launch_bounds__(256, kWalkBlocks<E>) k_walk_persistent(KParams p)
 {
-    __shared__ WarpQueue wq_all[8];
-    __shared__ uint32_t ps_all[BOUNDED ? 8 * 256 : 1];  // bounded step: each lane's pending search
-    const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    WarpQueue &wq = wq_all[wid];
-    const E edges = make_edges<E>(p.edges);
-    if (lane == 0) {
-        wq.issued = 0;
-        wq.total = 0;
-    }
-    __syncwarp();
-    bool queue_empty = false;
+    __shared__ WarpChunk chunk_all[8];
+    __shared__ ClassTab tab;
+    load_tab(tab, p.tab);
+    const uint32_t lane = threadIdx.x & 31;
+    WarpChunk &wc = chunk_all[threadIdx.x >> 5];
+    uint32_t issued = 0, total = 0;  // uniform: walks of the chunk handed out, and its walks
+    bool queue_empty = false;        // uniform
     bool active = false;
-    uint32_t src = 0, sctr = 0, j = 0, k = 0, u = 0, tag = 0, ctr_base = 0;
-    uint64_t slot = 0;  // endpoint index: (src - s_begin) * R + j
-    bool pend = false;  // bounded step: this lane's draw has a search in progress
+    uint32_t src = 0, sctr = 0, j = 0, k = 0, u = 0, tag = 0, pos = 0;
+    Pending pend;
     Tally tl;
 
     for (;;) {
         uint32_t idle = __ballot_sync(0xffffffffu, !active);
         // refill once p.refill lanes are idle, then every idle lane
-        if ((uint32_t)__popc(idle) < p.refill) idle = 0;
-        while (idle && !queue_empty) {
-            if (wq.issued == wq.total) {
-                unsigned long long c = 0;
-                if (lane == 0) c = atomicAdd(p.queue, 1ull);
-                c = __shfl_sync(0xffffffffu, c, 0);
-                const unsigned long long nch = p.nchunks_dev ? *p.nchunks_dev : p.nchunks;
-                if (c >= nch) {
-                    queue_empty = true;
-                    break;
-                }
-                if (lane == 0) {
-                    uint32_t nwalks;
+        if ((uint32_t)__popc(idle) >= p.refill) {
+            while (idle) {
+                if (issued == total) {
+                    if (queue_empty) break;
+                    unsigned long long c = 0;
+                    if (lane == 0) c = atomicAdd(p.queue, 1ull);
+                    c = __shfl_sync(0xffffffffu, c, 0);
+                    const unsigned long long nch = p.nchunks_dev ? *p.nchunks_dev : p.nchunks;
+                    if (c >= nch) {
+                        queue_empty = true;
+                        break;
+                    }
                     if (p.chunks) {  // whole sources of one instance
                         const int4 d = p.chunks[c];
-                        wq.base = (uint32_t)d.x;
-                        wq.ctr_base = (uint32_t)p.inst_off[d.z];
-                        wq.tag = (uint32_t)d.z;
-                        wq.j0 = 0;
-                        nwalks = (uint32_t)d.y * p.R;
+                        if (lane == 0) wc = WarpChunk{(uint32_t)d.x, (uint32_t)p.inst_off[d.z], (uint32_t)d.z, 0u};
+                        total = (uint32_t)d.y * p.R;
                     } else {  // walks [c * CW, ...) of the whole launch
-                        const uint64_t b = c * (uint64_t)p.CW;
-                        const uint64_t i0 = b / p.R;
-                        wq.base = (uint32_t)i0;
-                        wq.j0 = (uint32_t)(b - i0 * p.R);
-                        nwalks = (uint32_t)min((uint64_t)p.CW, p.walks - b);
-                        wq.ctr_base = 0;
-                        wq.tag = p.tag;
+                        const uint64_t b = c * (uint64_t)p.CW, i0 = b / p.R;
+                        if (lane == 0) wc = WarpChunk{(uint32_t)i0, 0u, p.tag, (uint32_t)(b - i0 * p.R)};
+                        total = (uint32_t)min((uint64_t)p.CW, p.walks - b);
                     }
-                    wq.issued = 0;
-                    wq.total = nwalks;
+                    issued = 0;
+                    __syncwarp();
                 }
+                const uint32_t n = issued + __popc(idle & ((1u << lane) - 1));  // the walk this lane would take
+                if (!active && n < total) {
+                    const uint32_t w = wc.j0 + n;  // < 2^20: a chunk <= 2^19 walks, j0 < R <= 4096
+                    const uint32_t i = div_by_R(w, p.r_magic);
+                    j = w - i * p.R;
+                    pos = wc.base + i;
+                    src = p.src_list ? p.src_list[pos] : (uint32_t)(p.s_begin + pos);
+                    sctr = src - wc.ctr_base;  // draws keyed by the caller's source id
+                    src = p.code_of[src];      // start and restart node of the layout
+                    tag = wc.tag;
+                    k = 0;
+                    u = src;
+                    active = true;
+                }
+                const uint32_t want = __popc(idle);
+                if (want <= total - issued) {
+                    issued += want;
+                    break;
+                }
+                issued = total;  // the lanes left take walks of the next chunk
                 __syncwarp();
+                idle = __ballot_sync(0xffffffffu, !active);
             }
-            const uint32_t issued = wq.issued;
-            const uint32_t take = min(wq.total - issued, (uint32_t)__popc(idle));
-            const uint32_t rank = __popc(idle & ((1u << lane) - 1));
-            if (((idle >> lane) & 1) && rank < take) {
-                const uint32_t w = wq.j0 + issued + rank;  // < 2^20: CW <= 2^19, j0 < R <= 4096
-                const uint32_t i = div_by_R(w, p.r_magic);
-                j = w - i * p.R;
-                const uint32_t pos = wq.base + i;
-                src = p.src_list ? p.src_list[pos] : (uint32_t)(p.s_begin + pos);
-                ctr_base = wq.ctr_base;
-                sctr = src - ctr_base;  // draws keyed by the caller's source id
-                if (p.rank) src = (uint32_t)p.rank[src];  // start and restart node of the layout
-                tag = wq.tag;
-                slot = (uint64_t)pos * p.R + j;
-                k = 0;
-                u = src;
-                active = true;
-            }
-            __syncwarp();
-            if (lane == 0) wq.issued = issued + take;
-            __syncwarp();
-            idle = __ballot_sync(0xffffffffu, !active);
+            if (queue_empty && __ballot_sync(0xffffffffu, active) == 0) break;  // queue drained, every walk done
         }
-        if (__ballot_sync(0xffffffffu, active) == 0) break;  // queue drained and every walk done
-
-        uint32_t end = 0;
-        bool ended;
-        if constexpr (BOUNDED) {
-            ended = active && walk_step_bounded<SEG, SPLIT>(p, StepKey{p.k0, p.k1, p.T}, edges, src, sctr, j, tag, k, u, end,
-                                                     pend, PendRef{ps_all, blockDim.x, threadIdx.x}, tl);
-        } else {
-            ended = walk_step<E, SEG, true, STATS, SPLIT>(p, StepKey{p.k0, p.k1, p.T}, edges, active, src, sctr, j, tag, k, u,
-                                                   end, tl);
-        }
-        if (ended) {
+        if (active && walk_step<E, SEG, STATS>(p, tab, p.key, p.T, src, sctr, j, tag, k, u, pend, tl)) {
+            const uint64_t slot = (uint64_t)pos * p.R + j;
 #ifdef PPR_CHECKED
             if (slot >= (uint64_t)(p.s_end - p.s_begin) * p.R) atomicOr(p.err, 8ull);
             else
 #endif
-            p.ends[slot] = end - ctr_base;
+            p.ends[slot] = u;
+            if (!SEG) tl.steps += k;
             active = false;
         }
     }
@@ -214,7 +202,7 @@ static int walker_event(ppr_result *r, cudaStream_t st)
     return PPR_OK;
 }
 
-template <class E, bool SEG, bool STATS, bool BOUNDED = false, bool SPLIT = false>
+template <class E, bool SEG, bool STATS>
 static int launch_typed(ppr_ctx *ctx, const KParams &kp, const RunPlan &plan, int64_t S, cudaStream_t st,
                         ppr_result *r)
 {
@@ -224,11 +212,11 @@ static int launch_typed(ppr_ctx *ctx, const KParams &kp, const RunPlan &plan, in
         int blocks = (int)std::min<uint64_t>((total + 255) / 256, (uint64_t)ctx->sms * 64);
         if (blocks < 1) blocks = 1;
         if ((rc = walker_event(r, st))) return rc;
-        k_walk_plain<E, SEG, STATS, SPLIT><<<blocks, 256, 0, st>>>(kp);
+        k_walk_plain<E, SEG, STATS><<<blocks, 256, 0, st>>>(kp);
         note_launch();
         PPR_CUDA(cudaGetLastError());
         if ((rc = walker_event(r, st))) return rc;
-        return launch_aggregate(ctx, AggParams{kp.ends, kp.R, kp.P2, S, kp.out_row0, kp.out, kp.order}, st);
+        return launch_aggregate(ctx, AggParams{kp.ends, kp.R, kp.P2, S, kp.out_row0, kp.out, kp.order, kp.tab}, st);
     }
     // walkers per CTA: 32 * warps_per_block (4 or 8 warps; default 8)
     const int wpb = plan.warps_per_block == 4 ? 4 : 8;
@@ -239,7 +227,7 @@ static int launch_typed(ppr_ctx *ctx, const KParams &kp, const RunPlan &plan, in
     int per_sm = occ ? occ->load(std::memory_order_relaxed) : 0;
     if (per_sm < 1) {
         PPR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &per_sm, k_walk_persistent<E, SEG, STATS, BOUNDED, SPLIT>, 32 * wpb, 0));
+            &per_sm, k_walk_persistent<E, SEG, STATS>, 32 * wpb, 0));
         if (per_sm < 1) per_sm = 1;
         if (occ) occ->store(per_sm, std::memory_order_relaxed);
     }
@@ -253,15 +241,16 @@ static int launch_typed(ppr_ctx *ctx, const KParams &kp, const RunPlan &plan, in
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     if (plan.l2_persist && ctx->l2_persist_max > 0 && ctx->l2_window_max > 0) {
-        // node records persisting in L2: every step reads one, the rows'
-        // records stream past them
-        const size_t bytes = std::min((size_t)kp.n_nodes * sizeof(typename E::Node), ctx->l2_window_max);
+        // the alias node records, or the front of the slots, persisting in L2
+        constexpr bool alias = std::is_same<E, AliasEdges>::value;
+        const size_t all = alias ? (size_t)kp.n_anode * sizeof(AliasNode) : (size_t)kp.n_slots * sizeof(Sector);
+        const size_t bytes = std::min(all, ctx->l2_window_max);
         if (ctx->l2_persist_set < std::min(bytes, ctx->l2_persist_max)) {
             ctx->l2_persist_set = std::min(bytes, ctx->l2_persist_max);
             PPR_CUDA(cudaDeviceSetLimit(cudaLimitPersistingL2CacheSize, ctx->l2_persist_set));
         }
         attr[0].id = cudaLaunchAttributeAccessPolicyWindow;
-        attr[0].val.accessPolicyWindow.base_ptr = (void *)kp.node;
+        attr[0].val.accessPolicyWindow.base_ptr = alias ? (void *)kp.anode : (void *)kp.slots;
         attr[0].val.accessPolicyWindow.num_bytes = bytes;
         attr[0].val.accessPolicyWindow.hitRatio = std::min(1.0f, (float)ctx->l2_persist_set / (float)bytes);
         attr[0].val.accessPolicyWindow.hitProp = cudaAccessPropertyPersisting;
@@ -269,11 +258,11 @@ static int launch_typed(ppr_ctx *ctx, const KParams &kp, const RunPlan &plan, in
         cfg.attrs = attr;
         cfg.numAttrs = 1;
     }
-    PPR_CUDA(cudaLaunchKernelEx(&cfg, k_walk_persistent<E, SEG, STATS, BOUNDED, SPLIT>, kp));
+    PPR_CUDA(cudaLaunchKernelEx(&cfg, k_walk_persistent<E, SEG, STATS>, kp));
     note_launch();
     PPR_CUDA(cudaGetLastError());
     if ((rc = walker_event(r, st))) return rc;
-    return launch_aggregate(ctx, AggParams{kp.ends, kp.R, kp.P2, S, kp.out_row0, kp.out, kp.order}, st);
+    return launch_aggregate(ctx, AggParams{kp.ends, kp.R, kp.P2, S, kp.out_row0, kp.out, kp.order, kp.tab}, st);
 }
 
 // Chunk table of a batched graph, built on the device: chunks of at most CS
@@ -328,12 +317,12 @@ size_t launch_workspace_bytes(const ppr_graph *g, const RunPlan &plan, int64_t S
 // Every kernel a run can launch is loaded here, once per device.  With lazy
 // module loading the first launch of a kernel may wait for the device to go
 // idle; loaded up front, a run's launches stay asynchronous.
-template <class E, bool SEG, bool STATS, bool SPLIT = false>
+template <class E, bool SEG, bool STATS>
 static void preload_walkers()
 {
     cudaFuncAttributes a;
-    cudaFuncGetAttributes(&a, k_walk_plain<E, SEG, STATS, SPLIT>);
-    cudaFuncGetAttributes(&a, k_walk_persistent<E, SEG, STATS, false, SPLIT>);
+    cudaFuncGetAttributes(&a, k_walk_plain<E, SEG, STATS>);
+    cudaFuncGetAttributes(&a, k_walk_persistent<E, SEG, STATS>);
 }
 
 void preload_run_kernels()
@@ -342,15 +331,6 @@ void preload_run_kernels()
     preload_walkers<NarrowEdges, true, false>();
     preload_walkers<NarrowEdges, false, true>();
     preload_walkers<NarrowEdges, true, true>();
-    cudaFuncAttributes fa;
-    cudaFuncGetAttributes(&fa, k_walk_persistent<NarrowEdges, false, false, true>);
-    cudaFuncGetAttributes(&fa, k_walk_persistent<NarrowEdges, true, false, true>);
-    preload_walkers<NarrowEdges, false, false, true>();
-    preload_walkers<NarrowEdges, true, false, true>();
-    preload_walkers<NarrowEdges, false, true, true>();
-    preload_walkers<NarrowEdges, true, true, true>();
-    cudaFuncGetAttributes(&fa, k_walk_persistent<NarrowEdges, false, false, true, true>);
-    cudaFuncGetAttributes(&fa, k_walk_persistent<NarrowEdges, true, false, true, true>);
     preload_walkers<WideEdges, false, false>();
     preload_walkers<WideEdges, true, false>();
     preload_walkers<WideEdges, false, true>();
@@ -367,27 +347,46 @@ void preload_run_kernels()
     cudaFuncGetAttributes(&a, k_aggregate<32>);
     cudaFuncGetAttributes(&a, k_chunk_count);
     cudaFuncGetAttributes(&a, k_chunk_fill);
+    cudaFuncGetAttributes(&a, k_scan_one);
     cudaFuncGetAttributes(&a, k_scan_tile_sums);
     cudaFuncGetAttributes(&a, k_scan_tile_offsets);
     cudaFuncGetAttributes(&a, k_scan_apply);
     cudaGetLastError();
 }
 
-// Narrow layout: SPLIT for a renumbered graph's layout (summary array,
-// evict-first bottom blocks), else summaries before each row's blocks.
-template <bool SPLIT>
-static int launch_narrow(ppr_ctx *ctx, const KParams &kp, const RunPlan &plan, int64_t S, cudaStream_t st,
+template <class E>
+static int launch_layout(ppr_ctx *ctx, const KParams &kp, const RunPlan &plan, int64_t S, cudaStream_t st,
                          ppr_result *ev_owner)
 {
     if (plan.stats)
-        return plan.segments ? launch_typed<NarrowEdges, true, true, false, SPLIT>(ctx, kp, plan, S, st, ev_owner)
-                             : launch_typed<NarrowEdges, false, true, false, SPLIT>(ctx, kp, plan, S, st, ev_owner);
-    // the bounded step: persistent kernel, no cooperative search (statistics launches took the branch above)
-    if (plan.step_loads > 0 && plan.kernel == PPR_KERNEL_PERSISTENT && kp.large == 0xffffffffu)
-        return plan.segments ? launch_typed<NarrowEdges, true, false, true, SPLIT>(ctx, kp, plan, S, st, ev_owner)
-                             : launch_typed<NarrowEdges, false, false, true, SPLIT>(ctx, kp, plan, S, st, ev_owner);
-    return plan.segments ? launch_typed<NarrowEdges, true, false, false, SPLIT>(ctx, kp, plan, S, st, ev_owner)
-                         : launch_typed<NarrowEdges, false, false, false, SPLIT>(ctx, kp, plan, S, st, ev_owner);
+        return plan.segments ? launch_typed<E, true, true>(ctx, kp, plan, S, st, ev_owner)
+                             : launch_typed<E, false, true>(ctx, kp, plan, S, st, ev_owner);
+    return plan.segments ? launch_typed<E, true, false>(ctx, kp, plan, S, st, ev_owner)
+                         : launch_typed<E, false, false>(ctx, kp, plan, S, st, ev_owner);
+}
+
+// The arrays a walk reads: the layout's, or those of its alias or segment tables.
+void set_layout(KParams &kp, const ppr_graph *g, bool segments, bool alias)
+{
+    kp.tab = alias ? g->alias.tab : (segments ? g->seg.tab : g->tab);
+    kp.slots = g->slots;
+    kp.seg_slots = g->seg.slots;
+    kp.aslots = g->alias.slots;
+    kp.single = segments ? g->seg.single : g->single;
+    kp.edges = g->edges;
+    kp.anode = g->alias.node;
+    kp.seg = g->seg.entries;
+    kp.seg_head = g->seg.head;
+    kp.node = g->node;
+    kp.code_of = g->code_of;
+    kp.order = g->order;
+    kp.n_nodes = (uint64_t)g->n;
+    kp.n_anode = (uint64_t)g->alias.nodes;
+    kp.n_slots = (uint64_t)g->n_slots;
+    kp.n_seg_slots = (uint64_t)g->seg.n_slots;
+    kp.n_single = (uint64_t)g->n_single;
+    kp.n_records = (uint64_t)g->m;
+    kp.n_seg = (uint64_t)g->seg.entries_cap;
 }
 
 int launch_walks(ppr_ctx *ctx, const ppr_graph *g, const RunPlan &plan, const Outputs &o, int64_t s_begin, int64_t S,
@@ -396,21 +395,15 @@ int launch_walks(ppr_ctx *ctx, const ppr_graph *g, const RunPlan &plan, const Ou
 {
     if (S <= 0) return PPR_OK;
     KParams kp{};
-    kp.node = plan.segments ? g->seg.node : (plan.sampler == 1 ? g->alias.node : g->node);
-    kp.edges = plan.sampler == 1 ? (const void *)g->alias.slots : g->edges;
-    kp.seg = g->seg.entries;
+    set_layout(kp, g, plan.segments, plan.sampler == 1);
     kp.R = plan.R;
     kp.T = plan.T;
-    kp.k0 = (uint32_t)plan.seed;
-    kp.k1 = (uint32_t)(plan.seed >> 32);
+    kp.key.set((uint32_t)plan.seed, (uint32_t)(plan.seed >> 32));
     kp.tag = plan.tag;
     kp.dangling = plan.dangling;
-    kp.large = plan.large_degree > 0 ? (uint32_t)plan.large_degree : 0xffffffffu;  // 0: off
     kp.s_begin = s_begin;
     kp.s_end = s_begin + S;
     kp.src_list = src_list;
-    kp.rank = g->rank;
-    kp.order = g->order;
     kp.out_row0 = out_row0;
     kp.out.nnz = o.nnz;
     kp.out.cols = o.cols;
@@ -425,13 +418,7 @@ int launch_walks(ppr_ctx *ctx, const ppr_graph *g, const RunPlan &plan, const Ou
     while (P2 < plan.R) P2 <<= 1;
     kp.P2 = P2;
     kp.r_magic = ((1ull << 40) + plan.R - 1) / plan.R;
-    kp.refill = plan.refill_lanes > 0 ? (uint32_t)std::min(plan.refill_lanes, 32) : 1u;
-    kp.step_loads = (uint32_t)std::max(plan.step_loads, 0);
-    kp.n_nodes = g->n;
-    kp.n_records = plan.sampler == 1 ? (uint64_t)g->m : (uint64_t)g->edge_records;
-    kp.sum = g->sum_base();
-    kp.n_sum = g->sum_extent();
-    kp.n_seg = (uint64_t)g->seg.entries_cap;
+    kp.refill = plan.refill_lanes > 0 ? (uint32_t)std::min(plan.refill_lanes, 32) : kDefaultRefill;
     kp.err = o.counters + 4;
     kp.ends = reinterpret_cast<uint32_t *>(ws);
     size_t off = align256((size_t)S * plan.R * sizeof(uint32_t));
@@ -482,15 +469,8 @@ int launch_walks(ppr_ctx *ctx, const ppr_graph *g, const RunPlan &plan, const Ou
     if (plan.sampler == 1)
         return plan.stats ? launch_typed<AliasEdges, false, true>(ctx, kp, plan, S, st, ev_owner)
                           : launch_typed<AliasEdges, false, false>(ctx, kp, plan, S, st, ev_owner);
-    if (g->wide) {
-        if (plan.stats)
-            return plan.segments ? launch_typed<WideEdges, true, true>(ctx, kp, plan, S, st, ev_owner)
-                                 : launch_typed<WideEdges, false, true>(ctx, kp, plan, S, st, ev_owner);
-        return plan.segments ? launch_typed<WideEdges, true, false>(ctx, kp, plan, S, st, ev_owner)
-                             : launch_typed<WideEdges, false, false>(ctx, kp, plan, S, st, ev_owner);
-    }
-    return g->sum ? launch_narrow<true>(ctx, kp, plan, S, st, ev_owner)
-                  : launch_narrow<false>(ctx, kp, plan, S, st, ev_owner);
+    return g->wide ? launch_layout<WideEdges>(ctx, kp, plan, S, st, ev_owner)
+                   : launch_layout<NarrowEdges>(ctx, kp, plan, S, st, ev_owner);
 }
 
 // ------------------------------------------------ allocation-free run ----
@@ -552,11 +532,11 @@ extern "C" int ppr_run_noalloc(ppr_ctx *ctx, const ppr_graph *g, const ppr_run_a
         set_error("the allocation-free run takes plain graphs only");
         return PPR_ENOTSUP;
     }
-    if (plan.segments && !(g->seg.T == plan.T && g->seg.node)) {
+    if (plan.segments && !(g->seg.T == plan.T && g->seg.tab)) {
         set_error("segment tables for this alpha are not built (a ppr_run with segments=1 builds them)");
         return PPR_ENOTSUP;
     }
-    if (plan.sampler == 1 && !g->alias.node) {
+    if (plan.sampler == 1 && !g->alias.tab) {
         set_error("alias sampler: needs tables built by an earlier ppr_run with sampler=1");
         return PPR_ENOTSUP;
     }

@@ -1,5 +1,5 @@
 """Tuning cache: the launch tuning chosen by ppr_autotune (native timing of
-candidate walkers-per-CTA, queue chunk and cooperative threshold), kept in a
+candidate walkers-per-CTA, queue chunk and refill threshold), kept in a
 JSON file keyed by the graph's shape, the run parameters and the device.
 Tuning never changes results; a stale entry only costs speed."""
 from __future__ import annotations
