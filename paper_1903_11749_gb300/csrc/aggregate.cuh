@@ -129,15 +129,16 @@ __device__ __forceinline__ void warp_sort_reg(uint32_t (&v)[E])
 }
 
 // Top-K of one row without sorting every run, for K <= 32 and K < nrun:
-// kv holds the keys (R - count) << 12 | run of runs e * 32 + lane (0xFFFFFFFF
-// past nrun), and the answer is the K smallest keys in ascending order.  The
+// kv holds the key (R - count) << 12 | run at each run's head element, v its
+// node id (kv 0xFFFFFFFF elsewhere; elements e * 32 + lane in order), and the
+// answer is the K smallest keys in ascending order.  The
 // count rank q = key >> 12 of the K-th smallest key is found by bisection
 // over [0, R - 1] with ballot counts; every key with q below it is taken (fewer
 // than K, sorted in one register per lane), then the first keys with q equal
 // to it in run order (= ascending key, as runs are numbered in id order)
 // fill the remaining places.  cbuf: 32 uint32 of per-warp shared memory.
 template <int E>
-__device__ __forceinline__ void topk_select_reg(const uint32_t (&kv)[E], uint32_t K, uint32_t R,
+__device__ __forceinline__ void topk_select_reg(const uint32_t (&kv)[E], const uint32_t (&v)[E], uint32_t K, uint32_t R,
                                                 const uint32_t *run_id, uint32_t *cbuf, const AggOut &o, uint64_t tb)
 {
     const uint32_t lane = threadIdx.x & 31, below = (1u << lane) - 1;
@@ -168,11 +169,11 @@ __device__ __forceinline__ void topk_select_reg(const uint32_t (&kv)[E], uint32_
     }
     __syncwarp();
     // nlt < K places for the keys below t, sorted; then K - nlt keys equal to t
-    uint32_t v[1] = {lane < nlt ? cbuf[lane] : 0xffffffffu};
-    warp_sort_reg<1>(v);
+    uint32_t x[1] = {lane < nlt ? cbuf[lane] : 0xffffffffu};
+    warp_sort_reg<1>(x);
     if (lane < nlt) {
-        o.topk_idx[tb + lane] = (int32_t)run_id[v[0] & 0xfffu];
-        o.topk_cnt[tb + lane] = R - (v[0] >> 12);
+        o.topk_idx[tb + lane] = (int32_t)run_id[x[0] & 0xfffu];
+        o.topk_cnt[tb + lane] = R - (x[0] >> 12);
     }
     uint32_t seen = 0;
 #pragma unroll
@@ -181,7 +182,7 @@ __device__ __forceinline__ void topk_select_reg(const uint32_t (&kv)[E], uint32_
         const uint32_t me = __ballot_sync(0xffffffffu, eq);
         const uint32_t pos = nlt + seen + __popc(me & below);
         if (eq && pos < K) {
-            o.topk_idx[tb + pos] = (int32_t)run_id[kv[e] & 0xfffu];
+            o.topk_idx[tb + pos] = (int32_t)v[e];
             o.topk_cnt[tb + pos] = R - t;
         }
         seen += __popc(me);
@@ -195,8 +196,9 @@ __device__ __forceinline__ void topk_select_reg(const uint32_t (&kv)[E], uint32_
 // placed by ballot prefix counts.  Returns false (nothing written) when more
 // than 32 runs repeat; the caller then sorts every key.
 template <int E>
-__device__ __forceinline__ bool topk_all_reg(const uint32_t (&kv)[E], uint32_t nrun, uint32_t K, uint32_t R,
-                                             const uint32_t *run_id, uint32_t *cbuf, const AggOut &o, uint64_t tb)
+__device__ __forceinline__ bool topk_all_reg(const uint32_t (&kv)[E], const uint32_t (&v)[E], uint32_t nrun, uint32_t K,
+                                             uint32_t R, const uint32_t *run_id, uint32_t *cbuf, const AggOut &o,
+                                             uint64_t tb)
 {
     const uint32_t lane = threadIdx.x & 31, below = (1u << lane) - 1;
     const uint32_t t1 = (R - 1) << 12;  // keys from here on: count 1 (or no run)
@@ -213,21 +215,20 @@ __device__ __forceinline__ bool topk_all_reg(const uint32_t (&kv)[E], uint32_t n
         seen += __popc(mr);
     }
     __syncwarp();
-    uint32_t v[1] = {lane < nm ? cbuf[lane] : 0xffffffffu};
-    warp_sort_reg<1>(v);
+    uint32_t x[1] = {lane < nm ? cbuf[lane] : 0xffffffffu};
+    warp_sort_reg<1>(x);
     if (lane < nm && lane < K) {
-        o.topk_idx[tb + lane] = (int32_t)run_id[v[0] & 0xfffu];
-        o.topk_cnt[tb + lane] = R - (v[0] >> 12);
+        o.topk_idx[tb + lane] = (int32_t)run_id[x[0] & 0xfffu];
+        o.topk_cnt[tb + lane] = R - (x[0] >> 12);
     }
     uint32_t ones = 0;
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-        const uint32_t i = (uint32_t)e * 32 + lane;
-        const bool one = i < nrun && kv[e] >= t1;
+        const bool one = kv[e] >= t1 && kv[e] != 0xffffffffu;
         const uint32_t m1 = __ballot_sync(0xffffffffu, one);
         const uint32_t pos = nm + ones + __popc(m1 & below);
         if (one && pos < K) {
-            o.topk_idx[tb + pos] = (int32_t)run_id[kv[e] & 0xfffu];
+            o.topk_idx[tb + pos] = (int32_t)v[e];
             o.topk_cnt[tb + pos] = 1;
         }
         ones += __popc(m1);
@@ -239,13 +240,21 @@ __device__ __forceinline__ bool topk_all_reg(const uint32_t (&kv)[E], uint32_t n
     return true;
 }
 
-// scratch: 3 * R uint32 of per-warp shared memory
+// scratch: R + 32 uint32 of per-warp shared memory.
+//
+// Bound by the ALU pipe, so what follows the sort is kept short: run heads
+// come from one shuffle and one ballot per register; a run's count is the
+// distance to the next head, read off the same ballots; and the top-k keys
+// stay at their heads (0xFFFFFFFF elsewhere), so a selected run has its node
+// id in the lane that holds its key.  (A tenth fewer instructions than with run
+// starts and keys passed through shared memory: 256-graph batch, R 200, 4.28 ->
+// 3.96 ms.)
 template <int E>
 __device__ inline void aggregate_source_reg(const uint32_t *ends, uint32_t R, uint32_t *scratch, const AggOut &o,
                                             uint64_t out_row, const CallerIds &ids = CallerIds())
 {
     const uint32_t lane = threadIdx.x & 31;
-    uint32_t *start_pos = scratch, *run_id = scratch + R, *kbuf = scratch + 2 * R;
+    uint32_t *run_id = scratch, *cbuf = scratch + R;
     uint32_t v[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) {
@@ -281,51 +290,47 @@ __device__ inline void aggregate_source_reg(const uint32_t *ends, uint32_t R, ui
     for (int e = 0; e < E; ++e)
         if ((uint32_t)e * 32 + lane < R) v[e] = ids(v[e]);
     warp_sort_reg<E>(v);
-    uint32_t nrun = 0;
+    uint32_t hb[E], nxt[E];  // heads of each register; first head in a later register (R: none)
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-        const uint32_t i = (uint32_t)e * 32 + lane;
-        const uint32_t pu = __shfl_up_sync(0xffffffffu, v[e], 1);
-        const uint32_t pe = __shfl_sync(0xffffffffu, v[e > 0 ? e - 1 : 0], 31);
-        const uint32_t nd = __shfl_down_sync(0xffffffffu, v[e], 1);
-        const uint32_t ne = __shfl_sync(0xffffffffu, v[e + 1 < E ? e + 1 : e], 0);
-        const uint32_t prev = lane == 0 ? pe : pu;
-        const uint32_t next = lane == 31 ? ne : nd;
-        const bool valid = i < R;
-        const bool head = valid && (i == 0 || prev != v[e]);
-        const bool tail = valid && (i == R - 1 || next != v[e]);
-        const uint32_t hb = __ballot_sync(0xffffffffu, head);
-        const uint32_t run = nrun + __popc(hb & ((2u << lane) - 1)) - 1;  // run of element i
-        if (head) {
-            start_pos[run] = i;
-            run_id[run] = v[e];
-        }
-        __syncwarp();
-        if (tail) {
-            const uint32_t c = i - start_pos[run] + 1;
+        // the element before: lane 31 hands lane 0 the last one of the register before
+        const uint32_t mine = e > 0 && lane == 31 ? v[e > 0 ? e - 1 : 0] : v[e];
+        const uint32_t prev = __shfl_sync(0xffffffffu, mine, (lane + 31) & 31);
+        const bool head = (uint32_t)e * 32 + lane < R && ((e == 0 && lane == 0) || prev != v[e]);
+        hb[e] = __ballot_sync(0xffffffffu, head);
+    }
+    uint32_t after = R;
+#pragma unroll
+    for (int e = E - 1; e >= 0; --e) {
+        nxt[e] = after;
+        if (hb[e]) after = (uint32_t)e * 32 + __ffs(hb[e]) - 1;
+    }
+    uint32_t nrun = 0, kv[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        kv[e] = 0xffffffffu;
+        if ((hb[e] >> lane) & 1u) {
+            const uint32_t i = (uint32_t)e * 32 + lane, above = hb[e] & (0xfffffffeu << lane);
+            const uint32_t run = nrun + __popc(hb[e] & ((1u << lane) - 1));
+            const uint32_t c = (above ? (uint32_t)e * 32 + __ffs(above) - 1 : nxt[e]) - i;
             if (o.cols) {
                 o.cols[rbase + run] = (int32_t)v[e];
                 o.cnts[rbase + run] = c;
             }
-            kbuf[run] = ((R - c) << 12) | run;
+            run_id[run] = v[e];
+            kv[e] = ((R - c) << 12) | run;
         }
-        nrun += __popc(hb);
+        nrun += __popc(hb[e]);
     }
     if (lane == 0 && o.nnz) o.nnz[out_row] = nrun;
     if (o.topk > 0) {
         __syncwarp();
-        uint32_t kv[E];
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const uint32_t i = (uint32_t)e * 32 + lane;
-            kv[e] = i < nrun ? kbuf[i] : 0xffffffffu;
-        }
         const uint64_t tb = out_row * (uint64_t)o.topk;
         const uint32_t K = (uint32_t)o.topk;
         if (E > 1 && K <= 32 && K < nrun) {
-            topk_select_reg<E>(kv, K, R, run_id, start_pos, o, tb);
-        } else if (E > 1 && E <= 8 && K >= nrun && topk_all_reg<E>(kv, nrun, K, R, run_id, start_pos, o, tb)) {
-            // the whole row, in top-k order (R <= 256)
+            topk_select_reg<E>(kv, v, K, R, run_id, cbuf, o, tb);
+        } else if (E > 1 && K >= nrun && topk_all_reg<E>(kv, v, nrun, K, R, run_id, cbuf, o, tb)) {
+            // the whole row, in top-k order
         } else {
             warp_sort_reg<E>(kv);
 #pragma unroll
@@ -351,6 +356,196 @@ __device__ inline void aggregate_source_reg(const uint32_t *ends, uint32_t R, ui
     __syncwarp();
 }
 
+// ------------------------------------------------ one block per source ----
+// R > 256: a block of T threads reduces one source, I elements a thread
+// (T * I = next_pow2(R)).  One warp a source left the chip idle where there
+// are few sources (rankings over some hundred sources with R in the
+// thousands) and waited through a chain of shared-memory or 32-register
+// stages.  Reduction of 500 sources, R 4096, top-1000: 1262 -> 40 us; 1,000
+// sources, R 1000: 46 -> 18 us; and with the chip full, 2^25 walks in all: R
+// 300 .697 -> .505 ms, 500 .478 -> .324, 1000 .728 -> .392, 2000 7.80 -> .504,
+// 4000 17.5 -> .497.
+
+// Ascending sort of T * I elements, element t * I + k in register k of thread
+// t.  Bitonic network in the form whose first exchange of every level mirrors
+// (i with i ^ (size - 1)), so every exchange puts the smaller element first and
+// no direction is tracked: strides below I stay in the thread, below 32 I in
+// the warp, longer ones go through sm (T * I words).
+template <int T, int I>
+__device__ __forceinline__ void block_sort(uint32_t (&v)[I], uint32_t *sm)
+{
+    const uint32_t t = threadIdx.x;
+    // exchange with thread t ^ x; MIRROR: the partner's elements in reverse order
+    auto across = [&](uint32_t x, bool mirror) {
+        const bool lower = (t & (mirror ? (x + 1) >> 1 : x)) == 0;
+        uint32_t o[I];
+        if (x < 32) {
+#pragma unroll
+            for (int k = 0; k < I; ++k) o[k] = __shfl_xor_sync(0xffffffffu, v[mirror ? I - 1 - k : k], x);
+        } else {
+#pragma unroll
+            for (int k = 0; k < I; ++k) sm[k * T + t] = v[k];
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < I; ++k) o[k] = sm[(mirror ? I - 1 - k : k) * T + (t ^ x)];
+            __syncthreads();
+        }
+#pragma unroll
+        for (int k = 0; k < I; ++k) v[k] = lower ? min(v[k], o[k]) : max(v[k], o[k]);
+    };
+    auto within = [&](int a, int b) {
+        const uint32_t x = v[a], y = v[b];
+        v[a] = min(x, y);
+        v[b] = max(x, y);
+    };
+#pragma unroll
+    for (int size = 2; size <= T * I; size <<= 1) {
+        if (size <= I) {
+#pragma unroll
+            for (int k = 0; k < I; ++k)
+                if ((k ^ (size - 1)) > k) within(k, k ^ (size - 1));
+        } else {
+            across(size / I - 1, true);
+        }
+#pragma unroll
+        for (int stride = size >> 2; stride > 0; stride >>= 1) {
+            if (stride < I) {
+#pragma unroll
+                for (int k = 0; k < I; ++k)
+                    if ((k ^ stride) > k) within(k, k ^ stride);
+            } else {
+                across(stride / I, false);
+            }
+        }
+    }
+}
+
+// Exclusive sum over the block's threads; *total: of all.  s: T / 32 words.
+template <int T>
+__device__ __forceinline__ uint32_t block_sum_before(uint32_t x, uint32_t *s, uint32_t *total)
+{
+    const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint32_t y = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t z = __shfl_up_sync(0xffffffffu, y, o);
+        if (lane >= (uint32_t)o) y += z;
+    }
+    if (lane == 31) s[wid] = y;
+    __syncthreads();
+    uint32_t before = 0, all = 0;
+#pragma unroll
+    for (uint32_t w = 0; w < T / 32; ++w) {
+        if (w == wid) before = all;
+        all += s[w];
+    }
+    __syncthreads();
+    *total = all;
+    return before + y - x;
+}
+
+template <int T, int I>
+struct BlockScratch {
+    uint32_t id[T * I];         // sort exchange, then the runs' node ids
+    uint32_t start[T * I + 1];  // first element of each run
+    uint32_t key[T * I / 2];    // sort exchange of the runs met twice or more (R / 2 of them at most), then their keys
+    uint32_t sums[T / 32];
+    uint32_t edge[T / 32];      // last element of each warp
+};
+
+template <int T, int I>
+__device__ void aggregate_source_block(const uint32_t *ends, uint32_t R, BlockScratch<T, I> &sm, const AggOut &o,
+                                       uint64_t out_row, const CallerIds &ids)
+{
+    const uint32_t t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    uint32_t v[I];
+#pragma unroll
+    for (int k = 0; k < I; ++k) {
+        const uint32_t i = (uint32_t)k * T + t;
+        v[k] = i < R ? ids(ends[i]) : 0xffffffffu;
+    }
+    block_sort<T, I>(v, sm.id);
+    if (lane == 31) sm.edge[wid] = v[I - 1];
+    __syncthreads();
+    uint32_t prev = __shfl_up_sync(0xffffffffu, v[I - 1], 1);
+    if (lane == 0) prev = wid > 0 ? sm.edge[wid - 1] : 0u;
+    uint32_t heads = 0;
+#pragma unroll
+    for (int k = 0; k < I; ++k) {
+        const uint32_t i = t * I + k;
+        if (i < R && (i == 0 || v[k] != (k > 0 ? v[k > 0 ? k - 1 : 0] : prev))) heads |= 1u << k;
+    }
+    uint32_t nrun;
+    uint32_t run = block_sum_before<T>(__popc(heads), sm.sums, &nrun);
+#pragma unroll
+    for (int k = 0; k < I; ++k)
+        if ((heads >> k) & 1u) {
+            sm.id[run] = v[k];
+            sm.start[run++] = t * I + k;
+        }
+    if (t == 0) {
+        sm.start[nrun] = R;
+        if (o.nnz) o.nnz[out_row] = nrun;
+    }
+    __syncthreads();
+    if (o.cols) {
+        const uint64_t rbase = out_row * o.cap;
+        for (uint32_t r = t; r < nrun; r += T) {
+            o.cols[rbase + r] = (int32_t)sm.id[r];
+            o.cnts[rbase + r] = sm.start[r + 1] - sm.start[r];
+        }
+    }
+    if (o.topk > 0) {
+        const uint32_t K = (uint32_t)o.topk;
+        const uint64_t tb = out_row * (uint64_t)o.topk;
+        // runs met once come last, in id order, and need no sort
+        uint32_t c[I], many = 0, nm;
+#pragma unroll
+        for (int k = 0; k < I; ++k) {
+            const uint32_t r = t * I + k;
+            c[k] = r < nrun ? sm.start[r + 1] - sm.start[r] : 0u;
+            many += c[k] >= 2;
+        }
+        uint32_t mb = block_sum_before<T>(many, sm.sums, &nm);
+#pragma unroll
+        for (int k = 0; k < I; ++k) {
+            const uint32_t r = t * I + k;
+            if (c[k] >= 2) {
+                sm.key[mb++] = ((R - c[k]) << 12) | r;
+            } else if (c[k] == 1 && nm + r - mb < K) {
+                o.topk_idx[tb + nm + r - mb] = (int32_t)sm.id[r];
+                o.topk_cnt[tb + nm + r - mb] = 1;
+            }
+        }
+        __syncthreads();
+        auto put = [&](uint32_t i, uint32_t key) {
+            if (i < nm && i < K) {
+                o.topk_idx[tb + i] = (int32_t)sm.id[key & 0xfffu];
+                o.topk_cnt[tb + i] = R - (key >> 12);
+            }
+        };
+        if (nm <= T) {
+            uint32_t x[1] = {t < nm ? sm.key[t] : 0xffffffffu};
+            __syncthreads();
+            block_sort<T, 1>(x, sm.key);
+            put(t, x[0]);
+        } else {
+            uint32_t x[I / 2];
+#pragma unroll
+            for (int k = 0; k < I / 2; ++k) x[k] = (uint32_t)k * T + t < nm ? sm.key[k * T + t] : 0xffffffffu;
+            __syncthreads();
+            block_sort<T, I / 2>(x, sm.key);
+#pragma unroll
+            for (int k = 0; k < I / 2; ++k) put(t * (I / 2) + k, x[k]);
+        }
+        for (uint32_t i = nrun + t; i < K; i += T) {
+            o.topk_idx[tb + i] = -1;
+            o.topk_cnt[tb + i] = 0;
+        }
+    }
+    __syncthreads();
+}
+
 // Launch parameters of k_aggregate: S sources, R endpoints each, source-major.
 struct AggParams {
     const uint32_t *ends;
@@ -362,42 +557,53 @@ struct AggParams {
     const ClassTab *tab;
 };
 
-// E > 0: register-resident reduction for next_pow2(R) = 32 * E; E = 0:
-// shared-memory reduction (any R).  Four warps per block, 12 * P2 bytes of
-// shared scratch per warp.
-template <int E>
-__global__ void __launch_bounds__(128) k_aggregate(AggParams p)
+// The first seq of each class-table entry, for CallerIds.
+__device__ __forceinline__ CallerIds load_ids(uint32_t *first, const AggParams &p)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ uint32_t first[kTabEntries];
     for (uint32_t i = threadIdx.x; i < kTabEntries; i += blockDim.x) first[i] = p.tab->e[i].first;
     __syncthreads();
-    const CallerIds ids{p.order, first};
-    const uint32_t wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    unsigned char *scratch = smem_raw + (size_t)wid * p.P2 * 12;
+    return CallerIds{p.order, first};
+}
+
+// One warp per source, next_pow2(R) = 32 * E <= 256 (R <= 32: E = 1).
+constexpr int kAggWarps = 4;
+template <int E>
+__global__ void __launch_bounds__(32 * kAggWarps) k_aggregate(AggParams p)
+{
+    __shared__ uint32_t first[kTabEntries];
+    __shared__ uint32_t scratch[kAggWarps][32 * E + 32];
+    const CallerIds ids = load_ids(first, p);
+    const uint32_t wid = threadIdx.x >> 5;
     const uint64_t S = (uint64_t)p.S;
-    for (uint64_t i = (uint64_t)blockIdx.x * nw + wid; i < S; i += (uint64_t)gridDim.x * nw) {
-        if constexpr (E > 0) {
-            aggregate_source_reg<E>(p.ends + i * p.R, p.R, reinterpret_cast<uint32_t *>(scratch), p.out,
-                                    (uint64_t)p.out_row0 + i, ids);
-        } else {
-            uint64_t *keys = reinterpret_cast<uint64_t *>(scratch);
-            aggregate_source(p.ends + i * p.R, p.R, reinterpret_cast<uint32_t *>(keys + p.P2), keys, p.out,
-                             (uint64_t)p.out_row0 + i, ids);
-        }
-    }
+    for (uint64_t i = (uint64_t)blockIdx.x * kAggWarps + wid; i < S; i += (uint64_t)gridDim.x * kAggWarps)
+        aggregate_source_reg<E>(p.ends + i * p.R, p.R, scratch[wid], p.out, (uint64_t)p.out_row0 + i, ids);
+}
+
+template <int T, int I>
+__global__ void __launch_bounds__(T) k_aggregate_block(AggParams p)
+{
+    __shared__ uint32_t first[kTabEntries];
+    __shared__ BlockScratch<T, I> sm;
+    const CallerIds ids = load_ids(first, p);
+    for (uint64_t i = blockIdx.x; i < (uint64_t)p.S; i += gridDim.x)
+        aggregate_source_block<T, I>(p.ends + i * p.R, p.R, sm, p.out, (uint64_t)p.out_row0 + i, ids);
 }
 
 template <int E>
 static int launch_aggregate_e(ppr_ctx *ctx, const AggParams &ap, cudaStream_t st)
 {
-    const int aw = 4;
-    size_t smem = (size_t)aw * ap.P2 * 12;
-    if (smem + sizeof(uint32_t) * kTabEntries > 48 * 1024)  // with the kernel's own table
-        PPR_CUDA(cudaFuncSetAttribute(k_aggregate<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    int ablocks = (int)std::min<int64_t>((ap.S + aw - 1) / aw, (int64_t)ctx->sms * 16);
-    if (ablocks < 1) ablocks = 1;
-    k_aggregate<E><<<ablocks, aw * 32, smem, st>>>(ap);
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((ap.S + kAggWarps - 1) / kAggWarps, (int64_t)ctx->sms * 16));
+    k_aggregate<E><<<blocks, 32 * kAggWarps, 0, st>>>(ap);
+    note_launch();
+    PPR_CUDA(cudaGetLastError());
+    return PPR_OK;
+}
+
+template <int T, int I>
+static int launch_aggregate_block(ppr_ctx *ctx, const AggParams &ap, cudaStream_t st)
+{
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(ap.S, (int64_t)ctx->sms * (4096 / T)));
+    k_aggregate_block<T, I><<<blocks, T, 0, st>>>(ap);
     note_launch();
     PPR_CUDA(cudaGetLastError());
     return PPR_OK;
@@ -410,9 +616,10 @@ static int launch_aggregate(ppr_ctx *ctx, const AggParams &ap, cudaStream_t st)
     case 64: return launch_aggregate_e<2>(ctx, ap, st);
     case 128: return launch_aggregate_e<4>(ctx, ap, st);
     case 256: return launch_aggregate_e<8>(ctx, ap, st);
-    case 512: return launch_aggregate_e<16>(ctx, ap, st);
-    case 1024: return launch_aggregate_e<32>(ctx, ap, st);
-    default: return launch_aggregate_e<0>(ctx, ap, st);
+    case 512: return launch_aggregate_block<128, 4>(ctx, ap, st);
+    case 1024: return launch_aggregate_block<256, 4>(ctx, ap, st);
+    case 2048: return launch_aggregate_block<512, 4>(ctx, ap, st);
+    default: return launch_aggregate_block<512, 8>(ctx, ap, st);  // R <= 4096
     }
 }
 

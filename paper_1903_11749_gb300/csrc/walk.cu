@@ -338,13 +338,14 @@ void preload_run_kernels()
     preload_walkers<AliasEdges, false, false>();
     preload_walkers<AliasEdges, false, true>();
     cudaFuncAttributes a;
-    cudaFuncGetAttributes(&a, k_aggregate<0>);
     cudaFuncGetAttributes(&a, k_aggregate<1>);
     cudaFuncGetAttributes(&a, k_aggregate<2>);
     cudaFuncGetAttributes(&a, k_aggregate<4>);
     cudaFuncGetAttributes(&a, k_aggregate<8>);
-    cudaFuncGetAttributes(&a, k_aggregate<16>);
-    cudaFuncGetAttributes(&a, k_aggregate<32>);
+    cudaFuncGetAttributes(&a, k_aggregate_block<128, 4>);
+    cudaFuncGetAttributes(&a, k_aggregate_block<256, 4>);
+    cudaFuncGetAttributes(&a, k_aggregate_block<512, 4>);
+    cudaFuncGetAttributes(&a, k_aggregate_block<512, 8>);
     cudaFuncGetAttributes(&a, k_chunk_count);
     cudaFuncGetAttributes(&a, k_chunk_fill);
     cudaFuncGetAttributes(&a, k_scan_one);
