@@ -73,10 +73,12 @@ void dev_free(void *p, cudaStream_t st)
 // reads their sizes and positions at once, so that no row's copy waits for
 // its own, and four rows' pairs are in flight at a time.  Bound by memory
 // (R-MAT scale 24, 600 M pairs: 4.36 -> 2.52 ms).
+// Nothing is written when the rows hold more than `limit` pairs.
 __global__ void __launch_bounds__(256) k_compact_rows(int64_t S, uint32_t cap, const uint32_t *nnz, const uint64_t *off,
-                                                      const int32_t *cols, const uint32_t *cnts, int32_t *ocol,
-                                                      uint32_t *ocnt)
+                                                      uint64_t limit, const int32_t *cols, const uint32_t *cnts,
+                                                      int32_t *ocol, uint32_t *ocnt)
 {
+    if (off[S] > limit) return;
     const uint32_t lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t s0 = 32 * (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5); s0 < S; s0 += 32 * warps) {
@@ -155,6 +157,19 @@ void ctx_release(ppr_ctx *ctx)
 }  // namespace ppr
 
 using namespace ppr;
+
+static size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
+
+// The context's copy stream and page-locked words, made on first use.
+static int copy_resources(ppr_ctx *ctx)
+{
+    cudaError_t e = cudaSuccess;
+    if (!ctx->copy_stream && (e = cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking)) != cudaSuccess)
+        return cuda_fail(e, "copy stream");
+    if (!ctx->pinned && (e = cudaHostAlloc((void **)&ctx->pinned, 16 * sizeof(unsigned long long), 0)) != cudaSuccess)
+        return cuda_fail(e, "page-locked words");
+    return PPR_OK;
+}
 
 static int set_device(const ppr_ctx *ctx)
 {
@@ -416,15 +431,18 @@ static void result_release(ppr_result *r)
 {
     if (!r) return;
     if (r->ctx) cudaSetDevice(r->ctx->device);
-    dev_free(r->d_nnz, r->stream);
-    dev_free(r->d_cols, r->stream);
-    dev_free(r->d_cnts, r->stream);
-    dev_free(r->d_topk_idx, r->stream);
-    dev_free(r->d_topk_cnt, r->stream);
-    dev_free(r->d_steps, r->stream);
-    for (void *p : r->scratch) dev_free(p, r->stream);
+    if (r->block) {
+        dev_free(r->block, r->stream);
+    } else {
+        dev_free(r->d_nnz, r->stream);
+        dev_free(r->d_cols, r->stream);
+        dev_free(r->d_cnts, r->stream);
+        dev_free(r->d_topk_idx, r->stream);
+        dev_free(r->d_topk_cnt, r->stream);
+        dev_free(r->d_steps, r->stream);
+        for (void *p : r->scratch) dev_free(p, r->stream);
+    }
     if (r->ev_start) cudaEventDestroy(r->ev_start);
-    if (r->ev_walk_end) cudaEventDestroy(r->ev_walk_end);
     if (r->ev_done) cudaEventDestroy(r->ev_done);
     for (cudaEvent_t ev : r->walk_events) cudaEventDestroy(ev);
     cudaGetLastError();  // a failed free must not surface in a later call
@@ -565,41 +583,71 @@ static int run_common(ppr_ctx *ctx, const ppr_graph *g, const ppr_run_args *a, c
         return code;
     };
     const size_t S = (size_t)r->S;
-    if ((rc = dev_alloc((void **)&r->d_nnz, sizeof(uint32_t) * S, "row sizes", st))) return fail(rc);
-    if ((rc = dev_alloc((void **)&r->d_cols, sizeof(int32_t) * S * r->cap, "row ids", st))) return fail(rc);
-    if ((rc = dev_alloc((void **)&r->d_cnts, sizeof(uint32_t) * S * r->cap, "row counts", st))) return fail(rc);
-    if (r->topk > 0) {
-        if ((rc = dev_alloc((void **)&r->d_topk_idx, sizeof(int32_t) * S * r->topk, "top-k ids", st))) return fail(rc);
-        if ((rc = dev_alloc((void **)&r->d_topk_cnt, sizeof(uint32_t) * S * r->topk, "top-k counts", st))) return fail(rc);
-    }
-    if ((rc = dev_alloc((void **)&r->d_steps, sizeof(unsigned long long) * 8, "counters", st))) return fail(rc);
-    uint32_t *d_list = nullptr;
-    if (list) {
-        if ((rc = dev_alloc((void **)&d_list, sizeof(uint32_t) * S, "source list", st))) return fail(rc);
-        r->scratch.push_back(d_list);
-        cudaError_t e = cudaMemcpyAsync(d_list, list, sizeof(uint32_t) * S, cudaMemcpyHostToDevice, st);
-        if (e != cudaSuccess) return fail(cuda_fail(e, "source list upload"));
-    }
-    cudaError_t e = cudaEventCreate(&r->ev_start);
-    if (e == cudaSuccess) e = cudaEventCreate(&r->ev_walk_end);
-    if (e == cudaSuccess) e = cudaEventCreate(&r->ev_done);
-    if (e != cudaSuccess) return fail(cuda_fail(e, "cudaEventCreate"));
-
     // Batch size (the paper's per-pipeline walk budget, gamma <= alpha*M/(n*c),
     // Sec. 4.3, becomes a source batch sized to device memory): every walk of
     // a batch keeps its 4-byte endpoint in HBM until the batch is aggregated;
     // that scratch is bounded to a quarter of the free memory.
     int64_t batch = r->S;
     if (a->max_batch_sources > 0) batch = std::min<int64_t>(batch, a->max_batch_sources);
-    {
+    // The buffers of a small run are one allocation (a query's time is mostly
+    // host calls); larger runs take them one by one.
+    const size_t row_bytes = sizeof(uint32_t) * S * r->cap, top_bytes = sizeof(uint32_t) * S * (size_t)r->topk;
+    uint32_t *d_list = nullptr;
+    unsigned char *ws = nullptr;
+    constexpr size_t kSmallRun = 64u << 20;
+    const size_t whole = align_up(sizeof(uint32_t) * S) + 2 * align_up(row_bytes) + 2 * align_up(top_bytes) +
+                         align_up(sizeof(unsigned long long) * 8) + (list ? align_up(sizeof(uint32_t) * S) : 0) +
+                         align_up(launch_workspace_bytes(g, plan, batch));
+    bool one = false;
+    if (whole <= kSmallRun) {
+        rc = dev_alloc(&r->block, whole, "run buffers", st);
+        one = rc == PPR_OK;
+    }
+    if (one) {
+        unsigned char *p = static_cast<unsigned char *>(r->block);
+        auto take = [&p](size_t bytes) {
+            unsigned char *q = p;
+            p += align_up(bytes);
+            return q;
+        };
+        r->d_nnz = reinterpret_cast<uint32_t *>(take(sizeof(uint32_t) * S));
+        r->d_cols = reinterpret_cast<int32_t *>(take(row_bytes));
+        r->d_cnts = reinterpret_cast<uint32_t *>(take(row_bytes));
+        if (r->topk > 0) {
+            r->d_topk_idx = reinterpret_cast<int32_t *>(take(top_bytes));
+            r->d_topk_cnt = reinterpret_cast<uint32_t *>(take(top_bytes));
+        }
+        r->d_steps = reinterpret_cast<unsigned long long *>(take(sizeof(unsigned long long) * 8));
+        if (list) d_list = reinterpret_cast<uint32_t *>(take(sizeof(uint32_t) * S));
+        ws = take(0);
+    } else {
+        if ((rc = dev_alloc((void **)&r->d_nnz, sizeof(uint32_t) * S, "row sizes", st))) return fail(rc);
+        if ((rc = dev_alloc((void **)&r->d_cols, row_bytes, "row ids", st))) return fail(rc);
+        if ((rc = dev_alloc((void **)&r->d_cnts, row_bytes, "row counts", st))) return fail(rc);
+        if (r->topk > 0) {
+            if ((rc = dev_alloc((void **)&r->d_topk_idx, top_bytes, "top-k ids", st))) return fail(rc);
+            if ((rc = dev_alloc((void **)&r->d_topk_cnt, top_bytes, "top-k counts", st))) return fail(rc);
+        }
+        if ((rc = dev_alloc((void **)&r->d_steps, sizeof(unsigned long long) * 8, "counters", st))) return fail(rc);
+        if (list) {
+            if ((rc = dev_alloc((void **)&d_list, sizeof(uint32_t) * S, "source list", st))) return fail(rc);
+            r->scratch.push_back(d_list);
+        }
         size_t free_b = 0, total_b = 0;
         cudaMemGetInfo(&free_b, &total_b);
         int64_t fit = (int64_t)(free_b / 4 / ((size_t)a->R * sizeof(uint32_t)));
         batch = std::max<int64_t>(1, std::min<int64_t>(batch, fit));
+        if ((rc = dev_alloc((void **)&ws, launch_workspace_bytes(g, plan, batch), "walk workspace", st))) return fail(rc);
+        r->scratch.push_back(ws);
     }
-    unsigned char *ws = nullptr;
-    if ((rc = dev_alloc((void **)&ws, launch_workspace_bytes(g, plan, batch), "walk workspace", st))) return fail(rc);
-    r->scratch.push_back(ws);
+    cudaError_t e = cudaSuccess;
+    if (list) {
+        e = cudaMemcpyAsync(d_list, list, sizeof(uint32_t) * S, cudaMemcpyHostToDevice, st);
+        if (e != cudaSuccess) return fail(cuda_fail(e, "source list upload"));
+    }
+    e = cudaEventCreate(&r->ev_start);
+    if (e == cudaSuccess) e = cudaEventCreate(&r->ev_done);
+    if (e != cudaSuccess) return fail(cuda_fail(e, "cudaEventCreate"));
     if ((e = cudaMemsetAsync(r->d_steps, 0, sizeof(unsigned long long) * 8, st)) != cudaSuccess)
         return fail(cuda_fail(e, "memset"));
     if ((e = cudaEventRecord(r->ev_start, st)) != cudaSuccess) return fail(cuda_fail(e, "cudaEventRecord"));
@@ -613,7 +661,6 @@ static int run_common(ppr_ctx *ctx, const ppr_graph *g, const ppr_run_args *a, c
             return fail(rc);
         }
     }
-    if ((e = cudaEventRecord(r->ev_walk_end, st)) != cudaSuccess) return fail(cuda_fail(e, "cudaEventRecord"));
     if ((e = cudaEventRecord(r->ev_done, st)) != cudaSuccess) return fail(cuda_fail(e, "cudaEventRecord"));
     *out = r;
     return PPR_OK;
@@ -659,11 +706,8 @@ int ppr_run_to_host(ppr_ctx *ctx, const ppr_graph *g, const ppr_run_args *a, int
     Range range("ppr_run_to_host");
     cudaStream_t st = (cudaStream_t)a->stream;
     if ((rc = prepare_tables(g, plan, st))) return rc;
+    if ((rc = copy_resources(ctx))) return rc;
     cudaError_t e = cudaSuccess;
-    if (!ctx->copy_stream && (e = cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking)) != cudaSuccess)
-        return cuda_fail(e, "copy stream");
-    if (!ctx->pinned && (e = cudaHostAlloc((void **)&ctx->pinned, 4 * sizeof(unsigned long long), 0)) != cudaSuccess)
-        return cuda_fail(e, "page-locked words");
     cudaStream_t cs = ctx->copy_stream;
     const int64_t S = a->src_end - a->src_begin;
     const uint32_t rcap = row_capacity(g, a->R);
@@ -757,7 +801,8 @@ int ppr_run_to_host(ppr_ctx *ctx, const ppr_graph *g, const ppr_run_args *a, int
             if ((rc = launch_walks(ctx, g, plan, o, a->src_begin + b0, nb, nullptr, 0, ws, st, r, i > 0)))
                 return finish(rc);
             exclusive_scan_u32(q.nnz, nb, q.off, q.tmp, st);
-            k_compact_rows<<<std::max(1, cblocks), 256, 0, st>>>(nb, rcap, q.nnz, q.off, q.cols, q.cnts, q.ccol, q.ccnt);
+            k_compact_rows<<<std::max(1, cblocks), 256, 0, st>>>(nb, rcap, q.nnz, q.off, ~0ull, q.cols, q.cnts, q.ccol,
+                                                                 q.ccnt);
             note_launch();
             // row starts made absolute here, so the copy stream runs copies only:
             // a kernel there would wait for SMs behind the next batch's walker
@@ -1032,22 +1077,25 @@ int ppr_wait(ppr_result *r, int64_t timeout_ms)
     int rc = set_device(r->ctx);
     if (rc) return rc;
     if (r->waited) return PPR_OK;
+    // a short run is waited for without sleeping (a sleep of 50 us takes 100);
+    // after two milliseconds the thread gives its core back between looks
     auto t0 = std::chrono::steady_clock::now();
     for (;;) {
         cudaError_t e = cudaEventQuery(r->ev_done);
         if (e == cudaSuccess) break;
         if (e != cudaErrorNotReady) return cuda_fail(e, "run");
-        if (timeout_ms >= 0) {
-            auto ms = std::chrono::duration_cast<std::chrono::milliseconds>(std::chrono::steady_clock::now() - t0).count();
-            if (ms >= timeout_ms) {
-                set_error("run not finished after %lld ms", (long long)timeout_ms);
-                return PPR_ETIMEOUT;
-            }
+        const auto us = std::chrono::duration_cast<std::chrono::microseconds>(std::chrono::steady_clock::now() - t0).count();
+        if (timeout_ms >= 0 && us >= 1000 * timeout_ms) {
+            set_error("run not finished after %lld ms", (long long)timeout_ms);
+            return PPR_ETIMEOUT;
         }
-        std::this_thread::sleep_for(std::chrono::microseconds(50));
+        if (us >= 2000) std::this_thread::sleep_for(std::chrono::microseconds(50));
     }
-    unsigned long long cnt[6] = {0, 0, 0, 0, 0, 0};
-    PPR_CUDA(cudaMemcpy(cnt, r->d_steps, sizeof(cnt), cudaMemcpyDeviceToHost));
+    // the run is over: its counters are read beside whatever the caller's streams do now
+    if ((rc = copy_resources(r->ctx))) return rc;
+    unsigned long long *cnt = r->ctx->pinned;
+    PPR_CUDA(cudaMemcpyAsync(cnt, r->d_steps, 6 * sizeof(cnt[0]), cudaMemcpyDeviceToHost, r->ctx->copy_stream));
+    PPR_CUDA(cudaStreamSynchronize(r->ctx->copy_stream));
     r->steps = cnt[0];
     r->sectors = cnt[2];
     r->model_sectors = cnt[5];
@@ -1057,7 +1105,7 @@ int ppr_wait(ppr_result *r, int64_t timeout_ms)
         return PPR_ECUDA;
     }
     float ms = 0.f;
-    PPR_CUDA(cudaEventElapsedTime(&ms, r->ev_start, r->ev_walk_end));
+    PPR_CUDA(cudaEventElapsedTime(&ms, r->ev_start, r->ev_done));
     r->run_ms = ms;
     float kms = 0.f;
     for (size_t i = 0; i + 1 < r->walk_events.size(); i += 2) {
@@ -1112,14 +1160,16 @@ int ppr_sparse_rows(const ppr_result *rc_, int64_t *row_ptr, int32_t *col, uint3
     cudaStream_t st = r->stream;
     const int64_t S = r->S;
     int64_t tiles = (S + kScanTile - 1) / kScanTile;
+    if ((rc = copy_resources(r->ctx))) return rc;
     uint64_t *d_off = nullptr, *d_tmp = nullptr;
-    if ((rc = dev_alloc((void **)&d_off, sizeof(uint64_t) * (S + 1), "row offsets", st))) return rc;
-    if ((rc = dev_alloc((void **)&d_tmp, sizeof(uint64_t) * (tiles + 2), "scan scratch", st)))
-        return dev_free(d_off, st), rc;
+    // row starts straight into the caller's device array when there is one
+    const bool own_off = !(dev_out && row_ptr);
+    if (!own_off) d_off = reinterpret_cast<uint64_t *>(row_ptr);
+    else if ((rc = dev_alloc((void **)&d_off, sizeof(uint64_t) * (S + 1), "row offsets", st))) return rc;
     int32_t *d_col = nullptr;
     uint32_t *d_cnt = nullptr;
     auto done = [&](int code) {
-        dev_free(d_off, st);
+        if (own_off) dev_free(d_off, st);
         dev_free(d_tmp, st);
         if (!dev_out) {
             dev_free(d_col, st);
@@ -1127,16 +1177,27 @@ int ppr_sparse_rows(const ppr_result *rc_, int64_t *row_ptr, int32_t *col, uint3
         }
         return code;
     };
+    if ((rc = dev_alloc((void **)&d_tmp, sizeof(uint64_t) * (tiles + 2), "scan scratch", st))) return done(rc);
     exclusive_scan_u32(r->d_nnz, S, d_off, d_tmp, st);
-    uint64_t total = 0;
-    cudaError_t e = cudaMemcpyAsync(&total, d_off + S, sizeof(uint64_t), cudaMemcpyDeviceToHost, st);
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((S + 255) / 256, (int64_t)r->ctx->sms * 32));
+    // into device arrays the rows are compacted at once, if they fit (the
+    // kernel looks); host arrays need the total first
+    const bool at_once = dev_out && col && cnt;
+    if (at_once) {
+        k_compact_rows<<<blocks, 256, 0, st>>>(S, r->cap, r->d_nnz, d_off, (uint64_t)std::max<int64_t>(cap, 0), r->d_cols,
+                                               r->d_cnts, col, cnt);
+        note_launch();
+    }
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(r->ctx->pinned, d_off + S, sizeof(uint64_t), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return done(cuda_fail(e, "row scan"));
+    const uint64_t total = r->ctx->pinned[0];
     r->nnz_total = (int64_t)total;
     if (nnz) *nnz = (int64_t)total;
-    if (row_ptr) {
-        e = cudaMemcpyAsync(row_ptr, d_off, sizeof(int64_t) * (S + 1),
-                            dev_out ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, st);
+    if (row_ptr && own_off) {
+        e = cudaMemcpyAsync(row_ptr, d_off, sizeof(int64_t) * (S + 1), cudaMemcpyDeviceToHost, st);
         if (e != cudaSuccess) return done(cuda_fail(e, "row_ptr copy"));
     }
     if (col || cnt) {
@@ -1148,19 +1209,13 @@ int ppr_sparse_rows(const ppr_result *rc_, int64_t *row_ptr, int32_t *col, uint3
             set_error("capacity %lld < nnz %llu", (long long)cap, (unsigned long long)total);
             return done(PPR_ERANGE);
         }
-        if (dev_out) {
-            d_col = col;
-            d_cnt = cnt;
-        } else {
-            if ((rc = dev_alloc((void **)&d_col, sizeof(int32_t) * (total + 1), "compacted ids", st))) return done(rc);
-            if ((rc = dev_alloc((void **)&d_cnt, sizeof(uint32_t) * (total + 1), "compacted counts", st))) return done(rc);
-        }
-        int blocks = (int)std::min<int64_t>((S + 255) / 256, (int64_t)r->ctx->sms * 32);
-        if (blocks < 1) blocks = 1;
-        k_compact_rows<<<blocks, 256, 0, st>>>(S, r->cap, r->d_nnz, d_off, r->d_cols, r->d_cnts, d_col, d_cnt);
+        if (at_once) return done(PPR_OK);
+        if ((rc = dev_alloc((void **)&d_col, sizeof(int32_t) * (total + 1), "compacted ids", st))) return done(rc);
+        if ((rc = dev_alloc((void **)&d_cnt, sizeof(uint32_t) * (total + 1), "compacted counts", st))) return done(rc);
+        k_compact_rows<<<blocks, 256, 0, st>>>(S, r->cap, r->d_nnz, d_off, total, r->d_cols, r->d_cnts, d_col, d_cnt);
         note_launch();
         e = cudaGetLastError();
-        if (e == cudaSuccess && !dev_out && total > 0) {
+        if (e == cudaSuccess && total > 0) {
             e = cudaMemcpyAsync(col, d_col, sizeof(int32_t) * total, cudaMemcpyDeviceToHost, st);
             if (e == cudaSuccess) e = cudaMemcpyAsync(cnt, d_cnt, sizeof(uint32_t) * total, cudaMemcpyDeviceToHost, st);
         }
@@ -1184,10 +1239,15 @@ int ppr_topk(const ppr_result *r, int32_t k, int32_t *idx, uint32_t *cnt, uint32
         return PPR_EINVAL;
     }
     cudaMemcpyKind kind = (flags & PPR_PTRS_DEVICE) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-    PPR_CUDA(cudaMemcpy2DAsync(idx, sizeof(int32_t) * k, r->d_topk_idx, sizeof(int32_t) * r->topk, sizeof(int32_t) * k,
-                               (size_t)r->S, kind, r->stream));
-    PPR_CUDA(cudaMemcpy2DAsync(cnt, sizeof(uint32_t) * k, r->d_topk_cnt, sizeof(uint32_t) * r->topk,
-                               sizeof(uint32_t) * k, (size_t)r->S, kind, r->stream));
+    if (k == r->topk) {  // whole rows: plain copies
+        PPR_CUDA(cudaMemcpyAsync(idx, r->d_topk_idx, sizeof(int32_t) * k * (size_t)r->S, kind, r->stream));
+        PPR_CUDA(cudaMemcpyAsync(cnt, r->d_topk_cnt, sizeof(uint32_t) * k * (size_t)r->S, kind, r->stream));
+    } else {
+        PPR_CUDA(cudaMemcpy2DAsync(idx, sizeof(int32_t) * k, r->d_topk_idx, sizeof(int32_t) * r->topk, sizeof(int32_t) * k,
+                                   (size_t)r->S, kind, r->stream));
+        PPR_CUDA(cudaMemcpy2DAsync(cnt, sizeof(uint32_t) * k, r->d_topk_cnt, sizeof(uint32_t) * r->topk,
+                                   sizeof(uint32_t) * k, (size_t)r->S, kind, r->stream));
+    }
     PPR_CUDA(cudaStreamSynchronize(r->stream));
     return PPR_OK;
 }

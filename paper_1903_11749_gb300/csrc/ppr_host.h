@@ -71,8 +71,8 @@ struct ppr_ctx {
     size_t l2_persist_set = 0;    // persisting set-aside this context asked for
     size_t l2_bytes = 0;          // L2 size (the layout's renumbering policy)
     size_t mem_bytes = 0;         // device memory (the layout's slot density)
-    cudaStream_t copy_stream = nullptr;  // output copies of ppr_run_to_host
-    unsigned long long *pinned = nullptr;  // page-locked words for per-batch totals
+    cudaStream_t copy_stream = nullptr;  // copies to the host beside the caller's streams
+    unsigned long long *pinned = nullptr;  // page-locked words: per-batch totals, a finished run's counters
     std::atomic<int> refs{1};  // the caller's handle plus every live graph and result
 };
 
@@ -128,7 +128,8 @@ struct ppr_result {
     uint32_t *d_topk_cnt = nullptr;
     unsigned long long *d_steps = nullptr;  // counters: [0] steps, [1] work queue, [2] sectors, [3] chunks,
                                             // [4] checked-build flags, [5] flat-CSR model sectors
-    cudaEvent_t ev_start = nullptr, ev_walk_end = nullptr, ev_done = nullptr;
+    cudaEvent_t ev_start = nullptr, ev_done = nullptr;
+    void *block = nullptr;       // one allocation behind the buffers of a small run, or null
     std::vector<cudaEvent_t> walk_events;  // (before, after) each walker launch
     bool waited = false;
     uint64_t steps = 0, sectors = 0, model_sectors = 0;

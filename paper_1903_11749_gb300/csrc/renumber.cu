@@ -172,7 +172,7 @@ int number_nodes(int64_t n, int64_t m, const int64_t *d_rp, const int64_t *d_off
     A.exact = g->instances == 0 && n > kExactMin && n <= kExactNodes;
     // nodes a warp takes in turn: few where the graph is small (a warp's chain
     // of rounds is then the kernel's time)
-    A.tile = n <= (1 << 18) ? 128u : 1024u;
+    A.tile = n <= 2048 ? 32u : (n <= (1 << 18) ? 128u : 1024u);
     A.tiles = (n + A.tile - 1) / A.tile;
     A.heads = heads;
     A.st = d_stats;
