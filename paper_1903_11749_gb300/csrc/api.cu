@@ -69,22 +69,23 @@ void dev_free(void *p, cudaStream_t st)
 }
 
 // Row compaction: the stored pairs of each source to the compacted position
-// given by the exclusive scan of the row sizes.  A warp takes 32 sources: it
-// reads their sizes and positions at once, so that no row's copy waits for
-// its own, and four rows' pairs are in flight at a time.  Bound by memory
+// given by the exclusive scan of the row sizes.  A warp takes `take` sources
+// (4 to 32): it reads their sizes and positions at once, so that no row's copy
+// waits for its own, and four rows' pairs are in flight at a time.  Bound by memory
 // (R-MAT scale 24, 600 M pairs: 4.36 -> 2.52 ms).
 // Nothing is written when the rows hold more than `limit` pairs.
 __global__ void __launch_bounds__(256) k_compact_rows(int64_t S, uint32_t cap, const uint32_t *nnz, const uint64_t *off,
-                                                      uint64_t limit, const int32_t *cols, const uint32_t *cnts,
-                                                      int32_t *ocol, uint32_t *ocnt)
+                                                      uint64_t limit, uint32_t take, const int32_t *cols,
+                                                      const uint32_t *cnts, int32_t *ocol, uint32_t *ocnt)
 {
     if (off[S] > limit) return;
     const uint32_t lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t s0 = 32 * (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5); s0 < S; s0 += 32 * warps) {
-        const uint32_t my_c = s0 + lane < S ? nnz[s0 + lane] : 0u;
-        const uint64_t my_o = s0 + lane < S ? off[s0 + lane] : 0ull;
-        for (uint32_t r0 = 0; r0 < 32; r0 += 4) {
+    for (int64_t s0 = take * (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5); s0 < S; s0 += take * warps) {
+        const bool mine = lane < take && s0 + lane < S;
+        const uint32_t my_c = mine ? nnz[s0 + lane] : 0u;
+        const uint64_t my_o = mine ? off[s0 + lane] : 0ull;
+        for (uint32_t r0 = 0; r0 < take; r0 += 4) {
             uint32_t c[4], longest = 0;
             uint64_t o[4];
 #pragma unroll
@@ -112,6 +113,19 @@ __global__ void __launch_bounds__(256) k_compact_rows(int64_t S, uint32_t cap, c
             }
         }
     }
+}
+
+// Sources a warp: 32 where that still fills the chip, else fewer.
+static int launch_compact(ppr_ctx *ctx, int64_t S, uint32_t cap, const uint32_t *nnz, const uint64_t *off, uint64_t limit,
+                          const int32_t *cols, const uint32_t *cnts, int32_t *ocol, uint32_t *ocnt, cudaStream_t st)
+{
+    const int64_t share = S / ((int64_t)ctx->sms * 32);
+    const uint32_t take = share >= 32 ? 32u : (share >= 16 ? 16u : (share >= 8 ? 8u : 4u));
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((S + 8 * take - 1) / (8 * take), (int64_t)ctx->sms * 32));
+    k_compact_rows<<<blocks, 256, 0, st>>>(S, cap, nnz, off, limit, take, cols, cnts, ocol, ocnt);
+    note_launch();
+    PPR_CUDA(cudaGetLastError());
+    return PPR_OK;
 }
 
 // Row starts of one batch made absolute: off[i] += *base, the entries of the
@@ -788,7 +802,6 @@ int ppr_run_to_host(ppr_ctx *ctx, const ppr_graph *g, const ppr_run_args *a, int
     if ((e = cudaMemsetAsync(r->d_steps, 0, sizeof(unsigned long long) * 8, st)) != cudaSuccess)
         return finish(cuda_fail(e, "memset"));
     unsigned long long *d_base = r->d_steps + 7;
-    const int cblocks = (int)std::min<int64_t>((B + 255) / 256, (int64_t)ctx->sms * 32);
     uint64_t base = 0;
     for (int64_t i = 0; i <= P; ++i) {
         if (i < P) {  // batch i: walk, reduce, compact on the run's stream
@@ -801,9 +814,8 @@ int ppr_run_to_host(ppr_ctx *ctx, const ppr_graph *g, const ppr_run_args *a, int
             if ((rc = launch_walks(ctx, g, plan, o, a->src_begin + b0, nb, nullptr, 0, ws, st, r, i > 0)))
                 return finish(rc);
             exclusive_scan_u32(q.nnz, nb, q.off, q.tmp, st);
-            k_compact_rows<<<std::max(1, cblocks), 256, 0, st>>>(nb, rcap, q.nnz, q.off, ~0ull, q.cols, q.cnts, q.ccol,
-                                                                 q.ccnt);
-            note_launch();
+            if ((rc = launch_compact(ctx, nb, rcap, q.nnz, q.off, ~0ull, q.cols, q.cnts, q.ccol, q.ccnt, st)))
+                return finish(rc);
             // row starts made absolute here, so the copy stream runs copies only:
             // a kernel there would wait for SMs behind the next batch's walker
             k_add_base<<<(int)std::min<int64_t>((nb + 256) / 256, (int64_t)ctx->sms * 8), 256, 0, st>>>(nb + 1, q.off,
@@ -1179,14 +1191,13 @@ int ppr_sparse_rows(const ppr_result *rc_, int64_t *row_ptr, int32_t *col, uint3
     };
     if ((rc = dev_alloc((void **)&d_tmp, sizeof(uint64_t) * (tiles + 2), "scan scratch", st))) return done(rc);
     exclusive_scan_u32(r->d_nnz, S, d_off, d_tmp, st);
-    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((S + 255) / 256, (int64_t)r->ctx->sms * 32));
     // into device arrays the rows are compacted at once, if they fit (the
     // kernel looks); host arrays need the total first
     const bool at_once = dev_out && col && cnt;
     if (at_once) {
-        k_compact_rows<<<blocks, 256, 0, st>>>(S, r->cap, r->d_nnz, d_off, (uint64_t)std::max<int64_t>(cap, 0), r->d_cols,
-                                               r->d_cnts, col, cnt);
-        note_launch();
+        if ((rc = launch_compact(r->ctx, S, r->cap, r->d_nnz, d_off, (uint64_t)std::max<int64_t>(cap, 0), r->d_cols,
+                                 r->d_cnts, col, cnt, st)))
+            return done(rc);
     }
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess)
@@ -1212,10 +1223,9 @@ int ppr_sparse_rows(const ppr_result *rc_, int64_t *row_ptr, int32_t *col, uint3
         if (at_once) return done(PPR_OK);
         if ((rc = dev_alloc((void **)&d_col, sizeof(int32_t) * (total + 1), "compacted ids", st))) return done(rc);
         if ((rc = dev_alloc((void **)&d_cnt, sizeof(uint32_t) * (total + 1), "compacted counts", st))) return done(rc);
-        k_compact_rows<<<blocks, 256, 0, st>>>(S, r->cap, r->d_nnz, d_off, total, r->d_cols, r->d_cnts, d_col, d_cnt);
-        note_launch();
-        e = cudaGetLastError();
-        if (e == cudaSuccess && total > 0) {
+        if ((rc = launch_compact(r->ctx, S, r->cap, r->d_nnz, d_off, total, r->d_cols, r->d_cnts, d_col, d_cnt, st)))
+            return done(rc);
+        if (total > 0) {
             e = cudaMemcpyAsync(col, d_col, sizeof(int32_t) * total, cudaMemcpyDeviceToHost, st);
             if (e == cudaSuccess) e = cudaMemcpyAsync(cnt, d_cnt, sizeof(uint32_t) * total, cudaMemcpyDeviceToHost, st);
         }
