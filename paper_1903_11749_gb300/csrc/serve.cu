@@ -17,7 +17,9 @@
 // the query's sources one at a time (the per-source reduction of
 // aggregate.cuh), writes each top-k row straight into pinned host memory and,
 // after the last row, marks the query done in host-mapped memory, where the
-// host's scheduler thread picks it up.  Every wait on the device is bounded in
+// host's scheduler thread picks it up.  A walking warp that has no walk left
+// and finds none to claim reduces sources too (queries of R <= 128), so the
+// end of a burst is not left to an eighth of the warps.  Every wait on the device is bounded in
 // time (%globaltimer): a loop without work exits after idle_us and the host
 // launches it again with the next query; a published slot whose descriptor
 // does not appear within a second ends the loop with an error status, which
@@ -214,40 +216,46 @@ __device__ __forceinline__ uint64_t block_tail(const LoopParams &P, unsigned lon
 
 // Work of one walker warp: a chunk of walks [g0, g0 + total) of query `id`.
 struct WalkChunk {
-    uint64_t id, magic;
+    uint64_t magic;
     const uint32_t *src;
     uint32_t slot, g0, issued, total, R, T, k0, k1;
 };
 
-// Lane 0: fills *c with chunk ci of the query whose descriptor is in slot s
-// (sequence number + 1 = tag), once that descriptor is in place (the host
-// writes it before the slot's counters; bounded wait).  1, or -1 when the
-// wait ran out.
-__device__ int take_chunk(const LoopParams &P, uint32_t s, uint32_t tag, uint32_t ci, WalkChunk *c)
+// The fields of a descriptor a chunk needs.
+struct ChunkDesc {
+    uint32_t cw, walks, nchunks, R, T, k0, k1;
+    uint64_t magic;
+    const uint32_t *src;
+};
+__device__ __forceinline__ ChunkDesc load_desc(const SDesc *d)
 {
-    const SDesc *d = P.desc + s;
-    const uint64_t t0 = gtime_ns();
-    while ((uint32_t)__ldcg(&d->seq1) != tag) {
-        if (gtime_ns() - t0 > kSlotWaitNs) {
-            flag_exit(P, PPR_LOOP_SLOT_TIMEOUT);
-            return -1;
-        }
-        __nanosleep(500);
-    }
-    atomicCAS(&P.slot[s].t_claim, 0ull, (unsigned long long)gtime_ns());
-    const uint32_t cw = __ldcg(&d->cw), walks = __ldcg(&d->walks);
-    c->id = __ldcg(&d->seq1) - 1;
+    ChunkDesc c;
+    c.cw = __ldcg(&d->cw);
+    c.walks = __ldcg(&d->walks);
+    c.nchunks = __ldcg(&d->nchunks);
+    c.R = __ldcg(&d->R);
+    c.T = __ldcg(&d->T);
+    c.k0 = __ldcg(&d->k0);
+    c.k1 = __ldcg(&d->k1);
+    c.magic = __ldcg(&d->r_magic);
+    c.src = reinterpret_cast<const uint32_t *>(__ldcg(reinterpret_cast<const unsigned long long *>(&d->src)));
+    return c;
+}
+
+// Lane 0: fills *c with chunk ci of the query in slot s (sequence number + 1 = tag).
+__device__ __forceinline__ void take_chunk(const LoopParams &P, uint32_t s, uint32_t ci, const ChunkDesc &d, WalkChunk *c)
+{
+    if (ci == 0) P.slot[s].t_claim = gtime_ns();
     c->slot = s;
-    c->g0 = ci * cw;
-    c->total = min(cw, walks - ci * cw);
+    c->g0 = ci * d.cw;
+    c->total = min(d.cw, d.walks - ci * d.cw);
     c->issued = 0;
-    c->R = __ldcg(&d->R);
-    c->T = __ldcg(&d->T);
-    c->k0 = __ldcg(&d->k0);
-    c->k1 = __ldcg(&d->k1);
-    c->magic = __ldcg(&d->r_magic);
-    c->src = reinterpret_cast<const uint32_t *>(__ldcg(reinterpret_cast<const unsigned long long *>(&d->src)));
-    return 1;
+    c->R = d.R;
+    c->T = d.T;
+    c->k0 = d.k0;
+    c->k1 = d.k1;
+    c->magic = d.magic;
+    c->src = d.src;
 }
 
 // Whole warp: hands out one chunk of some published query into *c (written by
@@ -314,15 +322,28 @@ __device__ int claim_chunk(const LoopParams &P, uint32_t start, WalkChunk *c, un
         int got = 0;
         if (lane == 0) {
             const uint32_t s = (uint32_t)((h + i) % kRing);
+            const SDesc *d = P.desc + s;
+            // The descriptor is read while the add is under way: the slot held
+            // query h + i when its claim word was read above, so if the add says
+            // that it still does, what was read in between is that query's.
+            ChunkDesc dc = load_desc(d);
             const unsigned long long old = atomicAdd(&P.slot[s].claim, 1ull);
             const uint32_t tag = (uint32_t)(old >> 32), ci = (uint32_t)old;
-            // the chunk exists if ci is below the chunk count of the query that holds the slot now
-            const SDesc *d = P.desc + s;
-            if (tag != 0) {
+            if (tag == (uint32_t)(h + i + 1)) {
+                got = ci < dc.nchunks;
+            } else if (tag != 0) {  // reused meanwhile: the query that holds it now, once its descriptor is in place
                 const uint64_t t0 = gtime_ns();
-                while ((uint32_t)__ldcg(&d->seq1) != tag && gtime_ns() - t0 < kSlotWaitNs) __nanosleep(500);
-                if ((uint32_t)__ldcg(&d->seq1) == tag && ci < __ldcg(&d->nchunks)) got = take_chunk(P, s, tag, ci, c);
+                bool there;
+                while (!(there = (uint32_t)__ldcg(&d->seq1) == tag) && gtime_ns() - t0 < kSlotWaitNs) __nanosleep(500);
+                if (there) {
+                    dc = load_desc(d);
+                    got = ci < dc.nchunks;
+                } else {
+                    flag_exit(P, PPR_LOOP_SLOT_TIMEOUT);
+                    got = -1;
+                }
             }
+            if (got > 0) take_chunk(P, s, ci, dc, c);
         }
         got = __shfl_sync(0xffffffffu, got, 0);
         if (got) return got;
@@ -338,9 +359,26 @@ __device__ __forceinline__ void count_walks(const LoopParams &P, uint32_t q, uin
     if (old + n == __ldcg(&P.desc[q].walks)) P.slot[q].t_walks = gtime_ns();
 }
 
+constexpr uint32_t kHelpMaxR = 128;  // walker warps without walks reduce sources of queries up to this R
+__device__ __noinline__ int claim_source(const LoopParams &P, unsigned long long *s_tail, bool refresh, uint32_t max_R,
+                            uint64_t &id_out, uint32_t &slot_out, uint32_t &i_out, uint32_t &n_out, bool &in_flight);
+__device__ __noinline__ void reduce_source(const LoopParams &P, const CallerIds &ids, uint32_t s, uint32_t i,
+                                           uint32_t *smem, uint32_t cap);
+__device__ void finish_source(const LoopParams &P, uint64_t id, uint32_t s, uint32_t n);
+
+// Activity of a walker warp since its last flush to P.glob (lane 0; shared memory).
+struct WarpActivity {
+    long long c_start;
+    unsigned long long c_sleep, c_claim;
+    uint32_t n_sleep, n_claim, n_miss;
+};
+
+// Walks until the warp has neither a walk nor a chunk to claim.  Returns 1 if
+// it walked, 0 if not, or -1 when the loop must end (a descriptor wait ran out).
 template <class E>
-__device__ void walker_warp(const LoopParams &P, const ClassTab &tab, WalkChunk &wc, uint32_t **ends_of,
-                            uint32_t gwarp, unsigned long long *s_tail)
+__device__ __forceinline__ int walk_until_idle(const LoopParams &P, const ClassTab &tab, WalkChunk &wc,
+                                               uint32_t **ends_of, uint32_t gwarp, unsigned long long *s_tail,
+                                               WarpActivity &act)
 {
     const uint32_t lane = threadIdx.x & 31;
     bool active = false;
@@ -351,11 +389,11 @@ __device__ void walker_warp(const LoopParams &P, const ClassTab &tab, WalkChunk 
     uint32_t T = 0;
     uint32_t pend_q = 0xffffffffu, pend_n = 0;  // uniform: walks of pend_q finished, not yet counted
     bool have = false;                          // uniform: wc holds walks left to issue
-    uint64_t idle_t0 = 0, flush_t = gtime_ns(), claim_after = 0;
-    uint32_t backoff = 256;
-    uint32_t n_iter = 0, n_claim = 0, n_miss = 0, n_sleep = 0;  // activity, flushed to P.glob
-    unsigned long long c_claim = 0, c_step = 0, c_sleep = 0;
-    long long c_start = clock64();
+    uint64_t flush_t = gtime_ns(), claim_after = 0;
+    uint32_t n_iter = 0, n_claim = 0, n_miss = 0;  // activity
+    uint32_t c_claim = 0, c_step = 0;              // clock cycles (flushed long before they wrap)
+    int status = 0;
+    bool walked = false;
     Tally tl;
     auto flush = [&]() {
         unsigned long long d = tl.steps;
@@ -365,32 +403,31 @@ __device__ void walker_warp(const LoopParams &P, const ClassTab &tab, WalkChunk 
             const long long now = clock64();
             atomicAdd(&P.glob->draws, d);
             atomicAdd(&P.glob->iterations, (unsigned long long)n_iter);
-            atomicAdd(&P.glob->claims, (unsigned long long)n_claim);
-            atomicAdd(&P.glob->claim_misses, (unsigned long long)n_miss);
-            atomicAdd(&P.glob->sleeps, (unsigned long long)n_sleep);
-            atomicAdd(&P.glob->cyc_claim, c_claim);
-            atomicAdd(&P.glob->cyc_step, c_step);
-            atomicAdd(&P.glob->cyc_sleep, c_sleep);
-            atomicAdd(&P.glob->cyc_total, (unsigned long long)(now - c_start));
-            c_start = now;
+            atomicAdd(&P.glob->claims, (unsigned long long)act.n_claim + n_claim);
+            atomicAdd(&P.glob->claim_misses, (unsigned long long)act.n_miss + n_miss);
+            atomicAdd(&P.glob->sleeps, (unsigned long long)act.n_sleep);
+            atomicAdd(&P.glob->cyc_claim, act.c_claim + c_claim);
+            atomicAdd(&P.glob->cyc_step, (unsigned long long)c_step);
+            atomicAdd(&P.glob->cyc_sleep, act.c_sleep);
+            atomicAdd(&P.glob->cyc_total, (unsigned long long)(now - act.c_start));
+            act = WarpActivity{now, 0, 0, 0, 0, 0};
         }
         tl.steps = 0;
-        n_iter = n_claim = n_miss = n_sleep = 0;
-        c_claim = c_step = c_sleep = 0;
+        n_iter = n_claim = n_miss = 0;
+        c_claim = c_step = 0;
     };
     for (;;) {
         uint32_t idle = __ballot_sync(0xffffffffu, !active);
         const bool all_idle = idle == 0xffffffffu;
         if ((uint32_t)__popc(idle) < P.refill) idle = 0;
         // after a claim found nothing, a warp with walks still running tries again only later
-        if (!all_idle && !have && claim_after && gtime_ns() < claim_after) idle = 0;
-        int status = 0;
+        if (idle && !all_idle && !have && claim_after && gtime_ns() < claim_after) idle = 0;
         while (idle) {
             if (!have) {
-                const long long c0 = clock64();
+                const uint32_t c0 = clock();
                 const int r = claim_chunk(P, gwarp, &wc, s_tail);
                 __syncwarp();
-                c_claim += clock64() - c0;
+                c_claim += clock() - c0;
                 ++n_claim;
                 n_miss += r <= 0;
                 claim_after = (r == 0 && !all_idle) ? gtime_ns() + kClaimRetryNs : 0;
@@ -434,27 +471,9 @@ __device__ void walker_warp(const LoopParams &P, const ClassTab &tab, WalkChunk 
             idle = __ballot_sync(0xffffffffu, !active);
         }
         if (status < 0) break;  // a descriptor wait ran out: the loop ends
-        if (__ballot_sync(0xffffffffu, active) == 0) {
-            // no walk and no chunk: stop, or wait (bounded) for the next query
-            if (ld_volatile(&P.ctl->stop)) {
-                if (lane == 0) flag_exit(P, PPR_LOOP_STOPPED);
-                break;
-            }
-            const uint64_t t = gtime_ns();
-            if (idle_t0 == 0) idle_t0 = t;
-            else if (t - idle_t0 > P.idle_ns) {
-                if (lane == 0) flag_exit(P, PPR_LOOP_IDLE);
-                break;
-            }
-            ++n_sleep;
-            const long long c0 = clock64();
-            __nanosleep(backoff);
-            c_sleep += clock64() - c0;
-            backoff = min(backoff * 2, 32768u);
-            continue;
-        }
-        idle_t0 = 0;
-        backoff = 256;
+        status = 0;
+        if (__ballot_sync(0xffffffffu, active) == 0) break;
+        walked = true;
         if (++n_iter % 1024 == 0) {
             const uint64_t t = gtime_ns();
             if (t - flush_t > 1000000) {
@@ -463,7 +482,7 @@ __device__ void walker_warp(const LoopParams &P, const ClassTab &tab, WalkChunk 
             }
         }
         bool fin = false;
-        const long long c0 = clock64();
+        const uint32_t c0 = clock();
         if (active && walk_step<E, false, false>(P.kp, tab, key, T, s0, src, j, 0, k, u, pend, tl)) {
             ends_of[q][g] = u;
             tl.steps += k;
@@ -471,7 +490,7 @@ __device__ void walker_warp(const LoopParams &P, const ClassTab &tab, WalkChunk 
             fin = true;
         }
         __syncwarp();
-        c_step += clock64() - c0;
+        c_step += clock() - c0;
         // completion counting: walks of pend_q add up in a register, others at once
         const uint32_t fin_m = __ballot_sync(0xffffffffu, fin);
         if (fin_m) {
@@ -497,14 +516,80 @@ __device__ void walker_warp(const LoopParams &P, const ClassTab &tab, WalkChunk 
         __syncwarp();
         if (lane == 0) count_walks(P, pend_q, pend_n);
     }
-    flush();
+    if (walked) {
+        flush();
+    } else if (lane == 0) {  // a look that found nothing: kept for the next flush
+        act.n_claim += n_claim;
+        act.n_miss += n_miss;
+        act.c_claim += c_claim;
+    }
+    return status < 0 ? status : (int)walked;
+}
+
+// A walker warp: walks, then helps reduce, then waits (bounded) for the next query.
+template <class E>
+__device__ __forceinline__ void walker_warp(const LoopParams &P, const ClassTab &tab, const CallerIds &ids, WalkChunk &wc,
+                                            uint32_t **ends_of, uint32_t *scratch, WarpActivity &act, uint32_t gwarp,
+                                            unsigned long long *s_tail)
+{
+    const uint32_t lane = threadIdx.x & 31;
+    if (lane == 0) act = WarpActivity{clock64(), 0, 0, 0, 0, 0};
+    __syncwarp();
+    uint64_t idle_t0 = 0;
+    uint32_t backoff = 256;
+    for (;;) {
+        const int walked = walk_until_idle<E>(P, tab, wc, ends_of, gwarp, s_tail, act);
+        if (walked < 0) break;
+        if (walked) {
+            idle_t0 = 0;
+            backoff = 256;
+        }
+        uint64_t id = 0;
+        uint32_t s = 0, i = 0, nb = 0;
+        bool in_flight = false;
+        const int r = claim_source(P, s_tail, false, kHelpMaxR, id, s, i, nb, in_flight);
+        if (r < 0) break;
+        if (r > 0) {
+            for (uint32_t b = 0; b < nb; ++b) reduce_source(P, ids, s, i + b, scratch, kHelpMaxR);
+            finish_source(P, id, s, nb);
+            idle_t0 = 0;
+            backoff = 256;
+            continue;
+        }
+        if (ld_volatile(&P.ctl->stop)) {
+            if (lane == 0) flag_exit(P, PPR_LOOP_STOPPED);
+            break;
+        }
+        const uint64_t t = gtime_ns();
+        if (idle_t0 == 0) idle_t0 = t;
+        else if (t - idle_t0 > P.idle_ns) {
+            if (lane == 0) flag_exit(P, PPR_LOOP_IDLE);
+            break;
+        }
+        if (in_flight) backoff = min(backoff, 1024u);  // other warps' walks are about to end: their sources come next
+        const long long c0 = clock64();
+        __nanosleep(backoff);
+        if (lane == 0) {
+            ++act.n_sleep;
+            act.c_sleep += clock64() - c0;
+        }
+        backoff = min(backoff * 2, 32768u);
+    }
+    if (lane == 0) {  // what is not flushed yet
+        atomicAdd(&P.glob->claims, (unsigned long long)act.n_claim);
+        atomicAdd(&P.glob->claim_misses, (unsigned long long)act.n_miss);
+        atomicAdd(&P.glob->sleeps, (unsigned long long)act.n_sleep);
+        atomicAdd(&P.glob->cyc_claim, act.c_claim);
+        atomicAdd(&P.glob->cyc_sleep, act.c_sleep);
+        atomicAdd(&P.glob->cyc_total, (unsigned long long)(clock64() - act.c_start));
+    }
 }
 
 // Whole warp: hands out one source of the oldest query whose walks are all
 // done.  Returns 1 (query id, slot, source i on every lane), 0 (none now),
 // -1 (the loop must end); *in_flight tells whether published queries still
 // have sources to hand out (ready or not).
-__device__ int claim_source(const LoopParams &P, unsigned long long *s_tail, bool refresh, uint32_t max_R,
+__device__ __noinline__ int claim_source(const LoopParams &P, unsigned long long *s_tail, bool refresh, uint32_t max_R,
                             uint64_t &id_out, uint32_t &slot_out, uint32_t &i_out, uint32_t &n_out, bool &in_flight)
 {
     const uint32_t lane = threadIdx.x & 31;
@@ -596,7 +681,7 @@ __device__ int claim_source(const LoopParams &P, unsigned long long *s_tail, boo
 
 // Reduction of source i of query slot s into its top-k row (host memory).
 // smem: cap endpoints, then the reduction's scratch (3 * cap words); cap >= R.
-__device__ void reduce_source(const LoopParams &P, const CallerIds &ids, uint32_t s, uint32_t i, uint32_t *smem,
+__device__ __noinline__ void reduce_source(const LoopParams &P, const CallerIds &ids, uint32_t s, uint32_t i, uint32_t *smem,
                               uint32_t cap)
 {
     const uint32_t lane = threadIdx.x & 31;
@@ -687,11 +772,13 @@ __device__ void aggregator_warp(const LoopParams &P, const CallerIds &ids, uint3
 }
 
 template <class E>
-__global__ void __launch_bounds__(32 * kLoopWarps, 4) k_serve_loop(LoopParams P)
+__global__ void __launch_bounds__(32 * kLoopWarps, 4) k_serve_loop(const __grid_constant__ LoopParams P)
 {
     __shared__ WalkChunk wc[kLoopWarps - 1];
     __shared__ uint32_t *ends_of[kRing];  // endpoint array of each slot, set by the warp that takes a chunk of it
     __shared__ __align__(16) uint32_t smem[kLoopMaxR + 3 * kLoopMaxR];  // the aggregator warp's endpoints and scratch
+    __shared__ __align__(16) uint32_t help[kLoopWarps - 1][2 * kHelpMaxR + 32];  // a helping warp's endpoints and scratch
+    __shared__ WarpActivity act[kLoopWarps - 1];
     __shared__ unsigned long long s_tail[2];  // the block's copy of the published tail, and when it was read
     __shared__ ClassTab tab;
     __shared__ uint32_t s_first[kTabEntries];
@@ -703,7 +790,8 @@ __global__ void __launch_bounds__(32 * kLoopWarps, 4) k_serve_loop(LoopParams P)
         aggregator_warp(P, CallerIds{P.kp.order, s_first}, smem, s_tail);
         return;
     }
-    walker_warp<E>(P, tab, wc[wid], ends_of, blockIdx.x * (kLoopWarps - 1) + wid, s_tail);
+    walker_warp<E>(P, tab, CallerIds{P.kp.order, s_first}, wc[wid], ends_of, help[wid], act[wid],
+                   blockIdx.x * (kLoopWarps - 1) + wid, s_tail);
 }
 
 // ============================================================ queries ====
@@ -958,7 +1046,7 @@ static int launch_loop_typed(Server *sv)
     P.slot = sv->d_slot;
     P.ctl = sv->ctl_dev;
     P.glob = sv->d_glob;
-    P.refill = sv->cfg.refill_lanes > 0 ? (uint32_t)std::min(sv->cfg.refill_lanes, 32) : 1u;
+    P.refill = sv->cfg.refill_lanes > 0 ? (uint32_t)std::min(sv->cfg.refill_lanes, 32) : 8u;
     P.idle_ns = (uint64_t)(sv->cfg.idle_us > 0 ? sv->cfg.idle_us : 200000) * 1000ull;
     if (!sv->grid) {
         int per_sm = 0;
@@ -1100,8 +1188,9 @@ static void scheduler_loop(Server *sv)
                 uint32_t P2 = 1;
                 while (P2 < R) P2 <<= 1;
                 d.P2 = P2;
-                // walks per chunk: about four chunks per walker warp for a large query
-                const uint64_t ww = std::max<uint64_t>(1, 4ull * sv->grid * (kLoopWarps - 1));
+                // walks per chunk: about two chunks per walker warp for a large query
+                // (a claim is two trips to L2 under contention)
+                const uint64_t ww = std::max<uint64_t>(1, 2ull * sv->grid * (kLoopWarps - 1));
                 uint64_t cw = sv->cfg.chunk_sources > 0 ? (uint64_t)sv->cfg.chunk_sources * R : (d.walks + ww - 1) / ww;
                 cw = std::min<uint64_t>(std::max<uint64_t>(cw, 32), 4096);
                 d.cw = (uint32_t)cw;
