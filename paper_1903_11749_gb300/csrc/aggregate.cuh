@@ -88,298 +88,27 @@ __device__ inline void aggregate_source(const uint32_t *ends, uint32_t R, uint32
     __syncwarp();
 }
 
-// Register-resident variant for next_pow2(R) = 32 * E <= 1024: the sorted
-// block lives in registers in striped order (element i = e * 32 + lane), a
-// bitonic network runs on shuffles (partner distance < 32) and in-register
-// exchanges (distance >= 32).  Runs are found from neighbour values; the
-// top-k sorts 32-bit keys (R - count) << 12 | run, whose order is count
-// descending then end id ascending because runs are numbered in id order.
-template <int E>
-__device__ __forceinline__ void warp_sort_reg(uint32_t (&v)[E])
-{
-    const uint32_t lane = threadIdx.x & 31;
-    constexpr int N = 32 * E;
-#pragma unroll
-    for (int k = 2; k <= N; k <<= 1) {
-#pragma unroll
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            if (j >= 32) {
-#pragma unroll
-                for (int e = 0; e < E; ++e) {
-                    const int f = e ^ (j >> 5);
-                    if (f > e) {
-                        const bool up = (((uint32_t)e * 32 + lane) & (uint32_t)k) == 0;
-                        const uint32_t a = v[e], b = v[f];
-                        const bool sw = (a > b) == up;
-                        v[e] = sw ? b : a;
-                        v[f] = sw ? a : b;
-                    }
-                }
-            } else {
-#pragma unroll
-                for (int e = 0; e < E; ++e) {
-                    const uint32_t o = __shfl_xor_sync(0xffffffffu, v[e], j);
-                    const bool up = (((uint32_t)e * 32 + lane) & (uint32_t)k) == 0;
-                    const bool lower = (lane & (uint32_t)j) == 0;
-                    v[e] = (lower == up) ? min(v[e], o) : max(v[e], o);
-                }
-            }
-        }
-    }
-}
-
-// Top-K of one row without sorting every run, for K <= 32 and K < nrun:
-// kv holds the key (R - count) << 12 | run at each run's head element, v its
-// node id (kv 0xFFFFFFFF elsewhere; elements e * 32 + lane in order), and the
-// answer is the K smallest keys in ascending order.  The
-// count rank q = key >> 12 of the K-th smallest key is found by bisection
-// over [0, R - 1] with ballot counts; every key with q below it is taken (fewer
-// than K, sorted in one register per lane), then the first keys with q equal
-// to it in run order (= ascending key, as runs are numbered in id order)
-// fill the remaining places.  cbuf: 32 uint32 of per-warp shared memory.
-template <int E>
-__device__ __forceinline__ void topk_select_reg(const uint32_t (&kv)[E], const uint32_t (&v)[E], uint32_t K, uint32_t R,
-                                                const uint32_t *run_id, uint32_t *cbuf, const AggOut &o, uint64_t tb)
-{
-    const uint32_t lane = threadIdx.x & 31, below = (1u << lane) - 1;
-    auto count_le = [&](uint32_t t) {
-        uint32_t c = 0;
-#pragma unroll
-        for (int e = 0; e < E; ++e) c += __popc(__ballot_sync(0xffffffffu, (kv[e] >> 12) <= t));
-        return c;
-    };
-    // smallest t with count_le(t) >= K; count_le(R - 1) = nrun > K.  Most rows
-    // have fewer than K runs of count >= 2, so t = R - 1 is tried first.
-    uint32_t lo = 0, hi = R - 1;
-    if (R >= 2 && count_le(R - 2) < K) lo = R - 1;
-    else hi = R >= 2 ? R - 2 : 0;
-    while (lo < hi) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if (count_le(mid) >= K) hi = mid;
-        else lo = mid + 1;
-    }
-    const uint32_t t = lo;
-    uint32_t nlt = 0;  // keys below t, gathered into cbuf in run order
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const bool lt = (kv[e] >> 12) < t;
-        const uint32_t ml = __ballot_sync(0xffffffffu, lt);
-        if (lt) cbuf[nlt + __popc(ml & below)] = kv[e];
-        nlt += __popc(ml);
-    }
-    __syncwarp();
-    // nlt < K places for the keys below t, sorted; then K - nlt keys equal to t
-    uint32_t x[1] = {lane < nlt ? cbuf[lane] : 0xffffffffu};
-    warp_sort_reg<1>(x);
-    if (lane < nlt) {
-        o.topk_idx[tb + lane] = (int32_t)run_id[x[0] & 0xfffu];
-        o.topk_cnt[tb + lane] = R - (x[0] >> 12);
-    }
-    uint32_t seen = 0;
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const bool eq = (kv[e] >> 12) == t;
-        const uint32_t me = __ballot_sync(0xffffffffu, eq);
-        const uint32_t pos = nlt + seen + __popc(me & below);
-        if (eq && pos < K) {
-            o.topk_idx[tb + pos] = (int32_t)v[e];
-            o.topk_cnt[tb + pos] = R - t;
-        }
-        seen += __popc(me);
-    }
-}
-
-// The whole row in top-k order (K >= nrun): kv as in topk_select_reg.  Runs
-// counted once come last (count 1 is the smallest) and already in run order,
-// so only the runs counted twice or more are sorted -- in one register per
-// lane when at most 32 of them (always when R <= 65) -- and the rest are
-// placed by ballot prefix counts.  Returns false (nothing written) when more
-// than 32 runs repeat; the caller then sorts every key.
-template <int E>
-__device__ __forceinline__ bool topk_all_reg(const uint32_t (&kv)[E], const uint32_t (&v)[E], uint32_t nrun, uint32_t K,
-                                             uint32_t R, const uint32_t *run_id, uint32_t *cbuf, const AggOut &o,
-                                             uint64_t tb)
-{
-    const uint32_t lane = threadIdx.x & 31, below = (1u << lane) - 1;
-    const uint32_t t1 = (R - 1) << 12;  // keys from here on: count 1 (or no run)
-    uint32_t nm = 0;
-#pragma unroll
-    for (int e = 0; e < E; ++e) nm += __popc(__ballot_sync(0xffffffffu, kv[e] < t1));
-    if (nm > 32) return false;
-    uint32_t seen = 0;
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const bool rep = kv[e] < t1;
-        const uint32_t mr = __ballot_sync(0xffffffffu, rep);
-        if (rep) cbuf[seen + __popc(mr & below)] = kv[e];
-        seen += __popc(mr);
-    }
-    __syncwarp();
-    uint32_t x[1] = {lane < nm ? cbuf[lane] : 0xffffffffu};
-    warp_sort_reg<1>(x);
-    if (lane < nm && lane < K) {
-        o.topk_idx[tb + lane] = (int32_t)run_id[x[0] & 0xfffu];
-        o.topk_cnt[tb + lane] = R - (x[0] >> 12);
-    }
-    uint32_t ones = 0;
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const bool one = kv[e] >= t1 && kv[e] != 0xffffffffu;
-        const uint32_t m1 = __ballot_sync(0xffffffffu, one);
-        const uint32_t pos = nm + ones + __popc(m1 & below);
-        if (one && pos < K) {
-            o.topk_idx[tb + pos] = (int32_t)v[e];
-            o.topk_cnt[tb + pos] = 1;
-        }
-        ones += __popc(m1);
-    }
-    for (uint32_t i = nrun + lane; i < K; i += 32) {
-        o.topk_idx[tb + i] = -1;
-        o.topk_cnt[tb + i] = 0;
-    }
-    return true;
-}
-
-// scratch: R + 32 uint32 of per-warp shared memory.
-//
-// Bound by the ALU pipe, so what follows the sort is kept short: run heads
-// come from one shuffle and one ballot per register; a run's count is the
-// distance to the next head, read off the same ballots; and the top-k keys
-// stay at their heads (0xFFFFFFFF elsewhere), so a selected run has its node
-// id in the lane that holds its key.  (A tenth fewer instructions than with run
-// starts and keys passed through shared memory: 256-graph batch, R 200, 4.28 ->
-// 3.96 ms.)
-template <int E>
-__device__ inline void aggregate_source_reg(const uint32_t *ends, uint32_t R, uint32_t *scratch, const AggOut &o,
-                                            uint64_t out_row, const CallerIds &ids = CallerIds())
-{
-    const uint32_t lane = threadIdx.x & 31;
-    uint32_t *run_id = scratch, *cbuf = scratch + R;
-    uint32_t v[E];
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const uint32_t i = (uint32_t)e * 32 + lane;
-        v[e] = i < R ? ends[i] : 0xffffffffu;
-    }
-    const uint64_t rbase = out_row * o.cap;
-    // A row whose R endpoints are all one node (a dangling source, whose walks
-    // restart where they began: 4-6 % of the sources of the R-MAT graphs) is
-    // one run of count R; it skips the sort.
-    const uint32_t v0 = __shfl_sync(0xffffffffu, v[0], 0);
-    bool same = true;
-#pragma unroll
-    for (int e = 0; e < E; ++e) same = same && ((uint32_t)e * 32 + lane >= R || v[e] == v0);
-    if (__all_sync(0xffffffffu, same)) {
-        const int32_t id = (int32_t)ids(v0);
-        if (lane == 0) {
-            if (o.cols) {
-                o.cols[rbase] = id;
-                o.cnts[rbase] = R;
-            }
-            if (o.nnz) o.nnz[out_row] = 1;
-        }
-        const uint64_t tb = out_row * (uint64_t)o.topk;
-        for (uint32_t i = lane; i < (uint32_t)max(o.topk, 0); i += 32) {
-            o.topk_idx[tb + i] = i == 0 ? id : -1;
-            o.topk_cnt[tb + i] = i == 0 ? R : 0u;
-        }
-        __syncwarp();
-        return;
-    }
-#pragma unroll
-    for (int e = 0; e < E; ++e)
-        if ((uint32_t)e * 32 + lane < R) v[e] = ids(v[e]);
-    warp_sort_reg<E>(v);
-    uint32_t hb[E], nxt[E];  // heads of each register; first head in a later register (R: none)
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        // the element before: lane 31 hands lane 0 the last one of the register before
-        const uint32_t mine = e > 0 && lane == 31 ? v[e > 0 ? e - 1 : 0] : v[e];
-        const uint32_t prev = __shfl_sync(0xffffffffu, mine, (lane + 31) & 31);
-        const bool head = (uint32_t)e * 32 + lane < R && ((e == 0 && lane == 0) || prev != v[e]);
-        hb[e] = __ballot_sync(0xffffffffu, head);
-    }
-    uint32_t after = R;
-#pragma unroll
-    for (int e = E - 1; e >= 0; --e) {
-        nxt[e] = after;
-        if (hb[e]) after = (uint32_t)e * 32 + __ffs(hb[e]) - 1;
-    }
-    uint32_t nrun = 0, kv[E];
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        kv[e] = 0xffffffffu;
-        if ((hb[e] >> lane) & 1u) {
-            const uint32_t i = (uint32_t)e * 32 + lane, above = hb[e] & (0xfffffffeu << lane);
-            const uint32_t run = nrun + __popc(hb[e] & ((1u << lane) - 1));
-            const uint32_t c = (above ? (uint32_t)e * 32 + __ffs(above) - 1 : nxt[e]) - i;
-            if (o.cols) {
-                o.cols[rbase + run] = (int32_t)v[e];
-                o.cnts[rbase + run] = c;
-            }
-            run_id[run] = v[e];
-            kv[e] = ((R - c) << 12) | run;
-        }
-        nrun += __popc(hb[e]);
-    }
-    if (lane == 0 && o.nnz) o.nnz[out_row] = nrun;
-    if (o.topk > 0) {
-        __syncwarp();
-        const uint64_t tb = out_row * (uint64_t)o.topk;
-        const uint32_t K = (uint32_t)o.topk;
-        if (E > 1 && K <= 32 && K < nrun) {
-            topk_select_reg<E>(kv, v, K, R, run_id, cbuf, o, tb);
-        } else if (E > 1 && K >= nrun && topk_all_reg<E>(kv, v, nrun, K, R, run_id, cbuf, o, tb)) {
-            // the whole row, in top-k order
-        } else {
-            warp_sort_reg<E>(kv);
-#pragma unroll
-            for (int e = 0; e < E; ++e) {
-                const uint32_t i = (uint32_t)e * 32 + lane;
-                if (i < K) {
-                    if (i < nrun) {
-                        o.topk_idx[tb + i] = (int32_t)run_id[kv[e] & 0xfffu];
-                        o.topk_cnt[tb + i] = R - (kv[e] >> 12);
-                    } else {
-                        o.topk_idx[tb + i] = -1;
-                        o.topk_cnt[tb + i] = 0;
-                    }
-                }
-            }
-            // k may exceed the sorted block (k > next_pow2(R) >= nnz): pad the rest
-            for (uint32_t i = 32u * E + lane; i < K; i += 32) {
-                o.topk_idx[tb + i] = -1;
-                o.topk_cnt[tb + i] = 0;
-            }
-        }
-    }
-    __syncwarp();
-}
-
-// ------------------------------------------------ one block per source ----
-// R > 256: a block of T threads reduces one source, I elements a thread
-// (T * I = next_pow2(R)).  One warp a source left the chip idle where there
-// are few sources (rankings over some hundred sources with R in the
-// thousands) and waited through a chain of shared-memory or 32-register
-// stages.  Reduction of 500 sources, R 4096, top-1000: 1262 -> 40 us; 1,000
-// sources, R 1000: 46 -> 18 us; and with the chip full, 2^25 walks in all: R
-// 300 .697 -> .505 ms, 500 .478 -> .324, 1000 .728 -> .392, 2000 7.80 -> .504,
-// 4000 17.5 -> .497.
-
+// Register-resident variant for next_pow2(R) = 32 * E <= 256 (R <= 32: E = 1).
+// The sort works on consecutive elements of a lane (its short strides are then
+// plain min and max, and of the 28 stages of R = 128 only 15 are shuffles); what
+// follows takes them in striped order (element e * 32 + lane in register e),
+// where ballots see them in order and rows are written in whole sectors.  Runs
+// are found from neighbour values; the top-k sorts 32-bit keys
+// (R - count) << 12 | run, whose order is count descending then end id
+// ascending because runs are numbered in id order.
 // Ascending sort of T * I elements, element t * I + k in register k of thread
-// t.  Bitonic network in the form whose first exchange of every level mirrors
+// t < T (a warp, or a block).  Bitonic network in the form whose first exchange of every level mirrors
 // (i with i ^ (size - 1)), so every exchange puts the smaller element first and
 // no direction is tracked: strides below I stay in the thread, below 32 I in
-// the warp, longer ones go through sm (T * I words).
+// the warp, longer ones (T > 32) go through sm (T * I words).
 template <int T, int I>
-__device__ __forceinline__ void block_sort(uint32_t (&v)[I], uint32_t *sm)
+__device__ __forceinline__ void sort_ascending(uint32_t (&v)[I], uint32_t *sm, uint32_t t)
 {
-    const uint32_t t = threadIdx.x;
     // exchange with thread t ^ x; MIRROR: the partner's elements in reverse order
     auto across = [&](uint32_t x, bool mirror) {
         const bool lower = (t & (mirror ? (x + 1) >> 1 : x)) == 0;
         uint32_t o[I];
-        if (x < 32) {
+        if (T == 32 || x < 32) {
 #pragma unroll
             for (int k = 0; k < I; ++k) o[k] = __shfl_xor_sync(0xffffffffu, v[mirror ? I - 1 - k : k], x);
         } else {
@@ -419,6 +148,251 @@ __device__ __forceinline__ void block_sort(uint32_t (&v)[I], uint32_t *sm)
         }
     }
 }
+
+// Top-K of one row without sorting every run, for K <= 32 and more than 32 runs
+// met twice or more:
+// kv holds the key (R - count) << 12 | run at each run's head element, v its
+// node id (kv 0xFFFFFFFF elsewhere; elements e * 32 + lane in order), and the
+// answer is the K smallest keys in ascending order.  The
+// count rank q = key >> 12 of the K-th smallest key is found by bisection
+// over [0, R - 2] with ballot counts; every key with q below it is taken (fewer
+// than K, sorted in one register per lane), then the first keys with q equal
+// to it in run order (= ascending key, as runs are numbered in id order)
+// fill the remaining places.  cbuf: 32 uint32 of per-warp shared memory.
+template <int E>
+__device__ __forceinline__ void topk_select_reg(const uint32_t (&kv)[E], const uint32_t (&v)[E], uint32_t K, uint32_t R,
+                                                const uint32_t *run_id, uint32_t *cbuf, const AggOut &o, uint64_t tb)
+{
+    const uint32_t lane = threadIdx.x & 31, below = (1u << lane) - 1;
+    auto count_le = [&](uint32_t t) {
+        uint32_t c = 0;
+#pragma unroll
+        for (int e = 0; e < E; ++e) c += __popc(__ballot_sync(0xffffffffu, (kv[e] >> 12) <= t));
+        return c;
+    };
+    // smallest t with count_le(t) >= K; count_le(R - 2) > 32 >= K here
+    uint32_t lo = 0, hi = R - 2;
+    while (lo < hi) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (count_le(mid) >= K) hi = mid;
+        else lo = mid + 1;
+    }
+    const uint32_t t = lo;
+    uint32_t nlt = 0;  // keys below t, gathered into cbuf in run order
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const bool lt = (kv[e] >> 12) < t;
+        const uint32_t ml = __ballot_sync(0xffffffffu, lt);
+        if (lt) cbuf[nlt + __popc(ml & below)] = kv[e];
+        nlt += __popc(ml);
+    }
+    __syncwarp();
+    // nlt < K places for the keys below t, sorted; then K - nlt keys equal to t
+    uint32_t x[1] = {lane < nlt ? cbuf[lane] : 0xffffffffu};
+    sort_ascending<32, 1>(x, nullptr, lane);
+    if (lane < nlt) {
+        o.topk_idx[tb + lane] = (int32_t)run_id[x[0] & 0xfffu];
+        o.topk_cnt[tb + lane] = R - (x[0] >> 12);
+    }
+    uint32_t seen = 0;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const bool eq = (kv[e] >> 12) == t;
+        const uint32_t me = __ballot_sync(0xffffffffu, eq);
+        const uint32_t pos = nlt + seen + __popc(me & below);
+        if (eq && pos < K) {
+            o.topk_idx[tb + pos] = (int32_t)v[e];
+            o.topk_cnt[tb + pos] = R - t;
+        }
+        seen += __popc(me);
+    }
+}
+
+// Top-K of a row in which nm <= 32 runs are met twice or more (most rows; all
+// of them when R <= 65): runs met once come last (count 1 is the smallest) and
+// already in run order, so only the nm others are sorted, in one register a
+// lane, and the rest are placed by their run index less the others before
+// them.  kv, v as above; many: ballots of the elements whose runs are met twice
+// or more.
+template <int E>
+__device__ __forceinline__ void topk_ones_reg(const uint32_t (&kv)[E], const uint32_t (&v)[E], const uint32_t (&many)[E],
+                                              uint32_t nm, uint32_t nrun, uint32_t K, uint32_t R, const uint32_t *run_id,
+                                              uint32_t *cbuf, const AggOut &o, uint64_t tb)
+{
+    const uint32_t lane = threadIdx.x & 31, below = (1u << lane) - 1;
+    uint32_t seen = 0;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const uint32_t before = seen + __popc(many[e] & below);
+        if ((many[e] >> lane) & 1u) {
+            cbuf[before] = kv[e];
+        } else if (kv[e] != 0xffffffffu) {
+            const uint32_t pos = nm + (kv[e] & 0xfffu) - before;
+            if (pos < K) {
+                o.topk_idx[tb + pos] = (int32_t)v[e];
+                o.topk_cnt[tb + pos] = 1;
+            }
+        }
+        seen += __popc(many[e]);
+    }
+    __syncwarp();
+    uint32_t x[1] = {lane < nm ? cbuf[lane] : 0xffffffffu};
+    if (nm > 1) sort_ascending<32, 1>(x, nullptr, lane);
+    if (lane < nm && lane < K) {
+        o.topk_idx[tb + lane] = (int32_t)run_id[x[0] & 0xfffu];
+        o.topk_cnt[tb + lane] = R - (x[0] >> 12);
+    }
+    for (uint32_t i = nrun + lane; i < K; i += 32) {
+        o.topk_idx[tb + i] = -1;
+        o.topk_cnt[tb + i] = 0;
+    }
+}
+
+// scratch: 32 * E + 32 uint32 of per-warp shared memory, 16-byte aligned.
+//
+// Bound by the ALU pipe, so what follows the sort is kept short: run heads
+// come from one shuffle and one ballot per register; a run's count is the
+// distance to the next head, read off the same ballots; and the top-k keys
+// stay at their heads (0xFFFFFFFF elsewhere), so a selected run has its node
+// id in the lane that holds its key.  Reductions with the chip full, ms, against
+// a sort in striped order with the top-k's ties found by a second pass of
+// ballots: R 50, top-64 .178 -> .156; R 100, top-32 .275 -> .232 (2^18 sources
+// each); R 200 .331 -> .267 (167,772 sources).
+template <int E>
+__device__ inline void aggregate_source_reg(const uint32_t *ends, uint32_t R, uint32_t *scratch, const AggOut &o,
+                                            uint64_t out_row, const CallerIds &ids = CallerIds())
+{
+    const uint32_t lane = threadIdx.x & 31;
+    uint32_t *run_id = scratch, *cbuf = scratch + 32 * E;
+    uint32_t v[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const uint32_t i = (uint32_t)e * 32 + lane;
+        v[e] = i < R ? ends[i] : 0xffffffffu;
+    }
+    const uint64_t rbase = out_row * o.cap;
+    // A row whose R endpoints are all one node (a dangling source, whose walks
+    // restart where they began: 4-6 % of the sources of the R-MAT graphs) is
+    // one run of count R; it skips the sort.
+    const uint32_t v0 = __shfl_sync(0xffffffffu, v[0], 0);
+    bool same = true;
+#pragma unroll
+    for (int e = 0; e < E; ++e) same = same && ((uint32_t)e * 32 + lane >= R || v[e] == v0);
+    if (__all_sync(0xffffffffu, same)) {
+        const int32_t id = (int32_t)ids(v0);
+        if (lane == 0) {
+            if (o.cols) {
+                o.cols[rbase] = id;
+                o.cnts[rbase] = R;
+            }
+            if (o.nnz) o.nnz[out_row] = 1;
+        }
+        const uint64_t tb = out_row * (uint64_t)o.topk;
+        for (uint32_t i = lane; i < (uint32_t)max(o.topk, 0); i += 32) {
+            o.topk_idx[tb + i] = i == 0 ? id : -1;
+            o.topk_cnt[tb + i] = i == 0 ? R : 0u;
+        }
+        __syncwarp();
+        return;
+    }
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+        if ((uint32_t)e * 32 + lane < R) v[e] = ids(v[e]);
+    sort_ascending<32, E>(v, nullptr, lane);
+    if (E > 1) {  // consecutive to striped
+        if constexpr (E == 2) {
+            reinterpret_cast<uint2 *>(scratch)[lane] = make_uint2(v[0], v[1]);
+        } else if constexpr (E >= 4) {
+#pragma unroll
+            for (int e = 0; e < E; e += 4)
+                reinterpret_cast<uint4 *>(scratch)[(lane * E + e) / 4] = make_uint4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int e = 0; e < E; ++e) v[e] = scratch[e * 32 + lane];
+        __syncwarp();
+    }
+    uint32_t hb[E], nxt[E];  // heads of each register; first head in a later register (R: none)
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        // the element before: lane 31 hands lane 0 the last one of the register before
+        const uint32_t mine = e > 0 && lane == 31 ? v[e > 0 ? e - 1 : 0] : v[e];
+        const uint32_t prev = __shfl_sync(0xffffffffu, mine, (lane + 31) & 31);
+        const bool head = (uint32_t)e * 32 + lane < R && ((e == 0 && lane == 0) || prev != v[e]);
+        hb[e] = __ballot_sync(0xffffffffu, head);
+    }
+    uint32_t after = R;
+#pragma unroll
+    for (int e = E - 1; e >= 0; --e) {
+        nxt[e] = after;
+        if (hb[e]) after = (uint32_t)e * 32 + __ffs(hb[e]) - 1;
+    }
+    uint32_t nrun = 0, kv[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        kv[e] = 0xffffffffu;
+        if ((hb[e] >> lane) & 1u) {
+            const uint32_t i = (uint32_t)e * 32 + lane, above = hb[e] & (0xfffffffeu << lane);
+            const uint32_t run = nrun + __popc(hb[e] & ((1u << lane) - 1));
+            const uint32_t c = (above ? (uint32_t)e * 32 + __ffs(above) - 1 : nxt[e]) - i;
+            if (o.cols) {
+                o.cols[rbase + run] = (int32_t)v[e];
+                o.cnts[rbase + run] = c;
+            }
+            run_id[run] = v[e];
+            kv[e] = ((R - c) << 12) | run;
+        }
+        nrun += __popc(hb[e]);
+    }
+    if (lane == 0 && o.nnz) o.nnz[out_row] = nrun;
+    if (o.topk > 0) {
+        __syncwarp();
+        const uint64_t tb = out_row * (uint64_t)o.topk;
+        const uint32_t K = (uint32_t)o.topk;
+        uint32_t many[E], nm = E > 1 ? 0 : 33;  // (one register: the whole row is sorted at once)
+#pragma unroll
+        for (int e = 0; e < (E > 1 ? E : 0); ++e) {
+            many[e] = __ballot_sync(0xffffffffu, kv[e] < (R - 1) << 12);
+            nm += __popc(many[e]);
+        }
+        if (nm <= 32) {
+            topk_ones_reg<E>(kv, v, many, nm, nrun, K, R, run_id, cbuf, o, tb);
+        } else if (E > 1 && K <= 32 && K < nrun) {
+            topk_select_reg<E>(kv, v, K, R, run_id, cbuf, o, tb);
+        } else {
+            sort_ascending<32, E>(kv, nullptr, lane);
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                const uint32_t i = lane * E + e;
+                if (i < K) {
+                    if (i < nrun) {
+                        o.topk_idx[tb + i] = (int32_t)run_id[kv[e] & 0xfffu];
+                        o.topk_cnt[tb + i] = R - (kv[e] >> 12);
+                    } else {
+                        o.topk_idx[tb + i] = -1;
+                        o.topk_cnt[tb + i] = 0;
+                    }
+                }
+            }
+            // k may exceed the sorted block (k > next_pow2(R) >= nnz): pad the rest
+            for (uint32_t i = 32u * E + lane; i < K; i += 32) {
+                o.topk_idx[tb + i] = -1;
+                o.topk_cnt[tb + i] = 0;
+            }
+        }
+    }
+    __syncwarp();
+}
+
+// ------------------------------------------------ one block per source ----
+// R > 256: a block of T threads reduces one source, I elements a thread
+// (T * I = next_pow2(R)).  One warp a source left the chip idle where there
+// are few sources (rankings over some hundred sources with R in the
+// thousands) and waited through a chain of shared-memory or 32-register
+// stages.  Reduction of 500 sources, R 4096, top-1000: 1262 -> 40 us; 1,000
+// sources, R 1000: 46 -> 18 us; and with the chip full, 2^25 walks in all: R
+// 300 .697 -> .505 ms, 500 .478 -> .324, 1000 .728 -> .392, 2000 7.80 -> .504,
+// 4000 17.5 -> .497.
 
 // Exclusive sum over the block's threads; *total: of all.  s: T / 32 words.
 template <int T>
@@ -464,7 +438,7 @@ __device__ void aggregate_source_block(const uint32_t *ends, uint32_t R, BlockSc
         const uint32_t i = (uint32_t)k * T + t;
         v[k] = i < R ? ids(ends[i]) : 0xffffffffu;
     }
-    block_sort<T, I>(v, sm.id);
+    sort_ascending<T, I>(v, sm.id, t);
     if (lane == 31) sm.edge[wid] = v[I - 1];
     __syncthreads();
     uint32_t prev = __shfl_up_sync(0xffffffffu, v[I - 1], 1);
@@ -527,14 +501,14 @@ __device__ void aggregate_source_block(const uint32_t *ends, uint32_t R, BlockSc
         if (nm <= T) {
             uint32_t x[1] = {t < nm ? sm.key[t] : 0xffffffffu};
             __syncthreads();
-            block_sort<T, 1>(x, sm.key);
+            sort_ascending<T, 1>(x, sm.key, t);
             put(t, x[0]);
         } else {
             uint32_t x[I / 2];
 #pragma unroll
             for (int k = 0; k < I / 2; ++k) x[k] = (uint32_t)k * T + t < nm ? sm.key[k * T + t] : 0xffffffffu;
             __syncthreads();
-            block_sort<T, I / 2>(x, sm.key);
+            sort_ascending<T, I / 2>(x, sm.key, t);
 #pragma unroll
             for (int k = 0; k < I / 2; ++k) put(t * (I / 2) + k, x[k]);
         }
@@ -571,7 +545,7 @@ template <int E>
 __global__ void __launch_bounds__(32 * kAggWarps) k_aggregate(AggParams p)
 {
     __shared__ uint32_t first[kTabEntries];
-    __shared__ uint32_t scratch[kAggWarps][32 * E + 32];
+    __shared__ __align__(16) uint32_t scratch[kAggWarps][32 * E + 32];
     const CallerIds ids = load_ids(first, p);
     const uint32_t wid = threadIdx.x >> 5;
     const uint64_t S = (uint64_t)p.S;
