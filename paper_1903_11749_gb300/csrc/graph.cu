@@ -263,12 +263,50 @@ __device__ __forceinline__ uint32_t first_above(const typename E::Edge *row, uin
     return lo;
 }
 
+// The same for 32 ascending x, one a lane, all 32 lanes taking part: a 32-ary
+// search for lane 0's edge (two or three dependent loads where bisection takes
+// ten), then the edges from there on, 32 at a time in one load, each lane
+// finding its place among them by shuffles.  A warp's ranges meet 16 to 64
+// edges on average; after kWarpChunks loads (runs of light edges) the lanes left
+// bisect what follows.
+constexpr uint32_t kWarpChunks = 8;
+template <class E, class P>
+__device__ __forceinline__ uint32_t first_above_warp(const typename E::Edge *row, uint32_t d, P x)
+{
+    const uint32_t lane = threadIdx.x & 31;
+    const P x0 = __shfl_sync(0xffffffffu, x, 0);
+    uint32_t lo = 0, n = d;
+    while (n > 32) {  // 32 parts; part i ends at edge lo + (i + 1) n / 32 - 1, the last one with P > x0
+        const uint32_t end = lo + (uint32_t)(((uint64_t)(lane + 1) * n) >> 5) - 1;
+        const uint32_t f = __popc(__ballot_sync(0xffffffffu, __ldg(&row[end].P) <= x0));
+        const uint32_t a = (uint32_t)(((uint64_t)f * n) >> 5), b = (uint32_t)(((uint64_t)(f + 1) * n) >> 5);
+        lo += a;
+        n = b - a;
+    }
+    uint32_t at = 0;
+    bool found = false;
+    for (uint32_t chunk = 0; chunk < kWarpChunks; ++chunk, lo += 32) {
+        const P v = lo + lane < d ? __ldg(&row[lo + lane].P) : (P)~(P)0;
+        uint32_t cnt = 0;  // edges of the chunk with P <= x (31 at most where the last one is above x)
+#pragma unroll
+        for (uint32_t s = 16; s > 0; s >>= 1) cnt += __shfl_sync(0xffffffffu, v, cnt + s - 1) <= x ? s : 0u;
+        const P last = __shfl_sync(0xffffffffu, v, 31);  // (by every lane, also those done)
+        if (!found && last > x) {
+            at = lo + cnt;
+            found = true;
+        }
+        if (__all_sync(0xffffffffu, found)) break;
+    }
+    if (!found) at = first_above<E, P>(row, lo, d - lo, x);
+    return at;
+}
+
 // One slot a thread.  The class-major numbering makes the slot's row and
 // range plain arithmetic, neighbouring threads hold neighbouring ranges of a
-// row (their probes of P share sectors), and every slot is one 32-byte store.
-// Bound by issue: the searches' instructions, so the narrow layout computes in
-// 32 bits and the table entry is found once a block (R-MAT scale 24, 394 M
-// slots: 7.9 -> 7.2 ms).
+// row, and every slot is one 32-byte store.  Bound by the latency of the
+// searches: where a warp has 32 ranges of one row they search together
+// (R-MAT scale 24, 394 M slots: 7.2 -> 5.3 ms; 64-bit keys and a table search a
+// thread before that: 7.9).
 template <class E>
 __global__ void __launch_bounds__(256) k_slots(SlotArgs A, E edges)
 {
@@ -294,6 +332,9 @@ __global__ void __launch_bounds__(256) k_slots(SlotArgs A, E edges)
     const TabEntry t = tab.e[entry];
     const uint32_t c = t.kind, rel = (uint32_t)((at - t.addr) / sizeof(Sector));  // below 2^32: a device holds fewer slots
     const uint32_t b = rel & ((1u << c) - 1);
+    // slots between the entry's last row and the next entry's start belong to no row (whole warps where c >= 5)
+    const uint32_t next = entry + 1 < kTabEntries ? tab.e[entry + 1].first : 0xffffffffu;
+    if (t.first + (rel >> c) >= (next == 0xffffffffu ? (uint32_t)A.n : next)) return;
     const NodeRec r = A.node[t.first + (rel >> c)];
     const typename E::Edge *row = edges.e + (r.word0 & kBeginMask);
     const uint32_t d = (uint32_t)(r.word0 >> 40) & kCountMask;
@@ -307,7 +348,9 @@ __global__ void __launch_bounds__(256) k_slots(SlotArgs A, E edges)
         X0 = (uint32_t)(lo >> c);
         X1 = (uint32_t)(up >> c) - (((uint32_t)up & ((1u << c) - 1)) == 0);
     }
-    const uint32_t lo = c ? first_above<E, P>(row, 0, d, X0) : 0u;
+    uint32_t lo = 0;
+    if (c >= 5) lo = first_above_warp<E, P>(row, d, X0);
+    else if (c) lo = first_above<E, P>(row, 0, d, X0);
     const uint32_t left = d - lo;  // edges from lo to the row's end
     constexpr uint32_t kFit = E::kWide ? 3 : 4;
     typename E::Rec rec[kFit];
@@ -1092,7 +1135,8 @@ int build_segments(ppr_graph *g, uint32_t T, cudaStream_t st)
     for (uint32_t e = 0; e < kTabEntries; ++e)
         if (tab.e[e].kind <= small) {
             const uint64_t next = e + 1 < kTabEntries && tab.e[e + 1].first != 0xffffffffu ? tab.e[e + 1].first : (uint64_t)n;
-            ns += (int64_t)(next - tab.e[e].first) << tab.e[e].kind;
+            ns = (int64_t)(reinterpret_cast<const Sector *>(tab.e[e].addr) - g->slots) +
+                 ((int64_t)(next - tab.e[e].first) << tab.e[e].kind);
         }
     if ((rc = dev_alloc((void **)&list, sizeof(uint32_t) * n, "segment node list", st)) ||
         (rc = dev_alloc((void **)&d_ct, sizeof(SegCounters), "segment counters", st)) ||

@@ -228,6 +228,8 @@ int number_nodes(int64_t n, int64_t m, const int64_t *d_rp, const int64_t *d_off
                 T.e[e].addr = sizeof(uint32_t) * (uint64_t)g->n_single;
                 g->n_single += (int64_t)cnt;
             } else if (c >= 2) {
+                // entries start on 32 slots, so that a warp of the slot build has one row where rows have 32 ranges
+                g->n_slots = (g->n_slots + 31) & ~31ll;
                 T.e[e].kind = c <= kExact ? ranges_log2(c, g->lam_bits, wide) : c - kExact - 1;
                 T.e[e].addr = sizeof(Sector) * (uint64_t)g->n_slots;
                 g->n_slots += (int64_t)(cnt << T.e[e].kind);
