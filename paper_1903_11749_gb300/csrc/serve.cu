@@ -80,12 +80,19 @@ struct __align__(16) SDesc {
 
 // Counters of a ring slot (device memory; the host writes them before
 // publishing).  claim and agg hold the low 32 bits of (sequence number + 1)
-// above the number of chunks / sources handed out so far: one load tells a
-// warp whether the slot holds the query it looks for and whether work is
-// left, and work is taken with one atomic add (no retries under contention);
-// the tag of the word an add returns says whose work it took, so a warp with
-// a stale view of the ring that lands on a reused slot takes work of the
-// query that holds it now (never work that no one else will do).
+// above a count that starts at kWordEnd less the chunks / sources and ends at
+// kWordEnd: the word alone, without the descriptor, says whose work it counts
+// and whether any is left, and work is taken with one atomic add (no retries
+// under contention).  The tag of the word an add returns says whose work it
+// took, so a warp with a stale view of the ring that lands on a reused slot
+// takes work of the query that holds it now (never work that no one else will
+// do).  Work taken keeps its query unfinished, and so its descriptor in place,
+// until it is done.
+constexpr uint32_t kWordEnd = 0x80000000u;
+__host__ __device__ __forceinline__ uint32_t word_left(unsigned long long w)
+{
+    return (uint32_t)w < kWordEnd ? kWordEnd - (uint32_t)w : 0u;
+}
 struct __align__(64) SSlot {
     unsigned long long claim;       // chunks still to hand out
     unsigned long long agg;         // sources still to hand to aggregators
@@ -181,6 +188,21 @@ __device__ int await_slot(const LoopParams &P, const unsigned long long *w, uint
             return -1;
         }
         __nanosleep(1000);
+    }
+    return 1;
+}
+
+// Lane 0, after taking work of a query that reused a slot: waits (bounded)
+// until its descriptor is seen (the host writes it before the slot's words).
+__device__ int await_desc(const LoopParams &P, const SDesc *d, uint32_t tag)
+{
+    const uint64_t t0 = gtime_ns();
+    while ((uint32_t)__ldcg(&d->seq1) != tag) {
+        if (gtime_ns() - t0 > kSlotWaitNs) {
+            flag_exit(P, PPR_LOOP_SLOT_TIMEOUT);
+            return -1;
+        }
+        __nanosleep(500);
     }
     return 1;
 }
@@ -287,7 +309,7 @@ __device__ int claim_chunk(const LoopParams &P, uint32_t start, WalkChunk *c, un
                 const uint32_t s = (uint32_t)(id % kRing);
                 const unsigned long long w = __ldcg(&P.slot[s].claim);
                 const int rel = tag_rel(w, id);
-                const bool left = rel == 0 && (uint32_t)w < __ldcg(&P.desc[s].nchunks);
+                const bool left = rel == 0 && word_left(w) > 0;
                 o = left;
                 if (rel < 0) unwritten = (int)i;
                 if (i == 0 && (rel > 0 || (rel == 0 && !left))) bump(&P.glob->head, h);
@@ -324,26 +346,20 @@ __device__ int claim_chunk(const LoopParams &P, uint32_t start, WalkChunk *c, un
             const uint32_t s = (uint32_t)((h + i) % kRing);
             const SDesc *d = P.desc + s;
             // The descriptor is read while the add is under way: the slot held
-            // query h + i when its claim word was read above, so if the add says
-            // that it still does, what was read in between is that query's.
+            // query h + i when its claim word was read above, so if the add took
+            // a chunk of it, the query was not finished in between and what was
+            // read is its descriptor.
             ChunkDesc dc = load_desc(d);
             const unsigned long long old = atomicAdd(&P.slot[s].claim, 1ull);
-            const uint32_t tag = (uint32_t)(old >> 32), ci = (uint32_t)old;
-            if (tag == (uint32_t)(h + i + 1)) {
-                got = ci < dc.nchunks;
-            } else if (tag != 0) {  // reused meanwhile: the query that holds it now, once its descriptor is in place
-                const uint64_t t0 = gtime_ns();
-                bool there;
-                while (!(there = (uint32_t)__ldcg(&d->seq1) == tag) && gtime_ns() - t0 < kSlotWaitNs) __nanosleep(500);
-                if (there) {
+            const uint32_t tag = (uint32_t)(old >> 32), left = word_left(old);
+            if (tag != 0 && left > 0) {
+                got = 1;
+                if (tag != (uint32_t)(h + i + 1)) {  // reused meanwhile: a chunk of the query that holds it now
+                    got = await_desc(P, d, tag);
                     dc = load_desc(d);
-                    got = ci < dc.nchunks;
-                } else {
-                    flag_exit(P, PPR_LOOP_SLOT_TIMEOUT);
-                    got = -1;
                 }
+                if (got > 0) take_chunk(P, s, dc.nchunks - left, dc, c);
             }
-            if (got > 0) take_chunk(P, s, ci, dc, c);
         }
         got = __shfl_sync(0xffffffffu, got, 0);
         if (got) return got;
@@ -361,7 +377,8 @@ __device__ __forceinline__ void count_walks(const LoopParams &P, uint32_t q, uin
 
 constexpr uint32_t kHelpMaxR = 128;  // walker warps without walks reduce sources of queries up to this R
 __device__ __noinline__ int claim_source(const LoopParams &P, unsigned long long *s_tail, bool refresh, uint32_t max_R,
-                            uint64_t &id_out, uint32_t &slot_out, uint32_t &i_out, uint32_t &n_out, bool &in_flight);
+                            bool wait, uint64_t &id_out, uint32_t &slot_out, uint32_t &i_out, uint32_t &n_out,
+                            bool &in_flight);
 __device__ __noinline__ void reduce_source(const LoopParams &P, const CallerIds &ids, uint32_t s, uint32_t i,
                                            uint32_t *smem, uint32_t cap);
 __device__ void finish_source(const LoopParams &P, uint64_t id, uint32_t s, uint32_t n);
@@ -526,11 +543,20 @@ __device__ __forceinline__ int walk_until_idle(const LoopParams &P, const ClassT
     return status < 0 ? status : (int)walked;
 }
 
+// Sources that a walker warp took of a query it may not be able to reduce (its
+// add landed on a reused slot): walks still to come, which a warp that waited
+// would keep from being walked, or an R beyond its scratch.  The block's
+// aggregator, which ends after the walker warps, reduces them.  n = 0: none.
+struct Handed {
+    unsigned long long id;
+    uint32_t s, i, n;
+};
+
 // A walker warp: walks, then helps reduce, then waits (bounded) for the next query.
 template <class E>
 __device__ __forceinline__ void walker_warp(const LoopParams &P, const ClassTab &tab, const CallerIds &ids, WalkChunk &wc,
-                                            uint32_t **ends_of, uint32_t *scratch, WarpActivity &act, uint32_t gwarp,
-                                            unsigned long long *s_tail)
+                                            uint32_t **ends_of, uint32_t *scratch, WarpActivity &act, Handed &handed,
+                                            uint32_t gwarp, unsigned long long *s_tail)
 {
     const uint32_t lane = threadIdx.x & 31;
     if (lane == 0) act = WarpActivity{clock64(), 0, 0, 0, 0, 0};
@@ -547,8 +573,21 @@ __device__ __forceinline__ void walker_warp(const LoopParams &P, const ClassTab 
         uint64_t id = 0;
         uint32_t s = 0, i = 0, nb = 0;
         bool in_flight = false;
-        const int r = claim_source(P, s_tail, false, kHelpMaxR, id, s, i, nb, in_flight);
+        int r = 0;
+        if (__shfl_sync(0xffffffffu, lane == 0 ? *(volatile uint32_t *)&handed.n : 0u, 0) == 0)
+            r = claim_source(P, s_tail, false, kHelpMaxR, false, id, s, i, nb, in_flight);
         if (r < 0) break;
+        if (r == 2) {  // of another query than it looked at: left to the aggregator
+            if (lane == 0) {
+                handed.id = id;
+                handed.s = s;
+                handed.i = i;
+                __threadfence_block();
+                *(volatile uint32_t *)&handed.n = nb;
+            }
+            __syncwarp();
+            continue;
+        }
         if (r > 0) {
             for (uint32_t b = 0; b < nb; ++b) reduce_source(P, ids, s, i + b, scratch, kHelpMaxR);
             finish_source(P, id, s, nb);
@@ -585,12 +624,29 @@ __device__ __forceinline__ void walker_warp(const LoopParams &P, const ClassTab 
     }
 }
 
-// Whole warp: hands out one source of the oldest query whose walks are all
-// done.  Returns 1 (query id, slot, source i on every lane), 0 (none now),
-// -1 (the loop must end); *in_flight tells whether published queries still
-// have sources to hand out (ready or not).
+// Lane 0: waits (bounded) until the walks of the query in slot s are done.
+__device__ int await_walks(const LoopParams &P, uint32_t s)
+{
+    const uint64_t t0 = gtime_ns();
+    while (__ldcg(&P.slot[s].walks_done) < __ldcg(&P.desc[s].walks)) {
+        if (gtime_ns() - t0 > kBusyWaitNs) {
+            flag_exit(P, PPR_LOOP_BUSY_TIMEOUT);
+            return -1;
+        }
+        __nanosleep(1000);
+    }
+    return 1;
+}
+
+// Whole warp: hands out a few sources of the oldest query of R <= max_R whose
+// walks are all done.  Returns 1 (query id, slot, sources from i on, on every
+// lane), 0 (none now), -1 (the loop must end); *in_flight tells whether
+// published queries still have sources to hand out (ready or not).  An add
+// that lands on a reused slot takes sources of a query of any R whose walks may
+// still run: with wait the warp waits for them (bounded), else it gets 2.
 __device__ __noinline__ int claim_source(const LoopParams &P, unsigned long long *s_tail, bool refresh, uint32_t max_R,
-                            uint64_t &id_out, uint32_t &slot_out, uint32_t &i_out, uint32_t &n_out, bool &in_flight)
+                            bool wait, uint64_t &id_out, uint32_t &slot_out, uint32_t &i_out, uint32_t &n_out,
+                            bool &in_flight)
 {
     const uint32_t lane = threadIdx.x & 31;
     const uint64_t t = block_tail(P, s_tail, refresh);
@@ -609,9 +665,8 @@ __device__ __noinline__ int claim_source(const LoopParams &P, unsigned long long
             const unsigned long long a = __ldcg(&P.slot[s].agg);
             const unsigned long long wd = __ldcg(&P.slot[s].walks_done);
             const uint32_t wk = __ldcg(&P.desc[s].walks);
-            const uint32_t S = __ldcg(&P.desc[s].S);
             const int rel = tag_rel(a, id);
-            const bool has = rel == 0 && (uint32_t)a < S;
+            const bool has = rel == 0 && word_left(a) > 0;
             o = has && wd >= wk && __ldcg(&P.desc[s].R) <= max_R;
             left |= has;
             if (rel < 0) unwritten = (int)i;
@@ -642,27 +697,18 @@ __device__ __noinline__ int claim_source(const LoopParams &P, unsigned long long
                 // a batch of sources per claim: a few batches per aggregating warp of the loop
                 const uint32_t batch = max(1u, min(32u, S / (4u * (P.walker_warps / (kLoopWarps - 1)))));
                 const unsigned long long old = atomicAdd(&P.slot[s].agg, (unsigned long long)batch);
-                const uint32_t tag = (uint32_t)(old >> 32), c = (uint32_t)old;
+                const uint32_t tag = (uint32_t)(old >> 32), have = word_left(old);
                 // the sources are those of the query that holds the slot now (another one if it was reused)
-                if (tag != 0 && (uint32_t)__ldcg(&d->seq1) == tag) {
-                    const uint32_t S2 = __ldcg(&d->S);
-                    if (c < S2) {
-                        src_i = c;
-                        take = min(batch, S2 - c);
-                        slot = s;
-                        qid = tag - 1;
-                        got = 1;
-                        // its walks may still be running if the slot was reused: wait for them (bounded)
-                        const uint64_t t0 = gtime_ns();
-                        while (__ldcg(&P.slot[s].walks_done) < __ldcg(&d->walks)) {
-                            if (gtime_ns() - t0 > kBusyWaitNs) {
-                                flag_exit(P, PPR_LOOP_BUSY_TIMEOUT);
-                                got = -1;
-                                break;
-                            }
-                            __nanosleep(1000);
-                        }
+                if (tag != 0 && have > 0) {
+                    take = min(batch, have);
+                    slot = s;
+                    qid = tag - 1;
+                    got = 1;
+                    if (tag != (uint32_t)(h + i + 1)) {
+                        got = await_desc(P, d, tag);
+                        if (got > 0) got = wait ? await_walks(P, s) : 2;
                     }
+                    src_i = __ldcg(&d->S) - have;
                 }
             }
             got = __shfl_sync(0xffffffffu, got, 0);
@@ -672,7 +718,7 @@ __device__ __noinline__ int claim_source(const LoopParams &P, unsigned long long
                 slot_out = __shfl_sync(0xffffffffu, slot, 0);
                 i_out = __shfl_sync(0xffffffffu, src_i, 0);
                 n_out = __shfl_sync(0xffffffffu, take, 0);
-                return 1;
+                return got;
             }
         }
     }
@@ -724,7 +770,8 @@ __device__ void finish_source(const LoopParams &P, uint64_t id, uint32_t s, uint
     }
 }
 
-__device__ void aggregator_warp(const LoopParams &P, const CallerIds &ids, uint32_t *smem, unsigned long long *s_tail)
+__device__ void aggregator_warp(const LoopParams &P, const CallerIds &ids, uint32_t *smem, Handed *handed,
+                                const uint32_t *walkers, unsigned long long *s_tail)
 {
     const uint32_t lane = threadIdx.x & 31;
     uint64_t idle_t0 = 0, busy_t0 = 0;
@@ -734,7 +781,29 @@ __device__ void aggregator_warp(const LoopParams &P, const CallerIds &ids, uint3
         uint64_t id = 0;
         uint32_t s = 0, i = 0, nb = 0;
         bool in_flight = false;
-        const int r = claim_source(P, s_tail, refresh, kLoopMaxR, id, s, i, nb, in_flight);
+        int r = 0;
+        // sources handed over by the block's walker warps come first; none
+        // follow once those have ended (read before the places)
+        const uint32_t left = __shfl_sync(0xffffffffu, lane == 0 ? *(const volatile uint32_t *)walkers : 0u, 0);
+        __threadfence_block();
+        const uint32_t hm = __ballot_sync(
+            0xffffffffu, lane < kLoopWarps - 1 && *(volatile uint32_t *)&handed[lane < kLoopWarps - 1 ? lane : 0].n != 0);
+        if (hm) {
+            __threadfence_block();
+            volatile Handed *h = handed + (__ffs(hm) - 1);
+            id = h->id;
+            s = h->s;
+            i = h->i;
+            nb = h->n;
+            __syncwarp();
+            if (lane == 0) {
+                r = await_walks(P, s);
+                h->n = 0;
+            }
+            r = __shfl_sync(0xffffffffu, r, 0);
+        } else {
+            r = claim_source(P, s_tail, refresh, kLoopMaxR, true, id, s, i, nb, in_flight);
+        }
         if (r < 0) break;
         if (r > 0) {
             for (uint32_t b = 0; b < nb; ++b) reduce_source(P, ids, s, i + b, smem, kLoopMaxR);
@@ -748,12 +817,12 @@ __device__ void aggregator_warp(const LoopParams &P, const CallerIds &ids, uint3
         const uint64_t t = gtime_ns();
         if (!in_flight) {  // nothing published is left to reduce
             busy_t0 = 0;
-            if (ld_volatile(&P.ctl->stop)) {
+            if (left == 0 && ld_volatile(&P.ctl->stop)) {
                 if (lane == 0) flag_exit(P, PPR_LOOP_STOPPED);
                 break;
             }
             if (idle_t0 == 0) idle_t0 = t;
-            else if (t - idle_t0 > P.idle_ns) {
+            else if (left == 0 && t - idle_t0 > P.idle_ns) {
                 if (lane == 0) flag_exit(P, PPR_LOOP_IDLE);
                 break;
             }
@@ -779,19 +848,28 @@ __global__ void __launch_bounds__(32 * kLoopWarps, 4) k_serve_loop(const __grid_
     __shared__ __align__(16) uint32_t smem[kLoopMaxR + 3 * kLoopMaxR];  // the aggregator warp's endpoints and scratch
     __shared__ __align__(16) uint32_t help[kLoopWarps - 1][2 * kHelpMaxR + 32];  // a helping warp's endpoints and scratch
     __shared__ WarpActivity act[kLoopWarps - 1];
+    __shared__ Handed handed[kLoopWarps - 1];
+    __shared__ uint32_t walkers;  // walker warps of the block that have not ended
     __shared__ unsigned long long s_tail[2];  // the block's copy of the published tail, and when it was read
     __shared__ ClassTab tab;
     __shared__ uint32_t s_first[kTabEntries];
     for (uint32_t i = threadIdx.x; i < kTabEntries; i += blockDim.x) s_first[i] = P.kp.tab->e[i].first;
-    if (threadIdx.x == 0) s_tail[0] = s_tail[1] = 0;
+    if (threadIdx.x < kLoopWarps - 1) handed[threadIdx.x].n = 0;
+    if (threadIdx.x == 0) {
+        s_tail[0] = s_tail[1] = 0;
+        walkers = kLoopWarps - 1;
+    }
     load_tab(tab, P.kp.tab);
     const uint32_t wid = threadIdx.x >> 5;
     if (wid == kLoopWarps - 1) {
-        aggregator_warp(P, CallerIds{P.kp.order, s_first}, smem, s_tail);
+        aggregator_warp(P, CallerIds{P.kp.order, s_first}, smem, handed, &walkers, s_tail);
         return;
     }
-    walker_warp<E>(P, tab, CallerIds{P.kp.order, s_first}, wc[wid], ends_of, help[wid], act[wid],
+    walker_warp<E>(P, tab, CallerIds{P.kp.order, s_first}, wc[wid], ends_of, help[wid], act[wid], handed[wid],
                    blockIdx.x * (kLoopWarps - 1) + wid, s_tail);
+    __syncwarp();
+    __threadfence_block();
+    if ((threadIdx.x & 31) == 0) atomicSub(&walkers, 1u);
 }
 
 // ============================================================ queries ====
@@ -1197,8 +1275,8 @@ static void scheduler_loop(Server *sv)
                 d.nchunks = (uint32_t)((d.walks + cw - 1) / cw);
                 SSlot &c = sv->h_slot[s];
                 const unsigned long long tag = (unsigned long long)(uint32_t)(f->seq + 1) << 32;
-                c.claim = tag;  // chunks handed out so far (counts up)
-                c.agg = tag;    // sources handed out so far (counts up)
+                c.claim = tag | (kWordEnd - d.nchunks);  // both count up to kWordEnd
+                c.agg = tag | (kWordEnd - d.S);
                 c.walks_done = 0;
                 c.agg_done = 0;
                 if (e == cudaSuccess)
