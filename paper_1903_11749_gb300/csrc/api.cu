@@ -174,16 +174,45 @@ using namespace ppr;
 
 static size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// The context's copy stream and page-locked words, made on first use.
-static int copy_resources(ppr_ctx *ctx)
-{
-    cudaError_t e = cudaSuccess;
-    if (!ctx->copy_stream && (e = cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking)) != cudaSuccess)
-        return cuda_fail(e, "copy stream");
-    if (!ctx->pinned && (e = cudaHostAlloc((void **)&ctx->pinned, 16 * sizeof(unsigned long long), 0)) != cudaSuccess)
-        return cuda_fail(e, "page-locked words");
-    return PPR_OK;
-}
+// The context's copy stream, and eight words of host memory for one call's
+// copies of counters and totals: a block of the context's page-locked words
+// (both made on first use), or, where 64 calls of as many threads hold them
+// all, words of the call's own.
+struct CopyResources {
+    ppr_ctx *ctx = nullptr;
+    int block = -1;
+    unsigned long long own[8];
+    unsigned long long *words = own;
+
+    int take(ppr_ctx *c)
+    {
+        ctx = c;
+        std::lock_guard<std::mutex> lock(ctx->mu);
+        cudaError_t e = cudaSuccess;
+        if (!ctx->copy_stream && (e = cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking)) != cudaSuccess)
+            return cuda_fail(e, "copy stream");
+        if (!ctx->pinned) {
+            if ((e = cudaHostAlloc((void **)&ctx->pinned, 64 * sizeof(own), 0)) != cudaSuccess)
+                return cuda_fail(e, "page-locked words");
+            ctx->pinned_free = ~0ull;
+        }
+        if (ctx->pinned_free) {
+            block = __builtin_ctzll(ctx->pinned_free);
+            ctx->pinned_free &= ctx->pinned_free - 1;
+            words = ctx->pinned + 8 * block;
+        }
+        return PPR_OK;
+    }
+    CopyResources() = default;
+    CopyResources(const CopyResources &) = delete;
+    CopyResources &operator=(const CopyResources &) = delete;
+    ~CopyResources()  // (the call has waited for its copies)
+    {
+        if (block < 0) return;
+        std::lock_guard<std::mutex> lock(ctx->mu);
+        ctx->pinned_free |= 1ull << block;
+    }
+};
 
 static int set_device(const ppr_ctx *ctx)
 {
@@ -720,7 +749,8 @@ int ppr_run_to_host(ppr_ctx *ctx, const ppr_graph *g, const ppr_run_args *a, int
     Range range("ppr_run_to_host");
     cudaStream_t st = (cudaStream_t)a->stream;
     if ((rc = prepare_tables(g, plan, st))) return rc;
-    if ((rc = copy_resources(ctx))) return rc;
+    CopyResources host;
+    if ((rc = host.take(ctx))) return rc;
     cudaError_t e = cudaSuccess;
     cudaStream_t cs = ctx->copy_stream;
     const int64_t S = a->src_end - a->src_begin;
@@ -823,7 +853,7 @@ int ppr_run_to_host(ppr_ctx *ctx, const ppr_graph *g, const ppr_run_args *a, int
             note_launch();
             k_next_base<<<1, 1, 0, st>>>(d_base, q.off + nb);
             note_launch();
-            if ((e = cudaMemcpyAsync(&ctx->pinned[i & 1], q.off + nb, sizeof(uint64_t), cudaMemcpyDeviceToHost, st)) !=
+            if ((e = cudaMemcpyAsync(&host.words[i & 1], q.off + nb, sizeof(uint64_t), cudaMemcpyDeviceToHost, st)) !=
                     cudaSuccess ||
                 (e = cudaEventRecord(q.ready, st)) != cudaSuccess)
                 return finish(cuda_fail(e, "batch"));
@@ -833,7 +863,7 @@ int ppr_run_to_host(ppr_ctx *ctx, const ppr_graph *g, const ppr_run_args *a, int
             Slot &q = slot[j & 1];
             const int64_t b0 = start[j], nb = start[j + 1] - b0;
             if ((e = cudaEventSynchronize(q.ready)) != cudaSuccess) return finish(cuda_fail(e, "batch"));
-            const uint64_t tot = ctx->pinned[j & 1] - base;  // the batch's last absolute row start, less the base
+            const uint64_t tot = host.words[j & 1] - base;  // the batch's last absolute row start, less the base
             if ((uint64_t)cap < base + tot) {
                 set_error("capacity %lld < nnz (at least %llu)", (long long)cap, (unsigned long long)(base + tot));
                 return finish(PPR_ERANGE);
@@ -1097,16 +1127,17 @@ int ppr_wait(ppr_result *r, int64_t timeout_ms)
         if (e == cudaSuccess) break;
         if (e != cudaErrorNotReady) return cuda_fail(e, "run");
         const auto us = std::chrono::duration_cast<std::chrono::microseconds>(std::chrono::steady_clock::now() - t0).count();
-        if (timeout_ms >= 0 && us >= 1000 * timeout_ms) {
+        if (timeout_ms >= 0 && us / 1000 >= timeout_ms) {
             set_error("run not finished after %lld ms", (long long)timeout_ms);
             return PPR_ETIMEOUT;
         }
         if (us >= 2000) std::this_thread::sleep_for(std::chrono::microseconds(50));
     }
     // the run is over: its counters are read beside whatever the caller's streams do now
-    if ((rc = copy_resources(r->ctx))) return rc;
-    unsigned long long *cnt = r->ctx->pinned;
-    PPR_CUDA(cudaMemcpyAsync(cnt, r->d_steps, 6 * sizeof(cnt[0]), cudaMemcpyDeviceToHost, r->ctx->copy_stream));
+    CopyResources host;
+    if ((rc = host.take(r->ctx))) return rc;
+    const unsigned long long *cnt = host.words;
+    PPR_CUDA(cudaMemcpyAsync(host.words, r->d_steps, 6 * sizeof(cnt[0]), cudaMemcpyDeviceToHost, r->ctx->copy_stream));
     PPR_CUDA(cudaStreamSynchronize(r->ctx->copy_stream));
     r->steps = cnt[0];
     r->sectors = cnt[2];
@@ -1172,7 +1203,8 @@ int ppr_sparse_rows(const ppr_result *rc_, int64_t *row_ptr, int32_t *col, uint3
     cudaStream_t st = r->stream;
     const int64_t S = r->S;
     int64_t tiles = (S + kScanTile - 1) / kScanTile;
-    if ((rc = copy_resources(r->ctx))) return rc;
+    CopyResources host;
+    if ((rc = host.take(r->ctx))) return rc;
     uint64_t *d_off = nullptr, *d_tmp = nullptr;
     // row starts straight into the caller's device array when there is one
     const bool own_off = !(dev_out && row_ptr);
@@ -1201,10 +1233,10 @@ int ppr_sparse_rows(const ppr_result *rc_, int64_t *row_ptr, int32_t *col, uint3
     }
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(r->ctx->pinned, d_off + S, sizeof(uint64_t), cudaMemcpyDeviceToHost, st);
+        e = cudaMemcpyAsync(host.words, d_off + S, sizeof(uint64_t), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return done(cuda_fail(e, "row scan"));
-    const uint64_t total = r->ctx->pinned[0];
+    const uint64_t total = host.words[0];
     r->nnz_total = (int64_t)total;
     if (nnz) *nnz = (int64_t)total;
     if (row_ptr && own_off) {

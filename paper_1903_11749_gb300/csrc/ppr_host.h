@@ -3,6 +3,7 @@
 
 #include <atomic>
 #include <cstdint>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -72,7 +73,9 @@ struct ppr_ctx {
     size_t l2_bytes = 0;          // L2 size (the layout's renumbering policy)
     size_t mem_bytes = 0;         // device memory (the layout's slot density)
     cudaStream_t copy_stream = nullptr;  // copies to the host beside the caller's streams
-    unsigned long long *pinned = nullptr;  // page-locked words: per-batch totals, a finished run's counters
+    unsigned long long *pinned = nullptr;  // 64 blocks of eight page-locked words, lent to the calls at work
+    uint64_t pinned_free = 0;              // bit i: block i is free
+    std::mutex mu;                         // guards pinned_free and the making of the stream and the words
     std::atomic<int> refs{1};  // the caller's handle plus every live graph and result
 };
 
