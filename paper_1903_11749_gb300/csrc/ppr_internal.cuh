@@ -205,27 +205,52 @@ __device__ __forceinline__ uint64_t mulhi64(uint64_t r, uint64_t W) { return __u
 
 // ---------------------------------------------------------------- loads ----
 // One 32-byte sector in a single 256-bit load (sm_100+ vector width).
+// FAR: fetched from DRAM by 64 bytes, where a load of any width moves 128 by
+// default (uniform 32-byte reads over 2 GB: 122.5 DRAM bytes a load, 62.6 with
+// the hint, both at 51 G loads a second: it is requests that are limited).
 struct Sector {
     uint32_t v[8];
 };
+template <bool FAR = false>
 __device__ __forceinline__ Sector ld_sector(const void *p)
 {
     Sector s;
-    asm("ld.global.nc.v8.u32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(s.v[0]), "=r"(s.v[1]), "=r"(s.v[2]), "=r"(s.v[3]), "=r"(s.v[4]), "=r"(s.v[5]), "=r"(s.v[6]),
-                   "=r"(s.v[7])
-                 : "l"(p));
+    if constexpr (FAR)
+        asm("ld.global.nc.L2::64B.v8.u32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+            : "=r"(s.v[0]), "=r"(s.v[1]), "=r"(s.v[2]), "=r"(s.v[3]), "=r"(s.v[4]), "=r"(s.v[5]), "=r"(s.v[6]),
+              "=r"(s.v[7])
+            : "l"(p));
+    else
+        asm("ld.global.nc.v8.u32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+            : "=r"(s.v[0]), "=r"(s.v[1]), "=r"(s.v[2]), "=r"(s.v[3]), "=r"(s.v[4]), "=r"(s.v[5]), "=r"(s.v[6]),
+              "=r"(s.v[7])
+            : "l"(p));
     return s;
 }
 
 // Eight bytes for the lanes with `on` set only (the others' are undefined),
 // without a branch that the compiler would carry what follows into.
+template <bool FAR>
 __device__ __forceinline__ uint2 ld_pair_if(const void *p, bool on)
 {
     uint2 v;
-    asm("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %3, 0;\n\t@q ld.global.nc.v2.u32 {%0,%1}, [%2];\n\t}"
-        : "=r"(v.x), "=r"(v.y)
-        : "l"(p), "r"((uint32_t)on));
+    if constexpr (FAR)
+        asm("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %3, 0;\n\t@q ld.global.nc.L2::64B.v2.u32 {%0,%1}, [%2];\n\t}"
+            : "=r"(v.x), "=r"(v.y)
+            : "l"(p), "r"((uint32_t)on));
+    else
+        asm("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %3, 0;\n\t@q ld.global.nc.v2.u32 {%0,%1}, [%2];\n\t}"
+            : "=r"(v.x), "=r"(v.y)
+            : "l"(p), "r"((uint32_t)on));
+    return v;
+}
+
+template <bool FAR>
+__device__ __forceinline__ uint4 ld_quad(const void *p)
+{
+    if constexpr (!FAR) return __ldg(static_cast<const uint4 *>(p));
+    uint4 v;
+    asm("ld.global.nc.L2::64B.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
     return v;
 }
 
@@ -237,7 +262,7 @@ __device__ __forceinline__ void st_sector(void *p, const Sector &s)
 }
 
 struct NarrowEdges {
-    static constexpr bool kWide = false;
+    static constexpr bool kWide = false, kFar = false, kAlias = false;
     using Edge = EdgeN;
     const EdgeN *e;
     __device__ __forceinline__ uint2 load(uint64_t i) const
@@ -250,7 +275,7 @@ struct NarrowEdges {
 };
 
 struct WideEdges {
-    static constexpr bool kWide = true;
+    static constexpr bool kWide = true, kFar = false, kAlias = false;
     using Edge = EdgeW;
     const EdgeW *e;
     __device__ __forceinline__ uint4 load(uint64_t i) const
@@ -263,7 +288,15 @@ struct WideEdges {
 };
 
 // Alias tables: walked with AliasNode records and AliasRec slots.
-struct AliasEdges {};
+struct AliasEdges {
+    static constexpr bool kWide = false, kFar = false, kAlias = true;
+};
+
+// The same layouts walked where they lie far beyond L2 (launch_walks).
+template <class E>
+struct Far : E {
+    static constexpr bool kFar = true;
+};
 
 // Segment entries have the same 16-byte shape as wide edges: key = cum,
 // target = node, and the fourth word carries mark_len.

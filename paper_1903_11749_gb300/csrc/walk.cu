@@ -8,7 +8,6 @@
 // turns each source's R endpoints into its count row and top-k.
 #include <algorithm>
 #include <atomic>
-#include <type_traits>
 #include <mutex>
 
 #include "ppr_host.h"
@@ -48,7 +47,7 @@ __device__ __forceinline__ void warp_add_tally(unsigned long long *dst, const Ta
 constexpr uint32_t kDefaultRefill = 8;
 
 template <class E>
-constexpr int kWalkBlocks = std::is_same<E, WideEdges>::value ? 8 : 6;
+constexpr int kWalkBlocks = E::kWide ? 8 : 6;
 
 template <class E, bool SEG, bool STATS>
 __global__ void __launch_bounds__(256, kWalkBlocks<E>) k_walk_plain(KParams p)
@@ -242,7 +241,7 @@ static int launch_typed(ppr_ctx *ctx, const KParams &kp, const RunPlan &plan, in
     cudaLaunchAttribute attr[1];
     if (plan.l2_persist && ctx->l2_persist_max > 0 && ctx->l2_window_max > 0) {
         // the alias node records, or the front of the slots, persisting in L2
-        constexpr bool alias = std::is_same<E, AliasEdges>::value;
+        constexpr bool alias = E::kAlias;
         const size_t all = alias ? (size_t)kp.n_anode * sizeof(AliasNode) : (size_t)kp.n_slots * sizeof(Sector);
         const size_t bytes = std::min(all, ctx->l2_window_max);
         if (ctx->l2_persist_set < std::min(bytes, ctx->l2_persist_max)) {
@@ -341,6 +340,9 @@ void preload_run_kernels()
     preload_walkers<NarrowEdges, true, false>();
     preload_walkers<NarrowEdges, false, true>();
     preload_walkers<NarrowEdges, true, true>();
+    preload_walkers<Far<NarrowEdges>, false, false>();
+    preload_walkers<Far<NarrowEdges>, true, false>();
+    preload_walkers<Far<AliasEdges>, false, false>();
     preload_walkers<WideEdges, false, false>();
     preload_walkers<WideEdges, true, false>();
     preload_walkers<WideEdges, false, true>();
@@ -398,6 +400,19 @@ void set_layout(KParams &kp, const ppr_graph *g, bool segments, bool alias)
     kp.n_single = (uint64_t)g->n_single;
     kp.n_records = (uint64_t)g->m;
     kp.n_seg = (uint64_t)g->seg.entries_cap;
+}
+
+// Whether a walk's random loads are fetched by 64 bytes (Far): where the slots
+// (the alias slots) are 16 times the L2 and more, a neighbour that comes along
+// is evicted before it is used.  R-MAT scale 24 on two GPUs, without / with:
+// job 109.05 / 105.63 and 103.57 / 103.51 ms, a quarter with segments 25.39 /
+// 24.59 and 24.09 / 23.99, with alias tables 24.34 / 24.03 and 23.50 / 23.22.
+// Scale 20 (three times the L2), where neighbours are used: 8.21 / 8.49 on the
+// first, and alias tables 5.48 / 5.90.
+static bool is_far(const ppr_ctx *ctx, const ppr_graph *g, bool alias)
+{
+    const double bytes = alias ? (double)g->m * sizeof(AliasRec) : (double)g->n_slots * sizeof(Sector);
+    return !g->wide && g->instances == 0 && bytes >= 16.0 * (double)ctx->l2_bytes;
 }
 
 int launch_walks(ppr_ctx *ctx, const ppr_graph *g, const RunPlan &plan, const Outputs &o, int64_t s_begin, int64_t S,
@@ -478,6 +493,10 @@ int launch_walks(ppr_ctx *ctx, const ppr_graph *g, const RunPlan &plan, const Ou
         }
         if (reset_queue) PPR_CUDA(cudaMemsetAsync(kp.queue, 0, sizeof(unsigned long long), st));
     }
+    const bool far = is_far(ctx, g, plan.sampler == 1) && !plan.stats;
+    if (far && plan.sampler == 1) return launch_typed<Far<AliasEdges>, false, false>(ctx, kp, plan, S, st, ev_owner);
+    if (far && plan.segments) return launch_typed<Far<NarrowEdges>, true, false>(ctx, kp, plan, S, st, ev_owner);
+    if (far) return launch_typed<Far<NarrowEdges>, false, false>(ctx, kp, plan, S, st, ev_owner);
     if (plan.sampler == 1)
         return plan.stats ? launch_typed<AliasEdges, false, true>(ctx, kp, plan, S, st, ev_owner)
                           : launch_typed<AliasEdges, false, false>(ctx, kp, plan, S, st, ev_owner);

@@ -9,8 +9,6 @@
 // depth 3) the same draw selects one outcome: a terminated outcome ends the
 // walk, an active one moves the walk and advances k by the outcome's length.
 #pragma once
-#include <type_traits>
-
 #include "ppr_host.h"
 #include "aggregate.cuh"
 
@@ -148,7 +146,7 @@ struct Pending {
 // the batch kernels, per lane in the serving loop).
 //
 // One step of one walk, or the rest of one.  Returns true when the walk has
-// ended, at node u.  E: NarrowEdges, WideEdges or AliasEdges.  STATS: count
+// ended, at node u.  E: NarrowEdges, WideEdges or AliasEdges, or Far of one.  STATS: count
 // the 32-byte sectors read.  k counts the draws of the walk (in segment mode
 // an outcome's length instead; tl.steps then counts the draws).
 template <class E, bool SEG, bool STATS, class K>
@@ -158,7 +156,7 @@ __device__ __forceinline__ bool walk_step(const KParams &p, const ClassTab &tab,
 {
     const uint32_t idx = u & kIdxMask;
     const TabEntry t = tab.e[u >> kIdxBits];  // (any u: 64 entries)
-    if constexpr (std::is_same<E, AliasEdges>::value) {
+    if constexpr (E::kAlias) {
         PPR_CHECK((uint64_t)t.first + idx < p.n_nodes, 1);
         // Integer alias method: slot i = floor(r*d / 2^64), y = floor(frac * W / 2^64).
         // What depends on the node alone, the record of a row that has to be
@@ -166,7 +164,7 @@ __device__ __forceinline__ bool walk_step(const KParams &p, const ClassTab &tab,
         const bool lookup = t.kind == kKindLookup, single = t.kind == kKindSingle, dang = t.kind == kKindDangling;
         if (dang && p.dangling == 1) return true;  // the walk ends here without a step
         const uint64_t at = t.addr + ((uint64_t)idx << (lookup ? 3 : 2));
-        const uint2 nr = ld_pair_if(reinterpret_cast<const void *>(at & ~7ull), lookup || single);
+        const uint2 nr = ld_pair_if<E::kFar>(reinterpret_cast<const void *>(at & ~7ull), lookup || single);
         const uint4 x = philox4x32_10(make_uint4(sctr, j, k, tag), key);
         uint32_t to = dang ? src : ((at & 4) ? nr.y : nr.x);
         if (!single && !dang) {
@@ -177,7 +175,7 @@ __device__ __forceinline__ bool walk_step(const KParams &p, const ClassTab &tab,
             const uint64_t r64 = (uint64_t)x.x | ((uint64_t)x.y << 32);
             const uint32_t i = (uint32_t)__umul64hi(r64, (uint64_t)cnt);
             const uint64_t frac = r64 * (uint64_t)cnt;
-            const uint4 rec = __ldg(reinterpret_cast<const uint4 *>(row) + i);  // {thr, col, alias col, W}
+            const uint4 rec = ld_quad<E::kFar>(row + i);  // {thr, col, alias col, W}
             const uint64_t y = mulhi64_by32((uint32_t)frac, (uint32_t)(frac >> 32), rec.w);
             to = y < rec.x ? rec.y : rec.z;
         }
@@ -220,7 +218,7 @@ __device__ __forceinline__ bool walk_step(const KParams &p, const ClassTab &tab,
                              : (at >= p.slots && at < p.slots + p.n_slots) ||
                                    (SEG && at >= p.seg_slots && at < p.seg_slots + p.n_seg_slots),
                       2);
-            const Sector s = ld_sector(at);
+            const Sector s = ld_sector<E::kFar>(at);
             if (STATS) ++tl.sectors;
             if (resume) {
                 next = pick_record(s, (pend.flags >> 8) & 3u, u);
