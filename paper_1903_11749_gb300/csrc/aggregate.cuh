@@ -566,7 +566,11 @@ __global__ void __launch_bounds__(T) k_aggregate_block(AggParams p)
 template <int E>
 static int launch_aggregate_e(ppr_ctx *ctx, const AggParams &ap, cudaStream_t st)
 {
-    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((ap.S + kAggWarps - 1) / kAggWarps, (int64_t)ctx->sms * 16));
+    // 128 blocks a SM, some ten times what is resident: sixteen left a second wave
+    // of a few blocks (R 50, 2^22 sources: 2.37 -> 1.98 ms; R 100, 2^20: .889 ->
+    // .796; R 200, 2^21: 3.19 -> 2.94; as many as are resident .97 ms at R 100,
+    // 512 a SM .81)
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((ap.S + kAggWarps - 1) / kAggWarps, (int64_t)ctx->sms * 128));
     k_aggregate<E><<<blocks, 32 * kAggWarps, 0, st>>>(ap);
     note_launch();
     PPR_CUDA(cudaGetLastError());
@@ -576,7 +580,9 @@ static int launch_aggregate_e(ppr_ctx *ctx, const AggParams &ap, cudaStream_t st
 template <int T, int I>
 static int launch_aggregate_block(ppr_ctx *ctx, const AggParams &ap, cudaStream_t st)
 {
-    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(ap.S, (int64_t)ctx->sms * (4096 / T)));
+    // many times what is resident, as above (R 300, 1000, 4000 of 2^16, 2^15, 2^13
+    // sources: 275, 344, 430 us; with an eighth of the blocks 291, 368, 462)
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(ap.S, (int64_t)ctx->sms * (32768 / T)));
     k_aggregate_block<T, I><<<blocks, T, 0, st>>>(ap);
     note_launch();
     PPR_CUDA(cudaGetLastError());
