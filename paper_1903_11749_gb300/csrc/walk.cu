@@ -35,20 +35,20 @@ __device__ __forceinline__ void warp_add_tally(unsigned long long *dst, const Ta
     }
 }
 
-// ------------------------------------------------------------ plain (K4) ----
-// Resident 256-thread blocks per SM asked of ptxas.  Narrow: 6 (40 registers;
-// 8 blocks at 32 gain nothing on the batch and lose 7 % on a small query).
-// Wide: 8 (R-MAT scale 18 with amounts as weights: 2.20 -> 2.08 ms).  Alias: 6 (R-MAT
-// scale 24, 2^22 sources: 20.4 ms; 8 blocks 21.4: more walks at once, fewer L2 hits).
 // Idle lanes before a warp starts new walks, unless the caller says: starting
 // them costs the whole warp some forty instructions (256-graph batch 17.6 ms
 // at one lane, 17.0 at four, 16.9 at eight, 17.9 at sixteen; the scale-24 and
 // scale-20 walkers, which wait for memory, are level from one to eight).
 constexpr uint32_t kDefaultRefill = 8;
 
+// Resident 256-thread blocks per SM asked of ptxas.  Narrow: 6 (38 registers;
+// 8 blocks at 32: 256-graph batch 18.75 against 18.55 ms, R-MAT scale-24 job
+// 103.7 against 102.9).  Wide: 8 (scale 18 with amounts as weights, 2.20 -> 2.08
+// ms).  Alias: 8 (scale 20 5.37 against 5.47 ms; a quarter of scale 24 level).
 template <class E>
-constexpr int kWalkBlocks = E::kWide ? 8 : 6;
+constexpr int kWalkBlocks = E::kWide || E::kAlias ? 8 : 6;
 
+// ------------------------------------------------------------ plain (K4) ----
 template <class E, bool SEG, bool STATS>
 __global__ void __launch_bounds__(256, kWalkBlocks<E>) k_walk_plain(KParams p)
 {
@@ -100,7 +100,14 @@ __global__ void __launch_bounds__(256, kWalkBlocks<E>) k_walk_plain(KParams p)
 struct WarpChunk {
     uint32_t base, ctr_base, tag;  // first position, counter base, tag
     uint32_t j0;                   // walk index (within source `base`) of the chunk's first walk
+    uint2 src[32];                 // counter id and code of the chunk's sources
 };
+// A chunk's sources are read when a warp takes it, one a lane, so that no
+// refill waits for them (256-graph batch 18.91 -> 18.55 ms, R-MAT scale-24 job
+// 103.8 -> 102.9, scale 20 8.10 -> 8.01; the wide walker, short of registers,
+// reads them as it starts walks: 2.200 ms, staged 2.227).  So a chunk has at
+// most 31 whole sources, or parts of 32.
+constexpr uint32_t kChunkSources = 31;
 
 __device__ __forceinline__ uint32_t div_by_R(uint32_t w, uint64_t magic)
 {
@@ -112,6 +119,8 @@ __global__ void __launch_bounds__(256, kWalkBlocks<E>) k_walk_persistent(KParams
 {
     __shared__ WarpChunk chunk_all[8];
     __shared__ ClassTab tab;
+    __shared__ unsigned long long nchunks;
+    if (threadIdx.x == 0) nchunks = p.nchunks_dev ? *p.nchunks_dev : p.nchunks;
     load_tab(tab, p.tab);
     const uint32_t lane = threadIdx.x & 31;
     WarpChunk &wc = chunk_all[threadIdx.x >> 5];
@@ -132,19 +141,35 @@ __global__ void __launch_bounds__(256, kWalkBlocks<E>) k_walk_persistent(KParams
                     unsigned long long c = 0;
                     if (lane == 0) c = atomicAdd(p.queue, 1ull);
                     c = __shfl_sync(0xffffffffu, c, 0);
-                    const unsigned long long nch = p.nchunks_dev ? *p.nchunks_dev : p.nchunks;
-                    if (c >= nch) {
+                    if (c >= nchunks) {
                         queue_empty = true;
                         break;
                     }
+                    uint32_t base, ctr_base = 0, ctag = p.tag, j0 = 0, nsrc;
                     if (p.chunks) {  // whole sources of one instance
                         const int4 d = p.chunks[c];
-                        if (lane == 0) wc = WarpChunk{(uint32_t)d.x, (uint32_t)p.inst_off[d.z], (uint32_t)d.z, 0u};
-                        total = (uint32_t)d.y * p.R;
+                        base = (uint32_t)d.x;
+                        ctr_base = (uint32_t)d.w;
+                        ctag = (uint32_t)d.z;
+                        nsrc = (uint32_t)d.y;
+                        total = nsrc * p.R;
                     } else {  // walks [c * CW, ...) of the whole launch
                         const uint64_t b = c * (uint64_t)p.CW, i0 = b / p.R;
-                        if (lane == 0) wc = WarpChunk{(uint32_t)i0, 0u, p.tag, (uint32_t)(b - i0 * p.R)};
+                        base = (uint32_t)i0;
+                        j0 = (uint32_t)(b - i0 * p.R);
                         total = (uint32_t)min((uint64_t)p.CW, p.walks - b);
+                        nsrc = div_by_R(j0 + total - 1, p.r_magic) + 1;
+                    }
+                    __syncwarp();  // the walks of the chunk before have been started
+                    if (lane == 0) {
+                        wc.base = base;
+                        wc.ctr_base = ctr_base;
+                        wc.tag = ctag;
+                        wc.j0 = j0;
+                    }
+                    if (!E::kWide && lane < nsrc) {  // draws are keyed by the caller's source id; walks start at its node of the layout
+                        const uint32_t id = p.src_list ? p.src_list[base + lane] : (uint32_t)(p.s_begin + base + lane);
+                        wc.src[lane] = make_uint2(id - ctr_base, p.code_of[id]);
                     }
                     issued = 0;
                     __syncwarp();
@@ -155,9 +180,15 @@ __global__ void __launch_bounds__(256, kWalkBlocks<E>) k_walk_persistent(KParams
                     const uint32_t i = div_by_R(w, p.r_magic);
                     j = w - i * p.R;
                     pos = wc.base + i;
-                    src = p.src_list ? p.src_list[pos] : (uint32_t)(p.s_begin + pos);
-                    sctr = src - wc.ctr_base;  // draws keyed by the caller's source id
-                    src = p.code_of[src];      // start and restart node of the layout
+                    if constexpr (!E::kWide) {
+                        const uint2 s = wc.src[i];
+                        sctr = s.x;
+                        src = s.y;
+                    } else {
+                        src = p.src_list ? p.src_list[pos] : (uint32_t)(p.s_begin + pos);
+                        sctr = src - wc.ctr_base;
+                        src = p.code_of[src];
+                    }
                     tag = wc.tag;
                     k = 0;
                     u = src;
@@ -294,16 +325,17 @@ __global__ void __launch_bounds__(256) k_chunk_fill(int32_t count, const int64_t
         }
         const int64_t a = max(node_off[lo], s_begin), b = min(node_off[lo + 1], s_end);
         const int64_t s = a + (int64_t)(c - offs[lo]) * CS;
-        chunks[c] = make_int4((int)(s - s_begin), (int)min((int64_t)CS, b - s), lo, 0);
+        chunks[c] = make_int4((int)(s - s_begin), (int)min((int64_t)CS, b - s), lo, (int)node_off[lo]);
     }
 }
 
-// sources per chunk; a chunk holds at most 2^19 walks (walk indices within a
-// chunk stay below 2^20 for the multiply-shift division by R)
+// sources per chunk, at most as many as a warp has places for; a chunk holds at
+// most 2^19 walks (walk indices within a chunk stay below 2^20 for the
+// multiply-shift division by R)
 static uint32_t chunk_sources(const RunPlan &plan)
 {
     const uint32_t cs = plan.chunk_sources > 0 ? (uint32_t)plan.chunk_sources : std::max(1u, 400u / plan.R);
-    return std::min(cs, std::max(1u, (1u << 19) / plan.R));
+    return std::min(std::min(cs, kChunkSources), std::max(1u, (1u << 19) / plan.R));
 }
 
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -476,7 +508,6 @@ int launch_walks(ppr_ctx *ctx, const ppr_graph *g, const RunPlan &plan, const Ou
             note_launch();
             PPR_CUDA(cudaGetLastError());
             kp.chunks = chunks;
-            kp.inst_off = g->d_node_off;
             kp.nchunks_dev = o.counters + 3;
             kp.nchunks = (uint32_t)((S + CS - 1) / CS + cnt);  // upper bound, for the grid size
         } else {

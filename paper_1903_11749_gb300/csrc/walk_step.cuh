@@ -36,7 +36,7 @@ struct KParams {
     uint64_t walks;           // S * R
     uint32_t nchunks;
     const unsigned long long *nchunks_dev;  // batched graphs: chunk count written on the device
-    const int4 *chunks;       // batched graphs: {position, nsrc, instance, 0}; else null
+    const int4 *chunks;       // batched graphs: {position, nsrc, instance, its first node}; else null
     const uint32_t *src_list; // explicit sources (position -> node id); null: s_begin + position
     const uint32_t *code_of;  // code of a caller node (the walk's start)
     const int32_t *order;     // caller id of a node by seq (endpoints)
