@@ -66,13 +66,12 @@ enum {
 /* flags */
 #define PPR_PTRS_DEVICE 0x1u /* pointer arguments are device pointers */
 /* Node numbering of the device layout (ppr_load_graph; plain graphs only).
- * The layout numbers nodes by the length class of their rows.  With
- * PPR_RENUMBER the nodes of a class follow in descending in-degree order
- * (counted on every fourth edge, two steps per power of two, ties in caller
- * order), so that the rows of the most visited nodes are contiguous;
- * PPR_KEEP_IDS keeps the caller's order within a class; with neither, the
- * layout takes the in-degree order when 32 bytes a node exceed twice the
- * device's L2.  The numbering is internal:
+ * The layout numbers nodes by the length class of their rows, in the caller's
+ * order within a class.  PPR_RENUMBER and PPR_KEEP_IDS, which chose the order
+ * within a class, are kept for callers that set them: a draw reads one slot of
+ * its row, and no order of the nodes makes that faster.  They decide what
+ * ppr_graph_info reports (with neither: renumbered when 32 bytes a node exceed
+ * twice the device's L2).  The numbering is internal:
  * sources, rows and top-k use the caller's ids, walks draw by the caller's
  * source id, and every result is the same either way. */
 #define PPR_RENUMBER 0x2u
@@ -174,7 +173,7 @@ typedef struct {
     int64_t device_bytes;    /* device memory held by the graph */
     int64_t segment_nodes;   /* nodes with a segment table (last built threshold) */
     int64_t segment_entries;
-    int32_t renumbered;      /* 1 if the layout numbers nodes by in-degree (PPR_RENUMBER) */
+    int32_t renumbered;      /* 1 where PPR_RENUMBER or the rule beside it applies */
     int32_t reserved;
 } ppr_graph_info;
 
@@ -204,7 +203,7 @@ typedef struct {
     int32_t large_degree;/* >= 0; kept for callers that set it: a draw reads one slot of its row
                             whatever the degree, so there is no search to share */
     int32_t warps_per_block;  /* persistent kernel: 4 or 8 warps per CTA (0 = 8) */
-    int32_t chunk_sources;    /* sources per queue item, 0 = default */
+    int32_t chunk_sources;    /* sources per queue item (31 at most are taken at once), 0 = default */
     int64_t max_batch_sources;/* sources per device batch, 0 = sized to free device memory */
     int32_t stats;       /* 1: also count the algorithmic 32-byte sectors of every step (slower;
                             rows, counts and steps are unchanged) */
@@ -219,8 +218,7 @@ typedef struct {
                             access-policy window; the device's persisting set-aside is raised
                             for this context on first use); 0: off.  Results are unchanged */
     int32_t refill_lanes;/* persistent kernel: a warp starts new walks once at least this many of
-                            its 32 lanes are idle, and then fills every idle lane (1..32; 0 = 1,
-                            at once).  32 starts a warp's walks together, like one thread per
+                            its 32 lanes are idle, and then fills every idle lane (1..32; 0 = 8).  32 starts a warp's walks together, like one thread per
                             walk, so the first steps of a source's walks share their loads.
                             Results are unchanged */
     void *stream;        /* cudaStream_t, NULL = legacy default stream */
@@ -283,8 +281,8 @@ typedef struct {
  * sample_sources, 0 = 65536; evenly strided for plain graphs, a leading range
  * for batched graphs) for each candidate of walkers per CTA (128, 256), queue
  * chunk (1/4x .. 4x of 400/R sources), then, with the fastest of those, for
- * refill thresholds of 8, 16, 24 and 32 idle lanes (against 1), and returns
- * the fastest.  Synchronous;
+ * refill thresholds of 1, 16, 24 and 32 idle lanes (against the run's, 8 unless
+ * set), and returns the fastest.  Synchronous;
  * allocates scratch for the sample.  Tuning never changes results.
  */
 int ppr_autotune(ppr_ctx *ctx, const ppr_graph *g, const ppr_run_args *args, int64_t sample_sources, ppr_tuning *best);
@@ -462,7 +460,7 @@ typedef struct {
                                takes chunk_sources only) */
     int32_t sampler;        /* neighbour choice of every query, as ppr_run_args.sampler; with 1
                                the graph's alias tables are built by ppr_serve_start */
-    int32_t refill_lanes;   /* as ppr_run_args.refill_lanes (0 = 1) */
+    int32_t refill_lanes;   /* as ppr_run_args.refill_lanes (0 = 8) */
     int32_t mode;           /* PPR_SERVE_DEVICE_LOOP (0) or PPR_SERVE_STREAMS (1) */
     int64_t idle_us;        /* device loop: idle time after which the resident kernel exits
                                (0 = 200,000 us); the next query launches it again */

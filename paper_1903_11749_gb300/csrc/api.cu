@@ -984,6 +984,7 @@ int ppr_autotune(ppr_ctx *ctx, const ppr_graph *g, const ppr_run_args *a, int64_
     if ((rc = set_device(ctx))) return rc;
     cudaStream_t st = (cudaStream_t)a->stream;
     if ((rc = prepare_tables(g, plan, st))) return rc;
+    if (plan.refill_lanes == 0) plan.refill_lanes = (int32_t)kDefaultRefill;  // (what is timed is what is returned)
     const int64_t S_all = a->src_end - a->src_begin;
     const int64_t S = std::max<int64_t>(1, std::min<int64_t>(S_all, sample_sources > 0 ? sample_sources : 65536));
     // batched graphs keep their instance structure: tune on a contiguous range
@@ -1062,12 +1063,12 @@ int ppr_autotune(ppr_ctx *ctx, const ppr_graph *g, const ppr_run_args *a, int64_
             if (bt.ms < 0 || ms_best < bt.ms) {
                 bt.chunk_sources = cs;
                 bt.warps_per_block = wpb;
-                bt.refill_lanes = plan.refill_lanes > 0 ? plan.refill_lanes : 1;
+                bt.refill_lanes = plan.refill_lanes;
                 bt.ms = ms_best;
             }
         }
     // refill thresholds with the fastest launch shape
-    const int rf_cands[] = {8, 16, 24, 32};
+    const int rf_cands[] = {plan.refill_lanes == 8 ? 1 : 8, 16, 24, 32};
     for (int rf : rf_cands) {
         if (rc || bt.ms < 0) break;
         RunPlan pl = plan;

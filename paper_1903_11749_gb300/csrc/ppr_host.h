@@ -163,6 +163,12 @@ int build_alias(ppr_graph *g, cudaStream_t st);
 
 // walk.cu
 void preload_run_kernels();  // loads every kernel a run launches (once per device)
+
+// Idle lanes before a warp starts new walks, unless the caller says: starting
+// them costs the whole warp some forty instructions (256-graph batch 17.6 ms
+// at one lane, 17.0 at four, 16.9 at eight, 17.9 at sixteen; the scale-24 and
+// scale-20 walkers, which wait for memory, are level from one to eight).
+constexpr uint32_t kDefaultRefill = 8;
 struct RunPlan {
     uint32_t T, R;
     uint64_t seed;
@@ -172,7 +178,7 @@ struct RunPlan {
     int32_t kernel;
     int32_t warps_per_block;
     int32_t chunk_sources;
-    int32_t refill_lanes;  // persistent kernel: idle lanes before a warp refills (0 = 1)
+    int32_t refill_lanes;  // persistent kernel: idle lanes before a warp refills (0 = kDefaultRefill)
     bool stats;
     int32_t sampler;  // 0 first-prefix-above rule, 1 integer alias method
     bool l2_persist;  // walker launches keep the front of the layout in L2 (access-policy window)

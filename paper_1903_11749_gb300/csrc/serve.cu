@@ -1124,7 +1124,7 @@ static int launch_loop_typed(Server *sv)
     P.slot = sv->d_slot;
     P.ctl = sv->ctl_dev;
     P.glob = sv->d_glob;
-    P.refill = sv->cfg.refill_lanes > 0 ? (uint32_t)std::min(sv->cfg.refill_lanes, 32) : 8u;
+    P.refill = sv->cfg.refill_lanes > 0 ? (uint32_t)std::min(sv->cfg.refill_lanes, 32) : kDefaultRefill;
     P.idle_ns = (uint64_t)(sv->cfg.idle_us > 0 ? sv->cfg.idle_us : 200000) * 1000ull;
     if (!sv->grid) {
         int per_sm = 0;

@@ -35,12 +35,6 @@ __device__ __forceinline__ void warp_add_tally(unsigned long long *dst, const Ta
     }
 }
 
-// Idle lanes before a warp starts new walks, unless the caller says: starting
-// them costs the whole warp some forty instructions (256-graph batch 17.6 ms
-// at one lane, 17.0 at four, 16.9 at eight, 17.9 at sixteen; the scale-24 and
-// scale-20 walkers, which wait for memory, are level from one to eight).
-constexpr uint32_t kDefaultRefill = 8;
-
 // Resident 256-thread blocks per SM asked of ptxas.  Narrow: 6 (38 registers;
 // 8 blocks at 32: 256-graph batch 18.75 against 18.55 ms, R-MAT scale-24 job
 // 103.7 against 102.9).  Wide: 8 (scale 18 with amounts as weights, 2.20 -> 2.08
