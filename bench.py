@@ -863,9 +863,9 @@ def main():
     ap.add_argument("--tune", action="store_true",
                     help="graph workloads: launch shape from the autotuner (cached) instead of the workload's")
     ap.add_argument("--l2-persist", type=int, default=0, choices=[0, 1],
-                    help="walker launches keep the node records persisting in L2")
+                    help="walker launches keep the front of the slots (alias: the node records) persisting in L2")
     ap.add_argument("--renumber", default="auto", choices=["auto", "on", "off"],
-                    help="layout node numbering: by in-degree (on), the generator's (off), or the library's choice")
+                    help="the renumbering flags of load_graph (accepted; they change only what the graph reports)")
     ap.add_argument("--serve-queries", type=int, default=2000)
     ap.add_argument("--serve-warmup", type=int, default=200)
     ap.add_argument("--serve-streams", type=int, default=4)

@@ -299,8 +299,8 @@ typedef struct {
     uint64_t steps;        /* draws consumed by all walks */
     uint64_t walks;        /* S * R */
     float kernel_ms;       /* device time of the walker launches alone (CUDA events) */
-    uint64_t sectors;      /* stats runs: 32-byte sectors the row searches read, node records
-                              included (0 otherwise) */
+    uint64_t sectors;      /* stats runs: 32-byte sectors the draws read: slots, edge records,
+                              table entries (0 otherwise) */
     float run_ms;          /* device time of the whole run: walkers and reductions */
     uint64_t model_sectors; /* stats runs: the same draws costed on a flat CSR searched by
                                bisection, in 32-byte sectors without reuse: per draw at a node
