@@ -87,8 +87,12 @@ struct __align__(16) SDesc {
 // took, so a warp with a stale view of the ring that lands on a reused slot
 // takes work of the query that holds it now (never work that no one else will
 // do).  Work taken keeps its query unfinished, and so its descriptor in place,
-// until it is done.
+// until it is done.  walks_done and agg_done count up to kCountEnd in the same
+// way: the warp whose add reaches the end knows it from what the add returns.
+// (After the add it may not look at the descriptor: another warp may have
+// finished the query in between and the host given the slot to the next one.)
 constexpr uint32_t kWordEnd = 0x80000000u;
+constexpr unsigned long long kCountEnd = 1ull << 62;
 __host__ __device__ __forceinline__ uint32_t word_left(unsigned long long w)
 {
     return (uint32_t)w < kWordEnd ? kWordEnd - (uint32_t)w : 0u;
@@ -96,8 +100,8 @@ __host__ __device__ __forceinline__ uint32_t word_left(unsigned long long w)
 struct __align__(64) SSlot {
     unsigned long long claim;       // chunks still to hand out
     unsigned long long agg;         // sources still to hand to aggregators
-    unsigned long long walks_done;  // walks finished
-    unsigned long long agg_done;    // sources reduced
+    unsigned long long walks_done;  // kCountEnd less the walks not yet finished
+    unsigned long long agg_done;    // kCountEnd less the sources not yet reduced
     unsigned long long t_claim, t_walks, t_done;  // %globaltimer: first chunk taken, last walk counted, last row
     unsigned long long pad;
 };
@@ -372,7 +376,7 @@ __device__ int claim_chunk(const LoopParams &P, uint32_t start, WalkChunk *c, un
 __device__ __forceinline__ void count_walks(const LoopParams &P, uint32_t q, uint32_t n)
 {
     const unsigned long long old = add_release(&P.slot[q].walks_done, (unsigned long long)n);
-    if (old + n == __ldcg(&P.desc[q].walks)) P.slot[q].t_walks = gtime_ns();
+    if (old + n == kCountEnd) P.slot[q].t_walks = gtime_ns();
 }
 
 constexpr uint32_t kHelpMaxR = 128;  // walker warps without walks reduce sources of queries up to this R
@@ -628,7 +632,7 @@ __device__ __forceinline__ void walker_warp(const LoopParams &P, const ClassTab 
 __device__ int await_walks(const LoopParams &P, uint32_t s)
 {
     const uint64_t t0 = gtime_ns();
-    while (__ldcg(&P.slot[s].walks_done) < __ldcg(&P.desc[s].walks)) {
+    while (__ldcg(&P.slot[s].walks_done) < kCountEnd) {
         if (gtime_ns() - t0 > kBusyWaitNs) {
             flag_exit(P, PPR_LOOP_BUSY_TIMEOUT);
             return -1;
@@ -664,10 +668,9 @@ __device__ __noinline__ int claim_source(const LoopParams &P, unsigned long long
             const uint32_t s = (uint32_t)(id % kRing);
             const unsigned long long a = __ldcg(&P.slot[s].agg);
             const unsigned long long wd = __ldcg(&P.slot[s].walks_done);
-            const uint32_t wk = __ldcg(&P.desc[s].walks);
             const int rel = tag_rel(a, id);
             const bool has = rel == 0 && word_left(a) > 0;
-            o = has && wd >= wk && __ldcg(&P.desc[s].R) <= max_R;
+            o = has && wd >= kCountEnd && __ldcg(&P.desc[s].R) <= max_R;
             left |= has;
             if (rel < 0) unwritten = (int)i;
             if (i == 0 && (rel > 0 || (rel == 0 && !has))) bump(&P.glob->agg_head, h);
@@ -762,7 +765,7 @@ __device__ void finish_source(const LoopParams &P, uint64_t id, uint32_t s, uint
     if ((threadIdx.x & 31) == 0) {
         atomicAdd(&P.glob->reduced, (unsigned long long)n);
         const unsigned long long old = atomicAdd(&P.slot[s].agg_done, (unsigned long long)n);
-        if (old + n == __ldcg(&P.desc[s].S)) {
+        if (old + n == kCountEnd) {
             P.slot[s].t_done = gtime_ns();
             __threadfence_system();
             st_release_sys(&P.ctl->done[s], id + 1);
@@ -1287,8 +1290,8 @@ static void scheduler_loop(Server *sv)
                 const unsigned long long tag = (unsigned long long)(uint32_t)(f->seq + 1) << 32;
                 c.claim = tag | (kWordEnd - d.nchunks);  // both count up to kWordEnd
                 c.agg = tag | (kWordEnd - d.S);
-                c.walks_done = 0;
-                c.agg_done = 0;
+                c.walks_done = kCountEnd - d.walks;
+                c.agg_done = kCountEnd - d.S;
                 if (e == cudaSuccess)
                     e = cudaMemcpyAsync((void *)d.src, pin, 4 * (size_t)S, cudaMemcpyHostToDevice, sv->ctl_stream);
                 // the descriptor first: a warp whose claim lands on the new counters finds it in place

@@ -1,0 +1,53 @@
+"""The serving loop's ring of 64 slots reused many times within a burst, by
+queries of every size of R that the loop's reductions tell apart (one to
+1,024: registers up to 128, shared memory above; walking warps help up to
+128).  Each answer must equal the rows of an ordinary run over its sources."""
+import threading
+
+import numpy as np
+import pytest
+
+from paper_1903_11749_gb300 import inputs as I
+from paper_1903_11749_gb300 import ppr
+
+pytestmark = pytest.mark.gpu
+
+RS = [1, 2, 31, 33, 64, 100, 128, 129, 200, 256, 257, 1000, 1024]
+
+
+@pytest.fixture(scope="module")
+def graph():
+    g = I.random_small_graph(6000, 60000, seed=51, wmax=50, dangling=60)
+    ctx = ppr.Context(0)
+    return ctx, ctx.load_graph(g.n, g.row_ptr, g.col, g.w)
+
+
+@pytest.mark.parametrize("smax,count", [(8, 600), (700, 200)])
+@pytest.mark.parametrize("sampler", [0, 1])
+def test_slots_reused_within_a_burst(graph, smax, count, sampler):
+    ctx, G = graph
+    want = {R: G.run(alpha=0.15, R=R, seed=R, topk=8, sampler=sampler).topk() for R in RS}
+    rng = np.random.default_rng(7)
+    qs = [(RS[i % len(RS)], rng.integers(0, 6000, int(rng.integers(1, smax + 1))).astype(np.int32))
+          for i in range(count)]
+    ctx.serve_start(G, max_sources=smax, max_topk=8, memory_budget=64 << 20, sampler=sampler)
+    try:
+        ids = [None] * count
+
+        def submitter(first):
+            for i in range(first, count, 2):
+                ids[i] = ctx.submit(qs[i][1], alpha=0.15, R=qs[i][0], seed=qs[i][0], topk=8)
+
+        threads = [threading.Thread(target=submitter, args=(k,)) for k in range(2)]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+        for i, (R, src) in enumerate(qs):
+            idx, cnt, _ = ctx.poll(ids[i], len(src), 8, timeout_ms=60000)
+            assert np.array_equal(idx, want[R][0][src]) and np.array_equal(cnt, want[R][1][src]), (i, R)
+        info = ctx.serve_info()
+        assert info["completed"] == count and info["in_flight"] == 0
+        assert info["reduced"] == sum(len(s) for _, s in qs)
+    finally:
+        ctx.serve_stop()
