@@ -21,7 +21,9 @@
 // and finds none to claim reduces sources too (queries of R <= 128), so the
 // end of a burst is not left to an eighth of the warps.  Every wait on the device is bounded in
 // time (%globaltimer): a loop without work exits after idle_us and the host
-// launches it again with the next query; a published slot whose descriptor
+// launches it again with the next query (walker warps stay while a published
+// query is unfinished; where they have all gone, what is in flight waits in the
+// slots for the next launch); a published slot whose descriptor
 // does not appear within a second ends the loop with an error status, which
 // fails the queries in flight.
 //
@@ -61,9 +63,10 @@ static int64_t now_ns()
 
 constexpr int kRing = 64;            // queries in flight at most (ring slots)
 constexpr int kLoopWarps = 8;        // per block: kLoopWarps - 1 walker warps, one aggregator
+constexpr int kLoopBlocks = 8;       // per SM at most
 constexpr uint32_t kLoopMaxR = 1024; // largest R the loop's reduction takes
 constexpr uint64_t kSlotWaitNs = 1000000000ull;   // bound on the wait for a published descriptor
-constexpr uint64_t kBusyWaitNs = 120000000000ull;  // bound on an aggregator waiting for walks in flight
+constexpr uint64_t kBusyWaitNs = 120000000000ull;  // bound on waiting for queries in flight without one finishing
 
 // Descriptor of a published query (device memory; the host writes it, then
 // publishes).  seq1 = the query's sequence number + 1 (0: never written).
@@ -114,13 +117,27 @@ struct SCtl {
     unsigned int status;                // device: exit reasons (PPR_LOOP_*)
 };
 
-struct SGlob {  // device memory, persists across launches of the loop
+struct __align__(32) SGlob {  // device memory, persists across launches of the loop
     unsigned long long head;      // oldest query that may still have chunks to hand out
+    unsigned long long gone;      // walker warps of this launch that have ended: the first one closes the loop
     unsigned long long agg_head;  // oldest query that may still have sources to reduce
+    unsigned long long finished;  // queries finished
     unsigned long long err;       // checked build: flags of indices that left their array
     // activity counters (ppr_serve_info)
     unsigned long long draws, iterations, claims, claim_misses, sleeps, reduced;
     unsigned long long cyc_claim, cyc_step, cyc_sleep, cyc_total;  // walker-warp clock cycles by activity
+};
+
+// Sources that a warp took of a query it may not be able to reduce (its add
+// landed on a reused slot): walks still to come, which a warp that waited
+// would keep from being walked, or an R beyond its scratch.  The block's
+// aggregator, which ends after the walker warps, reduces them once their walks
+// are done.  n = 0: none.  A block has one place a warp (the last one is the
+// aggregator's own); they are kept in device memory from one launch to the
+// next, as work taken is taken for good.
+struct Handed {
+    unsigned long long id;
+    uint32_t s, i, n;
 };
 
 struct LoopParams {
@@ -129,6 +146,7 @@ struct LoopParams {
     SSlot *slot;
     SCtl *ctl;   // device view of the host-mapped control block
     SGlob *glob;
+    Handed *handed;  // kLoopWarps places a block
     uint32_t refill;
     uint32_t walker_warps;  // in the whole grid
     uint64_t idle_ns;
@@ -291,7 +309,9 @@ __device__ __forceinline__ void take_chunk(const LoopParams &P, uint32_t s, uint
 // flight, and takes the next chunk of it with one atomic add (no retries under
 // contention).  The word's tag says which query the add landed on: if the
 // slot was reused in the meantime, the warp takes the chunk of the query that
-// now holds it.  Returns 1 (a chunk), 0 (none now), -1 (the loop must end: a
+// now holds it.  Once a walker warp has ended nothing is handed out: a query
+// published while the warps leave gets all those of the next launch, not the
+// few still here.  Returns 1 (a chunk), 0 (none now), -1 (the loop must end: a
 // published slot stayed unwritten).
 __device__ int claim_chunk(const LoopParams &P, uint32_t start, WalkChunk *c, unsigned long long *s_tail)
 {
@@ -299,7 +319,9 @@ __device__ int claim_chunk(const LoopParams &P, uint32_t start, WalkChunk *c, un
     bool refresh = false;
     for (int attempt = 0; attempt < 3; ++attempt) {
         const uint64_t t = block_tail(P, s_tail, refresh);
-        uint64_t h = __ldcg(&P.glob->head);
+        const ulonglong2 hg = __ldcg(reinterpret_cast<const ulonglong2 *>(&P.glob->head));
+        if (__shfl_sync(0xffffffffu, hg.y, 0) != 0) return 0;
+        uint64_t h = hg.x;
         if (t > kRing && h < t - kRing) h = t - kRing;  // ids below t - kRing are finished (their slots reused)
         const uint32_t n = h < t ? (uint32_t)(t - h < (uint64_t)kRing ? t - h : (uint64_t)kRing) : 0u;
         uint32_t ok[2];
@@ -381,8 +403,7 @@ __device__ __forceinline__ void count_walks(const LoopParams &P, uint32_t q, uin
 
 constexpr uint32_t kHelpMaxR = 128;  // walker warps without walks reduce sources of queries up to this R
 __device__ __noinline__ int claim_source(const LoopParams &P, unsigned long long *s_tail, bool refresh, uint32_t max_R,
-                            bool wait, uint64_t &id_out, uint32_t &slot_out, uint32_t &i_out, uint32_t &n_out,
-                            bool &in_flight);
+                            uint64_t &id_out, uint32_t &slot_out, uint32_t &i_out, uint32_t &n_out, bool &in_flight);
 __device__ __noinline__ void reduce_source(const LoopParams &P, const CallerIds &ids, uint32_t s, uint32_t i,
                                            uint32_t *smem, uint32_t cap);
 __device__ void finish_source(const LoopParams &P, uint64_t id, uint32_t s, uint32_t n);
@@ -547,31 +568,70 @@ __device__ __forceinline__ int walk_until_idle(const LoopParams &P, const ClassT
     return status < 0 ? status : (int)walked;
 }
 
-// Sources that a walker warp took of a query it may not be able to reduce (its
-// add landed on a reused slot): walks still to come, which a warp that waited
-// would keep from being walked, or an R beyond its scratch.  The block's
-// aggregator, which ends after the walker warps, reduces them.  n = 0: none.
-struct Handed {
-    unsigned long long id;
-    uint32_t s, i, n;
+// How long a warp has been without work (shared memory: the walking state
+// leaves no registers for it).
+struct WarpWait {
+    uint64_t idle_t0, busy_t0;  // since when nothing was in flight, since when no query in flight finished (0: from now)
+    unsigned long long seen;    // queries finished by busy_t0
 };
+
+// Lane 0: whether no published query has finished for kBusyWaitNs.
+__device__ __forceinline__ bool stalled(uint64_t t, unsigned long long finished, WarpWait &w)
+{
+    w.idle_t0 = 0;
+    if (w.busy_t0 == 0 || finished != w.seen) {
+        w.busy_t0 = t;
+        w.seen = finished;
+        return false;
+    }
+    return t - w.busy_t0 > kBusyWaitNs;
+}
+
+// Lane 0: whether nothing has been in flight for the loop's idle time.
+__device__ __forceinline__ bool idled(uint64_t t, uint64_t idle_ns, WarpWait &w)
+{
+    w.busy_t0 = 0;
+    if (w.idle_t0 == 0) w.idle_t0 = t;
+    return t - w.idle_t0 > idle_ns;
+}
+
+// Lane 0 of a walker warp without work: why it ends (PPR_LOOP_*), or 0.  The
+// walkers stay while a query is unfinished, so that one published meanwhile
+// finds them, and leave together; the first one looks at the host's tail itself.
+__device__ __noinline__ uint32_t walker_leaves(const LoopParams &P, WarpWait &w, unsigned long long *s_tail)
+{
+    if (ld_volatile(&P.ctl->stop)) return PPR_LOOP_STOPPED;
+    if (__ldcg(&P.glob->gone) != 0) return PPR_LOOP_IDLE;
+    const uint64_t t = gtime_ns();
+    const unsigned long long finished = __ldcg(&P.glob->finished);
+    if (finished < *(volatile unsigned long long *)&s_tail[0])
+        return stalled(t, finished, w) ? PPR_LOOP_BUSY_TIMEOUT : 0;
+    if (!idled(t, P.idle_ns, w)) return 0;
+    const unsigned long long tail = ld_tail(&P.ctl->tail);
+    if (tail == finished) return PPR_LOOP_IDLE;
+    atomicMax(&s_tail[0], tail);
+    w.idle_t0 = 0;
+    return 0;
+}
 
 // A walker warp: walks, then helps reduce, then waits (bounded) for the next query.
 template <class E>
 __device__ __forceinline__ void walker_warp(const LoopParams &P, const ClassTab &tab, const CallerIds &ids, WalkChunk &wc,
-                                            uint32_t **ends_of, uint32_t *scratch, WarpActivity &act, Handed &handed,
-                                            uint32_t gwarp, unsigned long long *s_tail)
+                                            uint32_t **ends_of, uint32_t *scratch, WarpActivity &act, WarpWait &wait,
+                                            Handed &handed, uint32_t gwarp, unsigned long long *s_tail)
 {
     const uint32_t lane = threadIdx.x & 31;
-    if (lane == 0) act = WarpActivity{clock64(), 0, 0, 0, 0, 0};
+    if (lane == 0) {
+        act = WarpActivity{clock64(), 0, 0, 0, 0, 0};
+        wait = WarpWait{0, 0, 0};
+    }
     __syncwarp();
-    uint64_t idle_t0 = 0;
     uint32_t backoff = 256;
     for (;;) {
         const int walked = walk_until_idle<E>(P, tab, wc, ends_of, gwarp, s_tail, act);
         if (walked < 0) break;
         if (walked) {
-            idle_t0 = 0;
+            if (lane == 0) wait = WarpWait{0, 0, 0};
             backoff = 256;
         }
         uint64_t id = 0;
@@ -579,7 +639,7 @@ __device__ __forceinline__ void walker_warp(const LoopParams &P, const ClassTab 
         bool in_flight = false;
         int r = 0;
         if (__shfl_sync(0xffffffffu, lane == 0 ? *(volatile uint32_t *)&handed.n : 0u, 0) == 0)
-            r = claim_source(P, s_tail, false, kHelpMaxR, false, id, s, i, nb, in_flight);
+            r = claim_source(P, s_tail, false, kHelpMaxR, id, s, i, nb, in_flight);
         if (r < 0) break;
         if (r == 2) {  // of another query than it looked at: left to the aggregator
             if (lane == 0) {
@@ -595,20 +655,13 @@ __device__ __forceinline__ void walker_warp(const LoopParams &P, const ClassTab 
         if (r > 0) {
             for (uint32_t b = 0; b < nb; ++b) reduce_source(P, ids, s, i + b, scratch, kHelpMaxR);
             finish_source(P, id, s, nb);
-            idle_t0 = 0;
+            if (lane == 0) wait = WarpWait{0, 0, 0};
             backoff = 256;
             continue;
         }
-        if (ld_volatile(&P.ctl->stop)) {
-            if (lane == 0) flag_exit(P, PPR_LOOP_STOPPED);
-            break;
-        }
-        const uint64_t t = gtime_ns();
-        if (idle_t0 == 0) idle_t0 = t;
-        else if (t - idle_t0 > P.idle_ns) {
-            if (lane == 0) flag_exit(P, PPR_LOOP_IDLE);
-            break;
-        }
+        uint32_t why = 0;
+        if (lane == 0 && (why = walker_leaves(P, wait, s_tail)) != 0) flag_exit(P, why);
+        if (__shfl_sync(0xffffffffu, why, 0)) break;
         if (in_flight) backoff = min(backoff, 1024u);  // other warps' walks are about to end: their sources come next
         const long long c0 = clock64();
         __nanosleep(backoff);
@@ -628,29 +681,14 @@ __device__ __forceinline__ void walker_warp(const LoopParams &P, const ClassTab 
     }
 }
 
-// Lane 0: waits (bounded) until the walks of the query in slot s are done.
-__device__ int await_walks(const LoopParams &P, uint32_t s)
-{
-    const uint64_t t0 = gtime_ns();
-    while (__ldcg(&P.slot[s].walks_done) < kCountEnd) {
-        if (gtime_ns() - t0 > kBusyWaitNs) {
-            flag_exit(P, PPR_LOOP_BUSY_TIMEOUT);
-            return -1;
-        }
-        __nanosleep(1000);
-    }
-    return 1;
-}
-
 // Whole warp: hands out a few sources of the oldest query of R <= max_R whose
 // walks are all done.  Returns 1 (query id, slot, sources from i on, on every
 // lane), 0 (none now), -1 (the loop must end); *in_flight tells whether
 // published queries still have sources to hand out (ready or not).  An add
 // that lands on a reused slot takes sources of a query of any R whose walks may
-// still run: with wait the warp waits for them (bounded), else it gets 2.
+// still run: 2.
 __device__ __noinline__ int claim_source(const LoopParams &P, unsigned long long *s_tail, bool refresh, uint32_t max_R,
-                            bool wait, uint64_t &id_out, uint32_t &slot_out, uint32_t &i_out, uint32_t &n_out,
-                            bool &in_flight)
+                            uint64_t &id_out, uint32_t &slot_out, uint32_t &i_out, uint32_t &n_out, bool &in_flight)
 {
     const uint32_t lane = threadIdx.x & 31;
     const uint64_t t = block_tail(P, s_tail, refresh);
@@ -709,7 +747,7 @@ __device__ __noinline__ int claim_source(const LoopParams &P, unsigned long long
                     got = 1;
                     if (tag != (uint32_t)(h + i + 1)) {
                         got = await_desc(P, d, tag);
-                        if (got > 0) got = wait ? await_walks(P, s) : 2;
+                        if (got > 0) got = 2;
                     }
                     src_i = __ldcg(&d->S) - have;
                 }
@@ -767,6 +805,7 @@ __device__ void finish_source(const LoopParams &P, uint64_t id, uint32_t s, uint
         const unsigned long long old = atomicAdd(&P.slot[s].agg_done, (unsigned long long)n);
         if (old + n == kCountEnd) {
             P.slot[s].t_done = gtime_ns();
+            atomicAdd(&P.glob->finished, 1ull);
             __threadfence_system();
             st_release_sys(&P.ctl->done[s], id + 1);
         }
@@ -776,8 +815,8 @@ __device__ void finish_source(const LoopParams &P, uint64_t id, uint32_t s, uint
 __device__ void aggregator_warp(const LoopParams &P, const CallerIds &ids, uint32_t *smem, Handed *handed,
                                 const uint32_t *walkers, unsigned long long *s_tail)
 {
-    const uint32_t lane = threadIdx.x & 31;
-    uint64_t idle_t0 = 0, busy_t0 = 0;
+    const uint32_t lane = threadIdx.x & 31, place = min(lane, (uint32_t)kLoopWarps - 1);
+    WarpWait wait{0, 0, 0};
     uint32_t backoff = 256;
     bool refresh = true;
     for (;;) {
@@ -785,62 +824,69 @@ __device__ void aggregator_warp(const LoopParams &P, const CallerIds &ids, uint3
         uint32_t s = 0, i = 0, nb = 0;
         bool in_flight = false;
         int r = 0;
-        // sources handed over by the block's walker warps come first; none
-        // follow once those have ended (read before the places)
+        // Read before anything is looked at: once the block's walker warps have
+        // ended none of them hands sources over, and once those of the whole
+        // grid have (gone), no walk that is not done yet will be.
         const uint32_t left = __shfl_sync(0xffffffffu, lane == 0 ? *(const volatile uint32_t *)walkers : 0u, 0);
+        const bool gone =
+            left == 0 && __shfl_sync(0xffffffffu, __ldcg(&P.glob->gone), 0) >= (unsigned long long)P.walker_warps;
+        __threadfence();
+        // sources handed over come first, as soon as their walks are done
+        const volatile Handed *h = handed + place;
+        const bool held = lane < kLoopWarps && h->n != 0;
         __threadfence_block();
-        const uint32_t hm = __ballot_sync(
-            0xffffffffu, lane < kLoopWarps - 1 && *(volatile uint32_t *)&handed[lane < kLoopWarps - 1 ? lane : 0].n != 0);
-        if (hm) {
-            __threadfence_block();
-            volatile Handed *h = handed + (__ffs(hm) - 1);
+        const bool ready = held && __ldcg(&P.slot[h->s].walks_done) >= kCountEnd;
+        const uint32_t hm = __ballot_sync(0xffffffffu, held), rm = __ballot_sync(0xffffffffu, ready);
+        if (rm) {
+            h = handed + (__ffs(rm) - 1);
             id = h->id;
             s = h->s;
             i = h->i;
             nb = h->n;
             __syncwarp();
-            if (lane == 0) {
-                r = await_walks(P, s);
-                h->n = 0;
+            if (lane == 0) *(volatile uint32_t *)&handed[__ffs(rm) - 1].n = 0;
+            __syncwarp();
+            r = 1;
+        } else if (!((hm >> (kLoopWarps - 1)) & 1u)) {
+            r = claim_source(P, s_tail, refresh, kLoopMaxR, id, s, i, nb, in_flight);
+            if (r == 2) {
+                if (lane == 0) handed[kLoopWarps - 1] = Handed{id, s, i, nb};
+                __syncwarp();
+                continue;
             }
-            r = __shfl_sync(0xffffffffu, r, 0);
-        } else {
-            r = claim_source(P, s_tail, refresh, kLoopMaxR, true, id, s, i, nb, in_flight);
         }
         if (r < 0) break;
         if (r > 0) {
             for (uint32_t b = 0; b < nb; ++b) reduce_source(P, ids, s, i + b, smem, kLoopMaxR);
             finish_source(P, id, s, nb);
-            idle_t0 = busy_t0 = 0;
+            wait = WarpWait{0, 0, 0};
             backoff = 256;
             refresh = false;
             continue;
         }
         refresh = true;
-        const uint64_t t = gtime_ns();
-        if (!in_flight) {  // nothing published is left to reduce
-            busy_t0 = 0;
-            if (left == 0 && ld_volatile(&P.ctl->stop)) {
-                if (lane == 0) flag_exit(P, PPR_LOOP_STOPPED);
-                break;
+        uint32_t why = 0;
+        if (lane == 0) {
+            const uint64_t t = gtime_ns();
+            if (!in_flight && !hm) {  // nothing published is left to reduce
+                const bool idle = idled(t, P.idle_ns, wait);
+                if (left == 0 && ld_volatile(&P.ctl->stop)) why = PPR_LOOP_STOPPED;
+                else if (left == 0 && (gone || idle)) why = PPR_LOOP_IDLE;
+            } else if (gone) {  // no warp is left to walk what is in flight: the next launch does
+                why = PPR_LOOP_IDLE;
+            } else if (stalled(t, __ldcg(&P.glob->finished), wait)) {
+                why = PPR_LOOP_BUSY_TIMEOUT;
+            } else {
+                why = ld_volatile(&P.ctl->status) & (PPR_LOOP_SLOT_TIMEOUT | PPR_LOOP_BUSY_TIMEOUT);
             }
-            if (idle_t0 == 0) idle_t0 = t;
-            else if (left == 0 && t - idle_t0 > P.idle_ns) {
-                if (lane == 0) flag_exit(P, PPR_LOOP_IDLE);
-                break;
-            }
-        } else {  // queries whose walks are still running: wait for them (bounded)
-            idle_t0 = 0;
-            if (busy_t0 == 0) busy_t0 = t;
-            else if (t - busy_t0 > kBusyWaitNs) {
-                if (lane == 0) flag_exit(P, PPR_LOOP_BUSY_TIMEOUT);
-                break;
-            }
-            if (ld_volatile(&P.ctl->status) & (PPR_LOOP_SLOT_TIMEOUT | PPR_LOOP_BUSY_TIMEOUT)) break;
+            if (why) flag_exit(P, why);
         }
+        if (__shfl_sync(0xffffffffu, why, 0)) break;
         __nanosleep(backoff);
         backoff = min(backoff * 2, 4096u);
     }
+    __syncwarp();
+    if (lane < kLoopWarps) P.handed[(uint64_t)blockIdx.x * kLoopWarps + lane] = handed[lane];
 }
 
 template <class E>
@@ -851,13 +897,14 @@ __global__ void __launch_bounds__(32 * kLoopWarps, 4) k_serve_loop(const __grid_
     __shared__ __align__(16) uint32_t smem[kLoopMaxR + 3 * kLoopMaxR];  // the aggregator warp's endpoints and scratch
     __shared__ __align__(16) uint32_t help[kLoopWarps - 1][2 * kHelpMaxR + 32];  // a helping warp's endpoints and scratch
     __shared__ WarpActivity act[kLoopWarps - 1];
-    __shared__ Handed handed[kLoopWarps - 1];
+    __shared__ WarpWait wait[kLoopWarps - 1];
+    __shared__ Handed handed[kLoopWarps];
     __shared__ uint32_t walkers;  // walker warps of the block that have not ended
     __shared__ unsigned long long s_tail[2];  // the block's copy of the published tail, and when it was read
     __shared__ ClassTab tab;
     __shared__ uint32_t s_first[kTabEntries];
     for (uint32_t i = threadIdx.x; i < kTabEntries; i += blockDim.x) s_first[i] = P.kp.tab->e[i].first;
-    if (threadIdx.x < kLoopWarps - 1) handed[threadIdx.x].n = 0;
+    if (threadIdx.x < kLoopWarps) handed[threadIdx.x] = P.handed[(uint64_t)blockIdx.x * kLoopWarps + threadIdx.x];
     if (threadIdx.x == 0) {
         s_tail[0] = s_tail[1] = 0;
         walkers = kLoopWarps - 1;
@@ -868,11 +915,15 @@ __global__ void __launch_bounds__(32 * kLoopWarps, 4) k_serve_loop(const __grid_
         aggregator_warp(P, CallerIds{P.kp.order, s_first}, smem, handed, &walkers, s_tail);
         return;
     }
-    walker_warp<E>(P, tab, CallerIds{P.kp.order, s_first}, wc[wid], ends_of, help[wid], act[wid], handed[wid],
+    walker_warp<E>(P, tab, CallerIds{P.kp.order, s_first}, wc[wid], ends_of, help[wid], act[wid], wait[wid], handed[wid],
                    blockIdx.x * (kLoopWarps - 1) + wid, s_tail);
     __syncwarp();
-    __threadfence_block();
-    if ((threadIdx.x & 31) == 0) atomicSub(&walkers, 1u);
+    __threadfence();  // its walks are counted and what it handed over is in place
+    if ((threadIdx.x & 31) == 0) {
+        atomicAdd(&P.glob->gone, 1ull);
+        __threadfence();
+        atomicSub(&walkers, 1u);
+    }
 }
 
 // ============================================================ queries ====
@@ -974,6 +1025,7 @@ struct Server {
     SDesc *d_desc = nullptr, *h_desc = nullptr;
     SSlot *d_slot = nullptr, *h_slot = nullptr;
     SGlob *d_glob = nullptr;
+    Handed *d_handed = nullptr;
     unsigned char *arena = nullptr;  // device
     unsigned char *pin = nullptr;    // pinned, mapped
     size_t pin_size = 0;
@@ -1127,14 +1179,16 @@ static int launch_loop_typed(Server *sv)
     P.slot = sv->d_slot;
     P.ctl = sv->ctl_dev;
     P.glob = sv->d_glob;
+    P.handed = sv->d_handed;
     P.refill = sv->cfg.refill_lanes > 0 ? (uint32_t)std::min(sv->cfg.refill_lanes, 32) : kDefaultRefill;
     P.idle_ns = (uint64_t)(sv->cfg.idle_us > 0 ? sv->cfg.idle_us : 200000) * 1000ull;
     if (!sv->grid) {
         int per_sm = 0;
         PPR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_serve_loop<E>, 32 * kLoopWarps, 0));
-        sv->grid = (uint32_t)(sv->ctx->sms * std::max(per_sm, 1));
+        sv->grid = (uint32_t)(sv->ctx->sms * std::min(std::max(per_sm, 1), kLoopBlocks));
     }
     P.walker_warps = sv->grid * (kLoopWarps - 1);
+    PPR_CUDA(cudaMemsetAsync(&sv->d_glob->gone, 0, sizeof(sv->d_glob->gone), sv->loop_stream));
     k_serve_loop<E><<<sv->grid, 32 * kLoopWarps, 0, sv->loop_stream>>>(P);
     note_launch();
     PPR_CUDA(cudaGetLastError());
@@ -1351,6 +1405,7 @@ static void free_loop(Server *sv)
     cudaFree(sv->d_desc);
     cudaFree(sv->d_slot);
     cudaFree(sv->d_glob);
+    cudaFree(sv->d_handed);
     if (sv->pin) cudaFreeHost(sv->pin);
     if (sv->ctl) cudaFreeHost(sv->ctl);
     if (sv->h_desc) cudaFreeHost(sv->h_desc);
@@ -1374,6 +1429,8 @@ static int start_loop(Server *sv)
     if (e == cudaSuccess) e = cudaMalloc((void **)&sv->d_desc, sizeof(SDesc) * kRing);
     if (e == cudaSuccess) e = cudaMalloc((void **)&sv->d_slot, sizeof(SSlot) * kRing);
     if (e == cudaSuccess) e = cudaMalloc((void **)&sv->d_glob, sizeof(SGlob));
+    const size_t handed_bytes = sizeof(Handed) * sv->ctx->sms * kLoopBlocks * kLoopWarps;
+    if (e == cudaSuccess) e = cudaMalloc((void **)&sv->d_handed, handed_bytes);
     if (e == cudaSuccess) e = cudaMalloc((void **)&sv->arena, sv->budget);
     // pinned output: room for several of the largest queries
     sv->pin_size = std::max<size_t>(64ull << 20, 4 * loop_pin_bytes(cfg.max_sources, cfg.max_topk));
@@ -1381,6 +1438,7 @@ static int start_loop(Server *sv)
     if (e == cudaSuccess) e = cudaMemsetAsync(sv->d_desc, 0, sizeof(SDesc) * kRing, sv->ctl_stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(sv->d_slot, 0, sizeof(SSlot) * kRing, sv->ctl_stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(sv->d_glob, 0, sizeof(SGlob), sv->ctl_stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(sv->d_handed, 0, handed_bytes, sv->ctl_stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(sv->ctl_stream);
     if (e != cudaSuccess) {
         const int rc = cuda_fail(e, "serving set-up");

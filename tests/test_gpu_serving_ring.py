@@ -51,3 +51,36 @@ def test_slots_reused_within_a_burst(graph, smax, count, sampler):
         assert info["reduced"] == sum(len(s) for _, s in qs)
     finally:
         ctx.serve_stop()
+
+
+def test_queries_published_while_the_walkers_leave(graph):
+    """With an idle time of a microsecond the loop ends at once whenever nothing
+    is in flight.  Queries that arrive while an earlier one is still being
+    reduced (R above what walking warps help with, so they have nothing to do)
+    or just as the warps leave are walked all the same, here or by the next
+    launch; none waits for the bound on queries in flight."""
+    import time
+    ctx, G = graph
+    want = {R: G.run(alpha=0.15, R=R, seed=R, topk=8).topk() for R in (40, 1000)}
+    rng = np.random.default_rng(3)
+    ctx.serve_start(G, max_sources=6000, max_topk=8, memory_budget=256 << 20, idle_us=1)
+    try:
+        for delay in np.linspace(0, 6e-3, 40):
+            work = []
+            for R, ns, pause in ((1000, 6000, delay), (40, 50, delay / 7), (40, 3, 0)):
+                src = rng.integers(0, 6000, ns).astype(np.int32)
+                work.append((R, src, ctx.submit(src, alpha=0.15, R=R, seed=R, topk=8)))
+                time.sleep(pause)
+            for R, src, q in work:
+                idx, cnt, _ = ctx.poll(q, len(src), 8, timeout_ms=20000)
+                assert np.array_equal(idx, want[R][0][src]) and np.array_equal(cnt, want[R][1][src])
+        for i in range(400):  # one small query at a time, at any moment of the loop's end
+            src = rng.integers(0, 6000, 3).astype(np.int32)
+            q = ctx.submit(src, alpha=0.15, R=40, seed=40, topk=8)
+            idx, cnt, _ = ctx.poll(q, 3, 8, timeout_ms=20000)
+            assert np.array_equal(idx, want[40][0][src]) and np.array_equal(cnt, want[40][1][src])
+            time.sleep((i % 50) * 2e-6)
+        info = ctx.serve_info()
+        assert info["launches"] > 1 and info["in_flight"] == 0
+    finally:
+        ctx.serve_stop()
