@@ -78,7 +78,8 @@ struct __align__(16) SDesc {
     uint64_t r_magic;     // ceil(2^40 / R): g / R by multiply-shift (exact for g < 2^40 / R)
     uint64_t seq1;
     uint32_t S, R, T, k0, k1, topk, cw, nchunks, walks, P2;
-    uint32_t pad[2];
+    uint32_t help;        // walker warps without walks reduce its sources too
+    uint32_t pad;
 };
 
 // Counters of a ring slot (device memory; the host writes them before
@@ -120,8 +121,9 @@ struct SCtl {
 struct __align__(32) SGlob {  // device memory, persists across launches of the loop
     unsigned long long head;      // oldest query that may still have chunks to hand out
     unsigned long long gone;      // walker warps of this launch that have ended: the first one closes the loop
-    unsigned long long agg_head;  // oldest query that may still have sources to reduce
     unsigned long long finished;  // queries finished
+    unsigned long long ready;     // queries whose walks are all done, of those that walker warps help reduce
+    unsigned long long agg_head;  // oldest query that may still have sources to reduce
     unsigned long long err;       // checked build: flags of indices that left their array
     // activity counters (ppr_serve_info)
     unsigned long long draws, iterations, claims, claim_misses, sleeps, reduced;
@@ -398,7 +400,11 @@ __device__ int claim_chunk(const LoopParams &P, uint32_t start, WalkChunk *c, un
 __device__ __forceinline__ void count_walks(const LoopParams &P, uint32_t q, uint32_t n)
 {
     const unsigned long long old = add_release(&P.slot[q].walks_done, (unsigned long long)n);
-    if (old + n == kCountEnd) P.slot[q].t_walks = gtime_ns();
+    if (old + n == kCountEnd) {
+        P.slot[q].t_walks = gtime_ns();
+        // (a hint: held up here, it may be the successor's)
+        if (__ldcg(&P.desc[q].help)) atomicAdd(&P.glob->ready, 1ull);
+    }
 }
 
 constexpr uint32_t kHelpMaxR = 128;  // walker warps without walks reduce sources of queries up to this R
@@ -573,7 +579,14 @@ __device__ __forceinline__ int walk_until_idle(const LoopParams &P, const ClassT
 struct WarpWait {
     uint64_t idle_t0, busy_t0;  // since when nothing was in flight, since when no query in flight finished (0: from now)
     unsigned long long seen;    // queries finished by busy_t0
+    unsigned long long looked;  // queries ready to reduce when a look found no source left
+    uint32_t backoff;           // ns of the next sleep
 };
+__device__ __forceinline__ void worked(WarpWait &w)
+{
+    w.idle_t0 = w.busy_t0 = 0;
+    w.backoff = 256;
+}
 
 // Lane 0: whether no published query has finished for kBusyWaitNs.
 __device__ __forceinline__ bool stalled(uint64_t t, unsigned long long finished, WarpWait &w)
@@ -623,23 +636,31 @@ __device__ __forceinline__ void walker_warp(const LoopParams &P, const ClassTab 
     const uint32_t lane = threadIdx.x & 31;
     if (lane == 0) {
         act = WarpActivity{clock64(), 0, 0, 0, 0, 0};
-        wait = WarpWait{0, 0, 0};
+        wait.looked = 0;
+        worked(wait);
     }
     __syncwarp();
-    uint32_t backoff = 256;
     for (;;) {
         const int walked = walk_until_idle<E>(P, tab, wc, ends_of, gwarp, s_tail, act);
         if (walked < 0) break;
-        if (walked) {
-            if (lane == 0) wait = WarpWait{0, 0, 0};
-            backoff = 256;
-        }
+        if (walked && lane == 0) worked(wait);
+        // A look for sources reads three words of every slot in view: with one
+        // a microsecond and warp while a query was in flight the warps without
+        // work held up the others' reads and counts (8 queries of up to 3,000
+        // sources, R 50: 1,650 us, now 620; 64 of up to 20,000, R 100: 4,960,
+        // now 4,780).  So a warp looks only when the count of ready queries has
+        // moved since its last, and sleeps longer and longer between.
         uint64_t id = 0;
         uint32_t s = 0, i = 0, nb = 0;
         bool in_flight = false;
         int r = 0;
-        if (__shfl_sync(0xffffffffu, lane == 0 ? *(volatile uint32_t *)&handed.n : 0u, 0) == 0)
-            r = claim_source(P, s_tail, false, kHelpMaxR, id, s, i, nb, in_flight);
+        unsigned long long ready = 0;
+        bool look = false;
+        if (lane == 0) {
+            ready = __ldcg(&P.glob->ready);
+            look = ready != wait.looked && *(volatile uint32_t *)&handed.n == 0;
+        }
+        if (__shfl_sync(0xffffffffu, look, 0)) r = claim_source(P, s_tail, false, kHelpMaxR, id, s, i, nb, in_flight);
         if (r < 0) break;
         if (r == 2) {  // of another query than it looked at: left to the aggregator
             if (lane == 0) {
@@ -655,21 +676,21 @@ __device__ __forceinline__ void walker_warp(const LoopParams &P, const ClassTab 
         if (r > 0) {
             for (uint32_t b = 0; b < nb; ++b) reduce_source(P, ids, s, i + b, scratch, kHelpMaxR);
             finish_source(P, id, s, nb);
-            if (lane == 0) wait = WarpWait{0, 0, 0};
-            backoff = 256;
+            if (lane == 0) worked(wait);
             continue;
         }
+        if (look) wait.looked = ready;  // (lane 0)
         uint32_t why = 0;
         if (lane == 0 && (why = walker_leaves(P, wait, s_tail)) != 0) flag_exit(P, why);
         if (__shfl_sync(0xffffffffu, why, 0)) break;
-        if (in_flight) backoff = min(backoff, 1024u);  // other warps' walks are about to end: their sources come next
-        const long long c0 = clock64();
-        __nanosleep(backoff);
         if (lane == 0) {
+            const long long c0 = clock64();
+            __nanosleep(wait.backoff);
+            wait.backoff = min(wait.backoff * 2, 32768u);
             ++act.n_sleep;
             act.c_sleep += clock64() - c0;
         }
-        backoff = min(backoff * 2, 32768u);
+        __syncwarp();
     }
     if (lane == 0) {  // what is not flushed yet
         atomicAdd(&P.glob->claims, (unsigned long long)act.n_claim);
@@ -816,8 +837,8 @@ __device__ void aggregator_warp(const LoopParams &P, const CallerIds &ids, uint3
                                 const uint32_t *walkers, unsigned long long *s_tail)
 {
     const uint32_t lane = threadIdx.x & 31, place = min(lane, (uint32_t)kLoopWarps - 1);
-    WarpWait wait{0, 0, 0};
-    uint32_t backoff = 256;
+    WarpWait wait;
+    worked(wait);
     bool refresh = true;
     for (;;) {
         uint64_t id = 0;
@@ -859,8 +880,7 @@ __device__ void aggregator_warp(const LoopParams &P, const CallerIds &ids, uint3
         if (r > 0) {
             for (uint32_t b = 0; b < nb; ++b) reduce_source(P, ids, s, i + b, smem, kLoopMaxR);
             finish_source(P, id, s, nb);
-            wait = WarpWait{0, 0, 0};
-            backoff = 256;
+            worked(wait);
             refresh = false;
             continue;
         }
@@ -882,8 +902,8 @@ __device__ void aggregator_warp(const LoopParams &P, const CallerIds &ids, uint3
             if (why) flag_exit(P, why);
         }
         if (__shfl_sync(0xffffffffu, why, 0)) break;
-        __nanosleep(backoff);
-        backoff = min(backoff * 2, 4096u);
+        __nanosleep(wait.backoff);
+        wait.backoff = min(wait.backoff * 2, 4096u);
     }
     __syncwarp();
     if (lane < kLoopWarps) P.handed[(uint64_t)blockIdx.x * kLoopWarps + lane] = handed[lane];
@@ -1329,6 +1349,8 @@ static void scheduler_loop(Server *sv)
                 uint32_t P2 = 1;
                 while (P2 < R) P2 <<= 1;
                 d.P2 = P2;
+                // up to one source an aggregator is taken by those at once
+                d.help = R <= kHelpMaxR && d.S > sv->grid ? 1u : 0u;
                 // Walks per chunk: about two chunks per walker warp for a query
                 // alone; with others in flight about as many for all together, as
                 // long as the query still has 64 (a claim is two trips to L2 under

@@ -84,3 +84,29 @@ def test_queries_published_while_the_walkers_leave(graph):
         assert info["launches"] > 1 and info["in_flight"] == 0
     finally:
         ctx.serve_stop()
+
+
+def test_warps_without_work_sleep(graph):
+    """While a few warps walk one query for a long time, those without work
+    sleep most of the time (up to 33 us between looks that take a few), so
+    that they do not stand in the way of the query's reads and counts."""
+    import time
+    ctx, G = graph
+
+    def ended():
+        deadline = time.time() + 20
+        while ctx.serve_info()["running"] and time.time() < deadline:
+            time.sleep(0.005)
+        return ctx.serve_info()
+
+    ctx.serve_start(G, max_sources=8, max_topk=8, memory_budget=64 << 20, idle_us=10_000)
+    try:
+        before = ended()
+        # 1,024 walks (32 warps' worth) of 20,000 steps on average
+        q = ctx.submit(np.array([5], np.int32), alpha=5e-5, R=1024, seed=1, topk=8)
+        ctx.poll(q, 1, 8, timeout_ms=60000)
+        after = ended()
+        slept = after["cycles_sleep"] - before["cycles_sleep"]
+        assert slept > 0.5 * (after["cycles_total"] - before["cycles_total"])
+    finally:
+        ctx.serve_stop()
