@@ -408,7 +408,7 @@ __device__ __forceinline__ void count_walks(const LoopParams &P, uint32_t q, uin
 }
 
 constexpr uint32_t kHelpMaxR = 128;  // walker warps without walks reduce sources of queries up to this R
-__device__ __noinline__ int claim_source(const LoopParams &P, unsigned long long *s_tail, bool refresh, uint32_t max_R,
+__device__ __noinline__ int claim_source(const LoopParams &P, uint32_t start, unsigned long long *s_tail, bool refresh, uint32_t max_R,
                             uint64_t &id_out, uint32_t &slot_out, uint32_t &i_out, uint32_t &n_out, bool &in_flight);
 __device__ __noinline__ void reduce_source(const LoopParams &P, const CallerIds &ids, uint32_t s, uint32_t i,
                                            uint32_t *smem, uint32_t cap);
@@ -660,7 +660,7 @@ __device__ __forceinline__ void walker_warp(const LoopParams &P, const ClassTab 
             ready = __ldcg(&P.glob->ready);
             look = ready != wait.looked && *(volatile uint32_t *)&handed.n == 0;
         }
-        if (__shfl_sync(0xffffffffu, look, 0)) r = claim_source(P, s_tail, false, kHelpMaxR, id, s, i, nb, in_flight);
+        if (__shfl_sync(0xffffffffu, look, 0)) r = claim_source(P, gwarp, s_tail, false, kHelpMaxR, id, s, i, nb, in_flight);
         if (r < 0) break;
         if (r == 2) {  // of another query than it looked at: left to the aggregator
             if (lane == 0) {
@@ -702,13 +702,13 @@ __device__ __forceinline__ void walker_warp(const LoopParams &P, const ClassTab 
     }
 }
 
-// Whole warp: hands out a few sources of the oldest query of R <= max_R whose
-// walks are all done.  Returns 1 (query id, slot, sources from i on, on every
+// Whole warp: hands out a few sources of a query of R <= max_R whose walks are
+// all done.  Returns 1 (query id, slot, sources from i on, on every
 // lane), 0 (none now), -1 (the loop must end); *in_flight tells whether
 // published queries still have sources to hand out (ready or not).  An add
 // that lands on a reused slot takes sources of a query of any R whose walks may
 // still run: 2.
-__device__ __noinline__ int claim_source(const LoopParams &P, unsigned long long *s_tail, bool refresh, uint32_t max_R,
+__device__ __noinline__ int claim_source(const LoopParams &P, uint32_t start, unsigned long long *s_tail, bool refresh, uint32_t max_R,
                             uint64_t &id_out, uint32_t &slot_out, uint32_t &i_out, uint32_t &n_out, bool &in_flight)
 {
     const uint32_t lane = threadIdx.x & 31;
@@ -716,7 +716,8 @@ __device__ __noinline__ int claim_source(const LoopParams &P, unsigned long long
     uint64_t h = __ldcg(&P.glob->agg_head);
     if (t > kRing && h < t - kRing) h = t - kRing;
     const uint32_t n = h < t ? (uint32_t)(t - h < (uint64_t)kRing ? t - h : (uint64_t)kRing) : 0u;
-    uint32_t ready[2], left = 0;
+    uint32_t left = 0;
+    unsigned long long ready = 0;
     int unwritten = -1;
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
@@ -734,7 +735,7 @@ __device__ __noinline__ int claim_source(const LoopParams &P, unsigned long long
             if (rel < 0) unwritten = (int)i;
             if (i == 0 && (rel > 0 || (rel == 0 && !has))) bump(&P.glob->agg_head, h);
         }
-        ready[r] = __ballot_sync(0xffffffffu, o);
+        ready |= (unsigned long long)__ballot_sync(0xffffffffu, o) << (32 * r);
     }
     in_flight = __ballot_sync(0xffffffffu, left) != 0;
     const uint32_t um = __ballot_sync(0xffffffffu, unwritten >= 0);
@@ -744,10 +745,18 @@ __device__ __noinline__ int claim_source(const LoopParams &P, unsigned long long
         if (lane == 0) r = await_slot(P, &P.slot[(h + ui) % kRing].agg, h + ui);
         return __shfl_sync(0xffffffffu, r, 0) < 0 ? -1 : 0;
     }
-    for (int r = 0; r < 2; ++r) {
-        uint32_t m = ready[r];
-        while (m) {  // oldest ready query first
-            const uint32_t i = r * 32 + __ffs(m) - 1;
+    // Every other warp takes of the oldest ready query, the rest share themselves
+    // out over all of them.  With the oldest first for all, small queries wait
+    // for the reductions of large ones published before them (64 queries of up
+    // to 20,000 sources, R 200: half of them answered within 5.6 ms, now .74);
+    // with all shared out, large ones finish together and the host copies
+    // nothing meanwhile (the whole burst 14.1 ms, now 12.7, oldest first 12.3).
+    unsigned long long m = ready;
+    for (uint32_t k = m && (start & 1) ? (start >> 1) % (uint32_t)__popcll(m) : 0u; k > 0; --k) m &= m - 1;
+    const unsigned long long before = ready ^ m;
+    for (int pass = 0; pass < 2; ++pass, m = before) {
+        while (m) {
+            const uint32_t i = __ffsll((long long)m) - 1;
             m &= m - 1;
             int got = 0;
             uint32_t src_i = 0, take = 0, slot = 0;
@@ -869,7 +878,7 @@ __device__ void aggregator_warp(const LoopParams &P, const CallerIds &ids, uint3
             __syncwarp();
             r = 1;
         } else if (!((hm >> (kLoopWarps - 1)) & 1u)) {
-            r = claim_source(P, s_tail, refresh, kLoopMaxR, id, s, i, nb, in_flight);
+            r = claim_source(P, blockIdx.x, s_tail, refresh, kLoopMaxR, id, s, i, nb, in_flight);
             if (r == 2) {
                 if (lane == 0) handed[kLoopWarps - 1] = Handed{id, s, i, nb};
                 __syncwarp();

@@ -110,3 +110,28 @@ def test_warps_without_work_sleep(graph):
         assert slept > 0.5 * (after["cycles_total"] - before["cycles_total"])
     finally:
         ctx.serve_stop()
+
+
+def test_a_small_query_does_not_wait_for_the_reductions_of_large_ones(graph):
+    """Eight queries of 6,000 sources with R 1,000 leave tens of milliseconds of
+    reductions; a query of three sources published when the first of them is
+    done is answered in well under half of what is left of that."""
+    ctx, G = graph
+    want = G.run(alpha=0.15, R=1000, seed=1, topk=8).topk()
+    large, small = np.arange(6000, dtype=np.int32), np.array([5, 17, 4000], np.int32)
+    ctx.serve_start(G, max_sources=6000, max_topk=8, memory_budget=512 << 20)
+    try:
+        for _ in range(2):  # (the first time warms up)
+            ids = [ctx.submit(large, alpha=0.15, R=1000, seed=1, topk=8) for _ in range(8)]
+            got = [ctx.poll(ids[0], 6000, 8, timeout_ms=60000)]
+            q = ctx.submit(small, alpha=0.15, R=1000, seed=1, topk=8)
+            idx, cnt, st = ctx.poll(q, 3, 8, timeout_ms=60000)
+            got += [ctx.poll(i, 6000, 8, timeout_ms=60000) for i in ids[1:]]
+        assert np.array_equal(idx, want[0][small]) and np.array_equal(cnt, want[1][small])
+        for a, b, _ in got:
+            assert np.array_equal(a, want[0]) and np.array_equal(b, want[1])
+        last = max(s["done_ns"] for _, _, s in got)
+        assert last > st["submit_ns"]
+        assert st["done_ns"] - st["submit_ns"] < 0.5 * (last - st["submit_ns"])
+    finally:
+        ctx.serve_stop()
