@@ -1,6 +1,7 @@
 // api.cu -- the extern "C" entry points of libppr.so (declared in
 // include/ppr.h): argument checks, ownership of device state, batching of a
 // source range into device-sized launches, and the row/top-k/dense readers.
+#include <algorithm>
 #include <chrono>
 #include <cmath>
 #include <cstdarg>
@@ -152,6 +153,12 @@ __global__ void k_dense(int64_t S, int64_t n, uint32_t cap, const uint32_t *nnz,
     }
 }
 
+// A run's counters (kWords of them) into host memory.
+__global__ void k_publish(const unsigned long long *counters, unsigned long long *host)
+{
+    if (threadIdx.x < kWords) host[threadIdx.x] = counters[threadIdx.x];
+}
+
 void ctx_retain(ppr_ctx *ctx)
 {
     if (ctx) ctx->refs.fetch_add(1);
@@ -160,12 +167,14 @@ void ctx_retain(ppr_ctx *ctx)
 void ctx_release(ppr_ctx *ctx)
 {
     if (!ctx || ctx->refs.fetch_sub(1) != 1) return;
-    if (ctx->copy_stream || ctx->pinned) {
-        cudaSetDevice(ctx->device);
-        if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
-        if (ctx->pinned) cudaFreeHost(ctx->pinned);
-        cudaGetLastError();
+    cudaSetDevice(ctx->device);
+    if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
+    for (int i = 0; i < ctx->n_late; ++i) {
+        cudaEventSynchronize(ctx->late[i].done);
+        cudaEventDestroy(ctx->late[i].done);
     }
+    if (ctx->pinned) cudaFreeHost(ctx->pinned);
+    cudaGetLastError();
     delete ctx;
 }
 }  // namespace ppr
@@ -174,43 +183,39 @@ using namespace ppr;
 
 static size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// The context's copy stream, and eight words of host memory for one call's
-// copies of counters and totals: a block of the context's page-locked words
-// (both made on first use), or, where 64 calls of as many threads hold them
-// all, words of the call's own.
-struct CopyResources {
-    ppr_ctx *ctx = nullptr;
-    int block = -1;
-    unsigned long long own[8];
-    unsigned long long *words = own;
-
-    int take(ppr_ctx *c)
-    {
-        ctx = c;
-        std::lock_guard<std::mutex> lock(ctx->mu);
-        cudaError_t e = cudaSuccess;
-        if (!ctx->copy_stream && (e = cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking)) != cudaSuccess)
-            return cuda_fail(e, "copy stream");
-        if (!ctx->pinned) {
-            if ((e = cudaHostAlloc((void **)&ctx->pinned, 64 * sizeof(own), 0)) != cudaSuccess)
-                return cuda_fail(e, "page-locked words");
-            ctx->pinned_free = ~0ull;
+// The context's page-locked words: blocks of kWords, lent to the calls and runs
+// at work.  Gives a block's index, or -1 when all are lent.
+static int take_words(ppr_ctx *ctx)
+{
+    std::lock_guard<std::mutex> lock(ctx->mu);
+    for (int i = 0; i < ctx->n_late;) {  // runs whose result was freed before they ended
+        if (cudaEventQuery(ctx->late[i].done) == cudaErrorNotReady) {
+            ++i;
+            continue;
         }
-        if (ctx->pinned_free) {
-            block = __builtin_ctzll(ctx->pinned_free);
-            ctx->pinned_free &= ctx->pinned_free - 1;
-            words = ctx->pinned + 8 * block;
-        }
-        return PPR_OK;
+        cudaEventDestroy(ctx->late[i].done);
+        ctx->free_words[ctx->n_free++] = ctx->late[i].block;
+        ctx->late[i] = ctx->late[--ctx->n_late];
     }
-    CopyResources() = default;
-    CopyResources(const CopyResources &) = delete;
-    CopyResources &operator=(const CopyResources &) = delete;
-    ~CopyResources()  // (the call has waited for its copies)
+    return ctx->n_free ? ctx->free_words[--ctx->n_free] : -1;
+}
+
+// The words of one call's copies of counters and totals: a block of the
+// context's, or, where all are lent, words of the call's own.
+struct CopyWords {
+    ppr_ctx *ctx;
+    int block;
+    unsigned long long own[kWords];
+    unsigned long long *words;
+
+    explicit CopyWords(ppr_ctx *c) : ctx(c), block(take_words(c)), words(block < 0 ? own : c->pinned + kWords * block) {}
+    CopyWords(const CopyWords &) = delete;
+    CopyWords &operator=(const CopyWords &) = delete;
+    ~CopyWords()  // (the call has waited for its copies)
     {
         if (block < 0) return;
         std::lock_guard<std::mutex> lock(ctx->mu);
-        ctx->pinned_free |= 1ull << block;
+        ctx->free_words[ctx->n_free++] = block;
     }
 };
 
@@ -294,9 +299,15 @@ int ppr_create(int device, ppr_ctx **out)
     cudaDeviceGetAttribute(&v, cudaDevAttrL2CacheSize, device);
     c->l2_bytes = (size_t)v;
     size_t free_b = 0;
-    if (cudaMemGetInfo(&free_b, &c->mem_bytes) != cudaSuccess) {
-        delete c;
-        return cuda_fail(cudaGetLastError(), "cudaMemGetInfo");
+    for (int i = 0; i < kWordBlocks; ++i) c->free_words[c->n_free++] = i;
+    e = cudaMemGetInfo(&free_b, &c->mem_bytes);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->copy_stream, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaHostAlloc((void **)&c->pinned, sizeof(unsigned long long) * kWords * kWordBlocks, cudaHostAllocMapped);
+    if (e == cudaSuccess) e = cudaHostGetDevicePointer((void **)&c->pinned_dev, c->pinned, 0);
+    if (e != cudaSuccess) {
+        const int rc = cuda_fail(e, "context set-up");
+        ctx_release(c);
+        return rc;
     }
     ppr::preload_run_kernels();
     {
@@ -305,6 +316,7 @@ int ppr_create(int device, ppr_ctx **out)
         cudaFuncGetAttributes(&fa, k_dense);
         cudaFuncGetAttributes(&fa, k_add_base);
         cudaFuncGetAttributes(&fa, k_next_base);
+        cudaFuncGetAttributes(&fa, k_publish);
         cudaGetLastError();
     }
     cudaMemPool_t pool;
@@ -474,6 +486,17 @@ static void result_release(ppr_result *r)
 {
     if (!r) return;
     if (r->ctx) cudaSetDevice(r->ctx->device);
+    if (r->words >= 0) {  // not waited for: the words are free when the run has written them
+        std::lock_guard<std::mutex> lock(r->ctx->mu);
+        if (!r->ev_counts) cudaStreamSynchronize(r->stream);  // (a launch that failed half way)
+        if (!r->ev_counts || cudaEventQuery(r->ev_counts) != cudaErrorNotReady) {
+            r->ctx->free_words[r->ctx->n_free++] = r->words;
+        } else {
+            r->ctx->late[r->ctx->n_late++] = {r->ev_counts, r->words};
+            r->ev_counts = nullptr;
+        }
+    }
+    if (r->ev_counts) cudaEventDestroy(r->ev_counts);
     if (r->block) {
         dev_free(r->block, r->stream);
     } else {
@@ -705,6 +728,18 @@ static int run_common(ppr_ctx *ctx, const ppr_graph *g, const ppr_run_args *a, c
         }
     }
     if ((e = cudaEventRecord(r->ev_done, st)) != cudaSuccess) return fail(cuda_fail(e, "cudaEventRecord"));
+    // The run itself stores its counters in host memory: a copy of theirs would
+    // queue behind the copies of other calls (beside a ppr_run_to_host of
+    // another thread ppr_wait took up to 27 ms, with any timeout, for a run
+    // that was over).
+    if ((r->words = take_words(ctx)) >= 0) {
+        k_publish<<<1, 32, 0, st>>>(r->d_steps, ctx->pinned_dev + kWords * r->words);
+        note_launch();
+        e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&r->ev_counts, cudaEventDisableTiming);
+        if (e == cudaSuccess) e = cudaEventRecord(r->ev_counts, st);
+        if (e != cudaSuccess) return fail(cuda_fail(e, "counters"));
+    }
     *out = r;
     return PPR_OK;
 }
@@ -749,8 +784,7 @@ int ppr_run_to_host(ppr_ctx *ctx, const ppr_graph *g, const ppr_run_args *a, int
     Range range("ppr_run_to_host");
     cudaStream_t st = (cudaStream_t)a->stream;
     if ((rc = prepare_tables(g, plan, st))) return rc;
-    CopyResources host;
-    if ((rc = host.take(ctx))) return rc;
+    CopyWords host(ctx);
     cudaError_t e = cudaSuccess;
     cudaStream_t cs = ctx->copy_stream;
     const int64_t S = a->src_end - a->src_begin;
@@ -1124,7 +1158,7 @@ int ppr_wait(ppr_result *r, int64_t timeout_ms)
     // after two milliseconds the thread gives its core back between looks
     auto t0 = std::chrono::steady_clock::now();
     for (;;) {
-        cudaError_t e = cudaEventQuery(r->ev_done);
+        cudaError_t e = cudaEventQuery(r->ev_counts ? r->ev_counts : r->ev_done);
         if (e == cudaSuccess) break;
         if (e != cudaErrorNotReady) return cuda_fail(e, "run");
         const auto us = std::chrono::duration_cast<std::chrono::microseconds>(std::chrono::steady_clock::now() - t0).count();
@@ -1134,12 +1168,23 @@ int ppr_wait(ppr_result *r, int64_t timeout_ms)
         }
         if (us >= 2000) std::this_thread::sleep_for(std::chrono::microseconds(50));
     }
-    // the run is over: its counters are read beside whatever the caller's streams do now
-    CopyResources host;
-    if ((rc = host.take(r->ctx))) return rc;
-    const unsigned long long *cnt = host.words;
-    PPR_CUDA(cudaMemcpyAsync(host.words, r->d_steps, 6 * sizeof(cnt[0]), cudaMemcpyDeviceToHost, r->ctx->copy_stream));
-    PPR_CUDA(cudaStreamSynchronize(r->ctx->copy_stream));
+    // the run's counters: in host memory by now, or (more than kWordBlocks
+    // results not yet waited for) read beside whatever the caller's streams do now
+    unsigned long long cnt[kWords];
+    bool have = false;
+    {
+        std::lock_guard<std::mutex> lock(r->ctx->mu);
+        if (r->words >= 0) {
+            std::copy_n(r->ctx->pinned + kWords * r->words, kWords, cnt);
+            r->ctx->free_words[r->ctx->n_free++] = r->words;
+            r->words = -1;
+            have = true;
+        }
+    }
+    if (!have) {
+        PPR_CUDA(cudaMemcpyAsync(cnt, r->d_steps, sizeof(cnt), cudaMemcpyDeviceToHost, r->ctx->copy_stream));
+        PPR_CUDA(cudaStreamSynchronize(r->ctx->copy_stream));
+    }
     r->steps = cnt[0];
     r->sectors = cnt[2];
     r->model_sectors = cnt[5];
@@ -1204,8 +1249,7 @@ int ppr_sparse_rows(const ppr_result *rc_, int64_t *row_ptr, int32_t *col, uint3
     cudaStream_t st = r->stream;
     const int64_t S = r->S;
     int64_t tiles = (S + kScanTile - 1) / kScanTile;
-    CopyResources host;
-    if ((rc = host.take(r->ctx))) return rc;
+    CopyWords host(r->ctx);
     uint64_t *d_off = nullptr, *d_tmp = nullptr;
     // row starts straight into the caller's device array when there is one
     const bool own_off = !(dev_out && row_ptr);

@@ -54,3 +54,70 @@ def test_results_of_several_threads(graph, threads):
         assert len(got[t]) == 60
         for g in got[t]:
             assert all(np.array_equal(a, b) for a, b in zip(g, want[t]))
+
+
+def test_a_finished_run_is_waited_for_beside_large_output_copies():
+    """Runs that are over are waited for while another thread's ppr_run_to_host
+    copies rows: the wait neither queues behind those copies (each takes more
+    than ten milliseconds here) nor overruns its timeout of 0."""
+    import time
+
+    import torch
+
+    n, R = 1 << 18, 1500
+    g = I.er_graph(n, 1 << 22, 1, 10, seed=5)
+    small = I.er_graph(2000, 16000, 1, 10, seed=5)
+    ctx = ppr.Context(0)
+    H = ctx.load_graph(g.n, g.row_ptr, g.col, g.w)
+    G = ctx.load_graph(small.n, small.row_ptr, small.col, small.w)
+    rows = [torch.zeros(n + 1, dtype=torch.int64, pin_memory=True)] + [
+        torch.zeros(n * R, dtype=torch.int32, pin_memory=True) for _ in range(2)]
+    H.run_to_host(*rows, alpha=0.15, R=R, seed=3, parts=1)
+    runs = [G.run(alpha=0.15, R=10, topk=4, src_end=50, wait=False) for _ in range(60)]
+    torch.cuda.synchronize()
+    busy = []
+
+    def host():
+        t = time.perf_counter()
+        for _ in range(3):
+            H.run_to_host(*rows, alpha=0.15, R=R, seed=3, parts=1)
+        busy.append(time.perf_counter() - t)
+
+    th = threading.Thread(target=host)
+    th.start()
+    waits = []
+    for r in runs:
+        if not th.is_alive():
+            break
+        t = time.perf_counter()
+        r.wait(0)
+        waits.append(time.perf_counter() - t)
+        time.sleep(0.001)
+    th.join()
+    assert busy[0] > 0.03 and len(waits) > 10
+    assert sorted(waits)[-2] < 0.003, sorted(waits)[-5:]  # (one may have been descheduled)
+    want = runs[0].info().steps
+    assert want > 0 and all(r.info().steps == want for r in runs[: len(waits)])
+
+
+def test_more_unread_runs_than_words():
+    """More runs than the context has words for their counters (1,024), some of
+    them freed before they end: every step count is the run's own."""
+    g = I.er_graph(2000, 16000, 1, 10, seed=5)
+    ctx = ppr.Context(0)
+    G = ctx.load_graph(g.n, g.row_ptr, g.col, g.w)
+
+    def start(i):
+        return G.run(alpha=0.15, R=8 + i % 5, seed=i % 7, src_end=100, wait=False)
+
+    want = [start(i).wait().info().steps for i in range(35)]
+    for _ in range(2):
+        runs = [start(i) for i in range(1400)]
+        for r in runs[::3]:
+            r.free()
+        runs += [start(i) for i in range(1400, 1900)]
+        for i, r in enumerate(runs):
+            if r.h:
+                assert r.wait().info().steps == want[i % 35]
+                r.free()
+    start(0).free()  # (the context goes with a run in flight)
