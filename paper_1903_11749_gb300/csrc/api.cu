@@ -1251,8 +1251,8 @@ int ppr_sparse_rows(const ppr_result *rc_, int64_t *row_ptr, int32_t *col, uint3
     int64_t tiles = (S + kScanTile - 1) / kScanTile;
     CopyWords host(r->ctx);
     uint64_t *d_off = nullptr, *d_tmp = nullptr;
-    // row starts straight into the caller's device array when there is one
-    const bool own_off = !(dev_out && row_ptr);
+    // row starts straight into the caller's device array when there is one the scan can store to
+    const bool own_off = !(dev_out && row_ptr && reinterpret_cast<uintptr_t>(row_ptr) % sizeof(int64_t) == 0);
     if (!own_off) d_off = reinterpret_cast<uint64_t *>(row_ptr);
     else if ((rc = dev_alloc((void **)&d_off, sizeof(uint64_t) * (S + 1), "row offsets", st))) return rc;
     int32_t *d_col = nullptr;
@@ -1277,6 +1277,8 @@ int ppr_sparse_rows(const ppr_result *rc_, int64_t *row_ptr, int32_t *col, uint3
             return done(rc);
     }
     cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess && row_ptr && dev_out && own_off)
+        e = cudaMemcpyAsync(row_ptr, d_off, sizeof(int64_t) * (S + 1), cudaMemcpyDeviceToDevice, st);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(host.words, d_off + S, sizeof(uint64_t), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -1284,7 +1286,7 @@ int ppr_sparse_rows(const ppr_result *rc_, int64_t *row_ptr, int32_t *col, uint3
     const uint64_t total = host.words[0];
     r->nnz_total = (int64_t)total;
     if (nnz) *nnz = (int64_t)total;
-    if (row_ptr && own_off) {
+    if (row_ptr && !dev_out) {
         e = cudaMemcpyAsync(row_ptr, d_off, sizeof(int64_t) * (S + 1), cudaMemcpyDeviceToHost, st);
         if (e != cudaSuccess) return done(cuda_fail(e, "row_ptr copy"));
     }
