@@ -280,7 +280,7 @@ typedef struct {
  * Times the persistent walker on a sample of the run's sources (at most
  * sample_sources, 0 = 65536; evenly strided for plain graphs, a leading range
  * for batched graphs) for each candidate of walkers per CTA (128, 256), queue
- * chunk (1/4x .. 4x of 400/R sources), then, with the fastest of those, for
+ * chunk (1/4x .. 4x of 400/R sources, at most 31), then, with the fastest of those, for
  * refill thresholds of 1, 16, 24 and 32 idle lanes (against the run's, 8 unless
  * set), and returns the fastest.  Synchronous;
  * allocates scratch for the sample.  Tuning never changes results.

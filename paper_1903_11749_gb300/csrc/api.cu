@@ -1032,7 +1032,20 @@ int ppr_autotune(ppr_ctx *ctx, const ppr_graph *g, const ppr_run_args *a, int64_
     const uint32_t cap = row_capacity(g, a->R);
     const int32_t topk = a->topk;
     unsigned char *buf = nullptr;
-    const size_t ws_bytes = launch_workspace_bytes(g, plan, S);
+    // chunks of a quarter of the library's choice to four times it, each as it would run, once
+    RunPlan by_default = plan;
+    by_default.chunk_sources = 0;
+    const int cs_base = (int)chunk_sources(by_default);
+    std::vector<int> cs_cands;
+    size_t ws_bytes = 0;  // (of a batch, the smaller the chunks the larger their table)
+    for (int cs : {std::max(1, cs_base / 4), std::max(1, cs_base / 2), cs_base, cs_base * 2, cs_base * 4}) {
+        RunPlan pl = plan;
+        pl.kernel = PPR_KERNEL_PERSISTENT;
+        pl.chunk_sources = cs;
+        cs = (int)chunk_sources(pl);
+        if (std::find(cs_cands.begin(), cs_cands.end(), cs) == cs_cands.end()) cs_cands.push_back(cs);
+        ws_bytes = std::max(ws_bytes, launch_workspace_bytes(g, pl, S));
+    }
     const size_t out_bytes = (size_t)S * (4 + 8ull * cap + 8ull * topk) + 256 + sizeof(uint32_t) * S + 1024;
     if ((rc = dev_alloc((void **)&buf, ws_bytes + out_bytes + 256, "autotune buffers", st))) return rc;
     unsigned char *p = buf;
@@ -1061,21 +1074,17 @@ int ppr_autotune(ppr_ctx *ctx, const ppr_graph *g, const ppr_run_args *a, int64_
         dev_free(buf, st);
         return cuda_fail(e, "autotune setup");
     }
-    const int cs_base = std::max(1, (int)(400 / a->R));
-    const int cs_cands[] = {std::max(1, cs_base / 4), std::max(1, cs_base / 2), cs_base, cs_base * 2, cs_base * 4};
     const int wpb_cands[] = {8, 4};
     ppr_tuning bt{};
     bt.ms = -1.f;
     int tried = 0;
     for (int wpb : wpb_cands)
         for (int cs : cs_cands) {
-            if ((uint64_t)cs * a->R > (1u << 20)) continue;
             RunPlan pl = plan;
             pl.kernel = PPR_KERNEL_PERSISTENT;
             pl.stats = false;
             pl.chunk_sources = cs;
             pl.warps_per_block = wpb;
-            if (launch_workspace_bytes(g, pl, S) > ws_bytes) continue;
             float ms_best = 1e30f;
             for (int rep = 0; rep < 2; ++rep) {
                 cudaMemsetAsync(o.counters, 0, 256, st);

@@ -217,6 +217,10 @@ struct Outputs {
 // Fills *plan; returns a PPR_* status with the message set.
 int check_run(const ppr_graph *g, const ppr_run_args *a, int64_t count, bool list, RunPlan *plan);
 
+// Sources a work chunk holds under a plan (its chunk_sources, or the library's
+// choice, as far as a warp has places for them).
+uint32_t chunk_sources(const RunPlan &p);
+
 // Device workspace one launch of S sources needs (endpoints, chunk table).
 size_t launch_workspace_bytes(const ppr_graph *g, const RunPlan &p, int64_t S);
 

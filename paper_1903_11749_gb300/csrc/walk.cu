@@ -326,7 +326,7 @@ __global__ void __launch_bounds__(256) k_chunk_fill(int32_t count, const int64_t
 // sources per chunk, at most as many as a warp has places for; a chunk holds at
 // most 2^19 walks (walk indices within a chunk stay below 2^20 for the
 // multiply-shift division by R)
-static uint32_t chunk_sources(const RunPlan &plan)
+uint32_t chunk_sources(const RunPlan &plan)
 {
     const uint32_t cs = plan.chunk_sources > 0 ? (uint32_t)plan.chunk_sources : std::max(1u, 400u / plan.R);
     return std::min(std::min(cs, kChunkSources), std::max(1u, (1u << 19) / plan.R));
