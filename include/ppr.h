@@ -400,6 +400,14 @@ int ppr_run_noalloc(ppr_ctx *ctx, const ppr_graph *g, const ppr_run_args *args, 
  * turns it off.  Process-wide. */
 void ppr_debug_fail_allocs(int64_t after);
 
+/* Test hook: what the library otherwise chooses by size.  -1: its choice.
+ * lam_bits (0..23): graphs loaded from now on have slots for ranges of
+ * 2^lam_bits edges on average; exact (0, 1): whether plain ones class rows of
+ * up to 24 edges by their degree; far (0, 1): whether runs on plain graphs
+ * with 32-bit row totals fetch by 64 bytes.  Results are unchanged.
+ * PPR_EINVAL for other values. */
+int ppr_debug_layout(ppr_ctx *ctx, int32_t lam_bits, int32_t exact, int32_t far_fetch);
+
 /* ------------------------------------------------------------- probes ----
  * Measurement beside the walk path; neither is part of a run.
  *

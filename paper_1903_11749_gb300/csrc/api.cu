@@ -241,6 +241,18 @@ uint32_t ppr_alpha_threshold(double alpha)
     return (uint32_t)t;
 }
 
+int ppr_debug_layout(ppr_ctx *ctx, int32_t lam_bits, int32_t exact, int32_t far_fetch)
+{
+    if (!ctx || lam_bits < -1 || lam_bits > 23 || exact < -1 || exact > 1 || far_fetch < -1 || far_fetch > 1) {
+        set_error("invalid layout choice");
+        return PPR_EINVAL;
+    }
+    ctx->force_lam = lam_bits;
+    ctx->force_exact = exact;
+    ctx->force_far = far_fetch;
+    return PPR_OK;
+}
+
 void ppr_debug_fail_allocs(int64_t after) { g_allocs_left.store(after < 0 ? -1 : after); }
 
 int ppr_walks_for_accuracy(double eps, double delta, double p_f, uint64_t *omega)

@@ -443,6 +443,7 @@ static int build_layout(ppr_ctx *ctx, int64_t n, int64_t m, const int64_t *d_rp,
     const double slot_bytes = 45.0 * (double)m * share, l2 = (double)ctx->l2_bytes;
     g->lam_bits = !E::kWide && slot_bytes > 1.75 * l2 && slot_bytes < 16.0 * l2 ? 1 : 0;
     while (g->lam_bits < 23 && (uint64_t)m * 64 >> g->lam_bits > ctx->mem_bytes / 8) ++g->lam_bits;
+    if (ctx->force_lam >= 0) g->lam_bits = (uint32_t)ctx->force_lam;
     uint32_t *heads;
     LayoutStats *d_ls;
     const int64_t tiles = (m + kEdgeTile - 1) / kEdgeTile;
@@ -459,7 +460,7 @@ static int build_layout(ppr_ctx *ctx, int64_t n, int64_t m, const int64_t *d_rp,
         return rc;
     PPR_CUDA(cudaMemsetAsync(heads, 0, sizeof(uint32_t) * head_words, st));
     PPR_CUDA(cudaMemsetAsync(d_ls, 0, sizeof(LayoutStats), st));
-    if ((rc = number_nodes(n, m, d_rp, d_off, heads, d_ls, E::kWide, st, g, tmp))) return rc;
+    if ((rc = number_nodes(ctx, n, m, d_rp, d_off, heads, d_ls, E::kWide, st, g, tmp))) return rc;
     const size_t run = kEdgeRun * sizeof(typename E::Edge);
     const size_t edge_bytes = (size_t)(tiles > 0 ? (m + kEdgeRun - 1) / kEdgeRun : 1) * run;
     if ((rc = dev_alloc(&g->edges, edge_bytes, "edge records", st)) ||

@@ -77,6 +77,7 @@ struct ppr_ctx {
     size_t l2_persist_set = 0;    // persisting set-aside this context asked for
     size_t l2_bytes = 0;          // L2 size (the layout's renumbering policy)
     size_t mem_bytes = 0;         // device memory (the layout's slot density)
+    int32_t force_lam = -1, force_exact = -1, force_far = -1;  // ppr_debug_layout
     cudaStream_t copy_stream = nullptr;  // output copies of ppr_run_to_host
     unsigned long long *pinned = nullptr;  // kWordBlocks blocks of page-locked words, lent to the calls and runs at work
     unsigned long long *pinned_dev = nullptr;  // their device address
@@ -169,7 +170,7 @@ struct LayoutStats {
     unsigned int status;
 };
 enum : uint32_t { kBadRowPtr = 1u, kBadCol = 2u, kBadWeight = 4u, kWide = 8u, kBigDegree = 16u };
-int number_nodes(int64_t n, int64_t m, const int64_t *d_rp, const int64_t *d_off, uint32_t *heads,
+int number_nodes(const ppr_ctx *ctx, int64_t n, int64_t m, const int64_t *d_rp, const int64_t *d_off, uint32_t *heads,
                  LayoutStats *d_stats, bool wide, cudaStream_t st, ppr_graph *g, std::vector<void *> &tmp);
 int build_segments(ppr_graph *g, uint32_t T, cudaStream_t st);
 int build_alias(ppr_graph *g, cudaStream_t st);

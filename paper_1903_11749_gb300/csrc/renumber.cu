@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(128) k_rn_scatter(NumberArgs A, ClassEntries C
     }
 }
 
-int number_nodes(int64_t n, int64_t m, const int64_t *d_rp, const int64_t *d_off, uint32_t *heads,
+int number_nodes(const ppr_ctx *ctx, int64_t n, int64_t m, const int64_t *d_rp, const int64_t *d_off, uint32_t *heads,
                  LayoutStats *d_stats, bool wide, cudaStream_t st, ppr_graph *g, std::vector<void *> &tmp)
 {
     Range range("number nodes");
@@ -169,7 +169,7 @@ int number_nodes(int64_t n, int64_t m, const int64_t *d_rp, const int64_t *d_off
     A.row_ptr = d_rp;
     A.lam_bits = g->lam_bits;
     A.wide = wide;
-    A.exact = g->instances == 0 && n > kExactMin && n <= kExactNodes;
+    A.exact = g->instances == 0 && n <= kExactNodes && (ctx->force_exact < 0 ? n > kExactMin : ctx->force_exact == 1);
     // nodes a warp takes in turn: few where the graph is small (a warp's chain
     // of rounds is then the kernel's time)
     A.tile = n <= 2048 ? 32u : (n <= (1 << 18) ? 128u : 1024u);

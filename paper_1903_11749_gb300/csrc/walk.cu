@@ -438,7 +438,8 @@ void set_layout(KParams &kp, const ppr_graph *g, bool segments, bool alias)
 static bool is_far(const ppr_ctx *ctx, const ppr_graph *g, bool alias)
 {
     const double bytes = alias ? (double)g->m * sizeof(AliasRec) : (double)g->n_slots * sizeof(Sector);
-    return !g->wide && g->instances == 0 && bytes >= 16.0 * (double)ctx->l2_bytes;
+    return !g->wide && g->instances == 0 &&
+           (ctx->force_far < 0 ? bytes >= 16.0 * (double)ctx->l2_bytes : ctx->force_far == 1);
 }
 
 int launch_walks(ppr_ctx *ctx, const ppr_graph *g, const RunPlan &plan, const Outputs &o, int64_t s_begin, int64_t S,

@@ -122,6 +122,7 @@ _SIGS = {
                              C.POINTER(C.c_uint64)]),
     "ppr_poll": (C.c_int, [C.c_void_p, C.c_uint64, C.c_void_p, C.c_void_p, C.c_int64, C.POINTER(QueryStats)]),
     "ppr_debug_fail_allocs": (None, [C.c_int64]),
+    "ppr_debug_layout": (C.c_int, [C.c_void_p, C.c_int32, C.c_int32, C.c_int32]),
     "ppr_probe_philox": (C.c_int, [C.c_void_p, C.c_uint64, C.c_void_p, C.c_int64, C.c_void_p]),
     "ppr_probe_rate": (C.c_int, [C.c_void_p, C.c_int32, C.c_int64, C.POINTER(C.c_double), C.POINTER(C.c_float)]),
     "ppr_run_to_host": (C.c_int, [C.c_void_p, C.c_void_p, C.POINTER(RunArgs), C.c_int32, C.c_void_p, C.c_void_p,
@@ -211,6 +212,10 @@ class Context:
             self.close()
         except Exception:
             pass
+
+    def debug_layout(self, lam_bits: int = -1, exact: int = -1, far: int = -1):
+        """Test hook: layout and fetch choices that sizes make otherwise (see include/ppr.h)."""
+        _check(lib().ppr_debug_layout(self.h, lam_bits, exact, far))
 
     # ---- serving
     def probe_philox(self, seed: int, counter, count: int) -> np.ndarray:
