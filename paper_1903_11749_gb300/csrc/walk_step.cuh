@@ -201,7 +201,10 @@ __device__ __forceinline__ bool walk_step(const KParams &p, const ClassTab &tab,
         const uint32_t slot = __funnelshift_l(x.y, idx, t.kind);
         if (t.kind >= kKindSingle && !resume) {
             if (t.kind == kKindDangling) {
-                if (p.dangling == 1) return true;  // the walk ends here without a step
+                if (p.dangling == 1) {  // the walk ends here without a step
+                    if (STATS) tl.model += flat_model_sectors(0);  // (a flat CSR is read to know)
+                    return true;
+                }
                 next = src;
             } else {
                 PPR_CHECK(idx < p.n_single, 2);

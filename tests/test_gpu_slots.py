@@ -113,3 +113,19 @@ def test_invalid_edges_are_still_refused(ppr, ctx, bad):
     with pytest.raises(ppr.PPRError) as e:
         ctx.load_graph(g.n, g.row_ptr, col, w)
     assert e.value.code == ppr.PPR_EINVAL
+
+
+@pytest.mark.parametrize("kernel", [0, 1])
+@pytest.mark.parametrize("segments", [False, True])
+def test_flat_model_counts_the_node_a_walk_ends_at(ppr, ctx, kernel, segments):
+    """In dangling mode 1 a walk that comes to a node without out-edges ends
+    there; the flat-CSR model reads one sector to find that out.  Here every
+    walk makes one draw at a row of 16 edges (row_ptr, three probe sectors, the
+    target) and ends at node 100; walks from node 100 make none."""
+    n, d, R = 101, 16, 50
+    rp = np.minimum(np.arange(n + 1, dtype=np.int64), n - 1) * d
+    G = ctx.load_graph(n, rp, np.full(d * (n - 1), n - 1, np.int32), np.ones(d * (n - 1), np.uint32))
+    r = G.run(alpha=1e-7, R=R, seed=1, dangling=1, stats=True, kernel=kernel, segments=segments)
+    i = r.info()
+    assert i.steps == (n - 1) * R
+    assert i.model_sectors == (n - 1) * R * (1 + 3 + 1) + n * R
