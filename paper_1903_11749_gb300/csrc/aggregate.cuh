@@ -30,6 +30,7 @@ struct CallerIds {
     }
 };
 
+// The serving loop's reduction for R above 128: one warp, in shared memory.
 // ends: the R endpoints of one source (shared memory).  sortbuf: next_pow2(R)
 // uint32 and keys: next_pow2(R) uint64 of per-warp shared scratch.  Writes
 // row `out_row` of the outputs.  All 32 lanes call it.
@@ -88,14 +89,6 @@ __device__ inline void aggregate_source(const uint32_t *ends, uint32_t R, uint32
     __syncwarp();
 }
 
-// Register-resident variant for next_pow2(R) = 32 * E <= 256 (R <= 32: E = 1).
-// The sort works on consecutive elements of a lane (its short strides are then
-// plain min and max, and of the 28 stages of R = 128 only 15 are shuffles); what
-// follows takes them in striped order (element e * 32 + lane in register e),
-// where ballots see them in order and rows are written in whole sectors.  Runs
-// are found from neighbour values; the top-k sorts 32-bit keys
-// (R - count) << 12 | run, whose order is count descending then end id
-// ascending because runs are numbered in id order.
 // Ascending sort of T * I elements, element t * I + k in register k of thread
 // t < T (a warp, or a block).  Bitonic network in the form whose first exchange of every level mirrors
 // (i with i ^ (size - 1)), so every exchange puts the smaller element first and
@@ -248,6 +241,14 @@ __device__ __forceinline__ void topk_ones_reg(const uint32_t (&kv)[E], const uin
     }
 }
 
+// Register-resident variant for next_pow2(R) = 32 * E <= 256 (R <= 32: E = 1).
+// The sort works on consecutive elements of a lane (its short strides are then
+// plain min and max, and of the 28 stages of R = 128 only 15 are shuffles); what
+// follows takes them in striped order (element e * 32 + lane in register e),
+// where ballots see them in order and rows are written in whole sectors.  Runs
+// are found from neighbour values; the top-k sorts 32-bit keys
+// (R - count) << 12 | run, whose order is count descending then end id
+// ascending because runs are numbered in id order.
 // scratch: 32 * E + 32 uint32 of per-warp shared memory, 16-byte aligned.
 //
 // Bound by the ALU pipe, so what follows the sort is kept short: run heads

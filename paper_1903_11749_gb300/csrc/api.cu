@@ -302,8 +302,6 @@ int ppr_create(int device, ppr_ctx **out)
     int v = 0;
     cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, device);
     c->sms = v;
-    cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
-    c->smem_optin = (size_t)v;
     cudaDeviceGetAttribute(&v, cudaDevAttrMaxPersistingL2CacheSize, device);
     c->l2_persist_max = (size_t)v;
     cudaDeviceGetAttribute(&v, cudaDevAttrMaxAccessPolicyWindowSize, device);

@@ -16,19 +16,6 @@
 
 namespace ppr {
 
-// Instance of global node u in a block-diagonal graph (node_off has count+1
-// entries); returns 0 for a plain graph.
-__device__ __forceinline__ int32_t instance_of(const int64_t *node_off, int32_t count, int64_t u)
-{
-    int32_t lo = 0, hi = count;  // find last g with node_off[g] <= u
-    while (hi - lo > 1) {
-        int32_t mid = (lo + hi) >> 1;
-        if (node_off[mid] <= u) lo = mid;
-        else hi = mid;
-    }
-    return lo;
-}
-
 // ------------------------------------------------------------ edge records ----
 // Prefixes by edge, not by row: a scan of the weights that restarts at every
 // row start (the bits number_nodes set) gives each edge its inclusive prefix
@@ -246,7 +233,7 @@ __global__ void __launch_bounds__(256) k_nodes(SlotArgs A, E edges)
         total = d == 1 ? (uint64_t)E::target(last) : E::key(last);
         if (d == 1) reinterpret_cast<uint32_t *>(A.tab->e[code >> kIdxBits].addr)[code & kIdxMask] = E::target(last);
     }
-    A.node[seq_of(*A.tab, code)] = NodeRec{pack_word0((uint64_t)a, d, false), total};
+    A.node[seq_of(*A.tab, code)] = NodeRec{pack_word0((uint64_t)a, d), total};
 }
 
 // Index of the first edge of a row whose prefix exceeds x, among its n edges
@@ -1016,7 +1003,7 @@ __global__ void __launch_bounds__(32 * WARPS) k_seg_fill(RowView<E> G, uint32_t 
             if (lane == 0) {
                 uint32_t *to = reinterpret_cast<uint32_t *>(te.addr) + idx;
                 *to = kMarkSeg;
-                links.head[to - links.single] = SegHead{pack_word0(base, K, false), carry};
+                links.head[to - links.single] = SegHead{pack_word0(base, K), carry};
             }
         } else {
             Sector *at = reinterpret_cast<Sector *>(te.addr) + ((uint64_t)idx << te.kind);
@@ -1260,7 +1247,7 @@ __global__ void __launch_bounds__(256) k_alias_small(AliasArgs A)
         const NodeRec nr = A.node[u];
         const uint32_t d = row_degree(nr);
         const uint64_t o = A.off[u];
-        if (u >= A.first_node) A.anode[u - A.first_node] = AliasNode{pack_word0(o, d, false)};
+        if (u >= A.first_node) A.anode[u - A.first_node] = AliasNode{pack_word0(o, d)};
         if (d < 2) continue;
         if (d > kAliasInline) {
             if (d > kAliasHuge) {

@@ -70,7 +70,6 @@ constexpr int kWordBlocks = 1024;  // of a context (64 KB)
 struct ppr_ctx {
     int device = 0;
     int sms = 0;
-    size_t smem_optin = 0;
     ppr::Server *server = nullptr;  // serving state (ppr_serve_start)
     size_t l2_persist_max = 0;    // device limits for L2 access-policy windows
     size_t l2_window_max = 0;
@@ -198,8 +197,7 @@ struct RunPlan {
     bool l2_persist;  // walker launches keep the front of the layout in L2 (access-policy window)
 };
 // Enqueues the walks of sources [s_begin, s_end) writing output rows from
-// out_row0.  ends: S * R endpoint scratch for the plain kernel (else unused);
-// queue: one device counter for the persistent kernel's work queue.
+// out_row0; their S * R endpoints go to the front of the workspace.
 // Where a launch writes: rows (nnz / cols / cnts at row * cap), top-k, and
 // the counters block: [0] steps, [1] work queue, [2] sectors, [3] chunk count.
 struct Outputs {

@@ -41,7 +41,6 @@ namespace ppr {
 
 constexpr uint64_t kBeginMask = (1ull << 40) - 1;
 constexpr uint32_t kCountMask = (1u << 23) - 1;
-constexpr uint64_t kSegFlag = 1ull << 63;
 
 struct __align__(16) NodeRec {
     uint64_t word0;
@@ -88,9 +87,9 @@ struct __align__(16) SegHead {
     uint64_t Q;
 };
 
-__host__ __device__ inline uint64_t pack_word0(uint64_t begin, uint32_t count, bool seg)
+__host__ __device__ inline uint64_t pack_word0(uint64_t begin, uint32_t count)
 {
-    return (begin & kBeginMask) | ((uint64_t)(count & kCountMask) << 40) | (seg ? kSegFlag : 0ull);
+    return (begin & kBeginMask) | ((uint64_t)(count & kCountMask) << 40);
 }
 
 // ------------------------------------------------------------- node codes ----
@@ -119,9 +118,12 @@ struct ClassTab {
 // ranges.  Plain graphs of more than kExactMin nodes class rows of up to kExact
 // edges by their degree, so that alias slots are found without a record: the
 // records of all nodes would not stay in L2 there, those of the longer rows (a
-// tenth) do (R-MAT scale 24, alias walker over 2^22 sources: 22.1 -> 20.9 ms).
-// Elsewhere the classes stay few: every class is an area of its own, and with
-// 23 more of them the walker of a 256-graph batch took 25.1 ms, not 17.6.
+// tenth) do.  Alias walker without / with such classes, R-MAT, R 100, up to
+// 2^20 sources: scale 18 .982 / .982 ms, 19 1.939 / 1.942, 20 4.583 / 4.500, 21
+// 5.97 / 5.86, 22 7.05 / 6.78, 23 7.81 / 7.40; scale 24, 2^22 sources, 22.1 /
+// 20.9.  The prefix walker and the load are level at every one of them, so the
+// line could lie at 2^20.  Batches keep few classes: every class is an area of
+// its own, and with 23 more the walker of 256 graphs took 25.1 ms, not 17.6.
 // More than kExactNodes nodes leave no room in the table for classes by degree.
 // 2^c is the smallest power of two >= d / 2^lam_bits, and a row that fits one
 // slot (four edges, three in the wide layout) is one range.
@@ -422,11 +424,8 @@ __device__ __forceinline__ uint32_t pick_record(const Sector &r, uint32_t first,
     return h0 ? r.v[1] : (h1 ? r.v[3] : (h2 ? r.v[5] : r.v[7]));
 }
 
-// ----------------------------------------------------------- aggregation ----
-// Per-source aggregation of R endpoints (Algorithm 2's final grouping of the
-// terminated walks by (head, tail)), done by one warp in shared memory:
-// bitonic sort of the endpoints, run-length counting, row write-out, then a
-// second bitonic sort of (count desc, end asc) keys for the top-k.
+// ------------------------------------------------------------------ sort ----
+// The sort of aggregate_source (aggregate.cuh), a warp's in shared memory.
 
 __device__ __forceinline__ uint32_t next_pow2(uint32_t v)
 {

@@ -1361,10 +1361,10 @@ static void scheduler_loop(Server *sv)
                 // up to one source an aggregator is taken by those at once
                 d.help = R <= kHelpMaxR && d.S > sv->grid ? 1u : 0u;
                 // Walks per chunk: about two chunks per walker warp for a query
-                // alone; with others in flight about as many for all together, as
-                // long as the query still has 64 (a claim is two trips to L2 under
+                // alone; with others in flight about four for all together, as long
+                // as the query still has 64 (a claim is two trips to L2 under
                 // contention: a burst of 64 queries made 165,000 of 80 walks each
-                // and took 7.0 ms, 31,000 and 6.5 ms now).
+                // and took 7.0 ms; with 31,000 it took 6.5).
                 const uint64_t ww = std::max<uint64_t>(1, 2ull * sv->grid * (kLoopWarps - 1));
                 uint64_t cw = std::max((d.walks + ww - 1) / ww, std::min<uint64_t>(load / (2 * ww), d.walks / 64));
                 if (sv->cfg.chunk_sources > 0) cw = (uint64_t)sv->cfg.chunk_sources * R;

@@ -100,7 +100,10 @@ struct WarpChunk {
 // refill waits for them (256-graph batch 18.91 -> 18.55 ms, R-MAT scale-24 job
 // 103.8 -> 102.9, scale 20 8.10 -> 8.01; the wide walker, short of registers,
 // reads them as it starts walks: 2.200 ms, staged 2.227).  So a chunk has at
-// most 31 whole sources, or parts of 32.
+// most 31 whole sources, or parts of 32, also where that is far less than 400
+// walks (R up to 12): with places for 63 or 127 sources scale 20 takes 568 or
+// 599 us, not 558, at R 2, 1,009 or 1,011, not 957, at R 6, and its alias
+// walker, which loses L1 to the places, 8.08 or 8.20 ms, not 7.52, at R 100.
 constexpr uint32_t kChunkSources = 31;
 
 __device__ __forceinline__ uint32_t div_by_R(uint32_t w, uint64_t magic)
@@ -483,7 +486,6 @@ int launch_walks(ppr_ctx *ctx, const ppr_graph *g, const RunPlan &plan, const Ou
         }
     } else {
         const uint32_t CS = chunk_sources(plan);
-        kp.CS = CS;
         if (g->instances > 0) {
             const int64_t cnt = g->instances;
             int4 *chunks = reinterpret_cast<int4 *>(ws + off);

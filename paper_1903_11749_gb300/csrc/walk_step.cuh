@@ -30,7 +30,6 @@ struct KParams {
     int32_t dangling;
     int64_t s_begin, s_end;   // sources of this launch (global ids)
     int64_t out_row0;         // output row of s_begin
-    uint32_t CS;              // sources per chunk (batched graphs)
     uint32_t CW;              // walks per chunk (plain graphs; a chunk may start inside a source)
     uint32_t refill;          // idle lanes before a warp starts new walks (1..32)
     uint64_t walks;           // S * R
