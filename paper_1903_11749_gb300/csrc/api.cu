@@ -169,11 +169,6 @@ void ctx_release(ppr_ctx *ctx)
     if (!ctx || ctx->refs.fetch_sub(1) != 1) return;
     cudaSetDevice(ctx->device);
     if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
-    for (int i = 0; i < ctx->n_late; ++i) {
-        cudaEventSynchronize(ctx->late[i].done);
-        cudaEventDestroy(ctx->late[i].done);
-    }
-    if (ctx->pinned) cudaFreeHost(ctx->pinned);
     cudaGetLastError();
     delete ctx;
 }
@@ -183,39 +178,70 @@ using namespace ppr;
 
 static size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// The context's page-locked words: blocks of kWords, lent to the calls and runs
-// at work.  Gives a block's index, or -1 when all are lent.
-static int take_words(ppr_ctx *ctx)
+// Page-locked words, kWordBlocks blocks of kWords, lent to the calls and runs at
+// work in the whole process.  They are made with the first context and kept:
+// freeing page-locked memory waits for the device, so that a context that took
+// its own along could not be closed while another one's serving loop is busy.
+constexpr int kWordBlocks = 1024;  // (64 KB)
+static struct {
+    std::mutex mu;
+    unsigned long long *host = nullptr, *dev = nullptr;
+    int free[kWordBlocks], n_free = 0;
+    struct {
+        cudaEvent_t done;
+        int block;
+    } late[kWordBlocks];  // blocks of runs whose result was freed before they ended: free after the event
+    int n_late = 0;
+} g_words;
+
+static cudaError_t make_words()
 {
-    std::lock_guard<std::mutex> lock(ctx->mu);
-    for (int i = 0; i < ctx->n_late;) {  // runs whose result was freed before they ended
-        if (cudaEventQuery(ctx->late[i].done) == cudaErrorNotReady) {
+    std::lock_guard<std::mutex> lock(g_words.mu);
+    if (g_words.host) return cudaSuccess;
+    void *p = nullptr, *d = nullptr;
+    cudaError_t e = cudaHostAlloc(&p, sizeof(unsigned long long) * kWords * kWordBlocks, cudaHostAllocMapped | cudaHostAllocPortable);
+    if (e != cudaSuccess) return e;
+    if ((e = cudaHostGetDevicePointer(&d, p, 0)) != cudaSuccess) {
+        cudaFreeHost(p);
+        return e;
+    }
+    g_words.host = static_cast<unsigned long long *>(p);
+    g_words.dev = static_cast<unsigned long long *>(d);
+    for (int i = 0; i < kWordBlocks; ++i) g_words.free[g_words.n_free++] = i;
+    return cudaSuccess;
+}
+
+// A block's index, or -1 when all are lent.
+static int take_words()
+{
+    std::lock_guard<std::mutex> lock(g_words.mu);
+    for (int i = 0; i < g_words.n_late;) {
+        if (cudaEventQuery(g_words.late[i].done) == cudaErrorNotReady) {
             ++i;
             continue;
         }
-        cudaEventDestroy(ctx->late[i].done);
-        ctx->free_words[ctx->n_free++] = ctx->late[i].block;
-        ctx->late[i] = ctx->late[--ctx->n_late];
+        cudaEventDestroy(g_words.late[i].done);
+        g_words.free[g_words.n_free++] = g_words.late[i].block;
+        g_words.late[i] = g_words.late[--g_words.n_late];
     }
-    return ctx->n_free ? ctx->free_words[--ctx->n_free] : -1;
+    return g_words.n_free ? g_words.free[--g_words.n_free] : -1;
 }
 
-// The words of one call's copies of counters and totals: a block of the
-// context's, or, where all are lent, words of the call's own.
+// The words of one call's copies of counters and totals: a lent block, or,
+// where all are lent, words of the call's own.
 struct CopyWords {
-    ppr_ctx *ctx;
     int block;
     unsigned long long own[kWords];
     unsigned long long *words;
 
-    explicit CopyWords(ppr_ctx *c) : ctx(c), block(take_words(c)), words(block < 0 ? own : c->pinned + kWords * block) {}
+    CopyWords() : block(take_words()), words(block < 0 ? own : g_words.host + kWords * block) {}
     CopyWords(const CopyWords &) = delete;
     CopyWords &operator=(const CopyWords &) = delete;
     ~CopyWords()  // (the call has waited for its copies)
     {
         if (block < 0) return;
-        std::lock_guard<std::mutex> lock(ctx->mu);
-        ctx->free_words[ctx->n_free++] = block;
+        std::lock_guard<std::mutex> lock(g_words.mu);
+        g_words.free[g_words.n_free++] = block;
     }
 };
 
@@ -309,11 +335,9 @@ int ppr_create(int device, ppr_ctx **out)
     cudaDeviceGetAttribute(&v, cudaDevAttrL2CacheSize, device);
     c->l2_bytes = (size_t)v;
     size_t free_b = 0;
-    for (int i = 0; i < kWordBlocks; ++i) c->free_words[c->n_free++] = i;
     e = cudaMemGetInfo(&free_b, &c->mem_bytes);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->copy_stream, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaHostAlloc((void **)&c->pinned, sizeof(unsigned long long) * kWords * kWordBlocks, cudaHostAllocMapped);
-    if (e == cudaSuccess) e = cudaHostGetDevicePointer((void **)&c->pinned_dev, c->pinned, 0);
+    if (e == cudaSuccess) e = make_words();
     if (e != cudaSuccess) {
         const int rc = cuda_fail(e, "context set-up");
         ctx_release(c);
@@ -497,12 +521,12 @@ static void result_release(ppr_result *r)
     if (!r) return;
     if (r->ctx) cudaSetDevice(r->ctx->device);
     if (r->words >= 0) {  // not waited for: the words are free when the run has written them
-        std::lock_guard<std::mutex> lock(r->ctx->mu);
+        std::lock_guard<std::mutex> lock(g_words.mu);
         if (!r->ev_counts) cudaStreamSynchronize(r->stream);  // (a launch that failed half way)
         if (!r->ev_counts || cudaEventQuery(r->ev_counts) != cudaErrorNotReady) {
-            r->ctx->free_words[r->ctx->n_free++] = r->words;
+            g_words.free[g_words.n_free++] = r->words;
         } else {
-            r->ctx->late[r->ctx->n_late++] = {r->ev_counts, r->words};
+            g_words.late[g_words.n_late++] = {r->ev_counts, r->words};
             r->ev_counts = nullptr;
         }
     }
@@ -742,8 +766,8 @@ static int run_common(ppr_ctx *ctx, const ppr_graph *g, const ppr_run_args *a, c
     // queue behind the copies of other calls (beside a ppr_run_to_host of
     // another thread ppr_wait took up to 27 ms, with any timeout, for a run
     // that was over).
-    if ((r->words = take_words(ctx)) >= 0) {
-        k_publish<<<1, 32, 0, st>>>(r->d_steps, ctx->pinned_dev + kWords * r->words);
+    if ((r->words = take_words()) >= 0) {
+        k_publish<<<1, 32, 0, st>>>(r->d_steps, g_words.dev + kWords * r->words);
         note_launch();
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&r->ev_counts, cudaEventDisableTiming);
@@ -794,7 +818,7 @@ int ppr_run_to_host(ppr_ctx *ctx, const ppr_graph *g, const ppr_run_args *a, int
     Range range("ppr_run_to_host");
     cudaStream_t st = (cudaStream_t)a->stream;
     if ((rc = prepare_tables(g, plan, st))) return rc;
-    CopyWords host(ctx);
+    CopyWords host;
     cudaError_t e = cudaSuccess;
     cudaStream_t cs = ctx->copy_stream;
     const int64_t S = a->src_end - a->src_begin;
@@ -1192,10 +1216,10 @@ int ppr_wait(ppr_result *r, int64_t timeout_ms)
     unsigned long long cnt[kWords];
     bool have = false;
     {
-        std::lock_guard<std::mutex> lock(r->ctx->mu);
+        std::lock_guard<std::mutex> lock(g_words.mu);
         if (r->words >= 0) {
-            std::copy_n(r->ctx->pinned + kWords * r->words, kWords, cnt);
-            r->ctx->free_words[r->ctx->n_free++] = r->words;
+            std::copy_n(g_words.host + kWords * r->words, kWords, cnt);
+            g_words.free[g_words.n_free++] = r->words;
             r->words = -1;
             have = true;
         }
@@ -1268,7 +1292,7 @@ int ppr_sparse_rows(const ppr_result *rc_, int64_t *row_ptr, int32_t *col, uint3
     cudaStream_t st = r->stream;
     const int64_t S = r->S;
     int64_t tiles = (S + kScanTile - 1) / kScanTile;
-    CopyWords host(r->ctx);
+    CopyWords host;
     uint64_t *d_off = nullptr, *d_tmp = nullptr;
     // row starts straight into the caller's device array when there is one the scan can store to
     const bool own_off = !(dev_out && row_ptr && reinterpret_cast<uintptr_t>(row_ptr) % sizeof(int64_t) == 0);

@@ -63,8 +63,7 @@ struct Server;
 }
 
 namespace ppr {
-constexpr int kWords = 8;          // a run's counters
-constexpr int kWordBlocks = 1024;  // of a context (64 KB)
+constexpr int kWords = 8;  // a run's counters
 }
 
 struct ppr_ctx {
@@ -78,15 +77,6 @@ struct ppr_ctx {
     size_t mem_bytes = 0;         // device memory (the layout's slot density)
     int32_t force_lam = -1, force_exact = -1, force_far = -1;  // ppr_debug_layout
     cudaStream_t copy_stream = nullptr;  // output copies of ppr_run_to_host
-    unsigned long long *pinned = nullptr;  // kWordBlocks blocks of page-locked words, lent to the calls and runs at work
-    unsigned long long *pinned_dev = nullptr;  // their device address
-    int free_words[ppr::kWordBlocks], n_free = 0;  // blocks not lent
-    struct {
-        cudaEvent_t done;
-        int block;
-    } late[ppr::kWordBlocks];              // blocks that are free once an event has passed
-    int n_late = 0;
-    std::mutex mu;                         // guards the words: free, late and those of results
     std::atomic<int> refs{1};  // the caller's handle plus every live graph and result
 };
 
@@ -143,7 +133,7 @@ struct ppr_result {
     unsigned long long *d_steps = nullptr;  // counters: [0] steps, [1] work queue, [2] sectors, [3] chunks,
                                             // [4] checked-build flags, [5] flat-CSR model sectors
     cudaEvent_t ev_start = nullptr, ev_done = nullptr;
-    int words = -1;                    // block of the context's words that the run stores its counters in
+    int words = -1;                    // block of the page-locked words that the run stores its counters in
     cudaEvent_t ev_counts = nullptr;   // when it has
     void *block = nullptr;       // one allocation behind the buffers of a small run, or null
     std::vector<cudaEvent_t> walk_events;  // (before, after) each walker launch

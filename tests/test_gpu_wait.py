@@ -101,8 +101,8 @@ def test_a_finished_run_is_waited_for_beside_large_output_copies():
 
 
 def test_more_unread_runs_than_words():
-    """More runs than the context has words for their counters (1,024), some of
-    them freed before they end: every step count is the run's own."""
+    """More runs than there are words for their counters (1,024), some of them
+    freed before they end: every step count is the run's own."""
     g = I.er_graph(2000, 16000, 1, 10, seed=5)
     ctx = ppr.Context(0)
     G = ctx.load_graph(g.n, g.row_ptr, g.col, g.w)
@@ -121,3 +121,33 @@ def test_more_unread_runs_than_words():
                 assert r.wait().info().steps == want[i % 35]
                 r.free()
     start(0).free()  # (the context goes with a run in flight)
+
+
+def test_a_context_closes_beside_a_busy_serving_loop():
+    """Another context's resident loop keeps the device busy with one long query;
+    contexts that have read runs are closed meanwhile without waiting for it."""
+    import time
+
+    g = I.random_small_graph(6000, 60000, seed=51, wmax=50, dangling=60)
+    one = ppr.Context(0)
+    G = one.load_graph(g.n, g.row_ptr, g.col, g.w)
+    used = []
+    for _ in range(3):
+        c = ppr.Context(0)
+        H = c.load_graph(g.n, g.row_ptr, g.col, g.w)
+        H.run(alpha=0.2, R=8, src_end=10).free()
+        H.free()
+        used.append(c)
+    one.serve_start(G)
+    try:
+        q = one.submit(np.array([3], np.int32), alpha=2e-5, R=1000, seed=1, topk=4)  # walks of 50,000 steps
+        time.sleep(0.01)
+        t0 = time.perf_counter()
+        for c in used:
+            c.close()
+        closed = time.perf_counter() - t0
+        one.poll(q, 1, 4, timeout_ms=60000)
+        answered = time.perf_counter() - t0
+        assert answered > 0.05 and closed < 0.2 * answered
+    finally:
+        one.serve_stop()
