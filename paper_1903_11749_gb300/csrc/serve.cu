@@ -66,7 +66,7 @@ constexpr int kLoopWarps = 8;        // per block: kLoopWarps - 1 walker warps, 
 constexpr int kLoopBlocks = 8;       // per SM at most
 constexpr uint32_t kLoopMaxR = 1024; // largest R the loop's reduction takes
 constexpr uint64_t kSlotWaitNs = 1000000000ull;   // bound on the wait for a published descriptor
-constexpr uint64_t kBusyWaitNs = 120000000000ull;  // bound on waiting for queries in flight without one finishing
+constexpr uint64_t kBusyWaitNs = 120000000000ull;  // bound on waiting for queries in flight without a source reduced
 
 // Descriptor of a published query (device memory; the host writes it, then
 // publishes).  seq1 = the query's sequence number + 1 (0: never written).
@@ -577,8 +577,8 @@ __device__ __forceinline__ int walk_until_idle(const LoopParams &P, const ClassT
 // How long a warp has been without work (shared memory: the walking state
 // leaves no registers for it).
 struct WarpWait {
-    uint64_t idle_t0, busy_t0;  // since when nothing was in flight, since when no query in flight finished (0: from now)
-    unsigned long long seen;    // queries finished by busy_t0
+    uint64_t idle_t0, busy_t0;  // since when nothing was in flight, since when none of it was reduced (0: from now)
+    unsigned long long seen;    // sources reduced by busy_t0
     unsigned long long looked;  // queries ready to reduce when a look found no source left
     uint32_t backoff;           // ns of the next sleep
 };
@@ -588,13 +588,14 @@ __device__ __forceinline__ void worked(WarpWait &w)
     w.backoff = 256;
 }
 
-// Lane 0: whether no published query has finished for kBusyWaitNs.
-__device__ __forceinline__ bool stalled(uint64_t t, unsigned long long finished, WarpWait &w)
+// Lane 0: whether no source of the queries in flight has been reduced for kBusyWaitNs.
+__device__ __forceinline__ bool stalled(const LoopParams &P, uint64_t t, WarpWait &w)
 {
     w.idle_t0 = 0;
-    if (w.busy_t0 == 0 || finished != w.seen) {
+    const unsigned long long reduced = __ldcg(&P.glob->reduced);
+    if (w.busy_t0 == 0 || reduced != w.seen) {
         w.busy_t0 = t;
-        w.seen = finished;
+        w.seen = reduced;
         return false;
     }
     return t - w.busy_t0 > kBusyWaitNs;
@@ -618,7 +619,7 @@ __device__ __noinline__ uint32_t walker_leaves(const LoopParams &P, WarpWait &w,
     const uint64_t t = gtime_ns();
     const unsigned long long finished = __ldcg(&P.glob->finished);
     if (finished < *(volatile unsigned long long *)&s_tail[0])
-        return stalled(t, finished, w) ? PPR_LOOP_BUSY_TIMEOUT : 0;
+        return stalled(P, t, w) ? PPR_LOOP_BUSY_TIMEOUT : 0;
     if (!idled(t, P.idle_ns, w)) return 0;
     const unsigned long long tail = ld_tail(&P.ctl->tail);
     if (tail == finished) return PPR_LOOP_IDLE;
@@ -903,7 +904,7 @@ __device__ void aggregator_warp(const LoopParams &P, const CallerIds &ids, uint3
                 else if (left == 0 && (gone || idle)) why = PPR_LOOP_IDLE;
             } else if (gone) {  // no warp is left to walk what is in flight: the next launch does
                 why = PPR_LOOP_IDLE;
-            } else if (stalled(t, __ldcg(&P.glob->finished), wait)) {
+            } else if (stalled(P, t, wait)) {
                 why = PPR_LOOP_BUSY_TIMEOUT;
             } else {
                 why = ld_volatile(&P.ctl->status) & (PPR_LOOP_SLOT_TIMEOUT | PPR_LOOP_BUSY_TIMEOUT);
