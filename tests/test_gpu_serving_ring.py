@@ -16,16 +16,23 @@ RS = [1, 2, 31, 33, 64, 100, 128, 129, 200, 256, 257, 1000, 1024]
 
 
 @pytest.fixture(scope="module")
-def graph():
-    g = I.random_small_graph(6000, 60000, seed=51, wmax=50, dangling=60)
+def graphs():
+    """The same edges with 32-bit and with 64-bit row totals."""
     ctx = ppr.Context(0)
-    return ctx, ctx.load_graph(g.n, g.row_ptr, g.col, g.w)
+    loaded = [I.random_small_graph(6000, 60000, seed=51, wmax=wmax, dangling=60) for wmax in (50, 1 << 31)]
+    return ctx, [ctx.load_graph(g.n, g.row_ptr, g.col, g.w) for g in loaded]
+
+
+@pytest.fixture(scope="module")
+def graph(graphs):
+    return graphs[0], graphs[1][0]
 
 
 @pytest.mark.parametrize("smax,count", [(8, 600), (700, 200)])
-@pytest.mark.parametrize("sampler", [0, 1])
-def test_slots_reused_within_a_burst(graph, smax, count, sampler):
-    ctx, G = graph
+@pytest.mark.parametrize("wide,sampler", [(0, 0), (0, 1), (1, 0)])
+def test_slots_reused_within_a_burst(graphs, smax, count, wide, sampler):
+    ctx, G = graphs[0], graphs[1][wide]
+    assert G.info().wide == wide
     want = {R: G.run(alpha=0.15, R=R, seed=R, topk=8, sampler=sampler).topk() for R in RS}
     rng = np.random.default_rng(7)
     qs = [(RS[i % len(RS)], rng.integers(0, 6000, int(rng.integers(1, smax + 1))).astype(np.int32))
