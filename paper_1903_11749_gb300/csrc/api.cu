@@ -216,7 +216,8 @@ static int take_words()
 {
     std::lock_guard<std::mutex> lock(g_words.mu);
     for (int i = 0; i < g_words.n_late;) {
-        if (cudaEventQuery(g_words.late[i].done) == cudaErrorNotReady) {
+        if (cudaEventQuery(g_words.late[i].done) != cudaSuccess) {  // not ready, or not to be asked (a capture elsewhere)
+            cudaGetLastError();
             ++i;
             continue;
         }
@@ -523,7 +524,7 @@ static void result_release(ppr_result *r)
     if (r->words >= 0) {  // not waited for: the words are free when the run has written them
         std::lock_guard<std::mutex> lock(g_words.mu);
         if (!r->ev_counts) cudaStreamSynchronize(r->stream);  // (a launch that failed half way)
-        if (!r->ev_counts || cudaEventQuery(r->ev_counts) != cudaErrorNotReady) {
+        if (!r->ev_counts || cudaEventQuery(r->ev_counts) == cudaSuccess) {
             g_words.free[g_words.n_free++] = r->words;
         } else {
             g_words.late[g_words.n_late++] = {r->ev_counts, r->words};
@@ -770,9 +771,14 @@ static int run_common(ppr_ctx *ctx, const ppr_graph *g, const ppr_run_args *a, c
         k_publish<<<1, 32, 0, st>>>(r->d_steps, g_words.dev + kWords * r->words);
         note_launch();
         e = cudaGetLastError();
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&r->ev_counts, cudaEventDisableTiming);
-        if (e == cudaSuccess) e = cudaEventRecord(r->ev_counts, st);
-        if (e != cudaSuccess) return fail(cuda_fail(e, "counters"));
+        cudaEvent_t ev = nullptr;
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+        if (e == cudaSuccess) e = cudaEventRecord(ev, st);
+        if (e != cudaSuccess) {
+            if (ev) cudaEventDestroy(ev);
+            return fail(cuda_fail(e, "counters"));
+        }
+        r->ev_counts = ev;
     }
     *out = r;
     return PPR_OK;
