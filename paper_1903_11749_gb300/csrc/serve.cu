@@ -746,14 +746,15 @@ __device__ __noinline__ int claim_source(const LoopParams &P, uint32_t start, un
         if (lane == 0) r = await_slot(P, &P.slot[(h + ui) % kRing].agg, h + ui);
         return __shfl_sync(0xffffffffu, r, 0) < 0 ? -1 : 0;
     }
-    // Every other warp takes of the oldest ready query, the rest share themselves
-    // out over all of them.  With the oldest first for all, small queries wait
-    // for the reductions of large ones published before them (64 queries of up
-    // to 20,000 sources, R 200: half of them answered within 5.6 ms, now .74);
-    // with all shared out, large ones finish together and the host copies
-    // nothing meanwhile (the whole burst 14.1 ms, now 12.7, oldest first 12.3).
+    // Three warps of four take of the oldest ready query, the fourth ones share
+    // themselves out over all of them.  With the oldest first for all, small
+    // queries wait for the reductions of large ones published before them (64
+    // queries of up to 20,000 sources, R 200: half of them answered within 5.6
+    // ms, now .82; every other warp .74).  With all shared out, large ones finish
+    // together and the host copies nothing meanwhile (the whole burst 14.1 ms;
+    // every other warp 12.65, one of four 12.24, oldest first 12.28).
     unsigned long long m = ready;
-    for (uint32_t k = m && (start & 1) ? (start >> 1) % (uint32_t)__popcll(m) : 0u; k > 0; --k) m &= m - 1;
+    for (uint32_t k = m && (start & 3) == 3 ? (start >> 2) % (uint32_t)__popcll(m) : 0u; k > 0; --k) m &= m - 1;
     const unsigned long long before = ready ^ m;
     for (int pass = 0; pass < 2; ++pass, m = before) {
         while (m) {
